@@ -1,6 +1,6 @@
 // Decode attention over the packed cache (Algorithm 2 lines 3 and 5; Eq. 2; Eq. 3; Section 4.4).
 //
-// Three launches on the caller's stream:
+// Two launches on the caller's stream:
 //   1. decode_prep_kernel   q' = T_K^{-T} q per query head (Algorithm 2 line 3), written as mma
 //                           B-fragments: for the quantized positions a 16-bit fixed-point copy of q' split
 //                           into two signed bytes per channel (the operand of the integer mma), for the
@@ -19,10 +19,11 @@
 //                               o        = sum_s (p_s Delta_v,s) c_v,s + (sum_s p_s x_min_v,s) 1.
 //                           Window units use ldmatrix + bf16 mma on the staged rows and fold into the
 //                           same accumulators.  Softmax is online (running max / sum) per warp; a warp
-//                           writes one partial (max, sum, o) per (sequence, KV head) it touched.
-//   3. decode_combine_kernel merges the partials of each (sequence, query head) into O.
+//                           writes the outputs of a (sequence, KV head) that lies inside its slice, and one
+//                           partial (max, sum, o) of one that it shares; the CTA's partials are merged when
+//                           its warps are done, the CTAs' by whichever of them arrives last.
 //
-// No kernel waits on another CTA.  The only waits are on a warp's own copy barriers, bounded by an
+// No CTA waits on another.  The only waits are on a warp's own copy barriers, bounded by an
 // iteration limit after which the kernel records WUSHKV_DEV_COPY_TIMEOUT and drains.
 //
 // Data that an earlier kernel of the same step may still be writing while a later one is already
@@ -223,6 +224,8 @@ __global__ void __launch_bounds__(PREP_THREADS) decode_prep_kernel(DecodeParams 
         }
         if (i == 0) P.plan[0] = 0;
     }
+    // arrival counters of this head's queries for the main kernel's merge: the third word of a partial record
+    if (i < G) P.part[((static_cast<long long>(b) * P.c.n_kv + h) * G + i) * PART_STRIDE + 2] = 0.f;
     if (i >= 128) return;                 // the fragment stage has one thread per channel
     float acc[8];
 #pragma unroll
@@ -485,9 +488,10 @@ struct WarpState {
     }
 };
 
-// Writes this warp's partial (max, sum, o[128]) of every head of one (sequence, KV head) to global memory.
-template <int BITS, int MODE>
-__device__ __forceinline__ void store_partial(const WarpState<MODE>& st, float* dst0, int lane, int G) {
+// Writes this warp's state of every query head of one (sequence, KV head) to global memory: a partial (max, sum, o[128]) in
+// records PART_STRIDE floats apart, or, WHOLE, the head's outputs o / sum in rows of D floats.
+template <int BITS, int MODE, bool WHOLE>
+__device__ __forceinline__ void store_state(const WarpState<MODE>& st, float* dst0, int lane, int G) {
     const int g = lane >> 2, t = lane & 3;
     constexpr int NH = WarpState<MODE>::NH;
 #pragma unroll
@@ -498,8 +502,11 @@ __device__ __forceinline__ void store_partial(const WarpState<MODE>& st, float* 
         l += __shfl_xor_sync(FULL, l, 16); z += __shfl_xor_sync(FULL, z, 16);
         const int head = MODE == 0 ? t : 2 * t + k;
         if (head < G) {
-            float* dst = dst0 + head * PART_STRIDE;
-            if (g == 0) { dst[0] = st.m[k]; dst[1] = l; }
+            float* dst = dst0 + head * (WHOLE ? D : PART_STRIDE);
+            if (!WHOLE) {
+                if (g == 0) { dst[0] = st.m[k]; dst[1] = l; }
+                dst += 4;
+            }
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
                 const float osc = exp2f(static_cast<float>(24 - field_shift<BITS>(i)));
@@ -511,8 +518,12 @@ __device__ __forceinline__ void store_partial(const WarpState<MODE>& st, float* 
                     lo_ch = st.o[i][k] * osc + z;
                     hi_ch = st.o[i][2 + k] * osc + z;
                 }
-                dst[4 + 16 * i + g] = lo_ch;
-                dst[4 + 16 * i + g + 8] = hi_ch;
+                if (WHOLE) {
+                    lo_ch = l > 0.f ? lo_ch / l : 0.f;
+                    hi_ch = l > 0.f ? hi_ch / l : 0.f;
+                }
+                dst[16 * i + g] = lo_ch;
+                dst[16 * i + g + 8] = hi_ch;
             }
         }
     }
@@ -572,8 +583,126 @@ __device__ __forceinline__ void window_unit(WarpState<MODE>& st, unsigned rec, i
 // units of WIN_TOKENS tokens.
 struct Segment {
     int b, h, slot, u0, u1, qp, first_page, q_lo, q_hi, n_win, n_sink, recent_lo;
+    long long head_first;                 // flattened index of the head's unit 0
 };
 constexpr int MAX_SEGMENTS = 6;           // per warp and round; more segments take further rounds
+
+// A (sequence, KV head) whose units are shared by several warps: its index, its first unit in the flattened list, its units.
+struct SharedHead {
+    int bh, n_units;
+    long long first;
+    const float* rec;                     // the warp's partials of the head's queries, in shared or global memory
+};
+// The warp whose slice [w total / ns, (w + 1) total / ns) holds unit u.
+__device__ __noinline__ int wide_quotient(long long a, long long b) { return static_cast<int>(a / b); }
+__device__ __forceinline__ int slice_owner(long long u, long long total, int ns) {
+    const long long x = (u + 1) * ns - 1;
+    if (x < (1LL << 32) && total < (1LL << 32)) return static_cast<int>(static_cast<unsigned>(x) / static_cast<unsigned>(total));
+    return wide_quotient(x, total);
+}
+// Merge of partial states (max, sum, o) of one query head by one warp: lane L holds channels 4L .. 4L+3.  The tail of the
+// kernel is a chain of latencies, so the rows of a batch and their maxima and sums are all requested together.
+constexpr int MERGE_BATCH = 8;
+struct MergedState {
+    float m, l;
+    float4 o;
+    __device__ __forceinline__ void reset() { m = -INFINITY; l = 0.f; o = make_float4(0.f, 0.f, 0.f, 0.f); }
+    // Adds n partials; next() returns the address of the next one.
+    template <class Next>
+    __device__ __forceinline__ void add(int n, int lane, Next next) {
+        for (int k = 0; k < n; k += MERGE_BATCH) {
+            float4 v[MERGE_BATCH];
+            float2 ml[MERGE_BATCH];
+            float mn = m;
+#pragma unroll
+            for (int e = 0; e < MERGE_BATCH; ++e) {
+                v[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+                ml[e] = make_float2(-INFINITY, 0.f);
+                if (k + e < n) {
+                    const float* rec = next();
+                    ml[e] = *reinterpret_cast<const float2*>(rec);
+                    v[e] = *(reinterpret_cast<const float4*>(rec + 4) + lane);
+                }
+            }
+#pragma unroll
+            for (int e = 0; e < MERGE_BATCH; ++e) mn = fmaxf(mn, ml[e].x);
+            if (mn == -INFINITY) continue;                       // nothing but empty partials so far
+            const float keep = ex2(m - mn);
+            l *= keep;
+            o.x *= keep; o.y *= keep; o.z *= keep; o.w *= keep;
+            m = mn;
+#pragma unroll
+            for (int e = 0; e < MERGE_BATCH; ++e) {
+                if (ml[e].x == -INFINITY) continue;
+                const float f = ex2(ml[e].x - mn);
+                l = fmaf(ml[e].y, f, l);
+                o.x = fmaf(v[e].x, f, o.x); o.y = fmaf(v[e].y, f, o.y);
+                o.z = fmaf(v[e].z, f, o.z); o.w = fmaf(v[e].w, f, o.w);
+            }
+        }
+    }
+    __device__ __forceinline__ void store(float* rec, int lane) const {
+        if (lane == 0) *reinterpret_cast<float2*>(rec) = make_float2(m, l);
+        reinterpret_cast<float4*>(rec + 4)[lane] = o;
+    }
+    __device__ __forceinline__ void finish(float* out, int lane) const {
+        const bool any = l > 0.f;
+        reinterpret_cast<float4*>(out)[lane] = any ? make_float4(o.x / l, o.y / l, o.z / l, o.w / l) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+};
+
+// Merge of the heads that several warps share, at the end of the main kernel.  First the shares of this CTA's warps (at most one
+// per warp) are merged, one warp per (head, query head).  Then the CTA that arrives last at the query head's counter merges
+// the CTAs' states, in CTA order, and writes the output: no CTA waits for another, and the result does not depend on which
+// one is last.
+template <int MAIN_WARPS>
+__device__ __forceinline__ void merge_shared_heads(const DecodeParams& P, const SharedHead* shared_s, const long long total) {
+    const CacheView& c = P.c;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, G = c.G;
+    const int my_bh = lane < 2 * MAIN_WARPS ? shared_s[lane].bh : -1;
+    const unsigned slots_of = __match_any_sync(FULL, my_bh);
+    const unsigned leaders = __ballot_sync(FULL, my_bh >= 0 && lane == __ffs(slots_of) - 1);
+    const int n_items = __popc(leaders) * G;
+    for (int item = warp; item < n_items; item += MAIN_WARPS) {
+        unsigned rest = leaders;
+        for (int k = item / G; k > 0; --k) rest &= rest - 1;
+        const int leader = __ffs(rest) - 1, head = item % G;
+        unsigned slots = __shfl_sync(FULL, slots_of, leader);
+        const SharedHead hd = shared_s[leader];
+        const int cta_warp0 = blockIdx.x * MAIN_WARPS;
+        float* rec0 = P.part + (static_cast<long long>(hd.bh) * G + head) * PART_STRIDE;     // the head's record of warp 0
+        const long long rec_step = static_cast<long long>(G) * PART_STRIDE;
+        MergedState ms;
+        ms.reset();
+        ms.add(__popc(slots), lane, [&] {
+            const float* rec = shared_s[__ffs(slots) - 1].rec + head * PART_STRIDE;
+            slots &= slots - 1;
+            return rec;
+        });
+        // The CTAs that share the head: all from the one that owns its first unit to the one that owns its last, or, when there
+        // are more CTAs than units, the owner of each unit.  A CTA's state is at the warp that owns its first unit of the head.
+        const bool every_cta = total >= gridDim.x, every_warp = total >= P.n_warps;
+        const int w_first = slice_owner(hd.first, total, P.n_warps), c_first = w_first / MAIN_WARPS;
+        const int n_ctas = every_cta ? slice_owner(hd.first + hd.n_units - 1, total, P.n_warps) / MAIN_WARPS - c_first + 1 : hd.n_units;
+        if (n_ctas > 1) {
+            ms.store(rec0 + (cta_warp0 + (leader >> 1)) * rec_step, lane);
+            __syncwarp();
+            int before = 0;                                          // the counter: a record's unused word, zeroed by the preparation kernel
+            if (lane == 0) asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(before) : "l"(rec0 + 2) : "memory");
+            if (__shfl_sync(FULL, before, 0) != n_ctas - 1) continue;
+            ms.reset();
+            int k = 0;
+            ms.add(n_ctas, lane, [&] {
+                int w = max(w_first, (c_first + k) * MAIN_WARPS);
+                if (!every_warp) w = slice_owner(every_cta ? max(hd.first, static_cast<long long>(c_first + k) * MAIN_WARPS * total / P.n_warps) : hd.first + k, total, P.n_warps);
+                ++k;
+                return rec0 + w * rec_step;
+            });
+        }
+        float* out = P.O + (static_cast<long long>(hd.bh / c.n_kv) * c.n_q + (hd.bh % c.n_kv) * G + head) * D;
+        ms.finish(out, lane);
+    }
+}
 
 // ------------------------------------------------------------------------------------------------
 // main kernel
@@ -656,9 +785,15 @@ __global__ void __launch_bounds__(main_warps(BITS, MODE) * 32, 1) decode_main_ke
         sh = static_cast<int>(rem / U);
         su = static_cast<int>(rem % U);
     }
+    for (int b = blockIdx.x; b < P.batch; b += gridDim.x)      // a sequence without units gets zeros
+        if (plan[b + 1] == plan[b])
+            for (int k = threadIdx.x; k < c.n_q * D; k += MAIN_WARPS * 32) P.O[static_cast<long long>(b) * c.n_q * D + k] = 0.f;
+    __shared__ SharedHead shared_s[2 * MAIN_WARPS];             // [2 warp]: head the warp entered in its middle, [2 warp + 1]: head it left unfinished
+    __shared__ long long total_s;           // kept for the merge at the end
+    if (threadIdx.x < 2 * MAIN_WARPS) shared_s[threadIdx.x].bh = -1;
+    if (threadIdx.x == 0) total_s = total;
     __syncthreads();                        // the staging area stops being plan scratch here
     pdl_launch_dependents();
-    if (L >= L1) return;
 
     // ---- barriers
     const unsigned bar0 = smem_u32(bars + warp * STAGES);
@@ -683,7 +818,7 @@ __global__ void __launch_bounds__(main_warps(BITS, MODE) * 32, 1) decode_main_ke
     bool timed_out = false;
     const int wait_limit = P.wait_limit > 0 ? P.wait_limit : (1 << 19);      // polls that may sleep ~2 us each: about a second
 
-    while (L < L1 && !timed_out) {
+    while (L < L1) {
         // ================= round set-up: list the next segments of the slice =====================
         int n_seg = 0, round_units = 0;
         while (n_seg < MAX_SEGMENTS && L < L1) {
@@ -694,6 +829,7 @@ __global__ void __launch_bounds__(main_warps(BITS, MODE) * 32, 1) decode_main_ke
                     Segment sg;
                     sg.b = sb; sg.h = sh; sg.slot = si.slot; sg.u0 = su; sg.u1 = u1; sg.qp = si.qp; sg.first_page = si.first_page;
                     sg.q_lo = si.q_lo; sg.q_hi = si.q_hi; sg.n_win = si.n_win; sg.n_sink = si.n_sink; sg.recent_lo = si.recent_lo;
+                    sg.head_first = L - su;
                     segs[n_seg] = sg;
                 }
                 ++n_seg;
@@ -763,12 +899,12 @@ __global__ void __launch_bounds__(main_warps(BITS, MODE) * 32, 1) decode_main_ke
             ++p_u;
             ++issued;
         };
-        for (int k = 0; k < STAGES && k < round_units; ++k) issue_next((stage + k) % STAGES);
+        for (int k = 0; k < STAGES && k < round_units && !timed_out; ++k) issue_next((stage + k) % STAGES);
         TL(1);
 
         // ================= consumer ==============================================================
         pdl_wait();                                     // query fragments come from the preparation kernel
-        for (int cs = 0; cs < n_seg && !timed_out; ++cs) {
+        for (int cs = 0; cs < n_seg; ++cs) {
             const Segment& sg = segs[cs];               // rarely used fields are re-read from shared memory
             const long long bh = static_cast<long long>(sg.b) * c.n_kv + sg.h;
             const int u1 = sg.u1, qp = sg.qp, q_lo = sg.q_lo, q_hi = sg.q_hi;
@@ -795,10 +931,19 @@ __global__ void __launch_bounds__(main_warps(BITS, MODE) * 32, 1) decode_main_ke
                 }
                 st.reset();
             }
-            for (int u = sg.u0; u < u1; ++u, pos0 += PAGE_TOKENS) {
+            for (int u = sg.u0; u < u1 && !timed_out; ++u, pos0 += PAGE_TOKENS) {
                 const int s = stage;
                 // a phase that one lane saw complete is complete for all: keep the decision warp-uniform
-                if (!__any_sync(FULL, mbar_wait_bounded(bar0 + 8 * s, (phase_bits >> s) & 1u, wait_limit))) { timed_out = true; break; }
+                if (!__any_sync(FULL, mbar_wait_bounded(bar0 + 8 * s, (phase_bits >> s) & 1u, wait_limit))) {
+                    timed_out = true;
+                    if (lane == 0) atomicOr(c.dev_status, WUSHKV_DEV_COPY_TIMEOUT);
+                    // Copies of this warp's other stages may still be in flight: wait for each (bounded; a stage with nothing
+                    // pending simply runs the limit out) before its shared memory is used for anything else or released.
+                    const int drain_limit = min(wait_limit, 1 << 9);
+#pragma unroll
+                    for (int k = 0; k < STAGES; ++k) mbar_wait_bounded(bar0 + 8 * k, (phase_bits >> k) & 1u, drain_limit);
+                    break;
+                }
                 phase_bits ^= 1u << s;
 #if WUSHKV_ABL & 16
                 if (lane == 0 && g_timeline[((blockIdx.x * 16 + warp) & 8191) * 4 + 2] == 0) g_timeline[((blockIdx.x * 16 + warp) & 8191) * 4 + 2] = gtime();
@@ -981,107 +1126,31 @@ __global__ void __launch_bounds__(main_warps(BITS, MODE) * 32, 1) decode_main_ke
                 if (issued < round_units) issue_next(s);         // refill the stage just consumed
                 stage = (stage + 1 == STAGES) ? 0 : stage + 1;
             }
-            store_partial<BITS, MODE>(st, P.part + (wg + static_cast<long long>(sg.b) * c.n_kv + sg.h) * G * PART_STRIDE, lane, G);
+            // A head that lies inside this warp's slice is finished here.  One that is shared leaves a partial result (after a
+            // wait that ran out: of what was read until then, so that whoever merges the head still finds every share): in
+            // the warp's ring if that has served its last unit, else in global memory.
+            const int U = qp + (sg.n_win + WIN_TOKENS - 1) / WIN_TOKENS;
+            if (sg.u0 == 0 && u1 == U) {
+                store_state<BITS, MODE, true>(st, P.O + (static_cast<long long>(sg.b) * c.n_q + sg.h * G) * D, lane, G);
+            } else {
+                static_assert(8 * PART_STRIDE * 4 <= STAGES * REC, "the partials of 8 query heads must fit in a warp's ring");
+                const bool last = cs == n_seg - 1 && L >= L1;
+                float* rec = last ? reinterpret_cast<float*>(smem + warp * STAGES * REC) : P.part + (wg + bh) * G * PART_STRIDE;
+                if (last) __syncwarp();                      // every lane has read the last unit
+                store_state<BITS, MODE, false>(st, rec, lane, G);
+                if (lane == 0) {
+                    SharedHead& hd = shared_s[2 * warp + (sg.u0 == 0 ? 1 : 0)];
+                    hd.bh = static_cast<int>(bh); hd.n_units = U; hd.first = sg.head_first; hd.rec = rec;
+                }
+            }
         }
         __syncwarp();
     }
     TL(3);
-    if (timed_out) {
-        if (lane == 0) atomicOr(c.dev_status, WUSHKV_DEV_COPY_TIMEOUT);
-        // Copies of this warp's other stages may still be in flight: wait for each (bounded; a stage with nothing
-        // pending simply runs the limit out) before the CTA's shared memory can be released.
-        const int drain_limit = min(wait_limit, 1 << 9);
-#pragma unroll
-        for (int s = 0; s < STAGES; ++s) mbar_wait_bounded(bar0 + 8 * s, (phase_bits >> s) & 1u, drain_limit);
-    }
-}
-
-// ------------------------------------------------------------------------------------------------
-// 3. combine
-// ------------------------------------------------------------------------------------------------
-// One CTA per (sequence, query head): up to 8 thread groups of one thread per channel, each merging a
-// contiguous share of the head's partials.  The partials sit in L2, so the cost is load latency: a
-// group issues the loads of COMBINE_BATCH partials together before it merges them.
-constexpr int COMBINE_BATCH = 8;        // loads in flight per thread
-template <int MAX_GROUPS, int GS>      // GS: log2 of the warps per slice (compile-time copy of slice_shift)
-__global__ void __launch_bounds__(128 * MAX_GROUPS) decode_combine_kernel(DecodeParams P) {
-    __shared__ float red_m[MAX_GROUPS], red_l[MAX_GROUPS], red_o[MAX_GROUPS][D];
-    const CacheView& c = P.c;
-    const int j = blockIdx.x, b = blockIdx.y, ch = threadIdx.x, grp = threadIdx.y, n_grp = blockDim.y;
-    pdl_wait();                                         // partials and the plan come from the earlier kernels
-    pdl_launch_dependents();                            // a programmatically launched successor waits for us itself
-    float* out = P.O + (static_cast<long long>(b) * c.n_q + j) * D;
-    const long long U = P.plan[b + 1] - P.plan[b];
-    const long long total = P.plan[P.batch] * c.n_kv;
-    if (U <= 0 || total <= 0) { if (grp == 0) out[ch] = 0.f; return; }
-    const int h = j / c.G, head = j % c.G;
-    const long long La = P.plan[b] * c.n_kv + static_cast<long long>(h) * U, Lb = La + U;      // units [La, Lb)
-    // The unit list is cut into ns equal slices, slice i = [floor(i total / ns), floor((i+1) total / ns)); a
-    // slice belongs to one warp (slice_shift 0) or to the four warps of a CTA (slice_shift 2), and every
-    // warp of a slice that meets [La, Lb) wrote a partial, at slot (slice + bh) * warps_per_slice + warp.
-    constexpr int gs = GS, group_mask = (1 << gs) - 1;
-    const long long ns = static_cast<long long>(P.n_warps) >> gs;
-    const long long s_first = ((La + 1) * ns - 1) / total, s_last = (Lb * ns - 1) / total;   // owners of La and Lb-1
-    const long long bh = static_cast<long long>(b) * c.n_kv + h;
-    const long long stride = static_cast<long long>(c.G) * PART_STRIDE;
-    const int n = static_cast<int>(s_last - s_first + 1) << gs;
-    // thread group grp merges the contiguous share [k0, k1) of the n partials
-    const int share = (n + n_grp - 1) / n_grp;
-    const int k0 = min(grp * share, n), k1 = min(k0 + share, n);
-    const float* base = P.part + ((((s_first + bh) << gs) + k0) * c.G + head) * PART_STRIDE;
-    // slice bounds advance by q = total / ns with a carry of r = total % ns (no division in the loop)
-    const long long q = total / ns, r = total % ns;
-    const long long sl0 = s_first + (k0 >> gs);
-    long long lo_w = sl0 * total / ns, rem = (sl0 * total) % ns;
-    long long hi_w = lo_w + q;
-    rem += r;
-    if (rem >= ns) { rem -= ns; ++hi_w; }
-    float m = -INFINITY, l = 0.f, o = 0.f;
-    for (int s0 = k0; s0 < k1; s0 += COMBINE_BATCH) {
-        float pm[COMBINE_BATCH], pl[COMBINE_BATCH], po[COMBINE_BATCH];
-#pragma unroll
-        for (int k = 0; k < COMBINE_BATCH; ++k) {
-            pm[k] = -INFINITY; pl[k] = 0.f; po[k] = 0.f;
-            if (s0 + k < k1) {
-                const bool wrote = max(lo_w, La) < min(hi_w, Lb);     // a slice that misses the range wrote nothing
-                if (((s0 + k + 1) & group_mask) == 0) {               // next partial belongs to the next slice
-                    lo_w = hi_w;
-                    hi_w = lo_w + q;
-                    rem += r;
-                    if (rem >= ns) { rem -= ns; ++hi_w; }
-                }
-                if (wrote) {
-                    const float* p = base + (s0 - k0 + k) * stride;
-                    pm[k] = __ldcg(p); pl[k] = __ldcg(p + 1); po[k] = __ldcg(p + 4 + ch);
-                }
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < COMBINE_BATCH; ++k) {
-            if (pm[k] == -INFINITY) continue;
-            const float mn = fmaxf(m, pm[k]);
-            const float sa = exp2f(m - mn), sb = exp2f(pm[k] - mn);   // m = -inf on the first partial: sa = 0
-            l = l * sa + pl[k] * sb;
-            o = o * sa + po[k] * sb;
-            m = mn;
-        }
-    }
-    if (MAX_GROUPS > 1 && n_grp > 1) {                  // merge the groups' states, in group order
-        if (ch == 0) { red_m[grp] = m; red_l[grp] = l; }
-        red_o[grp][ch] = o;
-        __syncthreads();
-        if (grp != 0) return;
-        for (int k = 1; k < n_grp; ++k) {
-            const float pm = red_m[k];
-            if (pm == -INFINITY) continue;
-            const float mn = fmaxf(m, pm);
-            const float sa = exp2f(m - mn), sb = exp2f(pm - mn);
-            l = l * sa + red_l[k] * sb;
-            o = o * sa + red_o[k][ch] * sb;
-            m = mn;
-        }
-    }
-    out[ch] = l > 0.f ? o / l : 0.f;
+    // ---- heads that several warps share
+    pdl_wait();                             // warps without units: the counters were zeroed by the preparation kernel
+    __syncthreads();
+    merge_shared_heads<MAIN_WARPS>(P, shared_s, total_s);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1148,19 +1217,6 @@ static int launch_decode(const DecodeParams& P, int n_ctas, cudaStream_t st) {
     cfg.dynamicSmemBytes = SMEM;
     if (cudaLaunchKernelEx(&cfg, decode_main_kernel<BITS, MODE, STAGES>, P) != cudaSuccess) return WUSHKV_ECUDA;
     if (g_prof_stop) cudaEventRecord(g_prof_stop, st);
-    // Partials per (sequence, KV head) are about n_warps / (batch n_kv).  Short lists go to one thread
-    // group per CTA (a few rounds of COMBINE_BATCH loads); a long list (few sequences, long context)
-    // is shared by 8 groups.
-    const long long per_head = P.n_warps / (static_cast<long long>(P.batch) * P.c.n_kv) + 2;
-    cfg.gridDim = dim3(P.c.n_q, P.batch);
-    cfg.dynamicSmemBytes = 0;
-    if (per_head <= 4 * COMBINE_BATCH) {
-        cfg.blockDim = dim3(128, 1);
-        if (cudaLaunchKernelEx(&cfg, decode_combine_kernel<1, 0>, P) != cudaSuccess) return WUSHKV_ECUDA;
-    } else {
-        cfg.blockDim = dim3(128, 8);
-        if (cudaLaunchKernelEx(&cfg, decode_combine_kernel<8, 0>, P) != cudaSuccess) return WUSHKV_ECUDA;
-    }
     return WUSHKV_OK;
 }
 
