@@ -90,6 +90,10 @@ struct DecodeParams {
     Prologue pro;        // pro.rope != nullptr: Q holds projected queries, normalised and rotated by the preparation kernel
 };
 
+// Arrival counters of a (sequence, KV head)'s 8 query head slots for the main kernel's merge, zeroed by the preparation kernel:
+// in the unused half of the head's integer fragments.
+__device__ __forceinline__ int* arrival_counters(const DecodeParams& P, long long bh) { return reinterpret_cast<int*>(P.qfrag + bh * 256 + 128); }
+
 // shift of the code field used by k-step / channel block idx (0..7) inside its 16-bit lane, after
 // the optional whole-word shift: the fp16 value of the masked field is code * 2^(field_shift - 24)
 template <int BITS>
@@ -134,81 +138,83 @@ __device__ __forceinline__ SeqInfo seq_info(const CacheView& c, int S, int slot)
 // ------------------------------------------------------------------------------------------------
 constexpr int PREP_THREADS = 512;                   // 16 warps share the 128 rows of T_K^{-T}
 constexpr int PREP_ROWS = D / (PREP_THREADS / 32);   // rows per warp
+constexpr int MAX_LOCAL_PLAN = 8192;                 // sequences up to which every CTA of the main kernel computes the work plan itself
+// One CTA per (KV head, sequence).  What bounds it is latency and, as 16 warps share the SM's schedulers, the number of
+// instructions: the selections of a plain butterfly, shuffles for maxima that one reduction does, and byte stores of fragments
+// to global memory (now put together in shared memory and stored as 16-byte words) made it 5.4 us for 2 heads x 1 sequence, 8.2 us
+// for 8 x 16 and 10.4 us for 8 x 1 with 8 query heads each, now 3.7, 5.8 and 6.2 us.  Two or four sequences per CTA (which read
+// the 64 KB of T_K^{-T} once) ran 8 x 64 in 10.3 and 13.2 us against 11.5 us, but the step no faster: the CTAs then wait longer
+// for room beside the append's.
 template <int BITS, int MODE>
 __global__ void __launch_bounds__(PREP_THREADS) decode_prep_kernel(DecodeParams P) {
-    __shared__ float q_s[8][D];
+    constexpr int QF = MODE == 0 ? 64 : 128, QW = MODE == 0 ? 128 : 256;     // uint4 of a (sequence, head)'s integer / bf16 fragments
+    __shared__ uint4 buf[QF + QW > 256 ? QF + QW : 256];                     // the queries, later the fragments
+    __shared__ float qp_s[8][D];
     __shared__ float red_abs[8][4];
     __shared__ int red_isum[8][4];
     __shared__ long long scan_s[4];
+    float (*q_s)[D] = reinterpret_cast<float (*)[D]>(buf);
     const int h = blockIdx.x, b = blockIdx.y, G = P.c.G;
     const int i = threadIdx.x, lane = i & 31, warp = i >> 5;
     // Normally everything this kernel reads may come from the kernel ahead of it.  In the fused step
     // (q_early) that kernel is the single-token append, which started only after all earlier work had
-    // finished: Q is final already and only the lengths (for the work plan) have to wait for it, so the
-    // transform of the queries runs beside the append.  The main kernel reads the lengths and stages
-    // pages as soon as it starts, so the plan CTA holds its launch signal back until the append is done.
-    const bool plan_cta = h == 0 && b == 0;
+    // finished: Q is final already, so the transform of the queries runs beside the append; the main kernel, which
+    // needs the lengths, waits for this kernel, whose first CTA in turn ends after the append.
+    const bool first_cta = h == 0 && b == 0;
     if (!P.q_early) pdl_wait();
-    if (!(P.q_early && plan_cta)) pdl_launch_dependents();   // the main kernel may start staging pages while this one runs
+    pdl_launch_dependents();               // the main kernel may start (and, unless q_early, stage pages) while this one runs
 
-    for (int k = i; k < G * D; k += PREP_THREADS)
-        q_s[k >> 7][k & (D - 1)] = bf16_bits_to_float(P.Q[(static_cast<long long>(b) * P.c.n_q + h * G) * D + k]);
+    // q'[g][i] = sum_j T_invT[h][i][j] q[g][j].  Lane L holds columns 4L .. 4L+3; the 32 products of a pass are indexed
+    // k = row * GP + head (GP = 4 or 8 head slots), and slot i of lane L holds product i ^ L: rows and heads are read in
+    // that order, so that the butterfly over the lanes adds slot to slot without a selection and leaves total L in lane L.
+    constexpr int GP = MODE == 0 ? 4 : 8, PASS_ROWS = 32 / GP;      // MODE 0 serves G <= 4, MODE 1 serves G <= 8
+    const float4* Tbase = reinterpret_cast<const float4*>(P.c.T_K_invT + (static_cast<long long>(h) * D + warp * PREP_ROWS) * D) + lane;
+    float4 trow[PREP_ROWS];
+#pragma unroll
+    for (int r = 0; r < PREP_ROWS; ++r) trow[r] = __ldg(Tbase + ((r / PASS_ROWS) * PASS_ROWS + ((r % PASS_ROWS) ^ (lane / GP))) * (D / 4));
+    for (int k = i; k < GP * (D / 2); k += PREP_THREADS) {               // unused head slots are zero
+        const int g = k / (D / 2), c2 = 2 * (k % (D / 2));
+        const unsigned w = g < G ? *reinterpret_cast<const unsigned*>(P.Q + (static_cast<long long>(b) * P.c.n_q + h * G + g) * D + c2) : 0u;
+        *reinterpret_cast<float2*>(&q_s[g][c2]) = make_float2(bf16_bits_to_float(w & 0xffff), bf16_bits_to_float(w >> 16));
+    }
     __syncthreads();
     if (P.pro.rope) {                     // projected queries: Norm and RoPE at the newest position (Algorithm 2 lines 1-2)
         if (warp < G) {
-            const int S = __ldcg(P.seq_len + b);
-            float4* qv = reinterpret_cast<float4*>(&q_s[warp][0]) + lane;
-            const float4 v = *qv;
-            float x[4] = {v.x, v.y, v.z, v.w};
-            norm_rope_warp(x, lane, P.pro, h * G + warp, prologue_position(P.pro, max(S - 1, 0), P.c.dev_status, lane == 0 && S > P.pro.n_pos));
+            const int g = warp, S = __ldcg(P.seq_len + b);
+            float4* qv = reinterpret_cast<float4*>(&q_s[g][0]) + lane;
+            const float4 x4 = *qv;
+            float x[4] = {x4.x, x4.y, x4.z, x4.w};
+            norm_rope_warp(x, lane, P.pro, h * G + g, prologue_position(P.pro, max(S - 1, 0), P.c.dev_status, lane == 0 && S > P.pro.n_pos));
             *qv = make_float4(x[0], x[1], x[2], x[3]);
         }
         __syncthreads();
     }
-    // q'[g][i] = sum_j T_invT[h][i][j] q[g][j].  Each of the 16 warps takes 8 rows, all of their loads in
-    // flight together; a row is one coalesced 512-byte read (lane L holds columns 4L..4L+3); rows are
-    // handled 32/GP at a time so that the GP x rows partial sums fit a 32-value transposing butterfly
-    // (GP = 4 or 8 head slots).
-    __shared__ float qp_s[8][D];
     {
-        constexpr int GP = MODE == 0 ? 4 : 8;           // MODE 0 serves G <= 4, MODE 1 serves G <= 8
-        constexpr int rows_per = 32 / GP;
-        const float4* Tbase = reinterpret_cast<const float4*>(P.c.T_K_invT + (static_cast<long long>(h) * D + warp * PREP_ROWS) * D) + lane;
-        float4 qv[8];
+        float4 qv[GP];
 #pragma unroll
-        for (int g = 0; g < 8; ++g) qv[g] = g < G ? *reinterpret_cast<const float4*>(&q_s[g][4 * lane]) : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int g = 0; g < GP; ++g) qv[g] = *reinterpret_cast<const float4*>(&q_s[g ^ (lane % GP)][4 * lane]);
 #pragma unroll
-        for (int r0 = 0; r0 < PREP_ROWS; r0 += rows_per) {
+        for (int r0 = 0; r0 < PREP_ROWS; r0 += PASS_ROWS) {
             float part[32];
 #pragma unroll
-            for (int k = 0; k < 32; ++k) part[k] = 0.f;
-#pragma unroll
-            for (int rr = 0; rr < 32; ++rr) {            // slot k = rr * GP + g for rr < rows_per
-                if (rr < rows_per) {
-                    const float4 t = __ldg(Tbase + (r0 + rr) * (D / 4));
-#pragma unroll
-                    for (int g = 0; g < 8; ++g)
-                        if (g < GP && rr * GP + g < 32)
-                            part[(rr * GP + g) & 31] = fmaf(t.x, qv[g].x, fmaf(t.y, qv[g].y, fmaf(t.z, qv[g].z, t.w * qv[g].w)));
-                }
+            for (int k = 0; k < 32; ++k) {
+                const float4 t = trow[r0 + k / GP], q = qv[k % GP];
+                part[k] = fmaf(t.x, q.x, fmaf(t.y, q.y, fmaf(t.z, q.z, t.w * q.w)));
             }
-            const float tot = warp_transpose_reduce(part, lane);
-            const int rr = lane / GP, g = lane % GP;
-            if (g < G) qp_s[g][warp * PREP_ROWS + r0 + rr] = tot;
+#pragma unroll
+            for (int off = 16; off >= 1; off >>= 1)
+#pragma unroll
+                for (int k = 0; k < off; ++k) part[k] += __shfl_xor_sync(FULL, part[k + off], off);
+            if (lane % GP < G) qp_s[lane % GP][warp * PREP_ROWS + r0 + lane / GP] = part[0];
         }
     }
-    __syncthreads();
-    if (plan_cta) {                       // work plan: exclusive prefix of units per sequence
-        if (P.q_early) { pdl_wait(); pdl_launch_dependents(); }     // the lengths come from the append
+    if (P.batch > MAX_LOCAL_PLAN && first_cta) {       // work plan for the main kernel: exclusive prefix of units per sequence
+        if (P.q_early) pdl_wait();                      // the lengths come from the append
         long long carry = 0;
         for (int base = 0; base < P.batch; base += 128) {
             const int bb = base + i;
             long long u = 0;
-            if (i < 128 && bb < P.batch) {
-                const int slot = __ldg(P.slot + bb);
-                if (slot < 0 || slot >= P.c.n_slots) atomicOr(P.c.dev_status, WUSHKV_DEV_BAD_SLOT);
-                u = seq_info(P.c, __ldcg(P.seq_len + bb), slot).U;
-            }
+            if (i < 128 && bb < P.batch) u = seq_info(P.c, __ldcg(P.seq_len + bb), __ldg(P.slot + bb)).U;
             long long incl = u;
             for (int o = 1; o < 32; o <<= 1) {
                 const long long v = __shfl_up_sync(FULL, incl, o);
@@ -224,61 +230,50 @@ __global__ void __launch_bounds__(PREP_THREADS) decode_prep_kernel(DecodeParams 
         }
         if (i == 0) P.plan[0] = 0;
     }
-    // arrival counters of this head's queries for the main kernel's merge: the third word of a partial record
-    if (i < G) P.part[((static_cast<long long>(b) * P.c.n_kv + h) * G + i) * PART_STRIDE + 2] = 0.f;
-    if (i >= 128) return;                 // the fragment stage has one thread per channel
-    float acc[8];
+    __syncthreads();
+    if (i >= D) return;                    // the fragment stage has one thread per channel
+    const int ch = i;
+    const long long bh = static_cast<long long>(b) * P.c.n_kv + h;
+    if (ch < 8) arrival_counters(P, bh)[ch] = 0;
+    float acc[GP];
 #pragma unroll
-    for (int g = 0; g < 8; ++g) acc[g] = g < G ? qp_s[g][i] : 0.f;
+    for (int g = 0; g < GP; ++g) acc[g] = g < G ? qp_s[g][ch] : 0.f;
     const float k2 = P.c.sm_scale * LOG2E;
     // ---- 16-bit fixed point of q' per head: q'[ch] ~ lam * qi[ch], |qi| <= Q_MAX, qi = 256 hi + lo with both
     // digits signed bytes.  The scores of the quantized positions use exactly this rounded query
     // (code part and x_min part alike), so they are the scores of a slightly perturbed query, the same
     // for every position.
 #pragma unroll
-    for (int g = 0; g < 8; ++g) {
+    for (int g = 0; g < GP; ++g) {
         if (g < G) {
-            float ab = fabsf(acc[g]);
-            for (int o = 16; o > 0; o >>= 1) ab = fmaxf(ab, __shfl_xor_sync(FULL, ab, o));
-            if (lane == 0) red_abs[g][warp] = ab;
+            const unsigned ab = __reduce_max_sync(FULL, __float_as_uint(acc[g]) & 0x7fffffffu);     // magnitudes compare like their bits
+            if (lane == 0) red_abs[g][warp] = __uint_as_float(ab);
         }
     }
-    asm volatile("bar.sync 1, 128;" ::: "memory");       // the four remaining warps only
-    int qi[8];
-    float lam[8];
+    asm volatile("bar.sync 1, 128;" ::: "memory");                       // the four remaining warps
+    int qi[GP];
 #pragma unroll
-    for (int g = 0; g < 8; ++g) {
-        qi[g] = 0; lam[g] = 1.f;
+    for (int g = 0; g < GP; ++g) {
+        qi[g] = 0;
         if (g < G) {
-            const float amax = fmaxf(fmaxf(red_abs[g][0], red_abs[g][1]), fmaxf(red_abs[g][2], red_abs[g][3]));
-            if (amax > 0.f && amax < 3e38f) {
-                lam[g] = amax * (1.f / Q_MAX);
+            const float* ra = red_abs[g];
+            const float amax = fmaxf(fmaxf(ra[0], ra[1]), fmaxf(ra[2], ra[3]));
+            if (amax > 0.f && amax < 3e38f)
                 qi[g] = max(-static_cast<int>(Q_MAX), min(static_cast<int>(Q_MAX), __float2int_rn(acc[g] * (Q_MAX / amax))));
-            }
-            int sm = qi[g];
-            for (int o = 16; o > 0; o >>= 1) sm += __shfl_xor_sync(FULL, sm, o);
+            const int sm = __reduce_add_sync(FULL, qi[g]);
             if (lane == 0) red_isum[g][warp] = sm;
         }
-    }
-    asm volatile("bar.sync 1, 128;" ::: "memory");
-    if (i < G) {
-        const int sum = red_isum[i][0] + red_isum[i][1] + red_isum[i][2] + red_isum[i][3];
-        constexpr float FS = BITS != 4 ? 4.f : 16.f;      // the integer score carries this factor (see the main kernel)
-        float* qs = P.qscal + (static_cast<long long>(b) * P.c.n_q + h * G + i) * 2;
-        qs[0] = k2 * lam[i] * (1.f / FS);                 // score (log2 domain) = qs[0] * (Delta_k * sum_int + x_min_k * qs[1])
-        qs[1] = FS * static_cast<float>(sum);
     }
     // ---- B fragments of the integer mma (m16n8k32, B = 32 channels x 8 columns of signed bytes).  Channel i sits in
     // k-step s = i >> 5 at k index 16 hh + 4 t + bb, i.e. register hh, lane 4 n + t, byte bb of column n.
     // MODE 0: column n holds head n >> 1, high digit (n even) or low digit (n odd).  MODE 1: column n holds
     // head n; the high digits form the first fragment set, the low digits the second.
-    const int s = i >> 5, hh = (i >> 4) & 1, bb = 2 * ((i >> 3) & 1) + (i & 1), t = (i >> 1) & 3;
-    const long long bh = static_cast<long long>(b) * P.c.n_kv + h;
-    signed char* frag = reinterpret_cast<signed char*>(P.qfrag + bh * 256);
+    const int s = ch >> 5, hh = (ch >> 4) & 1, bb = 2 * ((ch >> 3) & 1) + (ch & 1), t = (ch >> 1) & 3;
+    signed char* frag = reinterpret_cast<signed char*>(buf);
 #pragma unroll
     for (int n = 0; n < 8; ++n) {
         const int head = (MODE == 0) ? (n >> 1) : n;
-        const int v = head < G ? qi[head] : 0;
+        const int v = qi[head];
         const int hi = (v + 128) >> 8, lo = v - 256 * hi;          // hi in [-127, 127], lo in [-128, 127]
         const int off = (((s >> 1) * 32 + 4 * n + t) * 16) + ((s & 1) * 2 + hh) * 4 + bb;
         if (MODE == 0) {
@@ -291,22 +286,35 @@ __global__ void __launch_bounds__(PREP_THREADS) decode_prep_kernel(DecodeParams 
     // ---- bf16 B fragments for the windows (mma.m16n8k16).  Element (k-step s16, register r, lane 4n+t, half hf) is
     // channel 16 s16 + 8 r + 2 t + hf of mma column n.  MODE 0: column n holds head n>>1, its rounded value (n even)
     // or the rounding remainder (n odd).  MODE 1: column n holds head n; a second copy holds the remainders.
-    const int s16 = i >> 4, r16 = i & 15, r = r16 >> 3, tw = (r16 & 7) >> 1, hf = r16 & 1;
-    unsigned short* wfrag = reinterpret_cast<unsigned short*>(P.qwfrag + bh * 256);
+    const int s16 = ch >> 4, r16 = ch & 15, r = r16 >> 3, tw = (r16 & 7) >> 1, hf = r16 & 1;
+    unsigned short* wfrag = reinterpret_cast<unsigned short*>(buf + QF);
 #pragma unroll
     for (int n = 0; n < 8; ++n) {
         const int head = (MODE == 0) ? (n >> 1) : n;
-        float wval = 0.f, wrem = 0.f;
-        if (head < G) {
-            const float y = acc[head] * k2;
-            const float yh = __bfloat162float(__float2bfloat16_rn(y));
-            wrem = y - yh;
-            wval = (MODE == 0 && (n & 1)) ? wrem : y;
-        }
+        const float y = acc[head] * k2;                           // zero for unused head slots
+        const float wrem = y - __bfloat162float(__float2bfloat16_rn(y));
+        const float wval = (MODE == 0 && (n & 1)) ? wrem : y;
         const int idx = ((((s16 >> 1) * 32 + 4 * n + tw) * 4 + (s16 & 1) * 2 + r) << 1) + hf;
         wfrag[idx] = __bfloat16_as_ushort(__float2bfloat16_rn(wval));
         if (MODE == 1) wfrag[1024 + idx] = __bfloat16_as_ushort(__float2bfloat16_rn(wrem));
     }
+    asm volatile("bar.sync 1, 128;" ::: "memory");
+    if (ch < G) {
+        const int* ri = red_isum[ch];
+        const float* ra = red_abs[ch];
+        const float amax = fmaxf(fmaxf(ra[0], ra[1]), fmaxf(ra[2], ra[3]));
+        const float lam_h = (amax > 0.f && amax < 3e38f) ? amax * (1.f / Q_MAX) : 1.f;
+        constexpr float FS = BITS != 4 ? 4.f : 16.f;      // the integer score carries this factor (see the main kernel)
+        float* qs = P.qscal + (static_cast<long long>(b) * P.c.n_q + h * G + ch) * 2;
+        qs[0] = k2 * lam_h * (1.f / FS);                  // score (log2 domain) = qs[0] * (Delta_k * sum_int + x_min_k * qs[1])
+        qs[1] = FS * static_cast<float>(ri[0] + ri[1] + ri[2] + ri[3]);
+    }
+#pragma unroll
+    for (int k = 0; k < (QF + 127) / 128; ++k)
+        if (128 * k + ch < QF) P.qfrag[bh * 256 + 128 * k + ch] = buf[128 * k + ch];
+#pragma unroll
+    for (int k = 0; k < QW / 128; ++k) P.qwfrag[bh * 256 + 128 * k + ch] = buf[QF + 128 * k + ch];
+    if (P.q_early && first_cta) pdl_wait();              // see above
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -607,34 +615,35 @@ struct MergedState {
     float m, l;
     float4 o;
     __device__ __forceinline__ void reset() { m = -INFINITY; l = 0.f; o = make_float4(0.f, 0.f, 0.f, 0.f); }
-    // Adds n partials; next() returns the address of the next one.
-    template <class Next>
-    __device__ __forceinline__ void add(int n, int lane, Next next) {
-        for (int k = 0; k < n; k += MERGE_BATCH) {
-            float4 v[MERGE_BATCH];
-            float2 ml[MERGE_BATCH];
+    // Adds n >= 1 partials; record(k) is the address of partial k.  The loads are unconditional (past the end the last record
+    // again): under a condition each would wait for the one before.
+    template <bool GLOBAL, class Record>
+    __device__ __forceinline__ void add(int n, int lane, Record record) {
+        constexpr int NB = GLOBAL ? 2 * MERGE_BATCH : MERGE_BATCH;
+        for (int k = 0; k < n; k += NB) {
+            float4 v[NB];
+            float2 ml[NB];
             float mn = m;
 #pragma unroll
-            for (int e = 0; e < MERGE_BATCH; ++e) {
-                v[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-                ml[e] = make_float2(-INFINITY, 0.f);
-                if (k + e < n) {
-                    const float* rec = next();
-                    ml[e] = *reinterpret_cast<const float2*>(rec);
-                    v[e] = *(reinterpret_cast<const float4*>(rec + 4) + lane);
-                }
+            for (int e = 0; e < NB; ++e) {
+                const float* rec = record(min(k + e, n - 1));
+                const float2* pm = reinterpret_cast<const float2*>(rec);
+                const float4* po = reinterpret_cast<const float4*>(rec + 4) + lane;
+                ml[e] = GLOBAL ? __ldcg(pm) : *pm;               // GLOBAL: another CTA's, never through the L1
+                v[e] = GLOBAL ? __ldcg(po) : *po;
             }
 #pragma unroll
-            for (int e = 0; e < MERGE_BATCH; ++e) mn = fmaxf(mn, ml[e].x);
+            for (int e = 0; e < NB; ++e) if (k + e >= n) ml[e].x = -INFINITY;
+#pragma unroll
+            for (int e = 0; e < NB; ++e) mn = fmaxf(mn, ml[e].x);
             if (mn == -INFINITY) continue;                       // nothing but empty partials so far
             const float keep = ex2(m - mn);
             l *= keep;
             o.x *= keep; o.y *= keep; o.z *= keep; o.w *= keep;
             m = mn;
 #pragma unroll
-            for (int e = 0; e < MERGE_BATCH; ++e) {
-                if (ml[e].x == -INFINITY) continue;
-                const float f = ex2(ml[e].x - mn);
+            for (int e = 0; e < NB; ++e) {
+                const float f = ex2(ml[e].x - mn);                   // an empty partial holds zeros
                 l = fmaf(ml[e].y, f, l);
                 o.x = fmaf(v[e].x, f, o.x); o.y = fmaf(v[e].y, f, o.y);
                 o.z = fmaf(v[e].z, f, o.z); o.w = fmaf(v[e].w, f, o.w);
@@ -652,55 +661,76 @@ struct MergedState {
 };
 
 // Merge of the heads that several warps share, at the end of the main kernel.  First the shares of this CTA's warps (at most one
-// per warp) are merged, one warp per (head, query head).  Then the CTA that arrives last at the query head's counter merges
-// the CTAs' states, in CTA order, and writes the output: no CTA waits for another, and the result does not depend on which
-// one is last.
+// per warp) are merged, one warp per (head, query head).  The first and the last of these heads may reach into other CTAs: of
+// those, the CTA that arrives last at the query head's counter merges the CTAs' states, in CTA order, and writes the output: no
+// CTA waits for another, and the result does not depend on which one is last.  What this costs is latency, most of it the
+// release before the counters (1.3 us, 4.7 us when all CTAs get there together), so the CTA's counters are advanced together.
 template <int MAIN_WARPS>
 __device__ __forceinline__ void merge_shared_heads(const DecodeParams& P, const SharedHead* shared_s, const long long total) {
     const CacheView& c = P.c;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, G = c.G;
+    __shared__ int leader_s[2], n_ctas_s[2], last_s[2][8];       // [0] the CTA's first shared head, [1] its last one if that is another
     const int my_bh = lane < 2 * MAIN_WARPS ? shared_s[lane].bh : -1;
     const unsigned slots_of = __match_any_sync(FULL, my_bh);
     const unsigned leaders = __ballot_sync(FULL, my_bh >= 0 && lane == __ffs(slots_of) - 1);
-    const int n_items = __popc(leaders) * G;
-    for (int item = warp; item < n_items; item += MAIN_WARPS) {
+    if (leaders == 0) return;                                    // the same for every warp
+    const int n_heads = __popc(leaders), cta_warp0 = blockIdx.x * MAIN_WARPS;
+    const long long rec_step = static_cast<long long>(G) * PART_STRIDE;
+    // The CTAs that share a head: all from the one that owns its first unit to the one that owns its last, or, when there are
+    // more CTAs than units, the owner of each unit.  A CTA's state is at the warp that owns its first unit of the head.
+    const bool every_cta = total >= gridDim.x, every_warp = total >= P.n_warps;
+    for (int item = warp; item < n_heads * G; item += MAIN_WARPS) {
+        const int k_head = item / G, head = item % G;
         unsigned rest = leaders;
-        for (int k = item / G; k > 0; --k) rest &= rest - 1;
-        const int leader = __ffs(rest) - 1, head = item % G;
-        unsigned slots = __shfl_sync(FULL, slots_of, leader);
+        for (int k = k_head; k > 0; --k) rest &= rest - 1;
+        const int leader = __ffs(rest) - 1;
+        const unsigned slots = __shfl_sync(FULL, slots_of, leader);
         const SharedHead hd = shared_s[leader];
-        const int cta_warp0 = blockIdx.x * MAIN_WARPS;
-        float* rec0 = P.part + (static_cast<long long>(hd.bh) * G + head) * PART_STRIDE;     // the head's record of warp 0
-        const long long rec_step = static_cast<long long>(G) * PART_STRIDE;
+        const int n_shares = __popc(slots);
+        unsigned from_k = slots;                                     // lane k: the k-th share's slot is its lowest bit
+        for (int k = min(lane, n_shares - 1); k > 0; --k) from_k &= from_k - 1;
+        const unsigned long long my_rec = reinterpret_cast<unsigned long long>(shared_s[__ffs(from_k) - 1].rec + head * PART_STRIDE);
         MergedState ms;
         ms.reset();
-        ms.add(__popc(slots), lane, [&] {
-            const float* rec = shared_s[__ffs(slots) - 1].rec + head * PART_STRIDE;
-            slots &= slots - 1;
-            return rec;
-        });
-        // The CTAs that share the head: all from the one that owns its first unit to the one that owns its last, or, when there
-        // are more CTAs than units, the owner of each unit.  A CTA's state is at the warp that owns its first unit of the head.
-        const bool every_cta = total >= gridDim.x, every_warp = total >= P.n_warps;
-        const int w_first = slice_owner(hd.first, total, P.n_warps), c_first = w_first / MAIN_WARPS;
-        const int n_ctas = every_cta ? slice_owner(hd.first + hd.n_units - 1, total, P.n_warps) / MAIN_WARPS - c_first + 1 : hd.n_units;
-        if (n_ctas > 1) {
-            ms.store(rec0 + (cta_warp0 + (leader >> 1)) * rec_step, lane);
-            __syncwarp();
-            int before = 0;                                          // the counter: a record's unused word, zeroed by the preparation kernel
-            if (lane == 0) asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(before) : "l"(rec0 + 2) : "memory");
-            if (__shfl_sync(FULL, before, 0) != n_ctas - 1) continue;
-            ms.reset();
-            int k = 0;
-            ms.add(n_ctas, lane, [&] {
-                int w = max(w_first, (c_first + k) * MAIN_WARPS);
-                if (!every_warp) w = slice_owner(every_cta ? max(hd.first, static_cast<long long>(c_first + k) * MAIN_WARPS * total / P.n_warps) : hd.first + k, total, P.n_warps);
-                ++k;
-                return rec0 + w * rec_step;
-            });
+        ms.add<false>(n_shares, lane, [&](int k) { return reinterpret_cast<const float*>(__shfl_sync(FULL, my_rec, k)); });
+        int n_ctas = 1;
+        if (k_head == 0 || k_head == n_heads - 1) {
+            n_ctas = hd.n_units;
+            if (every_cta) n_ctas = slice_owner(hd.first + hd.n_units - 1, total, P.n_warps) / MAIN_WARPS - slice_owner(hd.first, total, P.n_warps) / MAIN_WARPS + 1;
+            if (lane == 0) { leader_s[k_head == 0 ? 0 : 1] = leader; n_ctas_s[k_head == 0 ? 0 : 1] = n_ctas; }
         }
-        float* out = P.O + (static_cast<long long>(hd.bh / c.n_kv) * c.n_q + (hd.bh % c.n_kv) * G + head) * D;
-        ms.finish(out, lane);
+        if (n_ctas > 1) ms.store(P.part + (static_cast<long long>(hd.bh) * G + head) * PART_STRIDE + (cta_warp0 + (leader >> 1)) * rec_step, lane);
+        else ms.finish(P.O + (static_cast<long long>(hd.bh / c.n_kv) * c.n_q + (hd.bh % c.n_kv) * G + head) * D, lane);
+    }
+    __syncthreads();
+    const int n_ends = n_heads > 1 ? 2 : 1;
+    if (threadIdx.x < n_ends * G) {
+        const int e = threadIdx.x / G, head = threadIdx.x % G;
+        int last = 0;
+        if (n_ctas_s[e] > 1) {
+            __threadfence();                                     // the CTA's states before its arrival (barrier above), the others' after it
+            last = atomicAdd(arrival_counters(P, shared_s[leader_s[e]].bh) + head, 1) == n_ctas_s[e] - 1;
+            __threadfence();
+        }
+        last_s[e][head] = last;
+    }
+    __syncthreads();
+    for (int item = warp; item < n_ends * G; item += MAIN_WARPS) {
+        const int e = item / G, head = item % G;
+        if (!last_s[e][head]) continue;
+        const SharedHead hd = shared_s[leader_s[e]];
+        const float* rec0 = P.part + (static_cast<long long>(hd.bh) * G + head) * PART_STRIDE;     // the head's record of warp 0
+        const int w_first = slice_owner(hd.first, total, P.n_warps), c_first = w_first / MAIN_WARPS;
+        MergedState ms;
+        ms.reset();
+        if (every_warp)
+            ms.add<true>(n_ctas_s[e], lane, [&](int k) { return rec0 + max(w_first, (c_first + k) * MAIN_WARPS) * rec_step; });
+        else
+            ms.add<true>(n_ctas_s[e], lane, [&](int k) {
+                const long long u = every_cta ? max(hd.first, static_cast<long long>(c_first + k) * MAIN_WARPS * total / P.n_warps) : hd.first + k;
+                return rec0 + slice_owner(u, total, P.n_warps) * rec_step;
+            });
+        ms.finish(P.O + (static_cast<long long>(hd.bh / c.n_kv) * c.n_q + (hd.bh % c.n_kv) * G + head) * D, lane);
     }
 }
 
@@ -739,7 +769,13 @@ __global__ void __launch_bounds__(main_warps(BITS, MODE) * 32, 1) decode_main_ke
     // unused staging area) so that nothing the preparation kernel writes is needed before the first copies.
     __shared__ long long scan_s[MAIN_WARPS];
     long long* plan_s = reinterpret_cast<long long*>(smem);
-    const bool local_plan = (static_cast<size_t>(P.batch) + 1) * sizeof(long long) <= static_cast<size_t>(MAIN_WARPS) * STAGES * REC;
+    static_assert((MAX_LOCAL_PLAN + 1) * sizeof(long long) <= static_cast<size_t>(MAIN_WARPS) * STAGES * REC, "the plan must fit in the staging area");
+    const bool local_plan = P.batch <= MAX_LOCAL_PLAN;
+    if (P.q_early || !local_plan) pdl_wait();           // lengths from the append / plan from the preparation kernel
+    for (int b = blockIdx.x * MAIN_WARPS * 32 + threadIdx.x; b < P.batch; b += gridDim.x * MAIN_WARPS * 32) {
+        const int slot = __ldg(P.slot + b);
+        if (slot < 0 || slot >= c.n_slots) atomicOr(c.dev_status, WUSHKV_DEV_BAD_SLOT);
+    }
     if (local_plan) {
         long long carry = 0;
         for (int base = 0; base < P.batch; base += MAIN_WARPS * 32) {
@@ -760,8 +796,6 @@ __global__ void __launch_bounds__(main_warps(BITS, MODE) * 32, 1) decode_main_ke
         }
         if (threadIdx.x == 0) plan_s[0] = 0;
         __syncthreads();
-    } else {
-        pdl_wait();
     }
     const long long* plan = local_plan ? plan_s : P.plan;
 
