@@ -216,18 +216,18 @@ __device__ __forceinline__ bool locate_token(const AppendParams& P, int token, i
     int lo = 0, hi = P.batch;                 // largest b with cu_new[b] <= token
     while (hi - lo > 1) {
         const int mid = (lo + hi) >> 1;
-        if (__ldg(P.cu_new + mid) <= token) lo = mid; else hi = mid;
+        if (ld_in(P.cu_new + mid) <= token) lo = mid; else hi = mid;
     }
     ts.b = lo;
-    ts.slot = __ldg(P.slot + lo);
-    const int s0 = __ldg(P.seq_len + lo);
-    const int first = __ldg(P.cu_new + lo), last = __ldg(P.cu_new + lo + 1);
+    ts.slot = ld_in(P.slot + lo);
+    const int s0 = ld_in(P.seq_len + lo);
+    const int first = ld_in(P.cu_new + lo), last = ld_in(P.cu_new + lo + 1);
     ts.pos = s0 + (token - first);
     ts.s_final = s0 + (last - first);
     if (ts.slot < 0 || ts.slot >= P.c.n_slots || s0 < 0) { atomicOr(P.c.dev_status, WUSHKV_DEV_BAD_SLOT); return false; }
     const int pidx = ts.pos / PAGE_TOKENS;
     if (pidx >= P.c.max_pages) { atomicOr(P.c.dev_status, WUSHKV_DEV_PAGE_TABLE_FULL); return false; }
-    const int page = __ldg(P.c.page_table + static_cast<long long>(ts.slot) * P.c.max_pages + pidx);
+    const int page = ld_in(P.c.page_table + static_cast<long long>(ts.slot) * P.c.max_pages + pidx);
     if (page < 0 || page >= P.c.n_pages) { atomicOr(P.c.dev_status, WUSHKV_DEV_BAD_PAGE_ID); return false; }
     ts.rec = P.c.pages + (static_cast<long long>(page) * P.c.n_kv + head) * record_bytes(P.c.bits);
     ts.r = ts.pos % PAGE_TOKENS;
@@ -251,12 +251,20 @@ __device__ __forceinline__ void store_window_copy(const AppendParams& P, const T
 template <int BITS>
 __global__ void __launch_bounds__(256) append_rows_kernel(AppendParams P) {
     extern __shared__ __align__(16) float Tt[];          // Tt[j * TT_STRIDE + i] = T[i][j]
+    pdl_wait();
+    pdl_launch_dependents();
     const int head = blockIdx.y;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     const float* T = P.c.T_K + static_cast<long long>(head) * D * D;
-    for (int idx = threadIdx.x; idx < D * D; idx += blockDim.x) {
-        const int i = idx >> 7, j = idx & 127;
-        Tt[j * TT_STRIDE + i] = __ldg(T + idx);
+    for (int base = threadIdx.x; base < D * D; base += 8 * blockDim.x) {       // (eight loads in flight, D * D = 64 x 256 threads)
+        float t[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) t[k] = ld_in(T + base + k * blockDim.x);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const int idx = base + k * blockDim.x, i = idx >> 7, j = idx & 127;
+            Tt[j * TT_STRIDE + i] = t[k];
+        }
     }
     __syncthreads();
     const int tok0 = blockIdx.x * P.tokens_per_cta;
@@ -266,7 +274,7 @@ __global__ void __launch_bounds__(256) append_rows_kernel(AppendParams P) {
         if (!locate_token(P, token, head, ts)) continue;
         const long long row = (static_cast<long long>(token) * P.c.n_kv + head) * D;
         // ---------------- keys: k' = T k (Algorithm 2 line 3), fp32 accumulation of exact bf16 products
-        const uint2 kraw = __ldg(reinterpret_cast<const uint2*>(P.K_new + row) + lane);
+        const uint2 kraw = ld_in(reinterpret_cast<const uint2*>(P.K_new + row) + lane);
         float kin[4] = {bf16_bits_to_float(kraw.x & 0xffff), bf16_bits_to_float(kraw.x >> 16),
                         bf16_bits_to_float(kraw.y & 0xffff), bf16_bits_to_float(kraw.y >> 16)};
         if (P.pro.rope) norm_rope_warp(kin, lane, P.pro, head, prologue_position(P.pro, ts.pos, P.c.dev_status, lane == 0));
@@ -292,7 +300,7 @@ __global__ void __launch_bounds__(256) append_rows_kernel(AppendParams P) {
         kb.y = float_to_bf16_bits(x[2]) | (static_cast<unsigned>(float_to_bf16_bits(x[3])) << 16);
         store_window_copy(P, ts, head, 0, kb, lane);
         // ---------------- values: already in the folded basis, no transform
-        const uint2 vraw = __ldg(reinterpret_cast<const uint2*>(P.V_new + row) + lane);
+        const uint2 vraw = ld_in(reinterpret_cast<const uint2*>(P.V_new + row) + lane);
         float v[4] = {bf16_bits_to_float(vraw.x & 0xffff), bf16_bits_to_float(vraw.x >> 16),
                       bf16_bits_to_float(vraw.y & 0xffff), bf16_bits_to_float(vraw.y >> 16)};
         quantize_vec<BITS>(v, P.rule_v, lane, code, step_h, xmin_h, P.c.dev_status);
@@ -315,12 +323,12 @@ __global__ void __launch_bounds__(128) append_token_kernel(AppendParams P) {
     // Launched programmatically: the CTAs may be resident before the kernel ahead in the stream has
     // finished, so wait for it (and its memory) first; then let the next kernel's CTAs come in early
     // too (that kernel waits for this one itself).
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    pdl_wait();
+    pdl_launch_dependents();
     const int head = blockIdx.x, b = blockIdx.y;
     const int n_kv = P.c.n_kv;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int first = __ldg(P.cu_new + b), n_new = __ldg(P.cu_new + b + 1) - first;
+    const int first = ld_in(P.cu_new + b), n_new = ld_in(P.cu_new + b + 1) - first;
     const int s0 = n_new > 0 ? P.seq_len[b] : 0;         // written by this cluster: not through the read-only path
     // every CTA of the sequence has read the old length once all have arrived here
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
@@ -328,16 +336,16 @@ __global__ void __launch_bounds__(128) append_token_kernel(AppendParams P) {
     if (n_new > 1 && threadIdx.x == 0 && head == 0) atomicOr(P.c.dev_status, WUSHKV_DEV_BAD_COUNT);   // the host promised one token per sequence
     int slot0 = 0, page = -1;
     if (ok) {
-        slot0 = __ldg(P.slot + b);                       // the page lookup does not depend on the transform: start it now
+        slot0 = ld_in(P.slot + b);                       // the page lookup does not depend on the transform: start it now
         if (slot0 >= 0 && slot0 < P.c.n_slots && s0 >= 0 && s0 / PAGE_TOKENS < P.c.max_pages)
-            page = __ldg(P.c.page_table + static_cast<long long>(slot0) * P.c.max_pages + s0 / PAGE_TOKENS);
+            page = ld_in(P.c.page_table + static_cast<long long>(slot0) * P.c.max_pages + s0 / PAGE_TOKENS);
     }
     if (ok) {
         const long long row0 = (static_cast<long long>(first) * n_kv + head) * D;
         // the warp that will quantize the value vector requests it now; it is used after the transform
         uint2 v_pre = make_uint2(0u, 0u);
-        if (warp == 1) v_pre = __ldg(reinterpret_cast<const uint2*>(P.V_new + row0) + lane);
-        kin_s[threadIdx.x] = bf16_bits_to_float(__ldg(P.K_new + row0 + threadIdx.x));
+        if (warp == 1) v_pre = ld_in(reinterpret_cast<const uint2*>(P.V_new + row0) + lane);
+        kin_s[threadIdx.x] = bf16_bits_to_float(ld_in(P.K_new + row0 + threadIdx.x));
         __syncthreads();
         if (P.pro.rope) {                                // projected keys: Norm and RoPE first
             if (warp == 0) {
@@ -359,7 +367,7 @@ __global__ void __launch_bounds__(128) append_token_kernel(AppendParams P) {
             float part[32];
 #pragma unroll
             for (int r = 0; r < 32; ++r) {
-                const float4 t = __ldg(Tbase + r * (D / 4));
+                const float4 t = ld_in(Tbase + r * (D / 4));
                 part[r] = fmaf(t.x, kv.x, fmaf(t.y, kv.y, fmaf(t.z, kv.z, t.w * kv.w)));
             }
             kp_s[r0 + lane] = warp_transpose_reduce(part, lane);
@@ -607,6 +615,8 @@ __global__ void __launch_bounds__(TC_THREADS, 2) append_chunk_kernel(AppendParam
     const int head = blockIdx.y;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int n_tiles = (P.total_new + TC_TILE - 1) / TC_TILE;
+    pdl_wait();
+    pdl_launch_dependents();
 
     // ---- one-time set-up: tensor memory, barrier, T_K as bf16 operand
     if (warp == 0) {
@@ -623,10 +633,17 @@ __global__ void __launch_bounds__(TC_THREADS, 2) append_chunk_kernel(AppendParam
     {
         const float* T = P.c.T_K + static_cast<long long>(head) * D * D;
         const int r8 = lane & 7, cq = lane >> 3;
-        for (int item = warp; item < 64; item += TC_THREADS / 32) {     // 16 row groups x 4 groups of 4 k chunks
-            const int rg = item >> 2, kc = (item & 3) * 4 + cq;
+        float4 ta[4], tb[4];                                            // all in flight before the first store to shared memory
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {                                   // 16 row groups x 4 groups of 4 k chunks
+            const int item = warp + k * (TC_THREADS / 32), rg = item >> 2, kc = (item & 3) * 4 + cq;
             const float4* src = reinterpret_cast<const float4*>(T + (rg * 8 + r8) * D + kc * 8);
-            const float4 a = __ldg(src), b = __ldg(src + 1);
+            ta[k] = ld_in(src); tb[k] = ld_in(src + 1);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int item = warp + k * (TC_THREADS / 32), rg = item >> 2, kc = (item & 3) * 4 + cq;
+            const float4 a = ta[k], b = tb[k];
             uint4 v;
             v.x = float_to_bf16_bits(a.x) | (static_cast<unsigned>(float_to_bf16_bits(a.y)) << 16);
             v.y = float_to_bf16_bits(a.z) | (static_cast<unsigned>(float_to_bf16_bits(a.w)) << 16);
@@ -737,7 +754,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2) append_chunk_kernel(AppendParam
                     const float4* wa = reinterpret_cast<const float4*>(P.pro.weight + static_cast<long long>(head) * D + 16 * q);
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
-                        const float4 u = __ldg(wa + e), v = __ldg(wa + 16 + e);
+                        const float4 u = ld_in(wa + e), v = ld_in(wa + 16 + e);
                         a[4 * e] *= r * u.x; a[4 * e + 1] *= r * u.y; a[4 * e + 2] *= r * u.z; a[4 * e + 3] *= r * u.w;
                         b[4 * e] *= r * v.x; b[4 * e + 1] *= r * v.y; b[4 * e + 2] *= r * v.z; b[4 * e + 3] *= r * v.w;
                     }
@@ -751,7 +768,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2) append_chunk_kernel(AppendParam
             unsigned outa[8], outb[8];
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
-                const float4 cs = __ldg(tab + e);             // (cos, sin) of pairs 16q + 2e, 16q + 2e + 1
+                const float4 cs = ld_in(tab + e);             // (cos, sin) of pairs 16q + 2e, 16q + 2e + 1
                 const float ya0 = fmaf(a[2 * e], cs.x, -b[2 * e] * cs.y), yb0 = fmaf(a[2 * e], cs.y, b[2 * e] * cs.x);
                 const float ya1 = fmaf(a[2 * e + 1], cs.z, -b[2 * e + 1] * cs.w), yb1 = fmaf(a[2 * e + 1], cs.w, b[2 * e + 1] * cs.z);
                 outa[e] = float_to_bf16_bits(ya0) | (static_cast<unsigned>(float_to_bf16_bits(ya1)) << 16);
@@ -870,7 +887,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2) append_chunk_kernel(AppendParam
                 if (token >= P.total_new) break;
                 TokenSlot ts;
                 if (!locate_token(P, token, head, ts)) continue;
-                const uint2 vraw = __ldg(reinterpret_cast<const uint2*>(P.V_new + (static_cast<long long>(token) * P.c.n_kv + head) * D) + lane);
+                const uint2 vraw = ld_in(reinterpret_cast<const uint2*>(P.V_new + (static_cast<long long>(token) * P.c.n_kv + head) * D) + lane);
                 float x[4] = {bf16_bits_to_float(vraw.x & 0xffff), bf16_bits_to_float(vraw.x >> 16),
                               bf16_bits_to_float(vraw.y & 0xffff), bf16_bits_to_float(vraw.y >> 16)};
                 int code[4];
@@ -1031,8 +1048,12 @@ __global__ void __launch_bounds__(TC_THREADS, 2) append_chunk_kernel(AppendParam
 // Advances the lengths after a rows / chunk append.  A sequence one of whose tokens could not be stored
 // (bad slot, page table too short, page id outside the pool: the append kernel flagged it and skipped
 // that token) keeps its old length.
-__global__ void advance_len_kernel(CacheView c, int batch, const int* slot, int* seq_len, const int* cu_new) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
+// One warp per sequence: its lanes look at the sequence's new pages side by side (a thread per sequence, page after page, took
+// 12 us for 8 x 8192 tokens).
+__global__ void __launch_bounds__(256) advance_len_kernel(CacheView c, int batch, const int* slot, int* seq_len, const int* cu_new) {
+    pdl_wait();                                          // the append reads the old lengths
+    pdl_launch_dependents();
+    const int b = static_cast<int>(blockIdx.x * 8 + (threadIdx.x >> 5)), lane = threadIdx.x & 31;
     if (b >= batch) return;
     const int n_new = cu_new[b + 1] - cu_new[b];
     if (n_new <= 0) return;
@@ -1040,11 +1061,13 @@ __global__ void advance_len_kernel(CacheView c, int batch, const int* slot, int*
     if (sl < 0 || sl >= c.n_slots || s0 < 0) return;
     const int p0 = s0 / PAGE_TOKENS, p1 = (s0 + n_new - 1) / PAGE_TOKENS;
     if (p1 >= c.max_pages) return;
-    for (int p = p0; p <= p1; ++p) {
+    bool ok = true;
+#pragma unroll 4
+    for (int p = p0 + lane; p <= p1; p += 32) {
         const int page = c.page_table[static_cast<long long>(sl) * c.max_pages + p];
-        if (page < 0 || page >= c.n_pages) return;
+        ok &= page >= 0 && page < c.n_pages;
     }
-    seq_len[b] = s0 + n_new;
+    if (__all_sync(FULL, ok) && lane == 0) seq_len[b] = s0 + n_new;
 }
 
 __global__ void unpack_debug_kernel(CacheView c, int slot, int head, int which, int pos0, int n,
@@ -1184,8 +1207,7 @@ static int append_impl(const wushkv_cache* cache, int32_t batch, const int32_t* 
         P.use_tma = (mk && mv && !P.pro.rope && !knobs().append_no_tma) ? 1 : 0;
         auto launch = [&](auto kernel) -> bool {
             if (!opt_in_dynamic_smem(reinterpret_cast<const void*>(kernel), TC_SMEM_TOTAL)) return false;
-            kernel<<<grid_tc, TC_THREADS, TC_SMEM_TOTAL, st>>>(P, map_k, map_v);
-            return true;
+            return launch_pdl(kernel, grid_tc, dim3(TC_THREADS), TC_SMEM_TOTAL, st, P, map_k, map_v) == cudaSuccess;
         };
         bool ok;
         if (P.c.bits == 2) {
@@ -1212,8 +1234,7 @@ static int append_impl(const wushkv_cache* cache, int32_t batch, const int32_t* 
         }
         if (!ok) return WUSHKV_ECUDA;
         if (cudaGetLastError() != cudaSuccess) return WUSHKV_ECUDA;
-        advance_len_kernel<<<(batch + 127) / 128, 128, 0, st>>>(P.c, batch, slot, seq_len, cu_new);
-        return cudaGetLastError() == cudaSuccess ? WUSHKV_OK : WUSHKV_ECUDA;
+        return launch_pdl(advance_len_kernel, dim3((batch + 7) / 8), dim3(256), 0, st, P.c, batch, slot, seq_len, cu_new) == cudaSuccess ? WUSHKV_OK : WUSHKV_ECUDA;
     }
     // enough CTAs to fill the machine, but at least 8 tokens each to amortise the transform load
     const int want_ctas = std::max(1, 2 * sm_count() / P.c.n_kv);
@@ -1224,18 +1245,16 @@ static int append_impl(const wushkv_cache* cache, int32_t batch, const int32_t* 
     const size_t smem = static_cast<size_t>(D) * TT_STRIDE * sizeof(float);
     if (P.c.bits == 2) {
         if (!opt_in_dynamic_smem(reinterpret_cast<const void*>(append_rows_kernel<2>), static_cast<int>(smem))) return WUSHKV_ECUDA;
-        append_rows_kernel<2><<<grid, 256, smem, st>>>(P);
+        if (launch_pdl(append_rows_kernel<2>, grid, dim3(256), smem, st, P) != cudaSuccess) return WUSHKV_ECUDA;
     } else if (P.c.bits == 3) {
         if (!opt_in_dynamic_smem(reinterpret_cast<const void*>(append_rows_kernel<3>), static_cast<int>(smem))) return WUSHKV_ECUDA;
-        append_rows_kernel<3><<<grid, 256, smem, st>>>(P);
+        if (launch_pdl(append_rows_kernel<3>, grid, dim3(256), smem, st, P) != cudaSuccess) return WUSHKV_ECUDA;
     } else {
         if (!opt_in_dynamic_smem(reinterpret_cast<const void*>(append_rows_kernel<4>), static_cast<int>(smem))) return WUSHKV_ECUDA;
-        append_rows_kernel<4><<<grid, 256, smem, st>>>(P);
+        if (launch_pdl(append_rows_kernel<4>, grid, dim3(256), smem, st, P) != cudaSuccess) return WUSHKV_ECUDA;
     }
     if (cudaGetLastError() != cudaSuccess) return WUSHKV_ECUDA;
-    advance_len_kernel<<<(batch + 127) / 128, 128, 0, st>>>(P.c, batch, slot, seq_len, cu_new);
-    if (cudaGetLastError() != cudaSuccess) return WUSHKV_ECUDA;
-    return WUSHKV_OK;
+    return launch_pdl(advance_len_kernel, dim3((batch + 7) / 8), dim3(256), 0, st, P.c, batch, slot, seq_len, cu_new) == cudaSuccess ? WUSHKV_OK : WUSHKV_ECUDA;
 }
 
 extern "C" int wushkv_append(const wushkv_cache* cache, int32_t batch, const int32_t* slot, int32_t* seq_len,

@@ -63,12 +63,6 @@ constexpr int WIN_TOKENS = 8;             // window tokens per work unit
 constexpr int WIN_ROW = 272;              // padded bytes per staged bf16 row (conflict-free ldmatrix)
 constexpr int WIN_V_OFF = WIN_TOKENS * WIN_ROW;
 
-// Programmatic dependent launch: a kernel launched with the programmatic-serialization attribute may
-// start while its predecessor in the stream is still running; it must call pdl_wait() before it
-// touches anything the predecessor writes.  Without the attribute both calls are no-ops.
-__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
 struct DecodeParams {
     CacheView c;
     int batch;
@@ -171,7 +165,7 @@ __global__ void __launch_bounds__(PREP_THREADS) decode_prep_kernel(DecodeParams 
     const float4* Tbase = reinterpret_cast<const float4*>(P.c.T_K_invT + (static_cast<long long>(h) * D + warp * PREP_ROWS) * D) + lane;
     float4 trow[PREP_ROWS];
 #pragma unroll
-    for (int r = 0; r < PREP_ROWS; ++r) trow[r] = __ldg(Tbase + ((r / PASS_ROWS) * PASS_ROWS + ((r % PASS_ROWS) ^ (lane / GP))) * (D / 4));
+    for (int r = 0; r < PREP_ROWS; ++r) trow[r] = ld_in(Tbase + ((r / PASS_ROWS) * PASS_ROWS + ((r % PASS_ROWS) ^ (lane / GP))) * (D / 4));
     for (int k = i; k < GP * (D / 2); k += PREP_THREADS) {               // unused head slots are zero
         const int g = k / (D / 2), c2 = 2 * (k % (D / 2));
         const unsigned w = g < G ? *reinterpret_cast<const unsigned*>(P.Q + (static_cast<long long>(b) * P.c.n_q + h * G + g) * D + c2) : 0u;

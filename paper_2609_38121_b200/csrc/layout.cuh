@@ -143,6 +143,16 @@ __device__ __forceinline__ unsigned short float_to_bf16_bits(float x) {   // rou
     return static_cast<unsigned short>(u >> 16);
 }
 
+// Programmatic dependent launch: a kernel launched with the programmatic-serialization attribute may
+// start while its predecessor in the stream is still running; it must call pdl_wait() before it
+// touches anything the predecessor reads or writes.  Every kernel of a chain has at least one CTA that waits, so that a
+// kernel's end implies the end of everything ahead of it.  Without the attribute both calls are no-ops.
+__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Load of an input: an ordinary one, which stays behind pdl_wait() (a load through the read-only path may be moved ahead of it).
+template <class T>
+__device__ __forceinline__ T ld_in(const T* p) { return *p; }
+
 // Sum v[i] over the 32 lanes of a warp for i = 0..31 at once: on return lane L holds the total of
 // v[L] in v[0].  31 shuffles instead of 32 x 5 (a butterfly that halves the live values each step).
 __device__ __forceinline__ float warp_transpose_reduce(float (&v)[32], int lane) {

@@ -71,8 +71,12 @@ struct PrefillParams {
     int use_tma;                          // 1: the tcgen05 kernel stages the chunk's own tiles with bulk tensor copies
     Prologue pro;                         // pro.rope != nullptr: K_new / Q_new are projected; Norm and RoPE are applied by the
     const float* q_weight;                // transform kernel (pro.weight: key weights, q_weight: query weights)
-    int n_split;                          // warp-specialised kernel: CTAs per tile pair, each over a share of the key tiles (1: none)
-    float* part;                          // n_split > 1: [n_split][total_new][n_q][PART_W] partial outputs
+    int max_split;                        // warp-specialised kernel: most CTAs per tile pair, each over a share of the key tiles (1: none)
+    int fixed_split;                      // > 0: that many for every pair; 0: by the amount of work (see make_share_table)
+    int n_sm;
+    int n_slots;                          // entries of the table of shares (rows of CTAs of the attention kernel)
+    int4* shares;                         // max_split > 1: (sequence, pair, share, shares of the pair), sequence -1: none; one more: .x is 1 if any pair is shared
+    float* part;                          // [max_split][total_new][n_q][PART_W] partial outputs
     int wait_limit;                       // poll limit of the barrier waits (0: default, a second or more)
     int drop;                             // testing aid: 1 the first tile's score MMAs are never committed, 2 the first bulk copy of a
                                           // CTA's first chunk tile is announced but never issued, 3 the same in the transform kernel
@@ -130,7 +134,7 @@ __global__ void __launch_bounds__(256) prefill_prep_kernel(PrefillParams P) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
     for (int idx = tid; idx < D * D; idx += 256) {
         const int i = idx >> 7, j = idx & 127;
-        float x = __ldg(T + idx);
+        float x = ld_in(T + idx);
 #pragma unroll
         for (int term = 0; term < 3; ++term) {
             if (term < n_terms) {
@@ -148,7 +152,7 @@ __global__ void __launch_bounds__(256) prefill_prep_kernel(PrefillParams P) {
     for (int item = tid; item < PREP_TOK * 16; item += 256) {
         const int r = item >> 4, piece = item & 15, tok = tok0 + r;
         uint4 v = make_uint4(0, 0, 0, 0);
-        if (tok < P.total_new) v = __ldg(reinterpret_cast<const uint4*>(src + (static_cast<long long>(tok) * n_heads + head) * D + 8 * piece));
+        if (tok < P.total_new) v = ld_in(reinterpret_cast<const uint4*>(src + (static_cast<long long>(tok) * n_heads + head) * D + 8 * piece));
         *reinterpret_cast<uint4*>(Xs + r * PREP_PITCH + 8 * piece) = v;
     }
     if (is_key) {                                         // the chunk's values as fp16 (no transform)
@@ -156,7 +160,7 @@ __global__ void __launch_bounds__(256) prefill_prep_kernel(PrefillParams P) {
             const int r = item >> 4, piece = item & 15, tok = tok0 + r;
             if (tok < P.total_new) {
                 const long long off = (static_cast<long long>(tok) * P.c.n_kv + head) * D + 8 * piece;
-                const uint4 v = __ldg(reinterpret_cast<const uint4*>(P.V_new + off));
+                const uint4 v = ld_in(reinterpret_cast<const uint4*>(P.V_new + off));
                 const unsigned w[4] = {v.x, v.y, v.z, v.w};
                 unsigned o[4];
 #pragma unroll
@@ -185,23 +189,23 @@ __global__ void __launch_bounds__(256) prefill_prep_kernel(PrefillParams P) {
             const float* w = is_key ? P.pro.weight : P.q_weight;
 #pragma unroll
             for (int k = 0; k < 32; ++k) {
-                const float wa = w ? __ldg(w + static_cast<long long>(head) * D + 32 * u + k) : 1.f;
-                const float wb = w ? __ldg(w + static_cast<long long>(head) * D + 64 + 32 * u + k) : 1.f;
+                const float wa = w ? ld_in(w + static_cast<long long>(head) * D + 32 * u + k) : 1.f;
+                const float wb = w ? ld_in(w + static_cast<long long>(head) * D + 64 + 32 * u + k) : 1.f;
                 a[k] *= rn * wa; b[k] *= rn * wb;
             }
         }
         int pos = 0;
         if (tok < P.total_new) {                           // position of the token: its sequence's length before the chunk + its index
             int lo = 0, hi = P.batch;
-            while (hi - lo > 1) { const int mid = (lo + hi) >> 1; if (__ldg(P.cu_new + mid) <= tok) lo = mid; else hi = mid; }
-            const int f0 = __ldg(P.cu_new + lo), n_b = __ldg(P.cu_new + lo + 1) - f0;
-            pos = __ldg(P.seq_len + lo) - n_b + (tok - f0);
+            while (hi - lo > 1) { const int mid = (lo + hi) >> 1; if (ld_in(P.cu_new + mid) <= tok) lo = mid; else hi = mid; }
+            const int f0 = ld_in(P.cu_new + lo), n_b = ld_in(P.cu_new + lo + 1) - f0;
+            pos = ld_in(P.seq_len + lo) - n_b + (tok - f0);
         }
         pos = prologue_position(P.pro, pos, P.c.dev_status, u == 0 && tok < P.total_new);
         const float2* tab = P.pro.rope + static_cast<long long>(pos) * (D / 2) + 32 * u;
 #pragma unroll
         for (int k = 0; k < 32; ++k) {
-            const float2 cs = __ldg(tab + k);
+            const float2 cs = ld_in(tab + k);
             xa[k] = float_to_bf16_bits(fmaf(a[k], cs.x, -b[k] * cs.y));
             xb[k] = float_to_bf16_bits(fmaf(a[k], cs.y, b[k] * cs.x));
         }
@@ -291,9 +295,9 @@ __global__ void __launch_bounds__(PF_THREADS) prefill_attn_kernel(PrefillParams 
     const int g = lane >> 2, t = lane & 3;
     const int qt = blockIdx.x % P.tiles_per_seq, b = blockIdx.x / P.tiles_per_seq;
     const int jq = blockIdx.y, h = jq / c.G;
-    const int first = __ldg(P.cu_new + b), n_new = __ldg(P.cu_new + b + 1) - first;
+    const int first = ld_in(P.cu_new + b), n_new = ld_in(P.cu_new + b + 1) - first;
     if (qt * BM >= n_new) return;
-    const int S = __ldg(P.seq_len + b), sl = __ldg(P.slot + b);
+    const int S = ld_in(P.seq_len + b), sl = ld_in(P.slot + b);
     if (sl < 0 || sl >= c.n_slots || S < n_new) {
         if (tid == 0) atomicOr(c.dev_status, WUSHKV_DEV_BAD_SLOT);
         return;
@@ -442,12 +446,12 @@ __global__ void __launch_bounds__(PF_THREADS) prefill_attn_kernel(PrefillParams 
         for (int pg = page_first; pg <= page_last; ++pg) {
             __syncthreads();
             int page = -1;
-            if (pg < c.max_pages) page = __ldg(c.page_table + static_cast<long long>(sl) * c.max_pages + pg);
+            if (pg < c.max_pages) page = ld_in(c.page_table + static_cast<long long>(sl) * c.max_pages + pg);
             const bool page_ok = page >= 0 && page < c.n_pages;
             if (!page_ok && tid == 0) atomicOr(c.dev_status, pg < c.max_pages ? WUSHKV_DEV_BAD_PAGE_ID : WUSHKV_DEV_PAGE_TABLE_FULL);
             if (page_ok) {
                 const uint4* src = reinterpret_cast<const uint4*>(c.pages + (static_cast<long long>(page) * c.n_kv + h) * REC);
-                for (int k = tid; k < REC / 16; k += PF_THREADS) reinterpret_cast<uint4*>(ts.raw)[k] = __ldg(src + k);
+                for (int k = tid; k < REC / 16; k += PF_THREADS) reinterpret_cast<uint4*>(ts.raw)[k] = ld_in(src + k);
             }
             __syncthreads();
             // thread -> token r = tid & 63, channels (tid >> 6) * 64 .. + 63, two at a time
@@ -845,9 +849,9 @@ __global__ void __launch_bounds__(TM, 2) prefill_attn_tc_kernel(PrefillParams P,
     const int G = c.G, R = TM / G;                              // chunk positions per tile
     const int qt = P.tiles_per_seq - 1 - static_cast<int>(blockIdx.x % P.tiles_per_seq);      // long tiles first
     const int b = blockIdx.x / P.tiles_per_seq, h = blockIdx.y;
-    const int first = __ldg(P.cu_new + b), n_new = __ldg(P.cu_new + b + 1) - first;
+    const int first = ld_in(P.cu_new + b), n_new = ld_in(P.cu_new + b + 1) - first;
     if (qt * R >= n_new) return;
-    const int S = __ldg(P.seq_len + b), sl = __ldg(P.slot + b);
+    const int S = ld_in(P.seq_len + b), sl = ld_in(P.slot + b);
     if (sl < 0 || sl >= c.n_slots || S < n_new) {
         if (tid == 0) atomicOr(c.dev_status, WUSHKV_DEV_BAD_SLOT);
         return;
@@ -1104,7 +1108,7 @@ __global__ void __launch_bounds__(TM, 2) prefill_attn_tc_kernel(PrefillParams P,
         const int page_first = q_lo / PAGE_TOKENS, page_last = (q_hi - 1) / PAGE_TOKENS;
         for (int pg = page_first; pg <= page_last && !failed; ++pg) {
             int page = -1;
-            if (pg < c.max_pages) page = __ldg(c.page_table + static_cast<long long>(sl) * c.max_pages + pg);
+            if (pg < c.max_pages) page = ld_in(c.page_table + static_cast<long long>(sl) * c.max_pages + pg);
             const bool page_ok = page >= 0 && page < c.n_pages;
             if (!page_ok && tid == 0) atomicOr(c.dev_status, pg < c.max_pages ? WUSHKV_DEV_BAD_PAGE_ID : WUSHKV_DEV_PAGE_TABLE_FULL);
             if (!drain_pv()) { failed = true; break; }          // the record is staged in the value buffer of the previous tile
@@ -1112,7 +1116,7 @@ __global__ void __launch_bounds__(TM, 2) prefill_attn_tc_kernel(PrefillParams P,
             unsigned char* raw = sVb + (vb ^ 1) * TC_K_BYTES;
             if (page_ok) {
                 const uint4* src = reinterpret_cast<const uint4*>(c.pages + (static_cast<long long>(page) * c.n_kv + h) * REC);
-                for (int k = tid; k < REC / 16; k += TM) reinterpret_cast<uint4*>(raw)[k] = __ldg(src + k);
+                for (int k = tid; k < REC / 16; k += TM) reinterpret_cast<uint4*>(raw)[k] = ld_in(src + k);
             }
             __syncthreads();
             {   // thread -> token r = tid & 63, channels (tid >> 6) * 64 .. + 63, eight at a time
@@ -1230,12 +1234,12 @@ __global__ void __launch_bounds__(TM, 2) prefill_attn_tc_kernel(PrefillParams P,
 //   warps 12-15       write the other key / value tiles into the same rings: bf16 window rows, and packed pages (the raw
 //                     record arrives by a bulk copy one tile ahead and is unpacked into fp16 codes).
 // Registers are moved from warps 8-15 to the softmax warps (setmaxnreg, per group of four warps).
-// When the tile pairs of a call are too few to fill the GPU, n_split CTAs share a pair: each takes a contiguous share of the
-// pair's key tiles and writes a partial row (O, reference, sum) per query row; prefill_merge_kernel combines them.
+// When the tile pairs of a call are too few to fill the GPU evenly, several CTAs share a pair: each takes a contiguous share of
+// the pair's key tiles and writes a partial row (O, reference, sum) per query row; prefill_merge_kernel combines them.
 // Tensor memory (512 columns): query tile t owns columns 256 t .. 256 t + 255: O (128), two score buffers (64 each).
 // Every wait is bounded; a wait that runs out raises a CTA-wide flag that ends all roles.
 constexpr int WS_THREADS = 512;
-constexpr int PART_W = 132;                                      // floats of a partial row: O (128), reference, sum, padding
+constexpr int PART_W = 132;                                      // floats of a partial row: O (128), reference, sum, number of shares (share 0's row)
 constexpr int WS_KS = 2, WS_VS = 3;                              // ring depths of the key / value stages: a key stage is free again when
                                                                  // its scores are done, a value stage only after O += P V a softmax later
 constexpr int WS_OFF_Q = 0;                                      // (tile 0 value, remainder), (tile 1 value, remainder)
@@ -1310,6 +1314,133 @@ __device__ unsigned long long g_ws_t[32];
 #define WST_FLUSH do { } while (0)
 #endif
 
+// The table of shares: which CTAs work on which share of which tile pair's key tiles, for calls with few pairs.  Written by one CTA
+// ahead of the attention kernel, because the host does not have the lengths (when every attention CTA worked it out for itself
+// that took 5 us of each, those without a share included).  Per pair the number of shares follows its number of key tiles
+// and one target for the whole call; of 32 targets, up to two shares per SM, the one is taken with the smallest estimate
+// of the slowest SM's time, in key tiles (about 2 us): where all CTAs run at once, the largest share; else the average and
+// about half a share at the end.  A share costs about SHARE_COST tiles (start, first record, end), a merge MERGE_COST and its
+// rows' way through L2.  Shares are handed out largest first.
+constexpr int SHARE_COST = 5, MERGE_COST = 2;
+constexpr float MERGE_ROW_COST = 1.2e-4f;                        // a partial row written and read again, in key tiles of the whole GPU
+constexpr int MAX_SHARED_PAIRS = 1024;                           // tile pairs (per KV head) of a call that may share them, and its sequences
+struct ShareScratch {
+    unsigned pair_of[MAX_SHARED_PAIRS];                          // (sequence << 16) | pair
+    int tiles[MAX_SHARED_PAIRS], size[MAX_SHARED_PAIRS], order[MAX_SHARED_PAIRS];
+    int count[16][32], largest[16][32];
+    int scan[16];
+    long long sums[16];
+};
+__device__ __forceinline__ int key_shares(const PrefillParams& P, int tiles, float per_tile) {
+    if (P.fixed_split > 0) return min(P.fixed_split, P.max_split);
+    return max(1, min(static_cast<int>(static_cast<float>(tiles) * per_tile), min(P.max_split, tiles)));
+}
+constexpr int SHARE_THREADS = 512;
+__device__ __noinline__ void make_share_table(const PrefillParams& P, ShareScratch& sc) {       // the first 512 threads of a CTA
+    const CacheView& c = P.c;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, R = TM / c.G;
+    auto sync = [] { asm volatile("bar.sync 4, 512;" ::: "memory"); };
+    auto exclusive = [&](int mine, int& all) {                   // prefix sum over the 512 threads
+        int incl = mine;
+#pragma unroll 1
+        for (int o = 1; o < 32; o <<= 1) { const int v = __shfl_up_sync(FULLM, incl, o); if (lane >= o) incl += v; }
+        sync();
+        if (lane == 31) sc.scan[warp] = incl;
+        sync();
+        int before = 0;
+        all = 0;
+#pragma unroll 4
+        for (int k = 0; k < SHARE_THREADS / 32; ++k) { if (k < warp) before += sc.scan[k]; all += sc.scan[k]; }
+        return before + incl - mine;
+    };
+    // ---- the pairs and their key tiles: full-precision old positions, packed pages, the chunk up to the pair's last row
+    int n_pairs = 0;
+    long long total = 0;
+    for (int base = 0; base < P.batch; base += SHARE_THREADS) {
+        const int b = base + tid;
+        int pairs = 0, old_tiles = 0, n_new = 0;
+        if (b < P.batch) {
+            n_new = ld_in(P.cu_new + b + 1) - ld_in(P.cu_new + b);
+            const int S = __ldcg(P.seq_len + b), S0 = max(S - n_new, 0);
+            const int q_hi = min(c.s_sink + n_quantized(S - c.lag, c.s_sink, c.s_keep, c.s_flush), S0);
+            pairs = n_new > 0 ? (n_new + 2 * R - 1) / (2 * R) : 0;
+            old_tiles = (max(S0 - max(q_hi - c.s_sink, 0), 0) + TN - 1) / TN + (q_hi > c.s_sink ? (q_hi - 1) / PAGE_TOKENS - c.s_sink / PAGE_TOKENS + 1 : 0);
+        }
+        int all;
+        const int first = n_pairs + exclusive(pairs, all);
+#pragma unroll 1
+        for (int p = 0; p < pairs && first + p < MAX_SHARED_PAIRS; ++p) {
+            sc.pair_of[first + p] = (static_cast<unsigned>(b) << 16) | static_cast<unsigned>(p);
+            sc.tiles[first + p] = old_tiles + (min((2 * p + 2) * R, n_new) + TN - 1) / TN;
+            total += sc.tiles[first + p];
+        }
+        n_pairs += all;
+    }
+    n_pairs = min(n_pairs, MAX_SHARED_PAIRS);                    // (the host admits no more)
+#pragma unroll 1
+    for (int o = 16; o >= 1; o >>= 1) total += __shfl_xor_sync(FULLM, total, o);
+    if (lane == 0) sc.sums[warp] = total;
+    sync();
+    total = 0;
+#pragma unroll 4
+    for (int k = 0; k < SHARE_THREADS / 32; ++k) total += sc.sums[k];
+    total *= c.n_kv;
+    // ---- the target
+    bool one_wave = true;
+    float per_tile = 0.f;                                        // shares per key tile; per pair rounded down, at least one
+    if (P.fixed_split == 0) {
+        const float mine = static_cast<float>(lane * P.n_sm / 16) / static_cast<float>(max(total, 1LL)) * 1.000001f;      // lane 0: no shares
+        int count = 0, largest = 0;
+        for (int i = warp; i < n_pairs; i += SHARE_THREADS / 32) {
+            const int t = sc.tiles[i], n = key_shares(P, t, mine);
+            count += n;
+            largest = max(largest, (t + n - 1) / n);
+        }
+        sc.count[warp][lane] = count; sc.largest[warp][lane] = largest;
+        sync();
+        count = 0; largest = 0;
+#pragma unroll 4
+        for (int k = 0; k < SHARE_THREADS / 32; ++k) { count += sc.count[k][lane]; largest = max(largest, sc.largest[k][lane]); }
+        float cost = count * c.n_kv <= P.n_sm ? static_cast<float>(largest + SHARE_COST)
+                                              : (static_cast<float>(total) + static_cast<float>(SHARE_COST) * count * c.n_kv) / P.n_sm + 0.5f * largest;
+        if (count > n_pairs) cost += MERGE_COST + MERGE_ROW_COST * P.total_new * c.n_q * count / n_pairs;
+        if (count > P.n_slots) cost = 1e6f;                      // more than the grid has room for
+        const unsigned best = __reduce_min_sync(FULLM, (static_cast<unsigned>(fminf(cost, 1e6f) * 64.f) << 5) | static_cast<unsigned>(lane));
+        per_tile = __shfl_sync(FULLM, mine, best & 31u);
+        one_wave = __shfl_sync(FULLM, count * c.n_kv <= P.n_sm, best & 31u);
+    }
+    // ---- if not all run at once: pairs by the size of their shares, largest first
+    if (!one_wave) {
+        auto share_size = [&](int i) { const int t = sc.tiles[i], n = key_shares(P, t, per_tile); return (t + n - 1) / n; };
+        for (int i = tid; i < n_pairs; i += SHARE_THREADS) sc.size[i] = share_size(i);
+        sync();
+        for (int i = tid; i < n_pairs; i += SHARE_THREADS) {
+            const int mine = sc.size[i];
+            int rank = 0;
+#pragma unroll 4
+            for (int k = 0; k < n_pairs; ++k) rank += sc.size[k] > mine || (sc.size[k] == mine && k < i);
+            sc.order[rank] = i;
+        }
+        sync();
+    }
+    int used = 0;
+    for (int base = 0; base < n_pairs; base += SHARE_THREADS) {
+        const int r = base + tid, i = r >= n_pairs ? 0 : one_wave ? r : sc.order[r], n = r < n_pairs ? key_shares(P, sc.tiles[i], per_tile) : 0;
+        int all;
+        const int first = used + exclusive(n, all);
+#pragma unroll 1
+        for (int k = 0; k < n && first + k < P.n_slots; ++k)
+            P.shares[first + k] = make_int4(static_cast<int>(sc.pair_of[i] >> 16), static_cast<int>(sc.pair_of[i] & 0xffffu), k, n);
+        used += all;
+    }
+    for (int x = used + tid; x < P.n_slots; x += SHARE_THREADS) P.shares[x] = make_int4(-1, 0, 0, 0);
+    if (tid == 0) P.shares[P.n_slots] = make_int4(used > n_pairs, 0, 0, 0);
+}
+__global__ void __launch_bounds__(SHARE_THREADS) prefill_shares_kernel(const __grid_constant__ PrefillParams P) {       // where no transform kernel with room for it runs ahead
+    __shared__ ShareScratch sc;
+    make_share_table(P, sc);
+}
+
 template <int BITS>
 __global__ void __launch_bounds__(WS_THREADS, 1) prefill_attn_ws_kernel(PrefillParams P, const __grid_constant__ CUtensorMap map_k,
                                                                         const __grid_constant__ CUtensorMap map_v,
@@ -1321,16 +1452,29 @@ __global__ void __launch_bounds__(WS_THREADS, 1) prefill_attn_ws_kernel(PrefillP
     const CacheView& c = P.c;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int G = c.G, R = TM / G;                              // chunk positions per query tile
-    // n_split CTAs share a tile pair: each takes a contiguous share of the pair's key tiles and leaves a partial result
-    // (short chunks over long caches would otherwise occupy a few SMs only)
-    const int n_split = P.n_split, sp = static_cast<int>(blockIdx.x % n_split), bx = static_cast<int>(blockIdx.x / n_split);
-    const int pairs = (P.tiles_per_seq + 1) >> 1;
-    const int pr = pairs - 1 - bx % pairs;                      // long pairs first
-    const int b = bx / pairs, h = blockIdx.y;
-    const int first = __ldg(P.cu_new + b), n_new = __ldg(P.cu_new + b + 1) - first;
+    pdl_wait();                                                 // the transforms (and the table) of the kernel ahead
+    pdl_launch_dependents();
+    int b, pr, sp = 0, n_split = 1;
+    int h = blockIdx.y;
+    if (P.max_split > 1) {
+        // several CTAs may share a tile pair: each takes a contiguous share of the pair's key tiles and leaves a partial result
+        h = blockIdx.x;
+        const int4 slot = __ldcg(P.shares + blockIdx.y);
+        if (slot.x < 0) return;
+        b = slot.x; pr = slot.y; sp = slot.z; n_split = slot.w;
+    } else {
+        const int pairs = (P.tiles_per_seq + 1) >> 1;
+        b = static_cast<int>(blockIdx.x) / pairs;
+        pr = pairs - 1 - static_cast<int>(blockIdx.x) % pairs;  // long pairs first
+    }
+    const int first = ld_in(P.cu_new + b), n_new = ld_in(P.cu_new + b + 1) - first;
     if (2 * pr * R >= n_new) return;
-    const int S = __ldg(P.seq_len + b), sl = __ldg(P.slot + b);
-    if (sl < 0 || sl >= c.n_slots || S < n_new) {
+    const int S = ld_in(P.seq_len + b), sl = ld_in(P.slot + b);
+    const bool bad = sl < 0 || sl >= c.n_slots || S < n_new;
+    if (P.max_split > 1 && sp == 0)                              // for the merge: how many shares the pair's rows have (none to merge if it is skipped)
+        for (int k = tid; k < min(2 * R, n_new - 2 * pr * R) * G; k += WS_THREADS)
+            P.part[(static_cast<long long>(first + 2 * pr * R + k / G) * c.n_q + h * G + k % G) * PART_W + D + 2] = bad ? 0.f : static_cast<float>(n_split);
+    if (bad) {
         if (tid == 0) atomicOr(c.dev_status, WUSHKV_DEV_BAD_SLOT);
         return;
     }
@@ -1718,7 +1862,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) prefill_attn_ws_kernel(PrefillP
             // (the page id is read a record ahead, so that the wait for the buffer covers the load)
             auto page_id = [&](const int gb) {
                 const int pg = page_first + gb;
-                return (gb < gb_end && pg < c.max_pages) ? __ldg(c.page_table + static_cast<long long>(sl) * c.max_pages + pg) : -1;
+                return (gb < gb_end && pg < c.max_pages) ? ld_in(c.page_table + static_cast<long long>(sl) * c.max_pages + pg) : -1;
             };
             int page_ahead = page_id(gb_first);
             for (int gb = gb_first; gb < gb_end && ok; ++gb) {
@@ -1795,7 +1939,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) prefill_attn_ws_kernel(PrefillP
         // later, so that nothing waits for the load
         auto page_of = [&](const int gb) -> int {
             const int pg = page_first + gb;
-            return pg < c.max_pages ? __ldg(c.page_table + static_cast<long long>(sl) * c.max_pages + pg) : -1;
+            return pg < c.max_pages ? ld_in(c.page_table + static_cast<long long>(sl) * c.max_pages + pg) : -1;
         };
         auto page_valid = [&](const int page) { return page >= 0 && page < c.n_pages; };
         // (the records themselves are requested by warp 9, up to two ahead; a page that cannot be read is reported there and
@@ -1939,31 +2083,54 @@ __global__ void __launch_bounds__(WS_THREADS, 1) prefill_attn_ws_kernel(PrefillP
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
 }
 
-// Merge of the partial results of the n_split CTAs of a tile pair: one CTA of 128 threads (one per channel) per
-// (chunk token, query head).  A partial holds O relative to its own reference m (2^m was factored out of its
-// probabilities) and the sum l of those probabilities; the output is sum_s 2^(m_s - M) O_s / sum_s 2^(m_s - M) l_s.
-__global__ void __launch_bounds__(D) prefill_merge_kernel(PrefillParams P) {
-    const CacheView& c = P.c;
-    const int tok = blockIdx.x, jq = blockIdx.y, ch = threadIdx.x;
-    {   // a sequence the attention kernel skipped leaves no partials: its rows stay untouched here as well
-        int lo = 0, hi = P.batch;
-        while (hi - lo > 1) { const int mid = (lo + hi) >> 1; if (__ldg(P.cu_new + mid) <= tok) lo = mid; else hi = mid; }
-        const int n_new = __ldg(P.cu_new + lo + 1) - __ldg(P.cu_new + lo), sl = __ldg(P.slot + lo);
-        if (sl < 0 || sl >= c.n_slots || __ldg(P.seq_len + lo) < n_new) return;
-    }
-    const long long row = static_cast<long long>(tok) * c.n_q + jq, stride = static_cast<long long>(P.total_new) * c.n_q * PART_W;
+// Merge of the partial results of the CTAs that share a tile pair, one row (chunk token, query head) by one warp, lane L holding
+// channels 4L .. 4L+3.  A partial holds O relative to its own reference m (2^m was factored out of its probabilities) and the
+// sum l of those probabilities; the output is sum_s 2^(m_s - M) O_s / sum_s 2^(m_s - M) l_s.  The lanes read the shares'
+// references and sums side by side and the rows are requested eight at a time.  (One CTA per row and a loop of dependent loads took 11 us for a
+// 300-token prompt of 8 query heads, this 4 us; merged by the last CTA of a pair instead of a kernel of its own: 47 us, as one
+// SM's warps then wait for the rows of a whole pair one after the other.)
+constexpr int MERGE_WARPS = 8;
+__global__ void __launch_bounds__(32 * MERGE_WARPS) prefill_merge_kernel(PrefillParams P) {
+    pdl_wait();
+    if (__ldcg(&P.shares[P.n_slots].x) == 0) return;             // no pair is shared
+    const int lane = threadIdx.x & 31;
+    for (long long row = static_cast<long long>(blockIdx.x) * MERGE_WARPS + (threadIdx.x >> 5); row < static_cast<long long>(P.total_new) * P.c.n_q;
+         row += static_cast<long long>(gridDim.x) * MERGE_WARPS) {
+    const long long stride = static_cast<long long>(P.total_new) * P.c.n_q * PART_W;
     const float* p0 = P.part + row * PART_W;
-    float M = -INFINITY;
-    for (int s = 0; s < P.n_split; ++s) M = fmaxf(M, __ldcg(p0 + s * stride + D));
-    float acc = 0.f, lsum = 0.f;
-    for (int s = 0; s < P.n_split; ++s) {
-        const float m = __ldcg(p0 + s * stride + D);
-        if (m == -INFINITY) continue;
-        const float w = fast_ex2(m - M);
-        acc = fmaf(w, __ldcg(p0 + s * stride + ch), acc);
-        lsum = fmaf(w, __ldcg(p0 + s * stride + D + 1), lsum);
+    const int n_share = static_cast<int>(__ldcg(p0 + D + 2));
+    if (n_share <= 1) continue;                                  // a pair that one CTA finished
+    float m = -INFINITY, l = 0.f;
+    float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int s0 = 0; s0 < n_share; s0 += 32) {
+        float2 ml = make_float2(-INFINITY, 0.f);
+        if (s0 + lane < n_share) ml = __ldcg(reinterpret_cast<const float2*>(p0 + (s0 + lane) * stride + D));
+        float M = fmaxf(m, ml.x);
+#pragma unroll
+        for (int k = 16; k >= 1; k >>= 1) M = fmaxf(M, __shfl_xor_sync(FULLM, M, k));
+        if (M == -INFINITY) continue;
+        const float keep = fast_ex2(m - M), w = fast_ex2(ml.x - M);
+        float ls = w * ml.y;
+#pragma unroll
+        for (int k = 16; k >= 1; k >>= 1) ls += __shfl_xor_sync(FULLM, ls, k);
+        l = fmaf(l, keep, ls);
+        o.x *= keep; o.y *= keep; o.z *= keep; o.w *= keep;
+        m = M;
+        const int cnt = min(32, n_share - s0);
+        for (int k = 0; k < cnt; k += 8) {
+            float4 v[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) v[e] = __ldcg(reinterpret_cast<const float4*>(p0 + (s0 + min(k + e, cnt - 1)) * stride) + lane);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const float we = __shfl_sync(FULLM, w, (k + e) & 31), f = k + e < cnt ? we : 0.f;      // an empty share holds zeros
+                o.x = fmaf(v[e].x, f, o.x); o.y = fmaf(v[e].y, f, o.y);
+                o.z = fmaf(v[e].z, f, o.z); o.w = fmaf(v[e].w, f, o.w);
+            }
+        }
     }
-    P.O[row * D + ch] = lsum > 0.f ? acc / lsum : 0.f;
+    reinterpret_cast<float4*>(P.O + row * D)[lane] = l > 0.f ? make_float4(o.x / l, o.y / l, o.z / l, o.w / l) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -2006,35 +2173,51 @@ static_assert(PT_OFF_X % 1024 == 0, "swizzled tiles need 1024-byte alignment");
 #define PST(slot) do { } while (0)
 #define PST_FLUSH(base) do { } while (0)
 #endif
-__global__ void __launch_bounds__(PT_THREADS, 1) prefill_prep_tc_kernel(PrefillParams P, const __grid_constant__ CUtensorMap map_k,
+__global__ void __launch_bounds__(PT_THREADS, 1) prefill_prep_tc_kernel(const __grid_constant__ PrefillParams P, const __grid_constant__ CUtensorMap map_k,
                                                                         const __grid_constant__ CUtensorMap map_q) {
     extern __shared__ __align__(1024) unsigned char sm_pt[];
     const int hs = blockIdx.y;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    pdl_wait();
+    pdl_launch_dependents();
+    if (hs == 2 * P.c.n_kv + P.c.n_q) {                          // one CTA more: the attention kernel's table of shares
+        if (blockIdx.x == 0 && warp < SHARE_THREADS / 32) make_share_table(P, *reinterpret_cast<ShareScratch*>(sm_pt));
+        return;
+    }
     if (hs >= P.c.n_kv + P.c.n_q) {
-        // head slots past the query heads: the chunk's values of one KV head as fp16 (no transform), 16-byte pieces, four
-        // loads in flight per thread; the CTAs of a slot take interleaved 128-token tiles like the others
+        // head slots past the query heads: the chunk's values of one KV head as fp16 (no transform), 16-byte pieces; the CTAs of
+        // a slot take interleaved 128-token tiles like the others.  The next tile's loads are in flight while this one is stored.
         const int vh = hs - P.c.n_kv - P.c.n_q;
-        for (int tok0 = static_cast<int>(blockIdx.x) * PREP_TOK; tok0 < P.total_new; tok0 += static_cast<int>(gridDim.x) * PREP_TOK) {
-            uint4 v[4];
-            long long off[4];
-            bool in[4];
+        uint4 v[2][4];
+        auto piece_of = [&](int tok0, int k, long long& off) {
+            const int item = tid + k * PT_THREADS, r = item >> 4, piece = item & 15;
+            off = (static_cast<long long>(tok0 + r) * P.c.n_kv + vh) * D + 8 * piece;
+            return item < PREP_TOK * 16 && tok0 + r < P.total_new;
+        };
+        auto load = [&](int tok0, uint4 (&dst)[4]) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) { long long off; if (piece_of(tok0, k, off)) dst[k] = ld_in(reinterpret_cast<const uint4*>(P.V_new + off)); }
+        };
+        auto store = [&](int tok0, const uint4 (&src)[4]) {
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                const int item = tid + k * PT_THREADS, r = item >> 4, piece = item & 15;
-                in[k] = item < PREP_TOK * 16 && tok0 + r < P.total_new;
-                off[k] = (static_cast<long long>(tok0 + r) * P.c.n_kv + vh) * D + 8 * piece;
-                if (in[k]) v[k] = __ldg(reinterpret_cast<const uint4*>(P.V_new + off[k]));
-            }
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                if (!in[k]) continue;
-                const unsigned w[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
+                long long off;
+                if (!piece_of(tok0, k, off)) continue;
+                const unsigned w[4] = {src[k].x, src[k].y, src[k].z, src[k].w};
                 unsigned o[4];
 #pragma unroll
                 for (int e = 0; e < 4; ++e) o[e] = pack_half2(bf16_bits_to_float(w[e] & 0xffff), bf16_bits_to_float(w[e] >> 16));
-                *reinterpret_cast<uint4*>(P.VP + off[k]) = make_uint4(o[0], o[1], o[2], o[3]);
+                *reinterpret_cast<uint4*>(P.VP + off) = make_uint4(o[0], o[1], o[2], o[3]);
             }
+        };
+        const int step = static_cast<int>(gridDim.x) * PREP_TOK;
+        int tok0 = static_cast<int>(blockIdx.x) * PREP_TOK;
+        load(tok0, v[0]);
+        for (; tok0 < P.total_new; tok0 += 2 * step) {           // (past the end nothing is loaded or stored)
+            load(tok0 + step, v[1]);
+            store(tok0, v[0]);
+            load(tok0 + 2 * step, v[0]);
+            store(tok0 + step, v[1]);
         }
         return;
     }
@@ -2074,22 +2257,32 @@ __global__ void __launch_bounds__(PT_THREADS, 1) prefill_prep_tc_kernel(PrefillP
     const bool seq_in_smem = P.pro.rope != nullptr && P.batch <= PT_MAX_SEQ;
     if (seq_in_smem) {
         for (int bq = tid; bq <= P.batch; bq += PT_THREADS) {
-            const int f0 = __ldg(P.cu_new + bq);
+            const int f0 = ld_in(P.cu_new + bq);
             seq_first[bq] = f0;
-            if (bq < P.batch) seq_base[bq] = __ldg(P.seq_len + bq) - (__ldg(P.cu_new + bq + 1) - f0) - f0;
+            if (bq < P.batch) seq_base[bq] = ld_in(P.seq_len + bq) - (ld_in(P.cu_new + bq + 1) - f0) - f0;
         }
     }
     // the transform as the B operand: element (i, j) of term `term` at (i / 8) * 2048 + (j / 8) * 128 + (i % 8) * 16 + (j % 8) * 2
-    for (int idx = tid; idx < D * D; idx += PT_THREADS) {
-        const int i = idx >> 7, j = idx & 127;
-        float x = __ldg(T + idx);
-        const int off = (i >> 3) * 2048 + (j >> 3) * 128 + (i & 7) * 16 + (j & 7) * 2;
+    {   // (all of a thread's loads are in flight before the first store to shared memory, which they may not pass)
+        constexpr int N4 = (D * D / 4 + PT_THREADS - 1) / PT_THREADS;
+        float4 t4[N4];
 #pragma unroll
-        for (int term = 0; term < 3; ++term) {
-            if (term < n_terms) {
-                const unsigned short hb = float_to_bf16_bits(x);
-                *reinterpret_cast<unsigned short*>(sm_pt + PT_OFF_T + term * (D * D * 2) + off) = hb;
-                x -= bf16_bits_to_float(hb);
+        for (int k = 0; k < N4; ++k) t4[k] = ld_in(reinterpret_cast<const float4*>(T) + min(tid + k * PT_THREADS, D * D / 4 - 1));
+#pragma unroll
+        for (int k = 0; k < N4; ++k) {
+            const int idx = 4 * (tid + k * PT_THREADS), i = idx >> 7, j = idx & 127;
+            if (idx >= D * D) break;
+            float x[4] = {t4[k].x, t4[k].y, t4[k].z, t4[k].w};
+            unsigned char* dst = sm_pt + PT_OFF_T + (i >> 3) * 2048 + (j >> 3) * 128 + (i & 7) * 16 + (j & 7) * 2;
+#pragma unroll
+            for (int term = 0; term < 3; ++term) {
+                if (term < n_terms) {
+                    unsigned short hb[4];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) { hb[e] = float_to_bf16_bits(x[e]); x[e] -= bf16_bits_to_float(hb[e]); }
+                    *reinterpret_cast<uint2*>(dst + term * (D * D * 2)) =
+                        make_uint2(hb[0] | (static_cast<unsigned>(hb[1]) << 16), hb[2] | (static_cast<unsigned>(hb[3]) << 16));
+                }
             }
         }
     }
@@ -2192,9 +2385,9 @@ __global__ void __launch_bounds__(PT_THREADS, 1) prefill_prep_tc_kernel(PrefillP
                     while (hi - lo > 1) { const int mid = (lo + hi) >> 1; if (seq_first[mid] <= tok) lo = mid; else hi = mid; }
                     pos = seq_base[lo] + tok;
                 } else {
-                    while (hi - lo > 1) { const int mid = (lo + hi) >> 1; if (__ldg(P.cu_new + mid) <= tok) lo = mid; else hi = mid; }
-                    const int f0 = __ldg(P.cu_new + lo), n_b = __ldg(P.cu_new + lo + 1) - f0;
-                    pos = __ldg(P.seq_len + lo) - n_b + (tok - f0);
+                    while (hi - lo > 1) { const int mid = (lo + hi) >> 1; if (ld_in(P.cu_new + mid) <= tok) lo = mid; else hi = mid; }
+                    const int f0 = ld_in(P.cu_new + lo), n_b = ld_in(P.cu_new + lo + 1) - f0;
+                    pos = ld_in(P.seq_len + lo) - n_b + (tok - f0);
                 }
                 pos = prologue_position(pro, pos, P.c.dev_status, q == 0 && valid);
                 uint4* cell[4];                             // [box][chunk]
@@ -2207,7 +2400,7 @@ __global__ void __launch_bounds__(PT_THREADS, 1) prefill_prep_tc_kernel(PrefillP
                 const float4* tab = reinterpret_cast<const float4*>(pro.rope + static_cast<long long>(pos) * (D / 2) + 16 * q);
                 float4 cs[8];                               // (cos, sin) of pairs 16 q .. 16 q + 15, two per load
 #pragma unroll
-                for (int k = 0; k < 8; ++k) cs[k] = __ldg(tab + k);
+                for (int k = 0; k < 8; ++k) cs[k] = ld_in(tab + k);
                 float x[4][8];
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
@@ -2229,7 +2422,7 @@ __global__ void __launch_bounds__(PT_THREADS, 1) prefill_prep_tc_kernel(PrefillP
                         float wv[8] = {1.f, 1.f, 1.f, 1.f, 1.f, 1.f, 1.f, 1.f};
                         if (pro.weight) {
                             const float4* wp = reinterpret_cast<const float4*>(pro.weight + static_cast<long long>(head) * D + 64 * (k >> 1) + 16 * q + 8 * (k & 1));
-                            const float4 wa = __ldg(wp), wb = __ldg(wp + 1);
+                            const float4 wa = ld_in(wp), wb = ld_in(wp + 1);
                             wv[0] = wa.x; wv[1] = wa.y; wv[2] = wa.z; wv[3] = wa.w; wv[4] = wb.x; wv[5] = wb.y; wv[6] = wb.z; wv[7] = wb.w;
                         }
 #pragma unroll
@@ -2331,7 +2524,10 @@ __global__ void __launch_bounds__(PT_THREADS, 1) prefill_prep_tc_kernel(PrefillP
 
 size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 
-struct PrefillPlan { size_t off_kp, off_vp, off_qp, off_qsum, off_part, total; int max_split; };
+constexpr int MAX_SHARES_PER_SM = 2;      // of a call whose pairs are shared, see make_share_table
+constexpr int MAX_TABLE = 2 * MAX_SHARED_PAIRS;
+constexpr int MAX_SPLIT = 64;
+struct PrefillPlan { size_t off_kp, off_vp, off_qp, off_qsum, off_part, per_split, table, least, total; int max_split; };
 bool make_prefill_plan(const CacheView& c, int total_new, PrefillPlan& pl) {
     if (total_new <= 0) return false;
     size_t off = 0;
@@ -2339,14 +2535,19 @@ bool make_prefill_plan(const CacheView& c, int total_new, PrefillPlan& pl) {
     pl.off_vp = off;   off = align256(off + static_cast<size_t>(total_new) * c.n_kv * D * sizeof(__half));
     pl.off_qp = off;   off = align256(off + 2 * static_cast<size_t>(total_new) * c.n_q * D * sizeof(__half));
     pl.off_qsum = off; off = align256(off + static_cast<size_t>(total_new) * c.n_q * sizeof(float));
-    // Partial results of the warp-specialised attention kernel when a call has too few tile pairs to fill the GPU: at
-    // least ceil(total_new / (2 R)) pairs per KV head exist, so at most sm_count / that many CTAs per pair are worth it.
+    // Partial results of the warp-specialised attention kernel for calls whose tile pairs do not fill the GPU several times over: at
+    // least ceil(total_new / (2 R)) pairs per KV head exist.  A call is accepted with room for as many shares as fill the
+    // GPU once (`least`); given the whole `total` it may also cut long sequences finer than short ones.
     const int R = 128 / c.G;
-    const long long min_ctas = (static_cast<long long>(total_new) + 2 * R - 1) / (2 * R) * c.n_kv;
-    pl.max_split = static_cast<int>(std::max<long long>(1, std::min<long long>(16, sm_count() / std::max<long long>(min_ctas, 1))));
+    const long long min_ctas = std::max<long long>((static_cast<long long>(total_new) + 2 * R - 1) / (2 * R) * c.n_kv, 1);
+    const long long once = std::max<long long>(1, std::min<long long>(16, sm_count() / min_ctas));
+    const long long most = 2 * MAX_SHARES_PER_SM * sm_count() / min_ctas;
+    pl.max_split = static_cast<int>(std::max<long long>(once, std::min<long long>(MAX_SPLIT, most)));
     pl.off_part = off;
-    if (pl.max_split > 1) off = align256(off + static_cast<size_t>(pl.max_split) * total_new * c.n_q * 132 * sizeof(float));
-    pl.total = off;
+    pl.per_split = static_cast<size_t>(total_new) * c.n_q * PART_W * sizeof(float);
+    pl.least = once > 1 ? align256(off + once * pl.per_split) : off;
+    pl.table = pl.max_split > 1 ? (MAX_TABLE + 1) * sizeof(int4) : 0;
+    pl.total = pl.max_split > 1 ? align256(off + pl.max_split * pl.per_split) + pl.table : off;
     return true;
 }
 
@@ -2383,12 +2584,14 @@ static int prefill_attn_impl(const wushkv_cache* cache, int32_t batch, const int
         return WUSHKV_EINVAL;
     PrefillPlan pl;
     if (!make_prefill_plan(P.c, total_new, pl)) return WUSHKV_EINVAL;
-    if (workspace_bytes < pl.total) return WUSHKV_ECAPACITY;
+    if (workspace_bytes < pl.least) return WUSHKV_ECAPACITY;
+    const size_t for_parts = workspace_bytes - pl.off_part > pl.table + 256 ? workspace_bytes - pl.off_part - pl.table - 256 : 0;
+    if (workspace_bytes < pl.total) pl.max_split = static_cast<int>(std::max<size_t>(1, std::min<size_t>(pl.max_split, for_parts / pl.per_split)));
     unsigned char* ws = static_cast<unsigned char*>(workspace);
     P.batch = batch; P.total_new = total_new; P.slot = slot; P.seq_len = seq_len; P.cu_new = cu_new;
     P.K_new = K_new; P.V_new = V_new; P.Q_new = Q_new; P.O = O;
     P.use_tma = 0;
-    P.n_split = 1;
+    P.max_split = 1; P.fixed_split = 0; P.n_sm = sm_count(); P.n_slots = 0; P.shares = nullptr;
     P.part = nullptr;
     P.wait_limit = static_cast<int>(std::min<long long>(std::max<long long>(knobs().wait_limit, 0), 1 << 30));
     P.drop = knobs().drop_prefill;
@@ -2398,6 +2601,20 @@ static int prefill_attn_impl(const wushkv_cache* cache, int32_t batch, const int
     P.qsum = reinterpret_cast<float*>(ws + pl.off_qsum);
     P.tiles_per_seq = (max_new + BM - 1) / BM;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    if (!knobs().prefill_legacy && !knobs().prefill_one_tile) {
+        // warp-specialised attention: with few tile pairs (short chunks, or few) several CTAs share a pair's key tiles, and their
+        // results are merged.  Which pairs exist and how many shares they get only the device knows (make_share_table); the
+        // grid covers the most that it hands out.
+        const int R = TM / P.c.G;
+        const long long n_pairs = std::min<long long>(static_cast<long long>(batch) * ((max_new + 2 * R - 1) / (2 * R)), total_new / (2 * R) + batch);
+        if (knobs().prefill_split > 0) P.fixed_split = P.max_split = static_cast<int>(std::max<long long>(1, std::min<long long>(std::min(knobs().prefill_split, pl.max_split), MAX_TABLE / n_pairs)));
+        else if (n_pairs * P.c.n_kv < 2 * MAX_SHARES_PER_SM * sm_count()) P.max_split = pl.max_split;
+        if (n_pairs > MAX_SHARED_PAIRS || batch > 32767 || max_new > 65535 * R) P.max_split = 1;
+        P.n_slots = static_cast<int>(std::min<long long>(n_pairs * P.max_split, MAX_TABLE));
+        if (P.fixed_split == 0) P.n_slots = static_cast<int>(std::min<long long>(P.n_slots, MAX_SHARES_PER_SM * sm_count() / P.c.n_kv + n_pairs));
+        P.part = reinterpret_cast<float*>(ws + pl.off_part);
+        P.shares = reinterpret_cast<int4*>(ws + align256(pl.off_part + P.max_split * pl.per_split));
+    }
     const size_t smem_prep = static_cast<size_t>(PREP_TOK + 3 * D) * PREP_PITCH * sizeof(unsigned short);
     if (!opt_in_dynamic_smem(reinterpret_cast<const void*>(prefill_prep_kernel), static_cast<int>(smem_prep))) return WUSHKV_ECUDA;
     {   // about one wave of CTAs: each keeps its head's transform resident and walks over token tiles
@@ -2412,7 +2629,7 @@ static int prefill_attn_impl(const wushkv_cache* cache, int32_t batch, const int
                              opt_in_dynamic_smem(reinterpret_cast<const void*>(prefill_prep_tc_kernel), PT_SMEM);
         if (tc_prep) {      // head slots: key heads, query heads, then one per KV head for the values
             const int slots_tc = slots + P.c.n_kv, per_slot_tc = std::max(1, std::min(n_tok_tiles, sm_count() / slots_tc));
-            prefill_prep_tc_kernel<<<dim3(per_slot_tc, slots_tc), PT_THREADS, PT_SMEM, st>>>(P, in_k, in_q);
+            if (launch_pdl(prefill_prep_tc_kernel, dim3(per_slot_tc, slots_tc + (P.max_split > 1 ? 1 : 0)), dim3(PT_THREADS), PT_SMEM, st, P, in_k, in_q) != cudaSuccess) return WUSHKV_ECUDA;
         }
 #if WUSHKV_WS_TIMING
         if (tc_prep) {
@@ -2428,7 +2645,10 @@ static int prefill_attn_impl(const wushkv_cache* cache, int32_t batch, const int
             cudaMemcpyToSymbol(g_ws_t, t, sizeof(t));
         }
 #endif
-        else prefill_prep_kernel<<<dim3(per_slot, slots), 256, smem_prep, st>>>(P);
+        else {
+            prefill_prep_kernel<<<dim3(per_slot, slots), 256, smem_prep, st>>>(P);
+            if (P.max_split > 1) prefill_shares_kernel<<<1, SHARE_THREADS, 0, st>>>(P);
+        }
     }
     if (cudaGetLastError() != cudaSuccess) return WUSHKV_ECUDA;
     if (!knobs().prefill_legacy) {              // tcgen05 path: the G heads of a KV head share a 128-row tile
@@ -2442,13 +2662,7 @@ static int prefill_attn_impl(const wushkv_cache* cache, int32_t batch, const int
         const bool mv = make_row_tensor_map(map_v, false, P.VP, P.c.n_kv, total_new, TN);
         P.use_tma = (mk && mv && !knobs().prefill_no_tma) ? 1 : 0;
         if (!knobs().prefill_one_tile) {        // warp-specialised kernel: a pair of query tiles per CTA
-            // few pairs (a short chunk): several CTAs per pair, each over a share of the key tiles, then a merge
-            const long long n_pairs = static_cast<long long>(batch) * ((P.tiles_per_seq + 1) / 2) * P.c.n_kv;
-            int n_split = static_cast<int>(std::max<long long>(1, std::min<long long>(pl.max_split, sm_count() / std::max<long long>(n_pairs, 1))));
-            if (knobs().prefill_split > 0) n_split = std::min(knobs().prefill_split, pl.max_split);
-            P.n_split = n_split;
-            P.part = reinterpret_cast<float*>(ws + pl.off_part);
-            const dim3 grid_ws(static_cast<unsigned>(batch) * ((P.tiles_per_seq + 1) / 2) * n_split, P.c.n_kv);
+            const dim3 grid_ws = P.max_split > 1 ? dim3(P.c.n_kv, P.n_slots) : dim3(static_cast<unsigned>(batch) * ((P.tiles_per_seq + 1) / 2), P.c.n_kv);
             // the query operands (value, remainder) as [token][query head][128 channels]: a box is one tile's (G heads, R positions)
             CUtensorMap map_q0, map_q1;
             const bool mq = make_row_tensor_map(map_q0, false, P.QP, P.c.n_q, total_new, R, P.c.G) &&
@@ -2456,14 +2670,17 @@ static int prefill_attn_impl(const wushkv_cache* cache, int32_t batch, const int
             if (!mq) P.use_tma = 0;
             auto launch_ws = [&](auto kernel, const int smem) -> bool {
                 if (!opt_in_dynamic_smem(reinterpret_cast<const void*>(kernel), smem)) return false;
-                kernel<<<grid_ws, WS_THREADS, smem, st>>>(P, map_k, map_v, map_q0, map_q1);
-                return true;
+                return launch_pdl(kernel, grid_ws, dim3(WS_THREADS), smem, st, P, map_k, map_v, map_q0, map_q1) == cudaSuccess;
             };
             const bool ok = P.c.bits == 2   ? launch_ws(prefill_attn_ws_kernel<2>, ws_smem(2))
                             : P.c.bits == 3 ? launch_ws(prefill_attn_ws_kernel<3>, ws_smem(3))
                                             : launch_ws(prefill_attn_ws_kernel<4>, ws_smem(4));
             if (!ok) return WUSHKV_ECUDA;
-            if (n_split > 1) prefill_merge_kernel<<<dim3(total_new, P.c.n_q), D, 0, st>>>(P);
+            if (P.max_split > 1) {
+                const long long n_rows = static_cast<long long>(total_new) * P.c.n_q;
+                const unsigned ctas = static_cast<unsigned>(std::min<long long>((n_rows + MERGE_WARPS - 1) / MERGE_WARPS, 8LL * sm_count()));
+                if (launch_pdl(prefill_merge_kernel, dim3(ctas), dim3(32 * MERGE_WARPS), 0, st, P) != cudaSuccess) return WUSHKV_ECUDA;
+            }
 #if WUSHKV_WS_TIMING
             {
                 cudaDeviceSynchronize();

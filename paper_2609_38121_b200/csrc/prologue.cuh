@@ -61,7 +61,7 @@ __device__ __forceinline__ void norm_rope_warp_loaded(float (&x)[4], int lane, c
 }
 // the lane's weights of `head` and its (cos, sin) table entries at `pos`
 __device__ __forceinline__ float4 prologue_weights(const Prologue& pro, int lane, int head) {
-    return (pro.normalise && pro.weight) ? __ldg(reinterpret_cast<const float4*>(pro.weight + static_cast<long long>(head) * D) + lane)
+    return (pro.normalise && pro.weight) ? ld_in(reinterpret_cast<const float4*>(pro.weight + static_cast<long long>(head) * D) + lane)
                                          : make_float4(1.f, 1.f, 1.f, 1.f);
 }
 __device__ __forceinline__ const float4* prologue_table(const Prologue& pro, int lane, int pos) {
@@ -70,7 +70,7 @@ __device__ __forceinline__ const float4* prologue_table(const Prologue& pro, int
 __device__ __forceinline__ void norm_rope_warp(float (&x)[4], int lane, const Prologue& pro, int head, int pos) {
     const float4 w = prologue_weights(pro, lane, head);
     const float4* tab = prologue_table(pro, lane, pos);
-    const float4 cs0 = __ldg(tab), cs1 = __ldg(tab + 1);
+    const float4 cs0 = ld_in(tab), cs1 = ld_in(tab + 1);
     norm_rope_warp_loaded(x, lane, pro, w, cs0, cs1);
 }
 

@@ -1,0 +1,59 @@
+"""Chunk attention whose tile pairs are shared by several CTAs by the amount of work: ragged chunks on ragged contexts, sequences
+without new tokens, one long sequence among short ones, one key tile per share, and a workspace that holds fewer shares than
+the call would like.  Against the oracle on the library's own cache, with the repository's tolerance."""
+import numpy as np
+import pytest
+
+from paper_2609_38121_b200 import workloads as W
+from tests.harness import Layer
+
+pytestmark = pytest.mark.gpu
+
+
+def _wl(n_q, n_kv, batch):
+    return W.LayerWorkload(dict(seed=131, batch=batch, n_q=n_q, n_kv=n_kv, ctx=0, theta=1e4, bits=2, s_sink=4, s_keep=64, rmsnorm=False,
+                                ragged=None, prefill_chunk=0))
+
+
+@pytest.mark.parametrize("ctx,new,n_q,n_kv,bits", [
+    ([2500], [3], 8, 1, 2),                                     # one pair, many shares
+    ([0], [300], 8, 2, 2),                                      # no context: shares of one tile, causal pairs of different length
+    ([1800, 40, 0, 700], [5, 90, 17, 0], 8, 2, 3),              # one long among short, a sequence without new tokens
+    ([100] * 9 + [1500], [40] * 9 + [70], 14, 2, 4),            # one sequence worth several of the others
+])
+def test_shares_by_amount_of_work(ctx, new, n_q, n_kv, bits):
+    L = Layer(_wl(n_q, n_kv, len(ctx)), [c + n for c, n in zip(ctx, new)], bits, 4, 64, 1)
+    if sum(ctx):
+        L.append_step(ctx)
+    assert L.check_prefill_parity(new) <= 2e-3
+    assert L.cache.status() == 0
+
+
+def test_smaller_workspaces():
+    import torch
+    from paper_2609_38121_b200 import binding as B
+    ctx, new = [1200, 300], [20, 40]
+    L = Layer(_wl(8, 2, 2), [c + n for c, n in zip(ctx, new)], 2, 4, 64, 1)
+    L.append_step(ctx)
+    L.prefill(new)
+    full, total = L.first, sum(new)
+    bits16 = lambda x: torch.from_numpy(W.f32_to_bf16_bits(x).view(np.int16)).cuda()  # noqa: E731
+    K = bits16(np.concatenate([L.tokens[b][0][ctx[b]:ctx[b] + new[b]] for b in range(2)]))
+    V = bits16(np.concatenate([L.tokens[b][1][ctx[b]:ctx[b] + new[b]] for b in range(2)]))
+    Q = bits16(np.concatenate([L.wl.chunk_queries(b, np.arange(ctx[b], ctx[b] + new[b])) for b in range(2)]))
+    cu = torch.tensor([0, 20, 60], dtype=torch.int32, device="cuda")
+    # The least that is accepted: operands, then 16 shares of 528-byte rows (60 tokens x 8 heads; 2 CTAs without shares on the GPU).
+    up = lambda x: (x + 255) // 256 * 256  # noqa: E731
+    operands = 2 * up(total * 2 * 256) + up(2 * total * 8 * 256) + up(total * 8 * 4)
+    least = up(operands + 16 * total * 8 * 528)
+    asked = B.prefill_workspace_bytes(L.cache.desc, 2, total)
+    assert asked >= least
+    for nbytes in (asked, asked - 1, least):
+        ws = torch.full((nbytes,), 0xFF, dtype=torch.uint8, device="cuda")
+        O = torch.full((total, 8, 128), float("nan"), device="cuda")
+        B.prefill_attn(L.cache.desc, 2, L.slot, L.seq_len, cu, total, 40, K, V, Q, O, ws, nbytes)
+        torch.cuda.synchronize()
+        assert np.max(np.abs(O.cpu().numpy() - full)) <= 1e-3 * np.max(np.abs(full))
+    with pytest.raises(B.WushkvError) as e:
+        B.prefill_attn(L.cache.desc, 2, L.slot, L.seq_len, cu, total, 40, K, V, Q, O, ws, least - 1)
+    assert e.value.status == B.ECAPACITY
