@@ -6,10 +6,9 @@
 //   gram_kernel             X^T X of one head over a slice of tokens on tensor cores (bf16 operands are the inputs
 //                           themselves, products exact, fp32 accumulation within the slice), added to the float64
 //                           statistics with atomics.
-//   build_transforms_kernel one CTA per head, float64 throughout: damping, Cholesky, L^T M L, two-sided Jacobi
-//                           eigensolver with a round-robin ordering (64 disjoint rotations per step), canonical
-//                           order / sign, T = c Had Lam^(-1/4) U^T L^T rounded to bf16, Gauss-Jordan inverse of the
-//                           rounded matrix.
+//   build_transforms_kernel one CTA per head, float64 throughout: damping, Cholesky, L^T M L, one-sided Jacobi on its Cholesky
+//                           factor with a round-robin ordering (64 disjoint rotations per step), canonical order / sign,
+//                           T = c Had Lam^(-1/4) U^T L^T rounded to bf16, Gauss-Jordan inverse of the rounded matrix.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -114,199 +113,293 @@ __device__ double block_sum(double v, double* red) {
     return red[0];
 }
 
-// C = A^T B (ta) or A B, all d x d row-major in global memory
-__device__ void matmul(const double* A, const double* B, double* C, bool ta) {
-    for (int idx = threadIdx.x; idx < D * D; idx += BT_THREADS) {
-        const int i = idx >> 7, j = idx & 127;
-        double s = 0;
-        for (int k = 0; k < D; ++k) s += (ta ? A[k * D + i] : A[i * D + k]) * B[k * D + j];
-        C[idx] = s;
+constexpr int BT_PITCH = D + 4;                      // doubles per column (row) of the matrix in shared memory
+constexpr int BT_PANEL = 16;                         // k values of a product that are staged together
+constexpr size_t BT_SMEM = (static_cast<size_t>(D) * BT_PITCH + 2 * BT_PANEL * BT_PITCH) * sizeof(double);
+
+// One thread's 4 x 8 block of a 128 x 128 product sum_k a(i, k) b(k, j): rows 4 (tid >> 4) .., columns (tid & 15) + 16 e.  The
+// operands come through shared-memory panels of 16 k values: four elements per thread and panel.
+template <class LoadA, class LoadB>
+__device__ __forceinline__ void block_product(double (&acc)[4][8], double* panel, LoadA load_a, LoadB load_b) {
+    const int tid = threadIdx.x, i0 = 4 * (tid >> 4), j0 = tid & 15;
+    double* pa = panel;
+    double* pb = panel + BT_PANEL * BT_PITCH;
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int e = 0; e < 8; ++e) acc[a][e] = 0.0;
+#pragma unroll 1
+    for (int k0 = 0; k0 < D; k0 += BT_PANEL) {
+        double ta[4], tb[4];
+#pragma unroll
+        for (int n = 0; n < 4; ++n) { ta[n] = load_a(k0, tid + n * BT_THREADS); tb[n] = load_b(k0, tid + n * BT_THREADS); }
+        __syncthreads();                             // the previous panel has been read
+#pragma unroll
+        for (int n = 0; n < 4; ++n) {
+            load_a.store(pa, tid + n * BT_THREADS, ta[n]);
+            load_b.store(pb, tid + n * BT_THREADS, tb[n]);
+        }
+        __syncthreads();
+#pragma unroll 4
+        for (int kk = 0; kk < BT_PANEL; ++kk) {
+            double av[4], bv[8];
+#pragma unroll
+            for (int a = 0; a < 4; ++a) av[a] = pa[kk * BT_PITCH + i0 + a];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) bv[e] = pb[kk * BT_PITCH + j0 + 16 * e];
+#pragma unroll
+            for (int a = 0; a < 4; ++a)
+#pragma unroll
+                for (int e = 0; e < 8; ++e) acc[a][e] = fma(av[a], bv[e], acc[a][e]);
+        }
     }
-    __syncthreads();
+}
+// Panels of a row-major matrix X in global memory: element (k, x) of the panel is X[k][x] or X[x][k].
+template <bool ROWS_ARE_K>
+struct GlobalPanel {
+    const double* X;
+    __device__ __forceinline__ double operator()(int k0, int n) const {
+        return ROWS_ARE_K ? X[(k0 + (n >> 7)) * D + (n & 127)] : X[(n >> 4) * D + k0 + (n & 15)];
+    }
+    __device__ __forceinline__ void store(double* p, int n, double v) const {
+        if (ROWS_ARE_K) p[(n >> 7) * BT_PITCH + (n & 127)] = v; else p[(n & 15) * BT_PITCH + (n >> 4)] = v;
+    }
+};
+struct ColumnPanel {                                 // element (k, x) is W[k] of column order[x] of the matrix in shared memory
+    const double* W;
+    const int* order;
+    __device__ __forceinline__ double operator()(int k0, int n) const { return W[order[n >> 4] * BT_PITCH + k0 + (n & 15)]; }
+    __device__ __forceinline__ void store(double* p, int n, double v) const { p[(n & 15) * BT_PITCH + (n >> 4)] = v; }
+};
+
+// Cholesky of the lower triangle of S (column j at S + j BT_PITCH), in place, the upper triangle set to zero.  False: not
+// positive definite.
+__device__ bool cholesky_columns(double* S, int* fail) {
+    const int tid = threadIdx.x, i = tid & (D - 1), jg = tid >> 7;
+#pragma unroll 1
+    for (int k = 0; k < D; ++k) {
+        const double piv = S[k * BT_PITCH + k];
+        if (!(piv > 0.0) && tid == 0) *fail = 1;
+        const double r = piv > 0.0 ? 1.0 / sqrt(piv) : 1.0;
+        const double lik = i >= k ? S[k * BT_PITCH + i] * r : 0.0;
+        __syncthreads();                             // every thread has read the column
+        if (jg == 0) S[k * BT_PITCH + i] = lik;
+        __syncthreads();
+        for (int j = k + 1 + jg; j < D; j += 4)
+            if (i >= j) S[j * BT_PITCH + i] = fma(-lik, S[k * BT_PITCH + j], S[j * BT_PITCH + i]);
+        __syncthreads();
+    }
+    return *fail == 0;
 }
 
-// One CTA per head.  ws: 8 matrices of d x d float64 per head.
+// One CTA per head, float64.  ws: 8 matrices of d x d float64 per head (3 are used).
+//   L L^T = H (damped);  A = L^T M L (M damped), scaled to trace 1;  C C^T = A.
+//   One-sided Jacobi on the columns of C: rotations from the right until they are orthogonal, W = C V.  Then A = W W^T: the
+//   eigenvectors of A are W's columns over their lengths, the eigenvalues the lengths' squares.
+// What bounds it: 127 steps of 64 disjoint rotations per sweep, each step reading and writing the whole matrix, 128 KB, in shared
+// memory, and a chain of about 1000 cycles from the dot products to the rotated columns.  A two-sided Jacobi on A with the
+// rotations applied to A's columns, A's rows and the eigenvectors in global memory, four barriers per step, took 50.6 ms
+// for 8 heads.
 __global__ void __launch_bounds__(BT_THREADS) build_transforms_kernel(const double* Mall, const double* Hall, double gamma, float* Tall,
                                                                        float* Tinvall, double* wsall, int* status) {
+    extern __shared__ __align__(16) double S[];      // the matrix, then two product panels
+    double* panel = S + D * BT_PITCH;
     __shared__ double red[BT_THREADS];
-    __shared__ double w_s[D], cs_s[D / 2], sn_s[D / 2];
-    __shared__ int order_s[D], pp_s[D / 2], qq_s[D / 2], ring_s[D];
-    __shared__ int fail_s, piv_s;
-    const int h = blockIdx.x, tid = threadIdx.x;
+    __shared__ double w_s[D], scale_s[D];
+    __shared__ int order_s[D], piv_s[D];
+    __shared__ int fail_s, piv_row_s;
+    const int h = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const double* Mh = Mall + static_cast<long long>(h) * D * D;
     const double* Hh = Hall + static_cast<long long>(h) * D * D;
     double* ws = wsall + static_cast<long long>(h) * 8 * D * D;
-    double *Md = ws, *L = ws + D * D, *A = ws + 2 * D * D, *U = ws + 3 * D * D, *B = ws + 4 * D * D, *Tm = ws + 5 * D * D, *Aug = ws + 6 * D * D;   // Aug: d x 2d
+    double *Md = ws, *L = ws + D * D, *B = ws + 2 * D * D;
     if (tid == 0) fail_s = 0;
-    // ---- damping (Definition 1)
+    // ---- damping (Definition 1), Cholesky of the damped Hessian
     const double trM = block_sum(tid < D ? Mh[tid * D + tid] : 0.0, red);
     const double trH = block_sum(tid < D ? Hh[tid * D + tid] : 0.0, red);
     for (int idx = tid; idx < D * D; idx += BT_THREADS) {
         const int i = idx >> 7, j = idx & 127;
         Md[idx] = Mh[idx] + (i == j ? gamma * trM / D : 0.0);
-        L[idx] = Hh[idx] + (i == j ? gamma * trH / D : 0.0);
+        S[j * BT_PITCH + i] = Hh[idx] + (i == j ? gamma * trH / D : 0.0);
     }
     __syncthreads();
-    // ---- Cholesky of the damped Hessian, in place (lower triangle of L)
-    for (int k = 0; k < D; ++k) {
-        if (tid == 0) {
-            const double piv = L[k * D + k];
-            if (!(piv > 0.0)) fail_s = 1;
-            L[k * D + k] = piv > 0.0 ? sqrt(piv) : 1.0;
-        }
-        __syncthreads();
-        const double dk = L[k * D + k];
-        for (int i = k + 1 + tid; i < D; i += BT_THREADS) L[i * D + k] /= dk;
-        __syncthreads();
-        const int n = D - k - 1;
-        for (int idx = tid; idx < n * n; idx += BT_THREADS) {
-            const int i = k + 1 + idx / n, j = k + 1 + idx % n;
-            if (j <= i) L[i * D + j] -= L[i * D + k] * L[j * D + k];
-        }
-        __syncthreads();
-    }
-    for (int idx = tid; idx < D * D; idx += BT_THREADS) if ((idx & 127) > (idx >> 7)) L[idx] = 0.0;
+    if (!cholesky_columns(S, &fail_s)) { if (tid == 0) atomicOr(status, WUSHKV_ENOTPD); return; }
+    for (int idx = tid; idx < D * D; idx += BT_THREADS) L[idx] = S[(idx & 127) * BT_PITCH + (idx >> 7)];
+    // ---- A = L^T (Md L), symmetrised and scaled
+    double acc[4][8];
+    const int i0 = 4 * (tid >> 4), j0 = tid & 15;
     __syncthreads();
-    if (fail_s) { if (tid == 0) atomicOr(status, WUSHKV_ENOTPD); return; }
-    // ---- A = L^T Md L, symmetrised; U = I
-    matmul(Md, L, B, false);
-    matmul(L, B, A, true);
+    block_product(acc, panel, GlobalPanel<false>{Md}, GlobalPanel<true>{L});
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int e = 0; e < 8; ++e) B[(i0 + a) * D + j0 + 16 * e] = acc[a][e];
+    __syncthreads();
+    block_product(acc, panel, GlobalPanel<true>{L}, GlobalPanel<true>{B});
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int e = 0; e < 8; ++e) S[(i0 + a) * BT_PITCH + j0 + 16 * e] = acc[a][e];
+    __syncthreads();
+    const double trA = block_sum(tid < D ? S[tid * BT_PITCH + tid] : 0.0, red);
+    if (!(trA > 0.0)) { if (tid == 0) atomicOr(status, WUSHKV_ENOTPD); return; }
     for (int idx = tid; idx < D * D; idx += BT_THREADS) {
         const int i = idx >> 7, j = idx & 127;
-        if (j > i) { const double s = 0.5 * (A[i * D + j] + A[j * D + i]); A[i * D + j] = s; A[j * D + i] = s; }
-        U[idx] = (i == j) ? 1.0 : 0.0;
+        if (i >= j) S[j * BT_PITCH + i] = 0.5 * (S[i * BT_PITCH + j] + S[j * BT_PITCH + i]) / trA;      // (only this thread reads or writes the pair)
     }
-    if (tid < D) ring_s[tid] = tid;
     __syncthreads();
-    // ---- two-sided Jacobi, round-robin ordering: 127 steps of 64 disjoint rotations per sweep
-    for (int sweep = 0; sweep < 30; ++sweep) {
-        double off = 0.0, dia = 0.0;
-        for (int idx = tid; idx < D * D; idx += BT_THREADS) {
-            const double v = A[idx];
-            if ((idx >> 7) == (idx & 127)) dia += v * v; else off += v * v;
-        }
-        off = block_sum(off, red);
-        dia = block_sum(dia, red);
-        if (off <= 1e-30 * dia) break;
-        for (int step = 0; step < D - 1; ++step) {
-            if (tid < D / 2) {                              // pair k: players ring[k] and ring[D-1-k]
-                int p = ring_s[tid], q = ring_s[D - 1 - tid];
-                if (p > q) { const int x = p; p = q; q = x; }
-                const double apq = A[p * D + q], app = A[p * D + p], aqq = A[q * D + q];
-                double c = 1.0, s = 0.0;
-                if (fabs(apq) > 1e-300) {
-                    const double theta = (aqq - app) / (2.0 * apq);
-                    const double tt = (theta >= 0.0 ? 1.0 : -1.0) / (fabs(theta) + sqrt(theta * theta + 1.0));
-                    c = 1.0 / sqrt(tt * tt + 1.0);
-                    s = tt * c;
+    if (!cholesky_columns(S, &fail_s)) { if (tid == 0) atomicOr(status, WUSHKV_ENOTPD); return; }
+    // ---- one-sided Jacobi, round-robin ordering.  Eight lanes own a pair of columns, 16 rows each (as 8 x 16 bytes: the eight lanes
+    // read 128 consecutive bytes).  The angle is computed in fp32 (its error only delays convergence), the rotation from it in
+    // float64, so that it is orthogonal to rounding; the longer column goes to the lower index, which speeds convergence up.
+    {
+        constexpr double TOL2 = 1.6e-29;             // squared cosine below which a pair counts as orthogonal (its rounding is about 1e-30)
+        const int pair = 4 * warp + (lane >> 3), l8 = lane & 7;
+#pragma unroll 1
+        for (int sweep = 0; sweep < 30; ++sweep) {
+            int rotated = 0;
+#pragma unroll 1
+            for (int step = 0; step < D - 1; ++step) {
+                auto player = [&](int pos) { int x = pos - 1 - step; if (x < 0) x += D - 1; return pos == 0 ? 0 : 1 + x; };
+                const int pa = player(pair), pb = player(D - 1 - pair);
+                double2* P = reinterpret_cast<double2*>(S + min(pa, pb) * BT_PITCH) + l8;
+                double2* Q = reinterpret_cast<double2*>(S + max(pa, pb) * BT_PITCH) + l8;
+                double2 p[8], q[8];
+                double alpha = 0.0, beta = 0.0, g = 0.0;
+#pragma unroll
+                for (int k = 0; k < 8; ++k) { p[k] = P[8 * k]; q[k] = Q[8 * k]; }
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    alpha = fma(p[k].x, p[k].x, fma(p[k].y, p[k].y, alpha));
+                    beta = fma(q[k].x, q[k].x, fma(q[k].y, q[k].y, beta));
+                    g = fma(p[k].x, q[k].x, fma(p[k].y, q[k].y, g));
                 }
-                pp_s[tid] = p; qq_s[tid] = q; cs_s[tid] = c; sn_s[tid] = s;
+#pragma unroll
+                for (int o = 1; o <= 4; o <<= 1) {
+                    alpha += __shfl_xor_sync(0xffffffffu, alpha, o);
+                    beta += __shfl_xor_sync(0xffffffffu, beta, o);
+                    g += __shfl_xor_sync(0xffffffffu, g, o);
+                }
+                if (g * g > TOL2 * (alpha * beta)) {
+                    rotated = 1;
+                    const float zeta = static_cast<float>(beta - alpha) / (2.f * static_cast<float>(g));
+                    const double t = static_cast<double>(copysignf(1.f, zeta) / (fabsf(zeta) + sqrtf(fmaf(zeta, zeta, 1.f))));
+                    const double c = rsqrt(fma(t, t, 1.0)), s = c * t;
+                    const bool swap = alpha - t * g < beta + t * g;
+                    const double c1 = swap ? s : c, s1 = swap ? -c : s;       // first column: c1 p - s1 q, second: s2 p + c2 q
+                    const double c2 = swap ? -s : c, s2 = swap ? c : s;
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        P[8 * k] = make_double2(fma(c1, p[k].x, -s1 * q[k].x), fma(c1, p[k].y, -s1 * q[k].y));
+                        Q[8 * k] = make_double2(fma(s2, p[k].x, c2 * q[k].x), fma(s2, p[k].y, c2 * q[k].y));
+                    }
+                }
+                __syncthreads();
             }
-            __syncthreads();
-            // columns: A <- A J, U <- U J
-            for (int idx = tid; idx < D * (D / 2); idx += BT_THREADS) {
-                const int r = idx >> 6, k = idx & 63;
-                const int p = pp_s[k], q = qq_s[k];
-                const double c = cs_s[k], s = sn_s[k];
-                const double ap = A[r * D + p], aq = A[r * D + q];
-                A[r * D + p] = c * ap - s * aq; A[r * D + q] = s * ap + c * aq;
-                const double up = U[r * D + p], uq = U[r * D + q];
-                U[r * D + p] = c * up - s * uq; U[r * D + q] = s * up + c * uq;
-            }
-            __syncthreads();
-            // rows: A <- J^T A
-            for (int idx = tid; idx < D * (D / 2); idx += BT_THREADS) {
-                const int col = idx >> 6, k = idx & 63;
-                const int p = pp_s[k], q = qq_s[k];
-                const double c = cs_s[k], s = sn_s[k];
-                const double ap = A[p * D + col], aq = A[q * D + col];
-                A[p * D + col] = c * ap - s * aq; A[q * D + col] = s * ap + c * aq;
-            }
-            __syncthreads();
-            if (tid == 0) {                                  // rotate the tournament: player ring[0] stays
-                const int last = ring_s[D - 1];
-                for (int k = D - 1; k > 1; --k) ring_s[k] = ring_s[k - 1];
-                ring_s[1] = last;
-            }
-            __syncthreads();
+            if (!__syncthreads_or(rotated)) break;
         }
     }
     // ---- canonical form: eigenvalues ascending, largest-magnitude entry of each eigenvector positive
-    if (tid < D) w_s[tid] = A[tid * D + tid];
+    if (tid < D) {
+        double len2 = 0.0, top = 0.0;
+#pragma unroll 4
+        for (int k = 0; k < D; ++k) {
+            const double x = S[tid * BT_PITCH + k];
+            len2 = fma(x, x, len2);
+            if (fabs(x) > fabs(top)) top = x;
+        }
+        w_s[tid] = len2 * trA;
+        if (!(len2 > 0.0)) fail_s = 1;
+        red[tid] = (top < 0.0 ? -1.0 : 1.0) / sqrt(len2);
+    }
     __syncthreads();
+    if (fail_s) { if (tid == 0) atomicOr(status, WUSHKV_ENOTPD); return; }
     if (tid < D) {
         int rank = 0;
         for (int j = 0; j < D; ++j) rank += (w_s[j] < w_s[tid]) || (w_s[j] == w_s[tid] && j < tid);
         order_s[rank] = tid;
-        if (!(w_s[tid] > 0.0)) fail_s = 1;
+        scale_s[rank] = red[tid] * pow(w_s[tid], -0.25);         // sign and scale of row `rank` of Lam^(-1/4) U^T
     }
-    __syncthreads();
-    if (fail_s) { if (tid == 0) atomicOr(status, WUSHKV_ENOTPD); return; }
     const double sum_sqrt = block_sum(tid < D ? sqrt(w_s[tid]) : 0.0, red);
-    const double c_norm = sqrt(1.0 + gamma) * sqrt(trM) / sqrt(sum_sqrt);
-    if (tid < D) {                                           // sign and scale of row tid of Lam^(-1/4) U^T
-        const int col = order_s[tid];
-        int arg = 0;
-        for (int k = 1; k < D; ++k) if (fabs(U[k * D + col]) > fabs(U[arg * D + col])) arg = k;
-        red[tid] = (U[arg * D + col] < 0 ? -1.0 : 1.0) * pow(w_s[col], -0.25);
+    const double hn = sqrt(1.0 + gamma) * sqrt(trM) / sqrt(sum_sqrt) / sqrt(static_cast<double>(D));
+    // ---- Lam^(-1/4) U^T L^T: row i is scale_i sum_k W[k][order_i] L[j][k]
+    __syncthreads();
+    block_product(acc, panel, ColumnPanel{S, order_s}, GlobalPanel<false>{L});
+    __syncthreads();                                 // the eigenvectors have been read
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int e = 0; e < 8; ++e) S[(i0 + a) * BT_PITCH + j0 + 16 * e] = scale_s[i0 + a] * acc[a][e];
+    __syncthreads();
+    // ---- T = c Had (..): fast Walsh-Hadamard transform over the rows, rounded to bf16
+    const int j = tid & (D - 1), grp = tid >> 7;
+    {
+        double x[32];
+#pragma unroll
+        for (int r = 0; r < 32; ++r) x[r] = S[(32 * grp + r) * BT_PITCH + j];
+#pragma unroll
+        for (int bit = 1; bit < 32; bit <<= 1)
+#pragma unroll
+            for (int r = 0; r < 32; ++r)
+                if ((r & bit) == 0) { const double u = x[r], v = x[r | bit]; x[r] = u + v; x[r | bit] = u - v; }
+#pragma unroll
+        for (int r = 0; r < 32; ++r) S[(32 * grp + r) * BT_PITCH + j] = x[r];
     }
     __syncthreads();
-    // B = Lam^(-1/4) U^T L^T: B[i][j] = scale_i sum_k U[k][col_i] L[j][k]
-    for (int idx = tid; idx < D * D; idx += BT_THREADS) {
-        const int i = idx >> 7, j = idx & 127, col = order_s[i];
-        double s = 0;
-        for (int k = 0; k < D; ++k) s += U[k * D + col] * L[j * D + k];
-        B[idx] = red[i] * s;
-    }
-    __syncthreads();
-    // T = c Had B (normalized Sylvester Hadamard), rounded to bf16
-    const double hn = c_norm / sqrt(static_cast<double>(D));
     float* To = Tall + static_cast<long long>(h) * D * D;
-    for (int idx = tid; idx < D * D; idx += BT_THREADS) {
-        const int i = idx >> 7, j = idx & 127;
-        double s = 0;
-        for (int k = 0; k < D; ++k) s += (__popc(i & k) & 1) ? -B[k * D + j] : B[k * D + j];
-        const double v = round_double_to_bf16(hn * s);
-        Tm[idx] = v;
-        To[idx] = static_cast<float>(v);
+#pragma unroll 2
+    for (int r = 8 * grp; r < 8 * grp + 8; ++r) {
+        const double x0 = S[r * BT_PITCH + j], x1 = S[(r + 32) * BT_PITCH + j], x2 = S[(r + 64) * BT_PITCH + j], x3 = S[(r + 96) * BT_PITCH + j];
+        const double y[4] = {(x0 + x1) + (x2 + x3), (x0 - x1) + (x2 - x3), (x0 + x1) - (x2 + x3), (x0 - x1) - (x2 - x3)};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const double v = round_double_to_bf16(hn * y[e]);
+            S[(r + 32 * e) * BT_PITCH + j] = v;
+            To[(r + 32 * e) * D + j] = static_cast<float>(v);
+        }
     }
     __syncthreads();
-    // ---- inverse of the rounded T: Gauss-Jordan with partial pivoting on [T | I]
-    for (int idx = tid; idx < D * 2 * D; idx += BT_THREADS) {
-        const int i = idx / (2 * D), j = idx % (2 * D);
-        Aug[idx] = j < D ? Tm[i * D + j] : ((j - D) == i ? 1.0 : 0.0);
-    }
-    __syncthreads();
+    // ---- inverse of the rounded T: Gauss-Jordan with partial pivoting, in place; thread (j, grp) owns column j of rows grp + 4 m
+#pragma unroll 1
     for (int col = 0; col < D; ++col) {
-        if (tid == 0) {
-            int piv = col;
-            for (int r = col + 1; r < D; ++r) if (fabs(Aug[r * 2 * D + col]) > fabs(Aug[piv * 2 * D + col])) piv = r;
-            piv_s = piv;
-            if (Aug[piv * 2 * D + col] == 0.0) fail_s = 1;
+        if (warp == 0) {
+            double best = -1.0;
+            int at = col;
+            for (int r = lane; r < D; r += 32)
+                if (r >= col) { const double v = fabs(S[r * BT_PITCH + col]); if (v > best) { best = v; at = r; } }
+#pragma unroll
+            for (int o = 16; o >= 1; o >>= 1) {
+                const double v = __shfl_xor_sync(0xffffffffu, best, o);
+                const int r = __shfl_xor_sync(0xffffffffu, at, o);
+                if (v > best || (v == best && r < at)) { best = v; at = r; }
+            }
+            if (lane == 0) { piv_row_s = at; piv_s[col] = at; if (!(best > 0.0)) fail_s = 1; }
         }
         __syncthreads();
         if (fail_s) { if (tid == 0) atomicOr(status, WUSHKV_ENOTPD); return; }
-        const int piv = piv_s;
-        if (piv != col)
-            for (int j = tid; j < 2 * D; j += BT_THREADS) { const double x = Aug[piv * 2 * D + j]; Aug[piv * 2 * D + j] = Aug[col * 2 * D + j]; Aug[col * 2 * D + j] = x; }
+        const int piv = piv_row_s;
+        const double inv = 1.0 / S[piv * BT_PITCH + col];
+        const double rowk = (j == col ? 1.0 : S[piv * BT_PITCH + j]) * inv, old_k = S[col * BT_PITCH + j];
         __syncthreads();
-        const double inv = 1.0 / Aug[col * 2 * D + col];
+        if (grp == 0 && piv != col) S[piv * BT_PITCH + j] = old_k;       // row swap
         __syncthreads();
-        for (int j = tid; j < 2 * D; j += BT_THREADS) Aug[col * 2 * D + j] *= inv;
+        if (tid < D) red[tid] = tid == col ? 0.0 : S[tid * BT_PITCH + col];      // the column being eliminated, before it changes
         __syncthreads();
-        if (tid < D) red[tid] = Aug[tid * 2 * D + col];      // the column being eliminated, before it changes
-        __syncthreads();
-        for (int idx = tid; idx < D * 2 * D; idx += BT_THREADS) {
-            const int r = idx / (2 * D), j = idx % (2 * D);
-            if (r != col) Aug[idx] -= red[r] * Aug[col * 2 * D + j];
+#pragma unroll 8
+        for (int i = grp; i < D; i += 4) {
+            const double x = j == col ? 0.0 : S[i * BT_PITCH + j];
+            S[i * BT_PITCH + j] = i == col ? rowk : fma(-red[i], rowk, x);
         }
         __syncthreads();
     }
-    float* Ti = Tinvall + static_cast<long long>(h) * D * D;
-    for (int idx = tid; idx < D * D; idx += BT_THREADS) {
-        const int i = idx >> 7, j = idx & 127;
-        Ti[idx] = static_cast<float>(Aug[j * 2 * D + D + i]);      // (T^-1)^T
+#pragma unroll 1
+    for (int col = D - 1; col >= 0; --col) {          // the row swaps, undone as column swaps in reverse
+        const int piv = piv_s[col];
+        if (piv != col && tid < D) { const double x = S[tid * BT_PITCH + col]; S[tid * BT_PITCH + col] = S[tid * BT_PITCH + piv]; S[tid * BT_PITCH + piv] = x; }
     }
+    __syncthreads();
+    float* Ti = Tinvall + static_cast<long long>(h) * D * D;
+    for (int idx = tid; idx < D * D; idx += BT_THREADS) Ti[idx] = static_cast<float>(S[(idx & 127) * BT_PITCH + (idx >> 7)]);      // (T^-1)^T
 }
 
 }  // namespace
@@ -336,6 +429,7 @@ extern "C" int wushkv_build_transforms_device(int32_t n_heads, int32_t d, const 
     if (!M || !H || !T || !T_invT || !dev_status || !workspace || n_heads <= 0 || d != D || !(gamma >= 0.0)) return WUSHKV_EINVAL;
     if (!aligned(M, 8) || !aligned(H, 8) || !aligned(workspace, 16)) return WUSHKV_EINVAL;
     if (workspace_bytes < wushkv_build_transforms_workspace_bytes(n_heads, d)) return WUSHKV_ECAPACITY;
-    build_transforms_kernel<<<n_heads, BT_THREADS, 0, static_cast<cudaStream_t>(stream)>>>(M, H, gamma, T, T_invT, static_cast<double*>(workspace), dev_status);
+    if (!opt_in_dynamic_smem(reinterpret_cast<const void*>(build_transforms_kernel), static_cast<int>(BT_SMEM))) return WUSHKV_ECUDA;
+    build_transforms_kernel<<<n_heads, BT_THREADS, BT_SMEM, static_cast<cudaStream_t>(stream)>>>(M, H, gamma, T, T_invT, static_cast<double*>(workspace), dev_status);
     return cudaGetLastError() == cudaSuccess ? WUSHKV_OK : WUSHKV_ECUDA;
 }
