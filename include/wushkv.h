@@ -180,7 +180,7 @@ int wushkv_build_transforms_device(int32_t n_heads, int32_t d, const double* M, 
  *   total_new, max_new (host): total and per-sequence maximum of new tokens.
  *   K_new (device): bf16 [total_new][n_kv][d] post-Norm post-RoPE keys, 16-byte aligned.
  *   V_new (device): bf16 [total_new][n_kv][d] values in the folded basis, 16-byte aligned.
- * Chunks (max_new >= 128) take the tensor-core transform path (tcgen05, fp32 accumulation in
+ * Chunks (max_new >= 128, or many shorter ones) take the tensor-core transform path (tcgen05, fp32 accumulation in
  * tensor memory), max_new == 1 a single-launch decode-time path, anything else a CUDA-core path.
  * All produce the same codes up to fp32 summation order (wushkv_set_test_option("append_path_cuda", 1)
  * forces the CUDA-core path for chunks).

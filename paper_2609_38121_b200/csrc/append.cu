@@ -1,7 +1,7 @@
 // Quantize-on-append (Algorithm 2 lines 3-4 and 9-12; quantizer: Section 5.3 Eq. 6).
 //
 // Three kernels, chosen by wushkv_append from the shape of the call:
-//   append_chunk_kernel  prefill chunks (max_new >= 128): key transform on tcgen05, four lanes per vector
+//   append_chunk_kernel  prefill chunks (max_new >= 128, or many short ones): key transform on tcgen05, four lanes per vector
 //                        for the quantizer (described where it is defined, further down);
 //   append_token_kernel  one token per sequence (a decode step): one CTA per sequence, single launch;
 //   append_rows_kernel   everything else, and the chunk path when WUSHKV_APPEND_PATH=cuda.
@@ -1191,7 +1191,14 @@ static int append_impl(const wushkv_cache* cache, int32_t batch, const int32_t* 
         return e1 == cudaSuccess ? WUSHKV_OK : WUSHKV_ECUDA;
     }
     const bool force_cuda = knobs().append_path_cuda != 0;             // testing aid: CUDA-core path for chunks too
-    if (max_new >= TC_TILE && !force_cuda) {    // prefill chunk: tensor-core transform
+    // Tokens per CTA of the warp-per-vector path: enough CTAs to fill the machine, but at least one token for each of 8 warps.
+    const int want_ctas = std::max(1, 2 * sm_count() / P.c.n_kv);
+    const int tpc = std::max(8, ((total_new + want_ctas - 1) / want_ctas + 7) / 8 * 8);
+    // The tensor-core path takes about 15 us whatever it gets (23 us with projected keys) while one wave of it suffices, the
+    // warp-per-vector path about 10 us for every token of a warp: the line is at two tokens per warp (three).  16 ragged
+    // chunks of 5 to 90 tokens, 8 heads, 3 bits: 34.7 -> 20.2 us.
+    const bool many_short = max_new > 1 && tpc >= (P.pro.rope ? 24 : 16);
+    if ((max_new >= TC_TILE || many_short) && !force_cuda) {    // prefill chunk: tensor-core transform
         const int n_tiles = (total_new + TC_TILE - 1) / TC_TILE;
         const int per_head = std::max(1, std::min(n_tiles, 2 * sm_count() / P.c.n_kv));
         const dim3 grid_tc(per_head, P.c.n_kv);
@@ -1236,10 +1243,6 @@ static int append_impl(const wushkv_cache* cache, int32_t batch, const int32_t* 
         if (cudaGetLastError() != cudaSuccess) return WUSHKV_ECUDA;
         return launch_pdl(advance_len_kernel, dim3((batch + 7) / 8), dim3(256), 0, st, P.c, batch, slot, seq_len, cu_new) == cudaSuccess ? WUSHKV_OK : WUSHKV_ECUDA;
     }
-    // enough CTAs to fill the machine, but at least 8 tokens each to amortise the transform load
-    const int want_ctas = std::max(1, 2 * sm_count() / P.c.n_kv);
-    int tpc = (total_new + want_ctas - 1) / want_ctas;
-    tpc = std::max(8, ((tpc + 7) / 8) * 8);
     P.tokens_per_cta = tpc;
     const dim3 grid((total_new + tpc - 1) / tpc, P.c.n_kv);
     const size_t smem = static_cast<size_t>(D) * TT_STRIDE * sizeof(float);

@@ -1,0 +1,57 @@
+"""The transform builder on statistics at the edges of its arithmetic, against the oracle's eigensolver: very differently scaled
+M and H, strongly graded spectra, repeated eigenvalues, many heads in one call, and matrices that are not positive definite."""
+import numpy as np
+import pytest
+
+from oracle import wushkv_oracle as O
+from paper_2609_38121_b200 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+def _spd(rng, spread, scale):
+    q = np.linalg.qr(rng.standard_normal((128, 128)))[0]
+    m = (q * (scale * 10.0 ** np.linspace(-spread, 0, 128))) @ q.T
+    return 0.5 * (m + m.T)
+
+
+def _build(M, H, gamma):
+    import torch
+    from paper_2609_38121_b200 import binding as B
+    T, Ti = B.build_transforms_device(torch.from_numpy(M).cuda(), torch.from_numpy(H).cuda(), gamma)
+    return T.cpu().numpy().astype(np.float64), Ti.cpu().numpy().astype(np.float64)
+
+
+@pytest.mark.parametrize("m_scale,h_scale,spread", [(1.0, 1.0, 3.0), (1e20, 1e-15, 3.0), (1e-18, 1e12, 6.0)])
+def test_scales_and_graded_spectra(m_scale, h_scale, spread):
+    rng = np.random.default_rng(5)
+    M = np.stack([_spd(rng, spread, m_scale) for _ in range(20)])
+    H = np.stack([_spd(rng, spread, h_scale) for _ in range(20)])
+    T, Ti = _build(M, H, W.GAMMA)
+    ref, _ = O.build_transforms(M, H, W.GAMMA)
+    # Both sides round the same float64 matrix to bf16: entries differ by one unit in the last place where the solvers' last bits
+    # cross a rounding boundary, about (solver error / 2^-8) of them; an entry near zero differs by the solvers' error.
+    unit = np.maximum(np.abs(ref), 1e-9 * np.abs(ref).max()) * 2.0 ** -7
+    assert np.all(np.abs(T - ref) <= unit) and np.mean(T != ref) < 1e-3
+    for h in range(20):
+        np.testing.assert_allclose(Ti[h].T @ T[h], np.eye(128), atol=1e-4)
+
+
+def test_repeated_eigenvalues():
+    """M = H = I: any orthonormal basis diagonalises A, so T is compared through what defines it: T^T T = c^2 / 128^0 * I up to bf16."""
+    T, Ti = _build(np.eye(128)[None], np.eye(128)[None].copy(), 0.0)
+    g = T[0].T @ T[0]
+    np.testing.assert_allclose(g, g[0, 0] * np.eye(128), atol=2.0 ** -6 * g[0, 0])
+    np.testing.assert_allclose(Ti[0].T @ T[0], np.eye(128), atol=1e-4)
+
+
+@pytest.mark.parametrize("which", ["hessian", "gram"])
+def test_indefinite_statistics_are_refused(which):
+    from paper_2609_38121_b200 import binding as B
+    rng = np.random.default_rng(6)
+    good, bad = _spd(rng, 2.0, 1.0), _spd(rng, 2.0, 1.0)
+    bad -= 0.5 * np.eye(128)                            # eigenvalues on both sides of zero
+    M, H = (good, bad) if which == "hessian" else (bad, good)
+    with pytest.raises(B.WushkvError) as e:
+        _build(M[None].copy(), H[None].copy(), 0.0)
+    assert e.value.status == B.ENOTPD
