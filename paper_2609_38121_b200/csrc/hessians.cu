@@ -6,15 +6,19 @@
 // which is the appendix's key / value Hessian with the sums over s and t exchanged.  Expanding the bilinear form,
 //   A_{gg'}(t) = W2 - W1 . (Gamma_{gg'} o_{g',t}) - W1 . (Gamma_{g'g} o_{g,t}) + W0 o_{g,t} . (Gamma_{gg'} o_{g',t}),
 //   W0 = sum_s w_s,  W1 = sum_s w_s v_s,  W2 = sum_s w_s (v_s^T Gamma_{gg'} v_s),  w_s = p_{g,t,s} p_{g',t,s},
-// so one pass over the causal probabilities with attention-like reductions suffices; A_{gg'} = A_{g'g}.
+// and, with the sum over s kept together (no cancellation between the terms of the expansion),
+//   A_{gg'}(t) = sum_s w_s (alpha_{gg'}(s) - v_s . U_{gg'}(t) + kappa_{gg'}(t)),   alpha = v_s . Gamma_{gg'} v_s,
+//   U = Gamma_{gg'} o_{g',t} + Gamma_{g'g} o_{g,t},   kappa = o_{g,t} . Gamma_{gg'} o_{g',t},   A_{gg'} = A_{g'g}.
 //
-// Five small kernels, fp32 arithmetic with float64 accumulation of the final sums (calibration is offline: clarity
-// and exactness before speed; cost O(S^2 G^2 d) per head):
-//   gamma_kernel      Gamma_{gg'} for all ordered pairs
-//   rows_kernel       causal softmax statistics (max, 1 / sum) and head outputs o_{g,t}
-//   project_kernel    u_{gg'}(t) = Gamma_{gg'} o_{g',t} and alpha_{gg'}(s) = v_s^T Gamma_{gg'} v_s
-//   pairs_kernel      W0, W1, W2 per (t, pair g <= g'), then A_{gg'}(t)
-//   reduce_kernel     H_K and H_V (float64, added to the caller's accumulators)
+// Every step is a contraction over 128 channels or over positions, done as register-blocked fp32 products out of shared
+// memory (with a warp per row, a CTA per position and the sums over s as vectors of 128 channels per pair, 1024 tokens of 32 / 8
+// heads took 6.0 ms, every value fetched being used for one or two multiplications; now 1.4 ms, pairs_kernel 0.61, rows_kernel 0.37):
+//   gamma_kernel      Gamma_{gg'}, 128 x 128 x d_model, float64 across groups of 16
+//   rows_kernel       causal softmax statistics (max, 1 / sum) and head outputs o_{g,t}: 64 x 64 tiles
+//   project_kernel    U, kappa and alpha: 64 x 128 tiles
+//   pairs_kernel      logits and v_s . U for (position t; 4 keys s) per thread, all query heads and up to 10 pairs; A, W0
+//   key_kernel        H_K: sum over (t, g) of q_{g,t} (sum_g' A_{gg'}(t) q_{g',t})^T, float64 across groups of 16
+//   value_kernel      H_V = 2 sum_{gg'} (sum_t W0) Gamma_{gg'}
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -26,7 +30,6 @@
 namespace wushkv {
 namespace {
 
-constexpr int HS_TILE = 32;                // cache positions per staged tile
 constexpr int HS_PITCH = D + 4;            // floats per staged row
 
 struct HessParams {
@@ -37,264 +40,468 @@ struct HessParams {
     const unsigned short* V;     // [S][n_kv][D]
     const float* W_O;            // [n_q][D][d_model]
     float* gamma;                // [n_kv][G][G][D][D]
-    float* row_m;                // [S][n_q] running maximum of the logits (natural log domain)
+    float* row_m;                // [S][n_q] maximum of the logits (natural log domain)
     float* row_linv;             // [S][n_q] 1 / sum exp
     float* Oh;                   // [S][n_q][D]
-    float* U;                    // [S][n_kv][G][G][D]   u_{gg'}(t) = Gamma_{gg'} o_{g',t}
-    float* alpha;                // [S][n_kv][G][G]
+    float* U;                    // [S][n_kv][n_pairs][D]
+    float* kappa;                // [S][n_kv][n_pairs]
+    float* alpha;                // [S][n_kv][n_pairs]
     float* A;                    // [S][n_kv][n_pairs]   pairs g <= g' in row-major order
     float* W0;                   // [S][n_kv][n_pairs]
     double* H_K;                 // [n_kv][D][D]
     double* H_V;
 };
+__device__ __forceinline__ void pair_heads(int k, int G, int& g, int& gp) {
+    g = 0;
+    while (k >= G - g) { k -= G - g; ++g; }
+    gp = g + k;
+}
+__device__ __forceinline__ float4 bf16x4(const unsigned short* p) {
+    const uint2 r = *reinterpret_cast<const uint2*>(p);
+    return make_float4(bf16_bits_to_float(r.x & 0xffff), bf16_bits_to_float(r.x >> 16), bf16_bits_to_float(r.y & 0xffff), bf16_bits_to_float(r.y >> 16));
+}
+__device__ __forceinline__ void fma4(float& acc, const float4& a, const float4& b) { acc = fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.x, b.x, acc)))); }
 
-// Gamma_{gg'}[i][j] = sum_m W_g[i][m] W_g'[j][m]; grid (D/16, D/16, n_kv*G*G), 16 x 16 threads.
-__global__ void __launch_bounds__(256) gamma_kernel(HessParams P) {
-    __shared__ float a_s[16][17], b_s[16][17];
-    const int z = blockIdx.z, h = z / (P.G * P.G), g = (z / P.G) % P.G, gp = z % P.G;
+// C[i][j] += sum_k a[k][i] b[k][j] for one staged group of 16 k; thread: rows 4 (tid >> 4) .., columns (tid & 15) + 16 e.
+constexpr int OUTER_K = 16;
+__device__ __forceinline__ void outer_group(const float (*a)[HS_PITCH], const float (*b)[HS_PITCH], double (&acc)[4][8]) {
+    const int i0 = 4 * (threadIdx.x >> 4), j0 = threadIdx.x & 15;
+    float part[4][8];
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int e = 0; e < 8; ++e) part[r][e] = 0.f;
+#pragma unroll 4
+    for (int k = 0; k < OUTER_K; ++k) {
+        const float4 av = *reinterpret_cast<const float4*>(&a[k][i0]);
+        float bv[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) bv[e] = b[k][j0 + 16 * e];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            part[0][e] = fmaf(av.x, bv[e], part[0][e]); part[1][e] = fmaf(av.y, bv[e], part[1][e]);
+            part[2][e] = fmaf(av.z, bv[e], part[2][e]); part[3][e] = fmaf(av.w, bv[e], part[3][e]);
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int e = 0; e < 8; ++e) acc[r][e] += static_cast<double>(part[r][e]);
+}
+
+// Gamma_{gg'}[i][j] = sum_m W_g[i][m] W_g'[j][m] and its transpose Gamma_{g'g}; grid (pairs, n_kv), 512 threads.
+__global__ void __launch_bounds__(512) gamma_kernel(HessParams P) {
+    __shared__ __align__(16) float a_s[OUTER_K][HS_PITCH], b_s[OUTER_K][HS_PITCH];
+    int g, gp;
+    pair_heads(blockIdx.x, P.G, g, gp);
+    const int h = blockIdx.y, tid = threadIdx.x;
     const float* Wa = P.W_O + static_cast<long long>(h * P.G + g) * D * P.d_model;
     const float* Wb = P.W_O + static_cast<long long>(h * P.G + gp) * D * P.d_model;
-    const int tx = threadIdx.x, ty = threadIdx.y, i = blockIdx.y * 16 + ty, j = blockIdx.x * 16 + tx;
-    double acc = 0.0;
-    for (int m0 = 0; m0 < P.d_model; m0 += 16) {
-        a_s[ty][tx] = m0 + tx < P.d_model ? Wa[static_cast<long long>(blockIdx.y * 16 + ty) * P.d_model + m0 + tx] : 0.f;
-        b_s[ty][tx] = m0 + tx < P.d_model ? Wb[static_cast<long long>(blockIdx.x * 16 + ty) * P.d_model + m0 + tx] : 0.f;
-        __syncthreads();
-        float part = 0.f;
+    double acc[4][8] = {};
+    for (int m0 = 0; m0 < P.d_model; m0 += OUTER_K) {
+        float ta[4], tb[4];
 #pragma unroll
-        for (int m = 0; m < 16; ++m) part = fmaf(a_s[ty][m], b_s[tx][m], part);
-        acc += static_cast<double>(part);
+        for (int n = 0; n < 4; ++n) {
+            const int item = tid + 512 * n, i = item >> 4, m = m0 + (item & 15);
+            ta[n] = m < P.d_model ? Wa[static_cast<long long>(i) * P.d_model + m] : 0.f;
+            tb[n] = m < P.d_model ? Wb[static_cast<long long>(i) * P.d_model + m] : 0.f;
+        }
         __syncthreads();
+#pragma unroll
+        for (int n = 0; n < 4; ++n) { const int item = tid + 512 * n; a_s[item & 15][item >> 4] = ta[n]; b_s[item & 15][item >> 4] = tb[n]; }
+        __syncthreads();
+        outer_group(a_s, b_s, acc);
     }
-    P.gamma[(static_cast<long long>(z) * D + i) * D + j] = static_cast<float>(acc);
+    float* out = P.gamma + (static_cast<long long>(h * P.G + g) * P.G + gp) * D * D;
+    float* outT = P.gamma + (static_cast<long long>(h * P.G + gp) * P.G + g) * D * D;
+    const int i0 = 4 * (tid >> 4), j0 = tid & 15;
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const float v = static_cast<float>(acc[r][e]);
+            out[(i0 + r) * D + j0 + 16 * e] = v;
+            if (g != gp) outT[(j0 + 16 * e) * D + i0 + r] = v;
+        }
 }
 
-// One warp per (t, query head): causal softmax statistics and o = sum_s p_s v_s.  grid (S, n_kv), G warps.
-__global__ void rows_kernel(HessParams P) {
-    const int t = blockIdx.x, h = blockIdx.y, g = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int j = h * P.G + g;
-    const unsigned short* qrow = P.Q + (static_cast<long long>(t) * P.n_q + j) * D;
-    float q[4];
-    {
-        const uint2 raw = *reinterpret_cast<const uint2*>(qrow + 4 * lane);
-        q[0] = bf16_bits_to_float(raw.x & 0xffff); q[1] = bf16_bits_to_float(raw.x >> 16);
-        q[2] = bf16_bits_to_float(raw.y & 0xffff); q[3] = bf16_bits_to_float(raw.y >> 16);
+// Causal softmax statistics and o = sum_s p_s v_s of 64 positions of one query head, over tiles of 64 keys.  256 threads: thread
+// (r, c) = (tid >> 4, tid & 15) holds the logits of positions 4 r .. and keys c + 16 e, then the outputs of the same positions
+// and channels 4 c .., 64 + 4 c ...  grid (position tiles, n_q), the longest first.
+constexpr int RT = 64;
+struct RowsSmem { float q[RT][HS_PITCH], kv[RT][HS_PITCH], p[RT][RT + 4]; };
+__global__ void __launch_bounds__(256, 2) rows_kernel(HessParams P) {
+    extern __shared__ __align__(16) unsigned char hs_smem[];
+    RowsSmem& sm = *reinterpret_cast<RowsSmem*>(hs_smem);
+    const int t0 = (gridDim.x - 1 - blockIdx.x) * RT, j = blockIdx.y, h = j / P.G, tid = threadIdx.x, r = tid >> 4, c = tid & 15;
+    for (int item = tid; item < RT * 32; item += 256) {
+        const int row = item >> 5, piece = item & 31;
+        *reinterpret_cast<float4*>(&sm.q[row][4 * piece]) =
+            t0 + row < P.S ? bf16x4(P.Q + (static_cast<long long>(t0 + row) * P.n_q + j) * D + 4 * piece) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    float m = -INFINITY, l = 0.f, o[4] = {0.f, 0.f, 0.f, 0.f};
-    for (int s = 0; s <= t; ++s) {
-        const uint2 kr = __ldg(reinterpret_cast<const uint2*>(P.K + (static_cast<long long>(s) * P.n_kv + h) * D) + lane);
-        float part = q[0] * bf16_bits_to_float(kr.x & 0xffff) + q[1] * bf16_bits_to_float(kr.x >> 16) +
-                     q[2] * bf16_bits_to_float(kr.y & 0xffff) + q[3] * bf16_bits_to_float(kr.y >> 16);
+    float m[4], l[4], o[4][8];
 #pragma unroll
-        for (int off = 16; off >= 1; off >>= 1) part += __shfl_xor_sync(0xffffffffu, part, off);
-        const float z = part * P.inv_tau;
-        const float mn = fmaxf(m, z);
-        const float sc = __expf(m - mn), p = __expf(z - mn);
-        const uint2 vr = __ldg(reinterpret_cast<const uint2*>(P.V + (static_cast<long long>(s) * P.n_kv + h) * D) + lane);
-        l = l * sc + p;
-        o[0] = o[0] * sc + p * bf16_bits_to_float(vr.x & 0xffff); o[1] = o[1] * sc + p * bf16_bits_to_float(vr.x >> 16);
-        o[2] = o[2] * sc + p * bf16_bits_to_float(vr.y & 0xffff); o[3] = o[3] * sc + p * bf16_bits_to_float(vr.y >> 16);
-        m = mn;
+    for (int a = 0; a < 4; ++a) {
+        m[a] = -INFINITY; l[a] = 0.f;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) o[a][e] = 0.f;
     }
-    const float linv = 1.f / l;
-    if (lane == 0) { P.row_m[static_cast<long long>(t) * P.n_q + j] = m; P.row_linv[static_cast<long long>(t) * P.n_q + j] = linv; }
-    *reinterpret_cast<float4*>(P.Oh + (static_cast<long long>(t) * P.n_q + j) * D + 4 * lane) = make_float4(o[0] * linv, o[1] * linv, o[2] * linv, o[3] * linv);
+    for (int s0 = 0; s0 < min(t0 + RT, P.S); s0 += RT) {
+        auto stage = [&](const unsigned short* X) {
+            for (int item = tid; item < RT * 32; item += 256) {
+                const int row = item >> 5, piece = item & 31;
+                *reinterpret_cast<float4*>(&sm.kv[row][4 * piece]) =
+                    s0 + row < P.S ? bf16x4(X + (static_cast<long long>(s0 + row) * P.n_kv + h) * D + 4 * piece) : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+        };
+        __syncthreads();
+        stage(P.K);
+        __syncthreads();
+        float z[4][4] = {};
+#pragma unroll 2
+        for (int k = 0; k < D; k += 4) {
+            float4 qa[4], kb[4];
+#pragma unroll
+            for (int a = 0; a < 4; ++a) { qa[a] = *reinterpret_cast<const float4*>(&sm.q[4 * r + a][k]); kb[a] = *reinterpret_cast<const float4*>(&sm.kv[c + 16 * a][k]); }
+#pragma unroll
+            for (int a = 0; a < 4; ++a)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) fma4(z[a][e], qa[a], kb[e]);
+        }
+        __syncthreads();
+        stage(P.V);
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            const int t = t0 + 4 * r + a;
+            float mx = -INFINITY;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) { z[a][e] = s0 + c + 16 * e <= t ? z[a][e] * P.inv_tau : -INFINITY; mx = fmaxf(mx, z[a][e]); }
+#pragma unroll
+            for (int off = 8; off >= 1; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+            const float mn = fmaxf(m[a], mx), sc = __expf(m[a] - mn);        // every position sees a key of the first tile: mn is finite
+            float sum = 0.f;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) { const float p = __expf(z[a][e] - mn); sm.p[4 * r + a][c + 16 * e] = p; sum += p; }
+            l[a] = l[a] * sc + sum;                                      // of this thread's keys
+            m[a] = mn;
+#pragma unroll
+            for (int e = 0; e < 8; ++e) o[a][e] *= sc;
+        }
+        __syncthreads();
+#pragma unroll 2
+        for (int k = 0; k < RT; k += 4) {
+            float4 pa[4];
+#pragma unroll
+            for (int a = 0; a < 4; ++a) pa[a] = *reinterpret_cast<const float4*>(&sm.p[4 * r + a][k]);
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) {
+                const float4 va = *reinterpret_cast<const float4*>(&sm.kv[k + kk][4 * c]), vb = *reinterpret_cast<const float4*>(&sm.kv[k + kk][64 + 4 * c]);
+#pragma unroll
+                for (int a = 0; a < 4; ++a) {
+                    const float p = kk == 0 ? pa[a].x : kk == 1 ? pa[a].y : kk == 2 ? pa[a].z : pa[a].w;
+                    o[a][0] = fmaf(p, va.x, o[a][0]); o[a][1] = fmaf(p, va.y, o[a][1]); o[a][2] = fmaf(p, va.z, o[a][2]); o[a][3] = fmaf(p, va.w, o[a][3]);
+                    o[a][4] = fmaf(p, vb.x, o[a][4]); o[a][5] = fmaf(p, vb.y, o[a][5]); o[a][6] = fmaf(p, vb.z, o[a][6]); o[a][7] = fmaf(p, vb.w, o[a][7]);
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+#pragma unroll
+        for (int off = 8; off >= 1; off >>= 1) l[a] += __shfl_xor_sync(0xffffffffu, l[a], off);
+        const int t = t0 + 4 * r + a;
+        if (t >= P.S) continue;
+        const float linv = 1.f / l[a];
+        if (c == 0) { P.row_m[static_cast<long long>(t) * P.n_q + j] = m[a]; P.row_linv[static_cast<long long>(t) * P.n_q + j] = linv; }
+        float* dst = P.Oh + (static_cast<long long>(t) * P.n_q + j) * D + 4 * c;
+        *reinterpret_cast<float4*>(dst) = make_float4(o[a][0] * linv, o[a][1] * linv, o[a][2] * linv, o[a][3] * linv);
+        *reinterpret_cast<float4*>(dst + 64) = make_float4(o[a][4] * linv, o[a][5] * linv, o[a][6] * linv, o[a][7] * linv);
+    }
 }
 
-// y = Gamma x for a 128-vector x held as 4 values per lane; returns y[r0 + lane] for the 32 rows r0.. in turn.
-__device__ __noinline__ void gamma_matvec(const float* gam, const float (&x)[4], int lane, float (&y)[4]) {
+// U, kappa and alpha of 64 positions and one pair: y = Gamma x for 64 rows x, 256 threads; thread (r, c) holds positions 4 r .. and
+// channels 4 c .., 64 + 4 c ...  grid (position tiles, pairs, n_kv).
+struct ProjectSmem { float x[RT][HS_PITCH], gam[D][D]; };
+__global__ void __launch_bounds__(256, 2) project_kernel(HessParams P) {
+    extern __shared__ __align__(16) unsigned char hs_smem[];
+    ProjectSmem& sm = *reinterpret_cast<ProjectSmem*>(hs_smem);
+    int g, gp;
+    pair_heads(blockIdx.y, P.G, g, gp);
+    const int t0 = blockIdx.x * RT, h = blockIdx.z, tid = threadIdx.x, r = tid >> 4, c = tid & 15;
+    float y[4][8];
+    auto clear = [&] {
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+            for (int e = 0; e < 8; ++e) y[a][e] = 0.f;
+    };
+    auto stage_gamma = [&](int ga, int gb) {             // Gamma_{ga gb} x = sum_j x_j Gamma_{gb ga}[j][.]: rows of the transpose
+        const float4* src = reinterpret_cast<const float4*>(P.gamma + (static_cast<long long>(h * P.G + gb) * P.G + ga) * D * D);
+        float4* dst = reinterpret_cast<float4*>(&sm.gam[0][0]);
+#pragma unroll 4
+        for (int k = tid; k < D * D / 4; k += 256) dst[k] = src[k];
+    };
+    auto stage_o = [&](int gx) {
+#pragma unroll 4
+        for (int item = tid; item < RT * 32; item += 256) {
+            const int row = item >> 5, piece = item & 31;
+            *reinterpret_cast<float4*>(&sm.x[row][4 * piece]) =
+                t0 + row < P.S ? *reinterpret_cast<const float4*>(P.Oh + (static_cast<long long>(t0 + row) * P.n_q + h * P.G + gx) * D + 4 * piece) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    };
+    auto product = [&] {
+#pragma unroll 2
+        for (int k = 0; k < D; k += 4) {
+            float4 xa[4];
+#pragma unroll
+            for (int a = 0; a < 4; ++a) xa[a] = *reinterpret_cast<const float4*>(&sm.x[4 * r + a][k]);
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) {
+                const float4 ga = *reinterpret_cast<const float4*>(&sm.gam[k + kk][4 * c]), gb = *reinterpret_cast<const float4*>(&sm.gam[k + kk][64 + 4 * c]);
+#pragma unroll
+                for (int a = 0; a < 4; ++a) {
+                    const float x = kk == 0 ? xa[a].x : kk == 1 ? xa[a].y : kk == 2 ? xa[a].z : xa[a].w;
+                    y[a][0] = fmaf(x, ga.x, y[a][0]); y[a][1] = fmaf(x, ga.y, y[a][1]); y[a][2] = fmaf(x, ga.z, y[a][2]); y[a][3] = fmaf(x, ga.w, y[a][3]);
+                    y[a][4] = fmaf(x, gb.x, y[a][4]); y[a][5] = fmaf(x, gb.y, y[a][5]); y[a][6] = fmaf(x, gb.z, y[a][6]); y[a][7] = fmaf(x, gb.w, y[a][7]);
+                }
+            }
+        }
+    };
+    auto dot_rows = [&](float* out) {                    // out[t] = x_t . y_t with the staged rows
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            const float4 xa = *reinterpret_cast<const float4*>(&sm.x[4 * r + a][4 * c]), xb = *reinterpret_cast<const float4*>(&sm.x[4 * r + a][64 + 4 * c]);
+            float d = 0.f;
+            fma4(d, xa, make_float4(y[a][0], y[a][1], y[a][2], y[a][3]));
+            fma4(d, xb, make_float4(y[a][4], y[a][5], y[a][6], y[a][7]));
+#pragma unroll
+            for (int off = 8; off >= 1; off >>= 1) d += __shfl_xor_sync(0xffffffffu, d, off);
+            if (c == 0 && t0 + 4 * r + a < P.S) out[(static_cast<long long>(t0 + 4 * r + a) * P.n_kv + h) * P.n_pairs + blockIdx.y] = d;
+        }
+    };
+    // Gamma_{gg'} o_{g'}, its product with o_g, then + Gamma_{g'g} o_g
+    clear();
+    stage_gamma(g, gp);
+    stage_o(gp);
+    __syncthreads();
+    product();
+    __syncthreads();
+    stage_o(g);
+    if (g != gp) stage_gamma(gp, g);
+    __syncthreads();
+    dot_rows(P.kappa);
+    product();                                           // (g = g': the same once more)
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+        const int t = t0 + 4 * r + a;
+        if (t >= P.S) continue;
+        float* dst = P.U + ((static_cast<long long>(t) * P.n_kv + h) * P.n_pairs + blockIdx.y) * D + 4 * c;
+        *reinterpret_cast<float4*>(dst) = make_float4(y[a][0], y[a][1], y[a][2], y[a][3]);
+        *reinterpret_cast<float4*>(dst + 64) = make_float4(y[a][4], y[a][5], y[a][6], y[a][7]);
+    }
+    __syncthreads();
+    for (int item = tid; item < RT * 32; item += 256) {
+        const int row = item >> 5, piece = item & 31;
+        *reinterpret_cast<float4*>(&sm.x[row][4 * piece]) =
+            t0 + row < P.S ? bf16x4(P.V + (static_cast<long long>(t0 + row) * P.n_kv + h) * D + 4 * piece) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    __syncthreads();
+    clear();
+    product();                                           // v . Gamma_{g'g} v = v . Gamma_{gg'} v
+    dot_rows(P.alpha);
+}
+
+// A and W0 of 16 positions and NC pairs (from pair0 on): thread (t, c) holds the logits of all heads and v . U of the pairs for its
+// position and keys c + 16 e of a tile of 64.  grid (position tiles, pair chunks, n_kv), 256 threads.
+template <int G, int NC>
+struct PairsSmem { float q[G][16][HS_PITCH], u[NC][16][HS_PITCH], k[RT][HS_PITCH], v[RT][HS_PITCH], al[NC][RT]; };
+constexpr int pair_chunks(int G) { return (G * (G + 1) / 2 + 9) / 10; }      // what fits in shared memory beside the heads' queries
+constexpr int pairs_per_chunk(int G) { return (G * (G + 1) / 2 + pair_chunks(G) - 1) / pair_chunks(G); }
+template <int G, int NC>
+__global__ void __launch_bounds__(256, 1) pairs_kernel(HessParams P) {
+    extern __shared__ __align__(16) unsigned char hs_smem[];
+    PairsSmem<G, NC>& sm = *reinterpret_cast<PairsSmem<G, NC>*>(hs_smem);
+    const int t0 = (gridDim.x - 1 - blockIdx.x) * 16, pair0 = blockIdx.y * NC, h = blockIdx.z, tid = threadIdx.x, tr = tid >> 4, c = tid & 15;
+    const int t = t0 + tr, n_pairs = min(NC, P.n_pairs - pair0);
+    for (int item = tid; item < G * 16 * 32; item += 256) {
+        const int g = item >> 9, row = (item >> 5) & 15, piece = item & 31;
+        *reinterpret_cast<float4*>(&sm.q[g][row][4 * piece]) =
+            t0 + row < P.S ? bf16x4(P.Q + (static_cast<long long>(t0 + row) * P.n_q + h * G + g) * D + 4 * piece) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    for (int item = tid; item < NC * 16 * 32; item += 256) {
+        const int k = item >> 9, row = (item >> 5) & 15, piece = item & 31;
+        *reinterpret_cast<float4*>(&sm.u[k][row][4 * piece]) =
+            t0 + row < P.S && k < n_pairs ? *reinterpret_cast<const float4*>(P.U + ((static_cast<long long>(t0 + row) * P.n_kv + h) * P.n_pairs + pair0 + k) * D + 4 * piece)
+                                          : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    float rm[G], rl[G], kap[NC], asum[NC], wsum[NC];
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+        const long long row = static_cast<long long>(min(t, P.S - 1)) * P.n_q + h * G + g;
+        rm[g] = P.row_m[row]; rl[g] = P.row_linv[row];
+    }
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+        kap[k] = k < n_pairs ? P.kappa[(static_cast<long long>(min(t, P.S - 1)) * P.n_kv + h) * P.n_pairs + pair0 + k] : 0.f;
+        asum[k] = wsum[k] = 0.f;
+    }
+    for (int s0 = 0; s0 < min(t0 + 16, P.S); s0 += RT) {
+        __syncthreads();
+#pragma unroll 2
+        for (int item = tid; item < RT * 32; item += 256) {
+            const int row = item >> 5, piece = item & 31;
+            const bool in = s0 + row < P.S;
+            const long long off = (static_cast<long long>(in ? s0 + row : 0) * P.n_kv + h) * D + 4 * piece;
+            *reinterpret_cast<float4*>(&sm.k[row][4 * piece]) = in ? bf16x4(P.K + off) : make_float4(0.f, 0.f, 0.f, 0.f);
+            *reinterpret_cast<float4*>(&sm.v[row][4 * piece]) = in ? bf16x4(P.V + off) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+        for (int item = tid; item < NC * RT; item += 256) {
+            const int k = item / RT, row = item % RT;
+            sm.al[k][row] = s0 + row < P.S && k < n_pairs ? P.alpha[(static_cast<long long>(s0 + row) * P.n_kv + h) * P.n_pairs + pair0 + k] : 0.f;
+        }
+        __syncthreads();
+        float p[G][4], rr[NC][4];
+#pragma unroll
+        for (int g = 0; g < G; ++g) p[g][0] = p[g][1] = p[g][2] = p[g][3] = 0.f;
+#pragma unroll
+        for (int k = 0; k < NC; ++k) rr[k][0] = rr[k][1] = rr[k][2] = rr[k][3] = 0.f;
 #pragma unroll 1
-    for (int blk = 0; blk < 4; ++blk) {
-        float part[32];
+        for (int k4 = 0; k4 < D; k4 += 4) {
+            float4 b[4];
 #pragma unroll
-        for (int r = 0; r < 32; ++r) {
-            const float4 gr = __ldg(reinterpret_cast<const float4*>(gam + static_cast<long long>(32 * blk + r) * D) + lane);
-            part[r] = fmaf(gr.x, x[0], fmaf(gr.y, x[1], fmaf(gr.z, x[2], gr.w * x[3])));
+            for (int e = 0; e < 4; ++e) b[e] = *reinterpret_cast<const float4*>(&sm.k[c + 16 * e][k4]);
+#pragma unroll
+            for (int g = 0; g < G; ++g) {
+                const float4 a = *reinterpret_cast<const float4*>(&sm.q[g][tr][k4]);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) fma4(p[g][e], a, b[e]);
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e) b[e] = *reinterpret_cast<const float4*>(&sm.v[c + 16 * e][k4]);
+#pragma unroll
+            for (int k = 0; k < NC; ++k) {
+                const float4 a = *reinterpret_cast<const float4*>(&sm.u[k][tr][k4]);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) fma4(rr[k][e], a, b[e]);
+            }
         }
-        const float tot = warp_transpose_reduce(part, lane);  // lane L: y[32 blk + L]
-        if (blk == 0) y[0] = tot; else if (blk == 1) y[1] = tot; else if (blk == 2) y[2] = tot; else y[3] = tot;
+#pragma unroll
+        for (int g = 0; g < G; ++g)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) p[g][e] = s0 + c + 16 * e <= t ? __expf(p[g][e] * P.inv_tau - rm[g]) * rl[g] : 0.f;
+        // pairs in order, from the chunk's first one on (chunk boundaries are the same for every thread)
+        int index = 0;
+#pragma unroll
+        for (int g = 0; g < G; ++g)
+#pragma unroll
+            for (int gp = g; gp < G; ++gp, ++index) {
+#pragma unroll
+                for (int k = 0; k < NC; ++k) {
+                    if (NC < G * (G + 1) / 2 ? index == pair0 + k : index == k) {
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            const float w = p[g][e] * p[gp][e];
+                            wsum[k] += w;
+                            asum[k] = fmaf(w, (sm.al[k][c + 16 * e] - rr[k][e]) + kap[k], asum[k]);
+                        }
+                    }
+                }
+            }
+    }
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+#pragma unroll
+        for (int off = 8; off >= 1; off >>= 1) { asum[k] += __shfl_xor_sync(0xffffffffu, asum[k], off); wsum[k] += __shfl_xor_sync(0xffffffffu, wsum[k], off); }
+        if (c == 0 && t < P.S && k < n_pairs) {
+            const long long o = (static_cast<long long>(t) * P.n_kv + h) * P.n_pairs + pair0 + k;
+            P.A[o] = asum[k];
+            P.W0[o] = wsum[k];
+        }
     }
 }
 
-// One warp per (position, ordered pair): u_{gg'}(t) = Gamma_{gg'} o_{g',t} and alpha_{gg'}(s) = v_s . Gamma_{gg'} v_s.
-// grid (S, n_kv), up to 16 warps that share the G*G ordered pairs.
-__global__ void project_kernel(HessParams P) {
-    const int t = blockIdx.x, h = blockIdx.y, lane = threadIdx.x & 31;
-    for (int w = threadIdx.x >> 5; w < P.G * P.G; w += blockDim.x >> 5) {
-    const int g = w / P.G, gp = w % P.G;
-    const float* gam = P.gamma + (static_cast<long long>(h * P.G + g) * P.G + gp) * D * D;
-    float x[4], y[4];
-    {
-        const float4 o = *reinterpret_cast<const float4*>(P.Oh + (static_cast<long long>(t) * P.n_q + h * P.G + gp) * D + 4 * lane);
-        x[0] = o.x; x[1] = o.y; x[2] = o.z; x[3] = o.w;
-    }
-    gamma_matvec(gam, x, lane, y);
-    float* u = P.U + ((static_cast<long long>(t) * P.n_kv + h) * P.G * P.G + w) * D;
-#pragma unroll
-    for (int blk = 0; blk < 4; ++blk) u[32 * blk + lane] = y[blk];
-    {
-        const uint2 vr = *reinterpret_cast<const uint2*>(P.V + (static_cast<long long>(t) * P.n_kv + h) * D + 4 * lane);
-        x[0] = bf16_bits_to_float(vr.x & 0xffff); x[1] = bf16_bits_to_float(vr.x >> 16);
-        x[2] = bf16_bits_to_float(vr.y & 0xffff); x[3] = bf16_bits_to_float(vr.y >> 16);
-    }
-    gamma_matvec(gam, x, lane, y);
-    // v . y: lane L holds y[32 blk + L]; the matching v entries are fetched one by one
-    float dot = 0.f;
-#pragma unroll
-    for (int blk = 0; blk < 4; ++blk)
-        dot = fmaf(y[blk], bf16_bits_to_float(P.V[(static_cast<long long>(t) * P.n_kv + h) * D + 32 * blk + lane]), dot);
-#pragma unroll
-    for (int off = 16; off >= 1; off >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, off);
-    if (lane == 0) P.alpha[(static_cast<long long>(t) * P.n_kv + h) * P.G * P.G + w] = dot;
-    }
-}
-
-// One CTA of 128 threads (one per channel) per (t, h): the pair sums W0, W1, W2 over s <= t, then A_{gg'}(t).
+// H_K[h][i][j] += (2 / tau^2) sum_t sum_g q_{g,t}[i] (sum_g' A_{gg'}(t) q_{g',t}[j]): grid (slices of positions, n_kv), 512 threads.
+constexpr int KEY_SLICE = 64;
 template <int G>
-__global__ void __launch_bounds__(128) pairs_kernel(HessParams P) {
-    constexpr int NP = G * (G + 1) / 2;
-    __shared__ float k_s[HS_TILE][HS_PITCH], v_s[HS_TILE][HS_PITCH];
-    __shared__ float q_s[G][D];
-    __shared__ float p_s[G][HS_TILE];
-    __shared__ float al_s[HS_TILE][G * G];
-    __shared__ float red_s[4][3 * NP];
-    const int t = blockIdx.x, h = blockIdx.y, c = threadIdx.x, lane = c & 31, warp = c >> 5;
-    for (int g = 0; g < G; ++g) q_s[g][c] = bf16_bits_to_float(P.Q[(static_cast<long long>(t) * P.n_q + h * G + g) * D + c]);
-    float w1[NP];
-    float w0 = 0.f, w2 = 0.f;            // thread `pair` (< NP) accumulates W0 and W2 of its pair
-#pragma unroll
-    for (int k = 0; k < NP; ++k) w1[k] = 0.f;
-    int my_g = 0, my_gp = 0;
-    if (c < NP) { int k = c; while (k >= G - my_g) { k -= G - my_g; ++my_g; } my_gp = my_g + k; }
-    for (int s0 = 0; s0 <= t; s0 += HS_TILE) {
+__global__ void __launch_bounds__(512) key_kernel(HessParams P) {
+    __shared__ __align__(16) float a_s[OUTER_K][HS_PITCH], b_s[OUTER_K][HS_PITCH];
+    __shared__ float c_s[OUTER_K / G > 0 ? OUTER_K / G : 1][G][G];
+    constexpr int TG = OUTER_K / G;                      // positions per staged group (G = 1 .. 8: at least 2)
+    const int h = blockIdx.y, tid = threadIdx.x, t_end = min(static_cast<int>(blockIdx.x + 1) * KEY_SLICE, P.S);
+    double acc[4][8] = {};
+    for (int t0 = blockIdx.x * KEY_SLICE; t0 < t_end; t0 += TG) {
         __syncthreads();
-        const int n = min(HS_TILE, t + 1 - s0);
-        for (int r = 0; r < HS_TILE; ++r) {
-            const bool in = r < n;
-            k_s[r][c] = in ? bf16_bits_to_float(P.K[(static_cast<long long>(s0 + r) * P.n_kv + h) * D + c]) : 0.f;
-            v_s[r][c] = in ? bf16_bits_to_float(P.V[(static_cast<long long>(s0 + r) * P.n_kv + h) * D + c]) : 0.f;
+        for (int item = tid; item < TG * G * G; item += 512) {
+            const int t = t0 + item / (G * G), g = item / G % G, gp = item % G, lo = min(g, gp), hi = max(g, gp);
+            c_s[item / (G * G)][g][gp] = t < t_end ? P.A[(static_cast<long long>(t) * P.n_kv + h) * P.n_pairs + lo * G - lo * (lo - 1) / 2 + hi - lo] : 0.f;
         }
-        for (int idx = c; idx < HS_TILE * G * G; idx += 128) {
-            const int r = idx / (G * G);
-            al_s[r][idx % (G * G)] = r < n ? P.alpha[(static_cast<long long>(s0 + r) * P.n_kv + h) * G * G + idx % (G * G)] : 0.f;
+        for (int item = tid; item < OUTER_K * 32; item += 512) {
+            const int row = item >> 5, t = t0 + row / G, piece = item & 31;
+            *reinterpret_cast<float4*>(&a_s[row][4 * piece]) =
+                row < TG * G && t < t_end ? bf16x4(P.Q + (static_cast<long long>(t) * P.n_q + h * G + row % G) * D + 4 * piece) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
         __syncthreads();
-        // probabilities: warp w takes (g, s) items w, w + 4, ...
-        for (int item = warp; item < G * HS_TILE; item += 4) {
-            const int g = item / HS_TILE, r = item % HS_TILE;
-            float part = 0.f;
+        for (int item = tid; item < OUTER_K * D; item += 512) {
+            const int row = item >> 7, ch = item & 127, tl = row / G, g = row % G;
+            float x = 0.f;
+            if (row < TG * G)
 #pragma unroll
-            for (int e = 0; e < 4; ++e) part = fmaf(q_s[g][lane + 32 * e], k_s[r][lane + 32 * e], part);
-#pragma unroll
-            for (int off = 16; off >= 1; off >>= 1) part += __shfl_xor_sync(0xffffffffu, part, off);
-            if (lane == 0) {
-                const long long row = static_cast<long long>(t) * P.n_q + h * G + g;
-                p_s[g][r] = r < n ? __expf(part * P.inv_tau - P.row_m[row]) * P.row_linv[row] : 0.f;
-            }
+                for (int gp = 0; gp < G; ++gp) x = fmaf(c_s[tl][g][gp], a_s[tl * G + gp][ch], x);
+            b_s[row][ch] = x;
         }
         __syncthreads();
-        for (int r = 0; r < n; ++r) {
-            const float v = v_s[r][c];
-            int k = 0;
-#pragma unroll
-            for (int g = 0; g < G; ++g)
-#pragma unroll
-                for (int gp = g; gp < G; ++gp, ++k) w1[k] = fmaf(p_s[g][r] * p_s[gp][r], v, w1[k]);
-        }
-        if (c < NP)
-            for (int r = 0; r < n; ++r) {
-                const float w = p_s[my_g][r] * p_s[my_gp][r];
-                w0 += w;
-                w2 = fmaf(w, al_s[r][my_g * G + my_gp], w2);
-            }
+        outer_group(a_s, b_s, acc);
     }
-    // A_{gg'} = W2 - W1 . u_{gg'} - W1 . u_{g'g} + W0 (o_g . u_{gg'}): three channel-wise dot products per pair
-    const float* Ubase = P.U + (static_cast<long long>(t) * P.n_kv + h) * G * G * D;
-    float d1[NP], d2[NP], d3[NP];
-    {
-        int k = 0;
+    const double f = 2.0 * static_cast<double>(P.inv_tau) * static_cast<double>(P.inv_tau);
+    const int i0 = 4 * (tid >> 4), j0 = tid & 15;
 #pragma unroll
-        for (int g = 0; g < G; ++g)
+    for (int r = 0; r < 4; ++r)
 #pragma unroll
-            for (int gp = g; gp < G; ++gp, ++k) {
-                const float u_a = Ubase[(g * G + gp) * D + c], u_b = Ubase[(gp * G + g) * D + c];
-                const float og = P.Oh[(static_cast<long long>(t) * P.n_q + h * G + g) * D + c];
-                d1[k] = w1[k] * u_a; d2[k] = w1[k] * u_b; d3[k] = og * u_a;
-            }
-    }
-#pragma unroll
-    for (int k = 0; k < NP; ++k) {
-#pragma unroll
-        for (int off = 16; off >= 1; off >>= 1) {
-            d1[k] += __shfl_xor_sync(0xffffffffu, d1[k], off);
-            d2[k] += __shfl_xor_sync(0xffffffffu, d2[k], off);
-            d3[k] += __shfl_xor_sync(0xffffffffu, d3[k], off);
+        for (int e = 0; e < 8; ++e) {                    // half to either side of the diagonal: symmetric like the exact sum
+            double* H = P.H_K + static_cast<long long>(h) * D * D;
+            const int i = i0 + r, j = j0 + 16 * e;
+            atomicAdd(H + i * D + j, 0.5 * f * acc[r][e]);
+            atomicAdd(H + j * D + i, 0.5 * f * acc[r][e]);
         }
-        if (lane == 0) { red_s[warp][3 * k] = d1[k]; red_s[warp][3 * k + 1] = d2[k]; red_s[warp][3 * k + 2] = d3[k]; }
+}
+
+// H_V[h] += 2 sum_{g<=g'} c_{gg'} sym(Gamma_{gg'}), c = sum_t W0(t): grid (16 row groups, n_kv), 256 threads.
+__global__ void __launch_bounds__(256) value_kernel(HessParams P) {
+    __shared__ double c_s[36];
+    const int h = blockIdx.y, tid = threadIdx.x, lane = tid & 31;
+    for (int k = tid >> 5; k < P.n_pairs; k += 8) {
+        double sum = 0.0;
+        for (int t = lane; t < P.S; t += 32) sum += static_cast<double>(P.W0[(static_cast<long long>(t) * P.n_kv + h) * P.n_pairs + k]);
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        if (lane == 0) c_s[k] = sum;
     }
     __syncthreads();
-    if (c < NP) {
-        float s1 = 0.f, s2 = 0.f, s3 = 0.f;
-        for (int w = 0; w < 4; ++w) { s1 += red_s[w][3 * c]; s2 += red_s[w][3 * c + 1]; s3 += red_s[w][3 * c + 2]; }
-        const long long o = (static_cast<long long>(t) * P.n_kv + h) * NP + c;
-        P.A[o] = w2 - s1 - s2 + w0 * s3;
-        P.W0[o] = w0;
+    for (int idx = tid; idx < D * D / 16; idx += 256) {
+        const int ij = blockIdx.x * (D * D / 16) + idx;
+        double hv = 0.0;
+        int k = 0;
+        for (int g = 0; g < P.G; ++g)
+            for (int gp = g; gp < P.G; ++gp, ++k) {
+                const double a = P.gamma[(static_cast<long long>(h * P.G + g) * P.G + gp) * D * D + ij];
+                hv += c_s[k] * (g == gp ? a : a + static_cast<double>(P.gamma[(static_cast<long long>(h * P.G + gp) * P.G + g) * D * D + ij]));
+            }
+        P.H_V[static_cast<long long>(h) * D * D + ij] += 2.0 * hv;
     }
 }
 
-// H_K[h][i][j] += (2 / tau^2) sum_t sum_{g<=g'} A(t) sym(q_g[i] q_g'[j]);  H_V[h][i][j] += 2 sum_{g<=g'} c sym(Gamma_{gg'}[i][j]),
-// c = sum_t W0(t).  grid (D/16, D/16, n_kv), 16 x 16 threads; float64 accumulation.
 template <int G>
-__global__ void __launch_bounds__(256) reduce_kernel(HessParams P) {
-    constexpr int NP = G * (G + 1) / 2;
-    __shared__ float qi_s[G][16], qj_s[G][16], a_s[NP];
-    __shared__ double c_s[NP];
-    const int h = blockIdx.z, tx = threadIdx.x, ty = threadIdx.y, tid = ty * 16 + tx;
-    const int i = blockIdx.y * 16 + ty, j = blockIdx.x * 16 + tx;
-    double hk = 0.0;
-    double csum = 0.0;                   // threads < NP: their pair's sum of W0
-    for (int t = 0; t < P.S; ++t) {
-        __syncthreads();
-        if (tid < G * 16) qi_s[tid / 16][tid % 16] = bf16_bits_to_float(P.Q[(static_cast<long long>(t) * P.n_q + h * G + tid / 16) * D + blockIdx.y * 16 + tid % 16]);
-        else if (tid < 2 * G * 16) { const int u = tid - G * 16; qj_s[u / 16][u % 16] = bf16_bits_to_float(P.Q[(static_cast<long long>(t) * P.n_q + h * G + u / 16) * D + blockIdx.x * 16 + u % 16]); }
-        if (tid < NP) {
-            a_s[tid] = P.A[(static_cast<long long>(t) * P.n_kv + h) * NP + tid];
-            csum += static_cast<double>(P.W0[(static_cast<long long>(t) * P.n_kv + h) * NP + tid]);
-        }
-        __syncthreads();
-        float part = 0.f;
-        int k = 0;
-#pragma unroll
-        for (int g = 0; g < G; ++g)
-#pragma unroll
-            for (int gp = g; gp < G; ++gp, ++k) {
-                const float outer = g == gp ? qi_s[g][ty] * qj_s[g][tx] : qi_s[g][ty] * qj_s[gp][tx] + qi_s[gp][ty] * qj_s[g][tx];
-                part = fmaf(a_s[k], outer, part);
-            }
-        hk += static_cast<double>(part);
-    }
-    __syncthreads();
-    if (tid < NP) c_s[tid] = csum;
-    __syncthreads();
-    double hv = 0.0;
-    {
-        int k = 0;
-        for (int g = 0; g < G; ++g)
-            for (int gp = g; gp < G; ++gp, ++k) {
-                const float* gam = P.gamma + (static_cast<long long>(h * G + g) * G + gp) * D * D;
-                const float* gamT = P.gamma + (static_cast<long long>(h * G + gp) * G + g) * D * D;
-                const double sym = g == gp ? static_cast<double>(gam[i * D + j]) : static_cast<double>(gam[i * D + j]) + static_cast<double>(gamT[i * D + j]);
-                hv += c_s[k] * sym;
-            }
-    }
-    const long long o = (static_cast<long long>(h) * D + i) * D + j;
-    P.H_K[o] += 2.0 * static_cast<double>(P.inv_tau) * static_cast<double>(P.inv_tau) * hk;
-    P.H_V[o] += 2.0 * hv;
+bool launch_pairs(const HessParams& P, cudaStream_t st) {
+    constexpr int NC = pairs_per_chunk(G);
+    if (!opt_in_dynamic_smem(reinterpret_cast<const void*>(pairs_kernel<G, NC>), static_cast<int>(sizeof(PairsSmem<G, NC>)))) return false;
+    pairs_kernel<G, NC><<<dim3((P.S + 15) / 16, pair_chunks(G), P.n_kv), 256, sizeof(PairsSmem<G, NC>), st>>>(P);
+    key_kernel<G><<<dim3((P.S + KEY_SLICE - 1) / KEY_SLICE, P.n_kv), 512, 0, st>>>(P);
+    return true;
 }
 
 size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 
-struct HessLayout { size_t gamma, row_m, row_linv, Oh, U, alpha, A, W0, total; };
+struct HessLayout { size_t gamma, row_m, row_linv, Oh, U, kappa, alpha, A, W0, total; };
 HessLayout hess_layout(int n_kv, int n_q, long long S) {
     const int G = n_q / n_kv, NP = G * (G + 1) / 2;
     HessLayout L;
@@ -303,8 +510,9 @@ HessLayout hess_layout(int n_kv, int n_q, long long S) {
     L.row_m = off;    off = align256(off + static_cast<size_t>(S) * n_q * sizeof(float));
     L.row_linv = off; off = align256(off + static_cast<size_t>(S) * n_q * sizeof(float));
     L.Oh = off;       off = align256(off + static_cast<size_t>(S) * n_q * D * sizeof(float));
-    L.U = off;        off = align256(off + static_cast<size_t>(S) * n_kv * G * G * D * sizeof(float));
-    L.alpha = off;    off = align256(off + static_cast<size_t>(S) * n_kv * G * G * sizeof(float));
+    L.U = off;        off = align256(off + static_cast<size_t>(S) * n_kv * NP * D * sizeof(float));
+    L.kappa = off;    off = align256(off + static_cast<size_t>(S) * n_kv * NP * sizeof(float));
+    L.alpha = off;    off = align256(off + static_cast<size_t>(S) * n_kv * NP * sizeof(float));
     L.A = off;        off = align256(off + static_cast<size_t>(S) * n_kv * NP * sizeof(float));
     L.W0 = off;       off = align256(off + static_cast<size_t>(S) * n_kv * NP * sizeof(float));
     L.total = off;
@@ -340,22 +548,29 @@ extern "C" int wushkv_accumulate_attention_hessians_device(int32_t n_kv, int32_t
     P.gamma = reinterpret_cast<float*>(ws + L.gamma);
     P.row_m = reinterpret_cast<float*>(ws + L.row_m); P.row_linv = reinterpret_cast<float*>(ws + L.row_linv);
     P.Oh = reinterpret_cast<float*>(ws + L.Oh); P.U = reinterpret_cast<float*>(ws + L.U);
+    P.kappa = reinterpret_cast<float*>(ws + L.kappa);
     P.alpha = reinterpret_cast<float*>(ws + L.alpha); P.A = reinterpret_cast<float*>(ws + L.A); P.W0 = reinterpret_cast<float*>(ws + L.W0);
     P.H_K = H_K; P.H_V = H_V;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    gamma_kernel<<<dim3(D / 16, D / 16, n_kv * G * G), dim3(16, 16), 0, st>>>(P);
-    rows_kernel<<<dim3(P.S, n_kv), 32 * G, 0, st>>>(P);
-    project_kernel<<<dim3(P.S, n_kv), 32 * std::min(G * G, 16), 0, st>>>(P);
-    const dim3 grid_t(P.S, n_kv), grid_r(D / 16, D / 16, n_kv);
+    if (!opt_in_dynamic_smem(reinterpret_cast<const void*>(rows_kernel), static_cast<int>(sizeof(RowsSmem))) ||
+        !opt_in_dynamic_smem(reinterpret_cast<const void*>(project_kernel), static_cast<int>(sizeof(ProjectSmem))))
+        return WUSHKV_ECUDA;
+    const unsigned tiles = (P.S + RT - 1) / RT;
+    gamma_kernel<<<dim3(P.n_pairs, n_kv), 512, 0, st>>>(P);
+    rows_kernel<<<dim3(tiles, n_q), 256, sizeof(RowsSmem), st>>>(P);
+    project_kernel<<<dim3(tiles, P.n_pairs, n_kv), 256, sizeof(ProjectSmem), st>>>(P);
+    bool ok;
     switch (G) {
-        case 1: pairs_kernel<1><<<grid_t, 128, 0, st>>>(P); reduce_kernel<1><<<grid_r, dim3(16, 16), 0, st>>>(P); break;
-        case 2: pairs_kernel<2><<<grid_t, 128, 0, st>>>(P); reduce_kernel<2><<<grid_r, dim3(16, 16), 0, st>>>(P); break;
-        case 3: pairs_kernel<3><<<grid_t, 128, 0, st>>>(P); reduce_kernel<3><<<grid_r, dim3(16, 16), 0, st>>>(P); break;
-        case 4: pairs_kernel<4><<<grid_t, 128, 0, st>>>(P); reduce_kernel<4><<<grid_r, dim3(16, 16), 0, st>>>(P); break;
-        case 5: pairs_kernel<5><<<grid_t, 128, 0, st>>>(P); reduce_kernel<5><<<grid_r, dim3(16, 16), 0, st>>>(P); break;
-        case 6: pairs_kernel<6><<<grid_t, 128, 0, st>>>(P); reduce_kernel<6><<<grid_r, dim3(16, 16), 0, st>>>(P); break;
-        case 7: pairs_kernel<7><<<grid_t, 128, 0, st>>>(P); reduce_kernel<7><<<grid_r, dim3(16, 16), 0, st>>>(P); break;
-        default: pairs_kernel<8><<<grid_t, 128, 0, st>>>(P); reduce_kernel<8><<<grid_r, dim3(16, 16), 0, st>>>(P); break;
+        case 1: ok = launch_pairs<1>(P, st); break;
+        case 2: ok = launch_pairs<2>(P, st); break;
+        case 3: ok = launch_pairs<3>(P, st); break;
+        case 4: ok = launch_pairs<4>(P, st); break;
+        case 5: ok = launch_pairs<5>(P, st); break;
+        case 6: ok = launch_pairs<6>(P, st); break;
+        case 7: ok = launch_pairs<7>(P, st); break;
+        default: ok = launch_pairs<8>(P, st); break;
     }
+    if (!ok) return WUSHKV_ECUDA;
+    value_kernel<<<dim3(16, n_kv), 256, 0, st>>>(P);
     return cudaGetLastError() == cudaSuccess ? WUSHKV_OK : WUSHKV_ECUDA;
 }

@@ -1,0 +1,22 @@
+"""Attention-aware Hessians at the edges of the kernels' tiles (16 and 64 positions, 10 pairs per chunk, d_model no multiple of 16)
+for the group sizes with one, two and three chunks of pairs, against the oracle's literal Jacobian form."""
+import numpy as np
+import pytest
+
+from oracle import wushkv_oracle as O
+from tests.test_gpu_hessians import TOL, _gpu, _inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n_q,n_kv,n_tok,d_model", [(2, 1, 1, 32), (4, 2, 65, 20), (5, 1, 33, 32), (6, 1, 17, 48), (8, 1, 66, 16), (1, 1, 130, 8)])
+def test_tile_edges(n_q, n_kv, n_tok, d_model):
+    wl, K, Q, V, WO = _inputs(n_q, n_kv, n_tok, d_model, seed=71)
+    tau = float(np.sqrt(128))
+    HK, HV = _gpu(K, Q, V, WO, tau)
+    G = n_q // n_kv
+    for h in range(n_kv):
+        rk, rv = O.attention_hessians(Q[:, h * G:(h + 1) * G], K[:, h], V[:, h], WO[h * G:(h + 1) * G], tau)
+        if n_tok > 1:                                   # one position attends to itself only: v - o = 0
+            assert np.max(np.abs(HK[h] - rk)) <= TOL * np.max(np.abs(rk))
+        assert np.max(np.abs(HV[h] - rv)) <= TOL * np.max(np.abs(rv))
