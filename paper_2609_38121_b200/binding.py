@@ -146,16 +146,30 @@ def _ptr(t):
     """Device or host pointer of a torch tensor / numpy array (None -> NULL)."""
     if t is None:
         return None
-    if isinstance(t, np.ndarray):
+    try:
+        return t.data_ptr()
+    except AttributeError:
         return t.ctypes.data
-    return t.data_ptr()
+
+
+# The handle of the current stream without a torch.cuda.Stream object around it (2.5 us of a 20 us decode step of one sequence).
+_current_stream = None
 
 
 def _stream_ptr(stream):
-    import torch
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return C.c_void_p(stream.cuda_stream)
+    global _current_stream
+    if stream is not None:
+        return stream.cuda_stream
+    if _current_stream is None:
+        import torch
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        if raw is None:
+            _current_stream = lambda: torch.cuda.current_stream().cuda_stream  # noqa: E731
+        else:
+            torch.cuda.current_stream()                 # initialises CUDA
+            device = torch._C._cuda_getDevice
+            _current_stream = lambda: raw(device())  # noqa: E731
+    return _current_stream()
 
 
 def status_string(status: int) -> str:
