@@ -257,16 +257,16 @@ class Session:
 
     def launches_per_step(self):
         # chunk append: transform/quantize kernel + length update (+ prefill attention: preparation + attention);
-        # token append: one kernel; decode: prep + main + combine
-        n = (4 if self.chunk else 1) + 3
+        # token append: one kernel; decode: prep + main
+        n = (4 if self.chunk else 1) + 2
         if self.chunk:
-            # few query-tile pairs (a short chunk): the attention runs several CTAs per pair and a merge kernel follows
+            # few query-tile pairs (a short chunk): CTAs may share a pair's key tiles and a merge kernel follows
             R = 128 // (self.wl.n_q // self.wl.n_kv)
-            tiles = -(-self.chunk // R)
-            pairs = self.batch * ((tiles + 1) // 2) * self.wl.n_kv
-            min_ctas = -(-self.batch * self.chunk // (2 * R)) * self.wl.n_kv
+            total = self.batch * self.chunk
+            pairs = min(self.batch * -(-self.chunk // (2 * R)), total // (2 * R) + self.batch)
+            min_ctas = -(-total // (2 * R)) * self.wl.n_kv
             sms = self.torch.cuda.get_device_properties(self.cache.device).multi_processor_count
-            if min(max(1, min(16, sms // max(min_ctas, 1))), max(1, sms // pairs)) > 1:
+            if pairs <= 1024 and pairs * self.wl.n_kv < 4 * sms and max(min(16, sms // min_ctas), min(64, 4 * sms // min_ctas)) > 1:
                 n += 1
         return n
 

@@ -197,8 +197,8 @@ size_t wushkv_decode_workspace_bytes(const wushkv_cache* cache, int32_t batch, i
  * query column that sees all seq_len[b] cached positions, softmax temperature 1/sm_scale),
  * evaluated directly on the packed cache: quantized positions are dequantized in registers
  * (x_hat = x_min + Delta * code), window positions are read from the bf16 buffers.  The
- * context is split across thread blocks (partial softmax state per split) and merged by a
- * final combine pass.  Call after wushkv_append of the step's token.
+ * context is split across thread blocks (partial softmax state per split) and merged by the
+ * last block to finish a head.  Call after wushkv_append of the step's token.
  *   slot (device): int32 [batch];  seq_len (device): int32 [batch], each >= 1.
  *   max_seq_len (host): upper bound of seq_len[b] (sizes the launch; no device read-back).
  *   Q (device): bf16 [batch][n_q][d] post-Norm post-RoPE, NOT compensated; 16-byte aligned.

@@ -48,8 +48,8 @@ extern "C" int wushkv_decode_attn_static(const wushkv_cache* cache, int32_t batc
         if (cudaGetSymbolAddress(&p, g_static_scratch) != cudaSuccess || p == nullptr) return WUSHKV_ECUDA;
         g_scratch_addr[dev] = p;
     }
-    // Nothing in the scratch has to start at zero: every partial that the combine pass reads is
-    // written by the main kernel of the same call, so the previous call's leftovers are never seen.
+    // Nothing in the scratch has to start at zero: every partial that the merge reads, and the counters that it
+    // advances, are written by the kernels of the same call, so the previous call's leftovers are never seen.
     return wushkv_decode_attn(cache, batch, slot, seq_len, max_seq_len, Q, O, g_scratch_addr[dev],
                               WUSHKV_STATIC_SCRATCH_BYTES, stream);
 }
