@@ -12,7 +12,7 @@
 //
 // Every step is a contraction over 128 channels or over positions, done as register-blocked fp32 products out of shared
 // memory (with a warp per row, a CTA per position and the sums over s as vectors of 128 channels per pair, 1024 tokens of 32 / 8
-// heads took 6.0 ms, every value fetched being used for one or two multiplications; now 1.4 ms, pairs_kernel 0.61, rows_kernel 0.37):
+// heads took 6.0 ms, every value fetched being used for one or two multiplications; now 1.36 ms, pairs_kernel 0.59, rows_kernel 0.35):
 //   gamma_kernel      Gamma_{gg'}, 128 x 128 x d_model, float64 across groups of 16
 //   rows_kernel       causal softmax statistics (max, 1 / sum) and head outputs o_{g,t}: 64 x 64 tiles
 //   project_kernel    U, kappa and alpha: 64 x 128 tiles
@@ -158,7 +158,7 @@ __global__ void __launch_bounds__(256, 2) rows_kernel(HessParams P) {
         stage(P.K);
         __syncthreads();
         float z[4][4] = {};
-#pragma unroll 2
+#pragma unroll 4
         for (int k = 0; k < D; k += 4) {
             float4 qa[4], kb[4];
 #pragma unroll
@@ -365,7 +365,7 @@ __global__ void __launch_bounds__(256, 1) pairs_kernel(HessParams P) {
         for (int g = 0; g < G; ++g) p[g][0] = p[g][1] = p[g][2] = p[g][3] = 0.f;
 #pragma unroll
         for (int k = 0; k < NC; ++k) rr[k][0] = rr[k][1] = rr[k][2] = rr[k][3] = 0.f;
-#pragma unroll 1
+#pragma unroll 2
         for (int k4 = 0; k4 < D; k4 += 4) {
             float4 b[4];
 #pragma unroll
