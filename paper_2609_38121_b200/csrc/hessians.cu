@@ -89,32 +89,43 @@ __device__ __forceinline__ void outer_group(const float (*a)[HS_PITCH], const fl
         for (int e = 0; e < 8; ++e) acc[r][e] += static_cast<double>(part[r][e]);
 }
 
-// Gamma_{gg'}[i][j] = sum_m W_g[i][m] W_g'[j][m] and its transpose Gamma_{g'g}; grid (pairs, n_kv), 512 threads.
-__global__ void __launch_bounds__(512) gamma_kernel(HessParams P) {
+// Gamma_{gg'}[i][j] = sum_m W_g[i][m] W_g'[j][m] and its transpose Gamma_{g'g}; grid (pairs, n_kv, 4 blocks of 32 rows i), 128
+// threads: with few pairs the time is that of one CTA's groups of 16 m, whose loads are in flight while the group before
+// is multiplied (a CTA per pair with its loads waited for: 58 us for one pair and d_model 320).
+__global__ void __launch_bounds__(128) gamma_kernel(HessParams P) {
     __shared__ __align__(16) float a_s[OUTER_K][HS_PITCH], b_s[OUTER_K][HS_PITCH];
     int g, gp;
     pair_heads(blockIdx.x, P.G, g, gp);
-    const int h = blockIdx.y, tid = threadIdx.x;
-    const float* Wa = P.W_O + static_cast<long long>(h * P.G + g) * D * P.d_model;
+    const int h = blockIdx.y, tid = threadIdx.x, r0 = 32 * blockIdx.z;
+    const float* Wa = P.W_O + (static_cast<long long>(h * P.G + g) * D + r0) * P.d_model;
     const float* Wb = P.W_O + static_cast<long long>(h * P.G + gp) * D * P.d_model;
     double acc[4][8] = {};
-    for (int m0 = 0; m0 < P.d_model; m0 += OUTER_K) {
-        float ta[4], tb[4];
+    float ta[4], tb[16];
+    auto fetch = [&](int m0) {
+        const int m = m0 + (tid & 15);
+        const bool in = m < P.d_model;
 #pragma unroll
-        for (int n = 0; n < 4; ++n) {
-            const int item = tid + 512 * n, i = item >> 4, m = m0 + (item & 15);
-            ta[n] = m < P.d_model ? Wa[static_cast<long long>(i) * P.d_model + m] : 0.f;
-            tb[n] = m < P.d_model ? Wb[static_cast<long long>(i) * P.d_model + m] : 0.f;
+        for (int n = 0; n < 16; ++n) {
+            const long long off = static_cast<long long>((tid >> 4) + 8 * n) * P.d_model + m;
+            tb[n] = in ? Wb[off] : 0.f;
+            if (n < 4) ta[n] = in ? Wa[off] : 0.f;
+        }
+    };
+    fetch(0);
+    for (int m0 = 0; m0 < P.d_model; m0 += OUTER_K) {
+        __syncthreads();
+#pragma unroll
+        for (int n = 0; n < 16; ++n) {
+            b_s[tid & 15][(tid >> 4) + 8 * n] = tb[n];
+            if (n < 4) a_s[tid & 15][(tid >> 4) + 8 * n] = ta[n];
         }
         __syncthreads();
-#pragma unroll
-        for (int n = 0; n < 4; ++n) { const int item = tid + 512 * n; a_s[item & 15][item >> 4] = ta[n]; b_s[item & 15][item >> 4] = tb[n]; }
-        __syncthreads();
+        fetch(m0 + OUTER_K);
         outer_group(a_s, b_s, acc);
     }
     float* out = P.gamma + (static_cast<long long>(h * P.G + g) * P.G + gp) * D * D;
     float* outT = P.gamma + (static_cast<long long>(h * P.G + gp) * P.G + g) * D * D;
-    const int i0 = 4 * (tid >> 4), j0 = tid & 15;
+    const int i0 = r0 + 4 * (tid >> 4), j0 = tid & 15;
 #pragma unroll
     for (int r = 0; r < 4; ++r)
 #pragma unroll
@@ -556,7 +567,7 @@ extern "C" int wushkv_accumulate_attention_hessians_device(int32_t n_kv, int32_t
         !opt_in_dynamic_smem(reinterpret_cast<const void*>(project_kernel), static_cast<int>(sizeof(ProjectSmem))))
         return WUSHKV_ECUDA;
     const unsigned tiles = (P.S + RT - 1) / RT;
-    gamma_kernel<<<dim3(P.n_pairs, n_kv), 512, 0, st>>>(P);
+    gamma_kernel<<<dim3(P.n_pairs, n_kv, D / 32), 128, 0, st>>>(P);
     rows_kernel<<<dim3(tiles, n_q), 256, sizeof(RowsSmem), st>>>(P);
     project_kernel<<<dim3(tiles, P.n_pairs, n_kv), 256, sizeof(ProjectSmem), st>>>(P);
     bool ok;
