@@ -75,6 +75,7 @@ struct PrefillParams {
     int fixed_split;                      // > 0: that many for every pair; 0: by the amount of work (see make_share_table)
     int n_sm;
     int n_slots;                          // entries of the table of shares (rows of CTAs of the attention kernel)
+    int max_pairs;                        // tile pairs of max_new tokens
     int4* shares;                         // max_split > 1: (sequence, pair, share, shares of the pair), sequence -1: none; one more: .x is 1 if any pair is shared
     float* part;                          // [max_split][total_new][n_q][PART_W] partial outputs
     int wait_limit;                       // poll limit of the barrier waits (0: default, a second or more)
@@ -1320,7 +1321,9 @@ __device__ unsigned long long g_ws_t[32];
 // and one target for the whole call; of 32 targets, up to two shares per SM, the one is taken with the smallest estimate
 // of the slowest SM's time, in key tiles (about 2 us): where all CTAs run at once, the largest share; else the average and
 // about half a share at the end.  A share costs about SHARE_COST tiles (start, first record, end), a merge MERGE_COST and its
-// rows' way through L2.  Shares are handed out largest first.
+// rows' way through L2.  Shares are handed out largest first.  A sequence with more new tokens than the host promised gets the tile
+// pairs of max_new tokens, and its other rows are marked as having no shares to merge; more pairs than the table has room for
+// (chunk bounds that contradict total_new) are reported, and nothing is merged.
 constexpr int SHARE_COST = 5, MERGE_COST = 2;
 constexpr float MERGE_ROW_COST = 1.2e-4f;                        // a partial row written and read again, in key tiles of the whole GPU
 constexpr int MAX_SHARED_PAIRS = 1024;                           // tile pairs (per KV head) of a call that may share them, and its sequences
@@ -1360,10 +1363,13 @@ __device__ __noinline__ void make_share_table(const PrefillParams& P, ShareScrat
         const int b = base + tid;
         int pairs = 0, old_tiles = 0, n_new = 0;
         if (b < P.batch) {
-            n_new = ld_in(P.cu_new + b + 1) - ld_in(P.cu_new + b);
+            const int b_first = ld_in(P.cu_new + b);
+            n_new = ld_in(P.cu_new + b + 1) - b_first;
             const int S = __ldcg(P.seq_len + b), S0 = max(S - n_new, 0);
             const int q_hi = min(c.s_sink + n_quantized(S - c.lag, c.s_sink, c.s_keep, c.s_flush), S0);
-            pairs = n_new > 0 ? (n_new + 2 * R - 1) / (2 * R) : 0;
+            pairs = n_new > 0 ? min((n_new + 2 * R - 1) / (2 * R), P.max_pairs) : 0;
+            for (int t = 2 * R * P.max_pairs; t < n_new && b_first + t < P.total_new; ++t)
+                for (int j = 0; j < c.n_q; ++j) P.part[(static_cast<long long>(b_first + t) * c.n_q + j) * PART_W + D + 2] = 0.f;
             old_tiles = (max(S0 - max(q_hi - c.s_sink, 0), 0) + TN - 1) / TN + (q_hi > c.s_sink ? (q_hi - 1) / PAGE_TOKENS - c.s_sink / PAGE_TOKENS + 1 : 0);
         }
         int all;
@@ -1434,7 +1440,11 @@ __device__ __noinline__ void make_share_table(const PrefillParams& P, ShareScrat
         used += all;
     }
     for (int x = used + tid; x < P.n_slots; x += SHARE_THREADS) P.shares[x] = make_int4(-1, 0, 0, 0);
-    if (tid == 0) P.shares[P.n_slots] = make_int4(used > n_pairs, 0, 0, 0);
+    if (tid == 0) {
+        const bool fits = used <= P.n_slots;
+        if (!fits) atomicOr(c.dev_status, WUSHKV_DEV_BAD_COUNT);
+        P.shares[P.n_slots] = make_int4(fits && used > n_pairs, 0, 0, 0);
+    }
 }
 __global__ void __launch_bounds__(SHARE_THREADS) prefill_shares_kernel(const __grid_constant__ PrefillParams P) {       // where no transform kernel with room for it runs ahead
     __shared__ ShareScratch sc;
@@ -1469,6 +1479,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) prefill_attn_ws_kernel(PrefillP
     }
     const int first = ld_in(P.cu_new + b), n_new = ld_in(P.cu_new + b + 1) - first;
     if (2 * pr * R >= n_new) return;
+    if (n_new > 2 * R * P.max_pairs && tid == 0) atomicOr(c.dev_status, WUSHKV_DEV_BAD_COUNT);      // rows past max_new's tile pairs are left alone
     const int S = ld_in(P.seq_len + b), sl = ld_in(P.slot + b);
     const bool bad = sl < 0 || sl >= c.n_slots || S < n_new;
     if (P.max_split > 1 && sp == 0)                              // for the merge: how many shares the pair's rows have (none to merge if it is skipped)
@@ -2094,12 +2105,16 @@ __global__ void __launch_bounds__(32 * MERGE_WARPS) prefill_merge_kernel(Prefill
     pdl_wait();
     if (__ldcg(&P.shares[P.n_slots].x) == 0) return;             // no pair is shared
     const int lane = threadIdx.x & 31;
-    for (long long row = static_cast<long long>(blockIdx.x) * MERGE_WARPS + (threadIdx.x >> 5); row < static_cast<long long>(P.total_new) * P.c.n_q;
+    // Rows behind the last sequence's were visited by no CTA: the workspace holds there what it held.  So it does in a sequence whose
+    // pairs found no room in the table; a count that no CTA can have written is passed over, and nothing is read outside the workspace.
+    const long long n_rows = static_cast<long long>(min(ld_in(P.cu_new + P.batch), P.total_new)) * P.c.n_q;
+    for (long long row = static_cast<long long>(blockIdx.x) * MERGE_WARPS + (threadIdx.x >> 5); row < n_rows;
          row += static_cast<long long>(gridDim.x) * MERGE_WARPS) {
     const long long stride = static_cast<long long>(P.total_new) * P.c.n_q * PART_W;
     const float* p0 = P.part + row * PART_W;
-    const int n_share = static_cast<int>(__ldcg(p0 + D + 2));
-    if (n_share <= 1) continue;                                  // a pair that one CTA finished
+    const float count = __ldcg(p0 + D + 2);
+    if (!(count >= 2.f && count <= static_cast<float>(P.max_split))) continue;       // a pair that one CTA finished
+    const int n_share = static_cast<int>(count);
     float m = -INFINITY, l = 0.f;
     float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
     for (int s0 = 0; s0 < n_share; s0 += 32) {
@@ -2533,7 +2548,7 @@ static int prefill_attn_impl(const wushkv_cache* cache, int32_t batch, const int
     P.batch = batch; P.total_new = total_new; P.slot = slot; P.seq_len = seq_len; P.cu_new = cu_new;
     P.K_new = K_new; P.V_new = V_new; P.Q_new = Q_new; P.O = O;
     P.use_tma = 0;
-    P.max_split = 1; P.fixed_split = 0; P.n_sm = sm_count(); P.n_slots = 0; P.shares = nullptr;
+    P.max_split = 1; P.fixed_split = 0; P.n_sm = sm_count(); P.n_slots = 0; P.max_pairs = 0; P.shares = nullptr;
     P.part = nullptr;
     P.wait_limit = static_cast<int>(std::min<long long>(std::max<long long>(knobs().wait_limit, 0), 1 << 30));
     P.drop = knobs().drop_prefill;
@@ -2552,6 +2567,7 @@ static int prefill_attn_impl(const wushkv_cache* cache, int32_t batch, const int
         if (knobs().prefill_split > 0) P.fixed_split = P.max_split = static_cast<int>(std::max<long long>(1, std::min<long long>(std::min(knobs().prefill_split, pl.max_split), MAX_TABLE / n_pairs)));
         else if (n_pairs * P.c.n_kv < 2 * MAX_SHARES_PER_SM * sm_count()) P.max_split = pl.max_split;
         if (n_pairs > MAX_SHARED_PAIRS || batch > 32767 || max_new > 65535 * R) P.max_split = 1;
+        P.max_pairs = (max_new + 2 * R - 1) / (2 * R);
         P.n_slots = static_cast<int>(std::min<long long>(n_pairs * P.max_split, MAX_TABLE));
         if (P.fixed_split == 0) P.n_slots = static_cast<int>(std::min<long long>(P.n_slots, MAX_SHARES_PER_SM * sm_count() / P.c.n_kv + n_pairs));
         P.part = reinterpret_cast<float*>(ws + pl.off_part);

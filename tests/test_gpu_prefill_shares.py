@@ -57,3 +57,59 @@ def test_smaller_workspaces():
     with pytest.raises(B.WushkvError) as e:
         B.prefill_attn(L.cache.desc, 2, L.slot, L.seq_len, cu, total, 40, K, V, Q, O, ws, least - 1)
     assert e.value.status == B.ECAPACITY
+
+
+def _chunk(L, ctx, new, rows):
+    """Keys, values and queries of the chunk as device buffers of `rows` rows (zeros behind the last token) and its bounds."""
+    import torch
+    def bits16(parts, heads):
+        x = np.zeros((rows, heads, 128), np.float32)
+        x[:sum(new)] = np.concatenate(parts)
+        return torch.from_numpy(W.f32_to_bf16_bits(x).view(np.int16)).cuda()
+    n = range(len(new))
+    K = bits16([L.tokens[b][0][ctx[b]:ctx[b] + new[b]] for b in n], L.wl.n_kv)
+    V = bits16([L.tokens[b][1][ctx[b]:ctx[b] + new[b]] for b in n], L.wl.n_kv)
+    Q = bits16([L.wl.chunk_queries(b, np.arange(ctx[b], ctx[b] + new[b])) for b in n], L.wl.n_q)
+    return K, V, Q, torch.tensor([0] + list(np.cumsum(new)), dtype=torch.int32, device="cuda")
+
+
+@pytest.mark.parametrize("word", [0x00, 0x40, 0x4E, 0xFF])      # as counts of shares: 0, 3.0, 8.6e8, not a number
+def test_rows_without_a_sequence_are_left_alone(word):
+    """total_new above cu_new[batch] (a buffer padded to a fixed size): whatever the workspace held for the rows behind the last
+    sequence, they are not written and the others are right."""
+    import torch
+    from paper_2609_38121_b200 import binding as B
+    ctx, new, rows = [1200, 300], [20, 40], 67
+    L = Layer(_wl(8, 2, 2), [c + n for c, n in zip(ctx, new)], 2, 4, 64, 1)
+    L.append_step(ctx)
+    L.prefill(new)
+    full = L.first
+    K, V, Q, cu = _chunk(L, ctx, new, rows)
+    nbytes = B.prefill_workspace_bytes(L.cache.desc, 2, rows)
+    ws = torch.full((nbytes,), word, dtype=torch.uint8, device="cuda")
+    O = torch.full((rows, 8, 128), float("nan"), device="cuda")
+    B.prefill_attn(L.cache.desc, 2, L.slot, L.seq_len, cu, rows, 40, K, V, Q, O, ws, nbytes)
+    out = O.cpu().numpy()
+    assert L.cache.status() == 0
+    assert np.all(np.isnan(out[60:]))
+    assert np.max(np.abs(out[:60] - full)) <= 1e-3 * np.max(np.abs(full))
+
+
+def test_more_tokens_than_promised():
+    """A sequence with more new tokens than max_new: its rows past the tile pairs of max_new tokens have no output, and that is reported."""
+    import torch
+    from paper_2609_38121_b200 import binding as B
+    ctx, new = [1200, 300], [20, 200]
+    L = Layer(_wl(8, 2, 2), [c + n for c, n in zip(ctx, new)], 2, 4, 64, 1)
+    L.append_step(ctx)
+    L.prefill(new)
+    full = L.first
+    K, V, Q, cu = _chunk(L, ctx, new, 220)
+    nbytes = B.prefill_workspace_bytes(L.cache.desc, 2, 220)
+    ws = torch.full((nbytes,), 0x40, dtype=torch.uint8, device="cuda")
+    O = torch.full((220, 8, 128), float("nan"), device="cuda")
+    B.prefill_attn(L.cache.desc, 2, L.slot, L.seq_len, cu, 220, 64, K, V, Q, O, ws, nbytes)
+    out = O.cpu().numpy()
+    assert L.cache.status() == B.DEV_BAD_COUNT
+    assert np.all(np.isnan(out[20 + 64:]))              # one pair of 32-position tiles per sequence
+    assert np.max(np.abs(out[:84] - full[:84])) <= 1e-3 * np.max(np.abs(full))
