@@ -241,7 +241,7 @@ int wushkv_decode_attn(const wushkv_cache* cache, int32_t batch, const int32_t* 
  * an fp16 value plus its fp16 rounding remainder.  The query heads of a KV head share one 128-row tile.  A call with too
  * few tiles to keep the GPU evenly busy splits the keys of the longer ones over several CTAs and merges their partial
  * results (the workspace holds them; a smaller one than wushkv_prefill_workspace_bytes() that still has room for one wave
- * of CTAs is accepted and gives fewer splits); the result does not depend on timing, only on the call's shapes, lengths
+ * of CTAs is accepted and gives one split of all tiles alike); the result does not depend on timing, only on the call's shapes, lengths
  * and workspace.
  */
 size_t wushkv_prefill_workspace_bytes(const wushkv_cache* cache, int32_t batch, int32_t total_new);

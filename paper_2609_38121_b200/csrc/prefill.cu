@@ -76,7 +76,8 @@ struct PrefillParams {
     int n_sm;
     int n_slots;                          // entries of the table of shares (rows of CTAs of the attention kernel)
     int max_pairs;                        // tile pairs of max_new tokens
-    int4* shares;                         // max_split > 1: (sequence, pair, share, shares of the pair), sequence -1: none; one more: .x is 1 if any pair is shared
+    int4* shares;                         // (sequence, pair, share, shares of the pair), sequence -1: none; one more: .x is 1 if any pair is shared
+                                          // nullptr: every pair has max_split shares, in the order of the grid
     float* part;                          // [max_split][total_new][n_q][PART_W] partial outputs
     int wait_limit;                       // poll limit of the barrier waits (0: default, a second or more)
     int drop;                             // testing aid: 1 the first tile's score MMAs are never committed, 2 the first bulk copy of a
@@ -1322,8 +1323,8 @@ __device__ unsigned long long g_ws_t[32];
 // of the slowest SM's time, in key tiles (about 2 us): where all CTAs run at once, the largest share; else the average and
 // about half a share at the end.  A share costs about SHARE_COST tiles (start, first record, end), a merge MERGE_COST and its
 // rows' way through L2.  Shares are handed out largest first.  A sequence with more new tokens than the host promised gets the tile
-// pairs of max_new tokens, and its other rows are marked as having no shares to merge; more pairs than the table has room for
-// (chunk bounds that contradict total_new) are reported, and nothing is merged.
+// pairs of max_new tokens; more pairs than the table has room for (chunk bounds that contradict total_new) are reported, and
+// nothing is merged.
 constexpr int SHARE_COST = 5, MERGE_COST = 2;
 constexpr float MERGE_ROW_COST = 1.2e-4f;                        // a partial row written and read again, in key tiles of the whole GPU
 constexpr int MAX_SHARED_PAIRS = 1024;                           // tile pairs (per KV head) of a call that may share them, and its sequences
@@ -1363,13 +1364,10 @@ __device__ __noinline__ void make_share_table(const PrefillParams& P, ShareScrat
         const int b = base + tid;
         int pairs = 0, old_tiles = 0, n_new = 0;
         if (b < P.batch) {
-            const int b_first = ld_in(P.cu_new + b);
-            n_new = ld_in(P.cu_new + b + 1) - b_first;
+            n_new = ld_in(P.cu_new + b + 1) - ld_in(P.cu_new + b);
             const int S = __ldcg(P.seq_len + b), S0 = max(S - n_new, 0);
             const int q_hi = min(c.s_sink + n_quantized(S - c.lag, c.s_sink, c.s_keep, c.s_flush), S0);
             pairs = n_new > 0 ? min((n_new + 2 * R - 1) / (2 * R), P.max_pairs) : 0;
-            for (int t = 2 * R * P.max_pairs; t < n_new && b_first + t < P.total_new; ++t)
-                for (int j = 0; j < c.n_q; ++j) P.part[(static_cast<long long>(b_first + t) * c.n_q + j) * PART_W + D + 2] = 0.f;
             old_tiles = (max(S0 - max(q_hi - c.s_sink, 0), 0) + TN - 1) / TN + (q_hi > c.s_sink ? (q_hi - 1) / PAGE_TOKENS - c.s_sink / PAGE_TOKENS + 1 : 0);
         }
         int all;
@@ -1466,21 +1464,27 @@ __global__ void __launch_bounds__(WS_THREADS, 1) prefill_attn_ws_kernel(PrefillP
     pdl_launch_dependents();
     int b, pr, sp = 0, n_split = 1;
     int h = blockIdx.y;
-    if (P.max_split > 1) {
-        // several CTAs may share a tile pair: each takes a contiguous share of the pair's key tiles and leaves a partial result
+    // several CTAs may share a tile pair: each takes a contiguous share of the pair's key tiles and leaves a partial result
+    if (P.shares != nullptr) {
         h = blockIdx.x;
         const int4 slot = __ldcg(P.shares + blockIdx.y);
         if (slot.x < 0) return;
         b = slot.x; pr = slot.y; sp = slot.z; n_split = slot.w;
     } else {
-        const int pairs = (P.tiles_per_seq + 1) >> 1;
-        b = static_cast<int>(blockIdx.x) / pairs;
-        pr = pairs - 1 - static_cast<int>(blockIdx.x) % pairs;  // long pairs first
+        const int pairs = (P.tiles_per_seq + 1) >> 1, bx = static_cast<int>(blockIdx.x) / P.max_split;
+        n_split = P.max_split; sp = static_cast<int>(blockIdx.x) % n_split;
+        b = bx / pairs;
+        pr = pairs - 1 - bx % pairs;                            // long pairs first
     }
     const int first = ld_in(P.cu_new + b), n_new = ld_in(P.cu_new + b + 1) - first;
+    const int S = ld_in(P.seq_len + b), sl = ld_in(P.slot + b);        // (requested together)
     if (2 * pr * R >= n_new) return;
-    if (n_new > 2 * R * P.max_pairs && tid == 0) atomicOr(c.dev_status, WUSHKV_DEV_BAD_COUNT);      // rows past max_new's tile pairs are left alone
-    const int S = ld_in(P.seq_len + b), sl = ld_in(P.slot + b);
+    if (n_new > 2 * R * P.max_pairs) {                           // rows past the tile pairs of max_new tokens are left alone: nothing to merge
+        if (tid == 0) atomicOr(c.dev_status, WUSHKV_DEV_BAD_COUNT);
+        if (P.max_split > 1 && sp == 0 && pr == P.max_pairs - 1)
+            for (int k = 2 * R * P.max_pairs * G + tid; k < min(n_new, P.total_new - first) * G; k += WS_THREADS)
+                P.part[(static_cast<long long>(first + k / G) * c.n_q + h * G + k % G) * PART_W + D + 2] = 0.f;
+    }
     const bool bad = sl < 0 || sl >= c.n_slots || S < n_new;
     if (P.max_split > 1 && sp == 0)                              // for the merge: how many shares the pair's rows have (none to merge if it is skipped)
         for (int k = tid; k < min(2 * R, n_new - 2 * pr * R) * G; k += WS_THREADS)
@@ -2103,16 +2107,19 @@ __global__ void __launch_bounds__(WS_THREADS, 1) prefill_attn_ws_kernel(PrefillP
 constexpr int MERGE_WARPS = 8;
 __global__ void __launch_bounds__(32 * MERGE_WARPS) prefill_merge_kernel(PrefillParams P) {
     pdl_wait();
-    if (__ldcg(&P.shares[P.n_slots].x) == 0) return;             // no pair is shared
-    const int lane = threadIdx.x & 31;
     // Rows behind the last sequence's were visited by no CTA: the workspace holds there what it held.  So it does in a sequence whose
     // pairs found no room in the table; a count that no CTA can have written is passed over, and nothing is read outside the workspace.
+    const int lane = threadIdx.x & 31;
+    const long long first_row = static_cast<long long>(blockIdx.x) * MERGE_WARPS + (threadIdx.x >> 5), row_step = static_cast<long long>(gridDim.x) * MERGE_WARPS;
+    auto count_of = [&](long long row) { return __ldcg(P.part + min(row, static_cast<long long>(P.total_new) * P.c.n_q - 1) * PART_W + D + 2); };
+    float next = count_of(first_row);                            // (requested together with the two that say whether it is used)
     const long long n_rows = static_cast<long long>(min(ld_in(P.cu_new + P.batch), P.total_new)) * P.c.n_q;
-    for (long long row = static_cast<long long>(blockIdx.x) * MERGE_WARPS + (threadIdx.x >> 5); row < n_rows;
-         row += static_cast<long long>(gridDim.x) * MERGE_WARPS) {
+    if (P.shares != nullptr && __ldcg(&P.shares[P.n_slots].x) == 0) return;      // no pair is shared
+    for (long long row = first_row; row < n_rows; row += row_step) {
+    const float count = next;
+    next = count_of(row + row_step);
     const long long stride = static_cast<long long>(P.total_new) * P.c.n_q * PART_W;
     const float* p0 = P.part + row * PART_W;
-    const float count = __ldcg(p0 + D + 2);
     if (!(count >= 2.f && count <= static_cast<float>(P.max_split))) continue;       // a pair that one CTA finished
     const int n_share = static_cast<int>(count);
     float m = -INFINITY, l = 0.f;
@@ -2484,7 +2491,7 @@ size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 constexpr int MAX_SHARES_PER_SM = 2;      // of a call whose pairs are shared, see make_share_table
 constexpr int MAX_TABLE = 2 * MAX_SHARED_PAIRS;
 constexpr int MAX_SPLIT = 64;
-struct PrefillPlan { size_t off_kp, off_vp, off_qp, off_qsum, off_part, per_split, table, least, total; int max_split; };
+struct PrefillPlan { size_t off_kp, off_vp, off_qp, off_qsum, off_part, per_split, table, least, total; int once, max_split; };
 bool make_prefill_plan(const CacheView& c, int total_new, PrefillPlan& pl) {
     if (total_new <= 0) return false;
     size_t off = 0;
@@ -2494,10 +2501,12 @@ bool make_prefill_plan(const CacheView& c, int total_new, PrefillPlan& pl) {
     pl.off_qsum = off; off = align256(off + static_cast<size_t>(total_new) * c.n_q * sizeof(float));
     // Partial results of the warp-specialised attention kernel for calls whose tile pairs do not fill the GPU several times over: at
     // least ceil(total_new / (2 R)) pairs per KV head exist.  A call is accepted with room for as many shares as fill the
-    // GPU once (`least`); given the whole `total` it may also cut long sequences finer than short ones.
+    // GPU once (`least`: every pair gets as many, without a table); given the whole `total` it may also cut long sequences
+    // finer than short ones.
     const int R = 128 / c.G;
     const long long min_ctas = std::max<long long>((static_cast<long long>(total_new) + 2 * R - 1) / (2 * R) * c.n_kv, 1);
     const long long once = std::max<long long>(1, std::min<long long>(16, sm_count() / min_ctas));
+    pl.once = static_cast<int>(once);
     const long long most = 2 * MAX_SHARES_PER_SM * sm_count() / min_ctas;
     pl.max_split = static_cast<int>(std::max<long long>(once, std::min<long long>(MAX_SPLIT, most)));
     pl.off_part = off;
@@ -2542,8 +2551,14 @@ static int prefill_attn_impl(const wushkv_cache* cache, int32_t batch, const int
     PrefillPlan pl;
     if (!make_prefill_plan(P.c, total_new, pl)) return WUSHKV_EINVAL;
     if (workspace_bytes < pl.least) return WUSHKV_ECAPACITY;
-    const size_t for_parts = workspace_bytes - pl.off_part > pl.table + 256 ? workspace_bytes - pl.off_part - pl.table - 256 : 0;
-    if (workspace_bytes < pl.total) pl.max_split = static_cast<int>(std::max<size_t>(1, std::min<size_t>(pl.max_split, for_parts / pl.per_split)));
+    // A smaller workspace: the table beside fewer shares, if there is room for as many as fill the GPU once, else no table.
+    bool with_table = true;
+    if (workspace_bytes < pl.total) {
+        const size_t room = workspace_bytes - pl.off_part > pl.table + 256 ? workspace_bytes - pl.off_part - pl.table - 256 : 0;
+        const size_t fit = std::min<size_t>(pl.max_split, room / pl.per_split);
+        with_table = fit >= static_cast<size_t>(pl.once);
+        pl.max_split = with_table ? static_cast<int>(fit) : pl.once;
+    }
     unsigned char* ws = static_cast<unsigned char*>(workspace);
     P.batch = batch; P.total_new = total_new; P.slot = slot; P.seq_len = seq_len; P.cu_new = cu_new;
     P.K_new = K_new; P.V_new = V_new; P.Q_new = Q_new; P.O = O;
@@ -2564,14 +2579,17 @@ static int prefill_attn_impl(const wushkv_cache* cache, int32_t batch, const int
         // grid covers the most that it hands out.
         const int R = TM / P.c.G;
         const long long n_pairs = std::min<long long>(static_cast<long long>(batch) * ((max_new + 2 * R - 1) / (2 * R)), total_new / (2 * R) + batch);
-        if (knobs().prefill_split > 0) P.fixed_split = P.max_split = static_cast<int>(std::max<long long>(1, std::min<long long>(std::min(knobs().prefill_split, pl.max_split), MAX_TABLE / n_pairs)));
+        if (!with_table) {
+            const long long all = static_cast<long long>(batch) * ((max_new + 2 * R - 1) / (2 * R)) * P.c.n_kv;
+            P.max_split = knobs().prefill_split > 0 ? std::min(knobs().prefill_split, pl.max_split) : static_cast<int>(std::max<long long>(1, std::min<long long>(pl.max_split, sm_count() / all)));
+        } else if (knobs().prefill_split > 0) P.fixed_split = P.max_split = static_cast<int>(std::max<long long>(1, std::min<long long>(std::min(knobs().prefill_split, pl.max_split), MAX_TABLE / n_pairs)));
         else if (n_pairs * P.c.n_kv < 2 * MAX_SHARES_PER_SM * sm_count()) P.max_split = pl.max_split;
-        if (n_pairs > MAX_SHARED_PAIRS || batch > 32767 || max_new > 65535 * R) P.max_split = 1;
+        if (with_table && (n_pairs > MAX_SHARED_PAIRS || batch > 32767 || max_new > 65535 * R)) P.max_split = 1;
         P.max_pairs = (max_new + 2 * R - 1) / (2 * R);
         P.n_slots = static_cast<int>(std::min<long long>(n_pairs * P.max_split, MAX_TABLE));
         if (P.fixed_split == 0) P.n_slots = static_cast<int>(std::min<long long>(P.n_slots, MAX_SHARES_PER_SM * sm_count() / P.c.n_kv + n_pairs));
         P.part = reinterpret_cast<float*>(ws + pl.off_part);
-        P.shares = reinterpret_cast<int4*>(ws + align256(pl.off_part + P.max_split * pl.per_split));
+        if (with_table && P.max_split > 1) P.shares = reinterpret_cast<int4*>(ws + align256(pl.off_part + P.max_split * pl.per_split));
     }
     const size_t smem_prep = static_cast<size_t>(PREP_TOK + 3 * D) * PREP_PITCH * sizeof(unsigned short);
     if (!opt_in_dynamic_smem(reinterpret_cast<const void*>(prefill_prep_kernel), static_cast<int>(smem_prep))) return WUSHKV_ECUDA;
@@ -2592,7 +2610,7 @@ static int prefill_attn_impl(const wushkv_cache* cache, int32_t batch, const int
         }
         if (tc_prep) {      // head slots: key heads, query heads, then one per KV head for the values
             const int slots_tc = slots + P.c.n_kv, per_slot_tc = std::max(1, std::min(n_tok_tiles, sm_count() / slots_tc));
-            if (launch_pdl(prefill_prep_tc_kernel, dim3(per_slot_tc, slots_tc + (P.max_split > 1 ? 1 : 0)), dim3(PT_THREADS), PT_SMEM, st, P, in_k, in_q) != cudaSuccess) return WUSHKV_ECUDA;
+            if (launch_pdl(prefill_prep_tc_kernel, dim3(per_slot_tc, slots_tc + (P.shares ? 1 : 0)), dim3(PT_THREADS), PT_SMEM, st, P, in_k, in_q) != cudaSuccess) return WUSHKV_ECUDA;
         }
 #if WUSHKV_WS_TIMING
         if (tc_prep) {
@@ -2610,7 +2628,7 @@ static int prefill_attn_impl(const wushkv_cache* cache, int32_t batch, const int
 #endif
         else {
             prefill_prep_kernel<<<dim3(per_slot, slots), 256, smem_prep, st>>>(P);
-            if (P.max_split > 1) prefill_shares_kernel<<<1, SHARE_THREADS, 0, st>>>(P);
+            if (P.shares) prefill_shares_kernel<<<1, SHARE_THREADS, 0, st>>>(P);
         }
     }
     if (cudaGetLastError() != cudaSuccess) return WUSHKV_ECUDA;
@@ -2625,7 +2643,7 @@ static int prefill_attn_impl(const wushkv_cache* cache, int32_t batch, const int
         const bool mv = make_row_tensor_map(map_v, false, P.VP, P.c.n_kv, total_new, TN);
         P.use_tma = (mk && mv && !knobs().prefill_no_tma) ? 1 : 0;
         if (!knobs().prefill_one_tile) {        // warp-specialised kernel: a pair of query tiles per CTA
-            const dim3 grid_ws = P.max_split > 1 ? dim3(P.c.n_kv, P.n_slots) : dim3(static_cast<unsigned>(batch) * ((P.tiles_per_seq + 1) / 2), P.c.n_kv);
+            const dim3 grid_ws = P.shares ? dim3(P.c.n_kv, P.n_slots) : dim3(static_cast<unsigned>(batch) * ((P.tiles_per_seq + 1) / 2) * P.max_split, P.c.n_kv);
             // the query operands (value, remainder) as [token][query head][128 channels]: a box is one tile's (G heads, R positions)
             CUtensorMap map_q0, map_q1;
             const bool mq = make_row_tensor_map(map_q0, false, P.QP, P.c.n_q, total_new, R, P.c.G) &&

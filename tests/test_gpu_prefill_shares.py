@@ -113,3 +113,37 @@ def test_more_tokens_than_promised():
     assert L.cache.status() == B.DEV_BAD_COUNT
     assert np.all(np.isnan(out[20 + 64:]))              # one pair of 32-position tiles per sequence
     assert np.max(np.abs(out[:84] - full[:84])) <= 1e-3 * np.max(np.abs(full))
+
+
+@pytest.mark.parametrize("ctx,new,n_q,n_kv,shares", [
+    ([1200, 300], [20, 40], 8, 2, 16),                  # two pairs per KV head: as many shares as the workspace holds
+    ([2368], [2368], 8, 1, 2),                          # 74 pairs of one KV head: two shares fill 148 SMs once
+])
+def test_least_workspace_holds_one_wave(ctx, new, n_q, n_kv, shares):
+    """The least workspace that is accepted holds one wave of shares, and the call makes use of all of them: the number that it
+    leaves beside the partial results of every row (behind the operands; rows of 132 floats, the count is the last but one)."""
+    import torch
+    from paper_2609_38121_b200 import binding as B
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("counts of a GPU with 148 SMs")
+    total = sum(new)
+    L = Layer(_wl(n_q, n_kv, len(ctx)), [c + n for c, n in zip(ctx, new)], 2, 4, 64, 1)
+    L.append_step(ctx, oracle_too=False)
+    L.append_step(new, oracle_too=False)
+    K, V, Q, cu = _chunk(L, ctx, new, total)
+    up = lambda x: (x + 255) // 256 * 256  # noqa: E731
+    operands = 2 * up(total * n_kv * 256) + up(2 * total * n_q * 256) + up(total * n_q * 4)
+    least, asked = up(operands + shares * total * n_q * 528), B.prefill_workspace_bytes(L.cache.desc, len(ctx), total)
+    outs = []
+    for nbytes in (least, asked):
+        ws = torch.zeros(nbytes, dtype=torch.uint8, device="cuda")
+        O = torch.full((total, n_q, 128), float("nan"), device="cuda")
+        B.prefill_attn(L.cache.desc, len(ctx), L.slot, L.seq_len, cu, total, max(new), K, V, Q, O, ws, nbytes)
+        outs.append(O.cpu().numpy())
+        counts = ws[operands:operands + total * n_q * 528].view(torch.float32).view(-1, 132)[:, 130]
+        if nbytes == least:
+            assert torch.all(counts == shares)
+    assert np.max(np.abs(outs[0] - outs[1])) <= 1e-3 * np.max(np.abs(outs[1]))
+    with pytest.raises(B.WushkvError) as e:
+        B.prefill_attn(L.cache.desc, len(ctx), L.slot, L.seq_len, cu, total, max(new), K, V, Q, O, ws, least - 1)
+    assert e.value.status == B.ECAPACITY
