@@ -255,7 +255,8 @@ __device__ bool cholesky_pivoted(double* S, int* perm, int* pivot_s, int* fail) 
     return *fail == 0;
 }
 
-// One CTA per head, float64.  ws: 8 matrices of d x d float64 per head (3 are used).
+// One CTA per head, float64.  ws: 8 matrices of d x d float64 per head (3 are used; the first element of the fourth says how many
+// sweeps the Jacobi took).
 //   L L^T = H (damped);  A = L^T M L (M damped), scaled to trace 1;  C C^T = A with its rows and columns in pivot order.
 //   One-sided Jacobi on the columns of C: rotations from the right until they are orthogonal, W = C V.  Then A = W W^T: the
 //   eigenvectors of A are W's columns over their lengths, the eigenvalues the lengths' squares.
@@ -317,13 +318,15 @@ __global__ void __launch_bounds__(BT_THREADS) build_transforms_kernel(const doub
     __syncthreads();
     if (!cholesky_pivoted(S, perm_s, &piv_row_s, &fail_s)) { if (tid == 0) atomicOr(status, WUSHKV_ENOTPD); return; }
     // ---- one-sided Jacobi, round-robin ordering.  Eight lanes own a pair of columns, 16 rows each (as 8 x 16 bytes: the eight lanes
-    // read 128 consecutive bytes).  The angle is computed in fp32 (its error only delays convergence), the rotation from it in
+    // read 128 consecutive bytes).  The angle is computed in fp32 (its error only delays convergence; where its operands leave the fp32
+    // range, as for columns whose lengths differ by more than 1e5, in float64), the rotation from it in
     // float64, so that it is orthogonal to rounding; the longer column goes to the lower index, which speeds convergence up.
+    int sweeps = 0;
     {
         constexpr double TOL2 = 1.6e-29;             // squared cosine below which a pair counts as orthogonal (its rounding is about 1e-30)
         const int pair = 4 * warp + (lane >> 3), l8 = lane & 7;
 #pragma unroll 1
-        for (int sweep = 0; sweep < 30; ++sweep) {
+        for (; sweeps < 30; ++sweeps) {
             int rotated = 0;
 #pragma unroll 1
             for (int step = 0; step < D - 1; ++step) {
@@ -350,7 +353,9 @@ __global__ void __launch_bounds__(BT_THREADS) build_transforms_kernel(const doub
                 if (g * g > TOL2 * (alpha * beta)) {
                     rotated = 1;
                     const float zeta = static_cast<float>(beta - alpha) / (2.f * static_cast<float>(g));
-                    const double t = static_cast<double>(copysignf(1.f, zeta) / (fabsf(zeta) + sqrtf(fmaf(zeta, zeta, 1.f))));
+                    double t = static_cast<double>(copysignf(1.f, zeta) / (fabsf(zeta) + sqrtf(fmaf(zeta, zeta, 1.f))));
+                    // zeta^2 overflows from 1.8e19 on, and zeta itself where g underflows: 1 / (2 zeta), and no more than 45 degrees
+                    if (!(fabsf(zeta) < 1e15f)) t = fmin(fmax(g / (beta - alpha), -1.0), 1.0);
                     const double c = rsqrt(fma(t, t, 1.0)), s = c * t;
                     const bool swap = alpha - t * g < beta + t * g;
                     const double c1 = swap ? s : c, s1 = swap ? -c : s;       // first column: c1 p - s1 q, second: s2 p + c2 q
@@ -366,6 +371,7 @@ __global__ void __launch_bounds__(BT_THREADS) build_transforms_kernel(const doub
             if (!__syncthreads_or(rotated)) break;
         }
     }
+    if (tid == 0) ws[3 * D * D] = sweeps;            // for the tests: sweeps that rotated something
     // ---- canonical form: eigenvalues ascending, largest-magnitude entry of each eigenvector positive
     if (tid < D) {
         double len2 = 0.0, top = 0.0;

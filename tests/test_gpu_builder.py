@@ -55,3 +55,31 @@ def test_indefinite_statistics_are_refused(which):
     with pytest.raises(B.WushkvError) as e:
         _build(M[None].copy(), H[None].copy(), 0.0)
     assert e.value.status == B.ENOTPD
+
+
+@pytest.mark.parametrize("gamma", [0.0, 1e-8])
+def test_columns_of_very_different_length(gamma):
+    """Spectra of M and H over seven decades each and next to no damping: the columns that the Jacobi rotates then differ in length by
+    1e6, and the tangent of their angle is the reciprocal of numbers whose square is beyond the fp32 range.  A pair that counts
+    as rotated without being turned would keep the sweeps going to their limit of 30; 10 to 12 are enough (a numpy model of
+    the same rule)."""
+    import torch
+    from paper_2609_38121_b200 import binding as B
+    rng = np.random.default_rng(5)
+    M, H = np.stack([_spd(rng, 7.0, 1.0) for _ in range(3)]), np.stack([_spd(rng, 7.0, 1.0) for _ in range(3)])
+    nbytes = B.lib.wushkv_build_transforms_workspace_bytes(3, 128)
+    dev = lambda x: torch.from_numpy(x).cuda()  # noqa: E731
+    Md, Hd, ws = dev(M), dev(H), torch.zeros(nbytes // 8, dtype=torch.float64, device="cuda")
+    T, Ti = torch.zeros((3, 128, 128), device="cuda"), torch.zeros((3, 128, 128), device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    stream = torch.cuda.current_stream().cuda_stream
+    assert B.lib.wushkv_build_transforms_device(3, 128, Md.data_ptr(), Hd.data_ptr(), gamma, T.data_ptr(), Ti.data_ptr(), status.data_ptr(),
+                                                ws.data_ptr(), nbytes, stream) == B.OK
+    torch.cuda.synchronize()
+    assert status.item() == 0
+    sweeps = ws.view(3, 8, 128 * 128)[:, 3, 0].cpu().numpy()
+    assert np.all(sweeps >= 5) and np.all(sweeps <= 16), sweeps
+    ref, _ = O.build_transforms(M, H, gamma)            # compared as in test_scales_and_graded_spectra
+    Td = T.cpu().numpy().astype(np.float64)
+    unit = np.maximum(np.abs(ref), 1e-9 * np.abs(ref).max()) * 2.0 ** -7
+    assert np.all(np.abs(Td - ref) <= unit) and np.mean(Td != ref) < 1e-3
