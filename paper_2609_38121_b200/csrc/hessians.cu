@@ -18,7 +18,7 @@
 //   project_kernel    U, kappa and alpha: 64 x 128 tiles
 //   pairs_kernel      logits and v_s . U for (position t; 4 keys s) per thread, all query heads and up to 10 pairs; A, W0
 //   key_kernel        H_K: sum over (t, g) of q_{g,t} (sum_g' A_{gg'}(t) q_{g',t})^T, float64 across groups of 16
-//   value_kernel      H_V = 2 sum_{gg'} (sum_t W0) Gamma_{gg'}
+//   finish_kernel     H_V = 2 sum_{gg'} (sum_t W0) Gamma_{gg'}; the slices of H_K added up in order
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -48,6 +48,8 @@ struct HessParams {
     float* alpha;                // [S][n_kv][n_pairs]
     float* A;                    // [S][n_kv][n_pairs]   pairs g <= g' in row-major order
     float* W0;                   // [S][n_kv][n_pairs]
+    double* key_part;            // [n_slices][n_kv][36][16][16] sums of key_kernel over a slice of positions, over Oh and U
+    int n_slices, slice_len;
     double* H_K;                 // [n_kv][D][D]
     double* H_V;
 };
@@ -431,28 +433,46 @@ __global__ void __launch_bounds__(256, 1) pairs_kernel(HessParams P) {
     }
 }
 
-// H_K[h][i][j] += (2 / tau^2) sum_t sum_g q_{g,t}[i] (sum_g' A_{gg'}(t) q_{g',t}[j]): grid (slices of positions, n_kv), 512 threads.
-constexpr int KEY_SLICE = 64;
+// One entry on or above the diagonal, and its mirror image.
+__device__ __forceinline__ void add_key_entry(const HessParams& P, int h, int i, int j, double sum) {
+    if (i > j) return;                                   // the other half of a block on the diagonal
+    const double v = 2.0 * static_cast<double>(P.inv_tau) * static_cast<double>(P.inv_tau) * sum;
+    double* H = P.H_K + static_cast<long long>(h) * D * D;
+    H[i * D + j] += v;
+    if (i != j) H[j * D + i] += v;
+}
+
+// H_K[h][i][j] += (2 / tau^2) sum_t sum_g q_{g,t}[i] (sum_g' A_{gg'}(t) q_{g',t}[j]): the 36 blocks of 16 x 16 entries on and above
+// the diagonal, one per warp; the entries below are their mirror images (the sum is symmetric).  grid (slices of positions, n_kv, 3),
+// 384 threads; lane (r, c) = (lane >> 2, lane & 3) holds rows 2 r .. and columns 4 c .. of its warp's block.  With one slice the
+// sums go to H_K, else they are left in the workspace (over U and the head outputs, which nothing reads any more) and
+// finish_kernel adds them up in the order of the slices: the same bits on every run.
+constexpr int KEY_SLICE = 64, KEY_BLOCKS = 36, KEY_WARPS = 12;
+__device__ __forceinline__ void key_block(int k, int& bi, int& bj) { pair_heads(k, 8, bi, bj); }
 template <int G>
-__global__ void __launch_bounds__(512) key_kernel(HessParams P) {
+__global__ void __launch_bounds__(32 * KEY_WARPS) key_kernel(HessParams P) {
     __shared__ __align__(16) float a_s[OUTER_K][HS_PITCH], b_s[OUTER_K][HS_PITCH];
-    __shared__ float c_s[OUTER_K / G > 0 ? OUTER_K / G : 1][G][G];
+    __shared__ float c_s[OUTER_K / G][G][G];
     constexpr int TG = OUTER_K / G;                      // positions per staged group (G = 1 .. 8: at least 2)
-    const int h = blockIdx.y, tid = threadIdx.x, t_end = min(static_cast<int>(blockIdx.x + 1) * KEY_SLICE, P.S);
-    double acc[4][8] = {};
-    for (int t0 = blockIdx.x * KEY_SLICE; t0 < t_end; t0 += TG) {
+    const int h = blockIdx.y, tid = threadIdx.x, t_end = min(static_cast<int>(blockIdx.x + 1) * P.slice_len, P.S);
+    const int block = blockIdx.z * KEY_WARPS + (tid >> 5), lane = tid & 31;
+    int bi, bj;
+    key_block(block, bi, bj);
+    const int i0 = 16 * bi + 2 * (lane >> 2), j0 = 16 * bj + 4 * (lane & 3);
+    double acc[2][4] = {};
+    for (int t0 = blockIdx.x * P.slice_len; t0 < t_end; t0 += TG) {
         __syncthreads();
-        for (int item = tid; item < TG * G * G; item += 512) {
+        for (int item = tid; item < TG * G * G; item += 32 * KEY_WARPS) {
             const int t = t0 + item / (G * G), g = item / G % G, gp = item % G, lo = min(g, gp), hi = max(g, gp);
             c_s[item / (G * G)][g][gp] = t < t_end ? P.A[(static_cast<long long>(t) * P.n_kv + h) * P.n_pairs + lo * G - lo * (lo - 1) / 2 + hi - lo] : 0.f;
         }
-        for (int item = tid; item < OUTER_K * 32; item += 512) {
+        for (int item = tid; item < OUTER_K * 32; item += 32 * KEY_WARPS) {
             const int row = item >> 5, t = t0 + row / G, piece = item & 31;
             *reinterpret_cast<float4*>(&a_s[row][4 * piece]) =
                 row < TG * G && t < t_end ? bf16x4(P.Q + (static_cast<long long>(t) * P.n_q + h * G + row % G) * D + 4 * piece) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
         __syncthreads();
-        for (int item = tid; item < OUTER_K * D; item += 512) {
+        for (int item = tid; item < OUTER_K * D; item += 32 * KEY_WARPS) {
             const int row = item >> 7, ch = item & 127, tl = row / G, g = row % G;
             float x = 0.f;
             if (row < TG * G)
@@ -461,25 +481,52 @@ __global__ void __launch_bounds__(512) key_kernel(HessParams P) {
             b_s[row][ch] = x;
         }
         __syncthreads();
-        outer_group(a_s, b_s, acc);
-    }
-    const double f = 2.0 * static_cast<double>(P.inv_tau) * static_cast<double>(P.inv_tau);
-    const int i0 = 4 * (tid >> 4), j0 = tid & 15;
+        float part[2][4] = {};
 #pragma unroll
-    for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {                    // half to either side of the diagonal: symmetric like the exact sum
-            double* H = P.H_K + static_cast<long long>(h) * D * D;
-            const int i = i0 + r, j = j0 + 16 * e;
-            atomicAdd(H + i * D + j, 0.5 * f * acc[r][e]);
-            atomicAdd(H + j * D + i, 0.5 * f * acc[r][e]);
+        for (int k = 0; k < OUTER_K; ++k) {
+            const float2 av = *reinterpret_cast<const float2*>(&a_s[k][i0]);
+            const float4 bv = *reinterpret_cast<const float4*>(&b_s[k][j0]);
+            part[0][0] = fmaf(av.x, bv.x, part[0][0]); part[0][1] = fmaf(av.x, bv.y, part[0][1]);
+            part[0][2] = fmaf(av.x, bv.z, part[0][2]); part[0][3] = fmaf(av.x, bv.w, part[0][3]);
+            part[1][0] = fmaf(av.y, bv.x, part[1][0]); part[1][1] = fmaf(av.y, bv.y, part[1][1]);
+            part[1][2] = fmaf(av.y, bv.z, part[1][2]); part[1][3] = fmaf(av.y, bv.w, part[1][3]);
         }
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) acc[r][e] += static_cast<double>(part[r][e]);
+    }
+    if (P.n_slices > 1) {
+        double* dst = P.key_part + ((static_cast<long long>(blockIdx.x) * P.n_kv + h) * KEY_BLOCKS + block) * 256 + 32 * (lane >> 2) + 4 * (lane & 3);
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            reinterpret_cast<double2*>(dst + 16 * r)[0] = make_double2(acc[r][0], acc[r][1]);
+            reinterpret_cast<double2*>(dst + 16 * r)[1] = make_double2(acc[r][2], acc[r][3]);
+        }
+        return;
+    }
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) add_key_entry(P, h, i0 + r, j0 + e, acc[r][e]);
 }
 
-// H_V[h] += 2 sum_{g<=g'} c_{gg'} sym(Gamma_{gg'}), c = sum_t W0(t): grid (16 row groups, n_kv), 256 threads.
-__global__ void __launch_bounds__(256) value_kernel(HessParams P) {
+// H_V[h] += 2 sum_{g<=g'} c_{gg'} sym(Gamma_{gg'}), c = sum_t W0(t), and the sums of key_kernel's slices: grid (16 row groups of H_V
+// and, with several slices, the 36 blocks of H_K; n_kv), 256 threads.
+__global__ void __launch_bounds__(256) finish_kernel(HessParams P) {
     __shared__ double c_s[36];
     const int h = blockIdx.y, tid = threadIdx.x, lane = tid & 31;
+    if (blockIdx.x >= 16) {
+        const int block = blockIdx.x - 16;
+        int bi, bj;
+        key_block(block, bi, bj);
+        const double* src = P.key_part + (static_cast<long long>(h) * KEY_BLOCKS + block) * 256 + tid;
+        double sum = 0.0;
+#pragma unroll 8
+        for (int k = 0; k < P.n_slices; ++k) sum += src[static_cast<long long>(k) * P.n_kv * KEY_BLOCKS * 256];
+        add_key_entry(P, h, 16 * bi + (tid >> 4), 16 * bj + (tid & 15), sum);
+        return;
+    }
     for (int k = tid >> 5; k < P.n_pairs; k += 8) {
         double sum = 0.0;
         for (int t = lane; t < P.S; t += 32) sum += static_cast<double>(P.W0[(static_cast<long long>(t) * P.n_kv + h) * P.n_pairs + k]);
@@ -506,7 +553,7 @@ bool launch_pairs(const HessParams& P, cudaStream_t st) {
     constexpr int NC = pairs_per_chunk(G);
     if (!opt_in_dynamic_smem(reinterpret_cast<const void*>(pairs_kernel<G, NC>), static_cast<int>(sizeof(PairsSmem<G, NC>)))) return false;
     pairs_kernel<G, NC><<<dim3((P.S + 15) / 16, pair_chunks(G), P.n_kv), 256, sizeof(PairsSmem<G, NC>), st>>>(P);
-    key_kernel<G><<<dim3((P.S + KEY_SLICE - 1) / KEY_SLICE, P.n_kv), 512, 0, st>>>(P);
+    key_kernel<G><<<dim3(P.n_slices, P.n_kv, KEY_BLOCKS / KEY_WARPS), 32 * KEY_WARPS, 0, st>>>(P);
     return true;
 }
 
@@ -562,6 +609,12 @@ extern "C" int wushkv_accumulate_attention_hessians_device(int32_t n_kv, int32_t
     P.kappa = reinterpret_cast<float*>(ws + L.kappa);
     P.alpha = reinterpret_cast<float*>(ws + L.alpha); P.A = reinterpret_cast<float*>(ws + L.A); P.W0 = reinterpret_cast<float*>(ws + L.W0);
     P.H_K = H_K; P.H_V = H_V;
+    // Slices of 64 positions or more: no more of them than give every SM two waves of CTAs, nor than fit over Oh and U.
+    const long long room = static_cast<long long>(L.kappa - L.Oh) / (static_cast<long long>(n_kv) * KEY_BLOCKS * 256 * 8);
+    const long long want = std::max<long long>(1, std::min<long long>({(n_tokens + KEY_SLICE - 1) / KEY_SLICE, room, 2LL * sm_count() / n_kv}));
+    P.slice_len = static_cast<int>((n_tokens + want - 1) / want);
+    P.n_slices = static_cast<int>((n_tokens + P.slice_len - 1) / P.slice_len);
+    P.key_part = reinterpret_cast<double*>(ws + L.Oh);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (!opt_in_dynamic_smem(reinterpret_cast<const void*>(rows_kernel), static_cast<int>(sizeof(RowsSmem))) ||
         !opt_in_dynamic_smem(reinterpret_cast<const void*>(project_kernel), static_cast<int>(sizeof(ProjectSmem))))
@@ -582,6 +635,6 @@ extern "C" int wushkv_accumulate_attention_hessians_device(int32_t n_kv, int32_t
         default: ok = launch_pairs<8>(P, st); break;
     }
     if (!ok) return WUSHKV_ECUDA;
-    value_kernel<<<dim3(16, n_kv), 256, 0, st>>>(P);
+    finish_kernel<<<dim3(16 + (P.n_slices > 1 ? KEY_BLOCKS : 0), n_kv), 256, 0, st>>>(P);
     return cudaGetLastError() == cudaSuccess ? WUSHKV_OK : WUSHKV_ECUDA;
 }

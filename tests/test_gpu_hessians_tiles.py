@@ -20,3 +20,14 @@ def test_tile_edges(n_q, n_kv, n_tok, d_model):
         if n_tok > 1:                                   # one position attends to itself only: v - o = 0
             assert np.max(np.abs(HK[h] - rk)) <= TOL * np.max(np.abs(rk))
         assert np.max(np.abs(HV[h] - rv)) <= TOL * np.max(np.abs(rv))
+
+
+@pytest.mark.parametrize("n_q,n_kv,n_tok", [(8, 2, 510), (2, 2, 500), (3, 1, 200)])
+def test_runs_agree_bit_for_bit(n_q, n_kv, n_tok):
+    """Sums over several slices of positions are added in a fixed order."""
+    wl, K, Q, V, WO = _inputs(n_q, n_kv, n_tok, 16, seed=73)
+    first = _gpu(K, Q, V, WO, float(np.sqrt(128)))
+    assert np.array_equal(first[0], first[0].transpose(0, 2, 1))
+    for _ in range(5):
+        again = _gpu(K, Q, V, WO, float(np.sqrt(128)))
+        assert np.array_equal(first[0], again[0]) and np.array_equal(first[1], again[1])
