@@ -17,7 +17,7 @@
 //   rows_kernel       causal softmax statistics (max, 1 / sum) and head outputs o_{g,t}: 64 x 64 tiles
 //   project_kernel    U, kappa and alpha: 64 x 128 tiles
 //   pairs_kernel      logits and v_s . U for (position t; 4 keys s) per thread, all query heads and up to 10 pairs; A, W0
-//   key_kernel        H_K: sum over (t, g) of q_{g,t} (sum_g' A_{gg'}(t) q_{g',t})^T, float64 across groups of 16
+//   key_kernel        H_K: sum over (t, g) of q_{g,t} (sum_g' A_{gg'}(t) q_{g',t})^T, float64 across positions
 //   finish_kernel     H_V = 2 sum_{gg'} (sum_t W0) Gamma_{gg'}; the slices of H_K added up in order
 #include <cuda_runtime.h>
 
@@ -460,18 +460,35 @@ __global__ void __launch_bounds__(32 * KEY_WARPS) key_kernel(HessParams P) {
     key_block(block, bi, bj);
     const int i0 = 16 * bi + 2 * (lane >> 2), j0 = 16 * bj + 4 * (lane & 3);
     double acc[2][4] = {};
+    // the next group's queries and coefficients are requested while this one is multiplied
+    constexpr int N_Q = (OUTER_K * 32 + 32 * KEY_WARPS - 1) / (32 * KEY_WARPS);
+    static_assert(TG * G * G <= 32 * KEY_WARPS, "a coefficient per thread");
+    uint2 q_next[N_Q];
+    float c_next = 0.f;
+    auto request = [&](int t0) {
+#pragma unroll
+        for (int n = 0; n < N_Q; ++n) {
+            const int item = tid + n * 32 * KEY_WARPS, row = item >> 5, t = t0 + row / G;
+            q_next[n] = row < TG * G && t < t_end
+                            ? *reinterpret_cast<const uint2*>(P.Q + (static_cast<long long>(t) * P.n_q + h * G + row % G) * D + 4 * (item & 31)) : make_uint2(0u, 0u);
+        }
+        const int t = t0 + tid / (G * G), g = tid / G % G, gp = tid % G, lo = min(g, gp), hi = max(g, gp);
+        c_next = tid < TG * G * G && t < t_end ? P.A[(static_cast<long long>(t) * P.n_kv + h) * P.n_pairs + lo * G - lo * (lo - 1) / 2 + hi - lo] : 0.f;
+    };
+    request(blockIdx.x * P.slice_len);
     for (int t0 = blockIdx.x * P.slice_len; t0 < t_end; t0 += TG) {
         __syncthreads();
-        for (int item = tid; item < TG * G * G; item += 32 * KEY_WARPS) {
-            const int t = t0 + item / (G * G), g = item / G % G, gp = item % G, lo = min(g, gp), hi = max(g, gp);
-            c_s[item / (G * G)][g][gp] = t < t_end ? P.A[(static_cast<long long>(t) * P.n_kv + h) * P.n_pairs + lo * G - lo * (lo - 1) / 2 + hi - lo] : 0.f;
-        }
-        for (int item = tid; item < OUTER_K * 32; item += 32 * KEY_WARPS) {
-            const int row = item >> 5, t = t0 + row / G, piece = item & 31;
-            *reinterpret_cast<float4*>(&a_s[row][4 * piece]) =
-                row < TG * G && t < t_end ? bf16x4(P.Q + (static_cast<long long>(t) * P.n_q + h * G + row % G) * D + 4 * piece) : make_float4(0.f, 0.f, 0.f, 0.f);
+        if (tid < TG * G * G) c_s[tid / (G * G)][tid / G % G][tid % G] = c_next;
+#pragma unroll
+        for (int n = 0; n < N_Q; ++n) {
+            const int item = tid + n * 32 * KEY_WARPS;
+            const uint2 w = q_next[n];
+            if (item < OUTER_K * 32)
+                *reinterpret_cast<float4*>(&a_s[item >> 5][4 * (item & 31)]) =
+                    make_float4(bf16_bits_to_float(w.x & 0xffff), bf16_bits_to_float(w.x >> 16), bf16_bits_to_float(w.y & 0xffff), bf16_bits_to_float(w.y >> 16));
         }
         __syncthreads();
+        request(t0 + TG);
         for (int item = tid; item < OUTER_K * D; item += 32 * KEY_WARPS) {
             const int row = item >> 7, ch = item & 127, tl = row / G, g = row % G;
             float x = 0.f;
@@ -481,20 +498,23 @@ __global__ void __launch_bounds__(32 * KEY_WARPS) key_kernel(HessParams P) {
             b_s[row][ch] = x;
         }
         __syncthreads();
-        float part[2][4] = {};
 #pragma unroll
-        for (int k = 0; k < OUTER_K; ++k) {
-            const float2 av = *reinterpret_cast<const float2*>(&a_s[k][i0]);
-            const float4 bv = *reinterpret_cast<const float4*>(&b_s[k][j0]);
-            part[0][0] = fmaf(av.x, bv.x, part[0][0]); part[0][1] = fmaf(av.x, bv.y, part[0][1]);
-            part[0][2] = fmaf(av.x, bv.z, part[0][2]); part[0][3] = fmaf(av.x, bv.w, part[0][3]);
-            part[1][0] = fmaf(av.y, bv.x, part[1][0]); part[1][1] = fmaf(av.y, bv.y, part[1][1]);
-            part[1][2] = fmaf(av.y, bv.z, part[1][2]); part[1][3] = fmaf(av.y, bv.w, part[1][3]);
+        for (int tl = 0; tl < TG; ++tl) {                // a position's sum over the heads in fp32, beyond that float64
+            float part[2][4] = {};
+#pragma unroll
+            for (int k = tl * G; k < tl * G + G; ++k) {
+                const float2 av = *reinterpret_cast<const float2*>(&a_s[k][i0]);
+                const float4 bv = *reinterpret_cast<const float4*>(&b_s[k][j0]);
+                part[0][0] = fmaf(av.x, bv.x, part[0][0]); part[0][1] = fmaf(av.x, bv.y, part[0][1]);
+                part[0][2] = fmaf(av.x, bv.z, part[0][2]); part[0][3] = fmaf(av.x, bv.w, part[0][3]);
+                part[1][0] = fmaf(av.y, bv.x, part[1][0]); part[1][1] = fmaf(av.y, bv.y, part[1][1]);
+                part[1][2] = fmaf(av.y, bv.z, part[1][2]); part[1][3] = fmaf(av.y, bv.w, part[1][3]);
+            }
+#pragma unroll
+            for (int r = 0; r < 2; ++r)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) acc[r][e] += static_cast<double>(part[r][e]);
         }
-#pragma unroll
-        for (int r = 0; r < 2; ++r)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) acc[r][e] += static_cast<double>(part[r][e]);
     }
     if (P.n_slices > 1) {
         double* dst = P.key_part + ((static_cast<long long>(blockIdx.x) * P.n_kv + h) * KEY_BLOCKS + block) * 256 + 32 * (lane >> 2) + 4 * (lane & 3);

@@ -31,3 +31,28 @@ def test_runs_agree_bit_for_bit(n_q, n_kv, n_tok):
     for _ in range(5):
         again = _gpu(K, Q, V, WO, float(np.sqrt(128)))
         assert np.array_equal(first[0], again[0]) and np.array_equal(first[1], again[1])
+
+
+@pytest.mark.parametrize("n_q,n_kv,n_tok", [(1, 1, 500), (3, 1, 300), (8, 1, 200)])
+def test_positions_are_summed_in_float64(n_q, n_kv, n_tok):
+    """Channel 5 of the queries is repeated in channel 9 at even positions and in channel 70 at odd ones (zero otherwise), so that
+    every position contributes the same fp32 number to H_K[5][5] as to H_K[5][9] or H_K[5][70], and nothing to the other:
+    H_K[5][5] = H_K[5][9] + H_K[5][70] up to the float64 rounding of n_tok sums.  Any fp32 sum over positions breaks this at 1e-8."""
+    wl, K, Q, V, WO = _inputs(n_q, n_kv, n_tok, 16, seed=79)
+    Q = Q.copy()
+    Q[:, :, 9] = np.where(np.arange(n_tok)[:, None] % 2 == 0, Q[:, :, 5], 0)
+    Q[:, :, 70] = np.where(np.arange(n_tok)[:, None] % 2 == 1, Q[:, :, 5], 0)
+    HK, _ = _gpu(K, Q, V, WO, float(np.sqrt(128)))
+    assert HK[0, 5, 9] != 0 and HK[0, 5, 70] != 0
+    assert abs(HK[0, 5, 5] - HK[0, 5, 9] - HK[0, 5, 70]) <= n_tok * 2.0 ** -52 * abs(HK[0, 5, 5])
+
+
+def test_seven_heads_and_a_long_sequence():
+    """Three chunks of pairs, the last one short (28 pairs), and one head over many slices, against the literal form."""
+    for n_q, n_tok, d_model in [(7, 70, 16), (1, 400, 8)]:
+        wl, K, Q, V, WO = _inputs(n_q, 1, n_tok, d_model, seed=71)
+        tau = float(np.sqrt(128))
+        HK, HV = _gpu(K, Q, V, WO, tau)
+        rk, rv = O.attention_hessians(Q, K[:, 0], V[:, 0], WO, tau)
+        assert np.max(np.abs(HK[0] - rk)) <= TOL * np.max(np.abs(rk))
+        assert np.max(np.abs(HV[0] - rv)) <= TOL * np.max(np.abs(rv))
