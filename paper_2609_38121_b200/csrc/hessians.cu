@@ -44,7 +44,7 @@ struct HessParams {
     float* row_linv;             // [S][n_q] 1 / sum exp
     float* Oh;                   // [S][n_q][D]
     float* U;                    // [S][n_kv][n_pairs][D]
-    float* kappa;                // [S][n_kv][n_pairs]
+    float* kappa;                // [S][n_kv][n_pairs], where A goes: pairs_kernel reads a position's before it writes its A
     float* alpha;                // [S][n_kv][n_pairs]
     float* A;                    // [S][n_kv][n_pairs]   pairs g <= g' in row-major order
     float* W0;                   // [S][n_kv][n_pairs]
@@ -579,7 +579,7 @@ bool launch_pairs(const HessParams& P, cudaStream_t st) {
 
 size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 
-struct HessLayout { size_t gamma, row_m, row_linv, Oh, U, kappa, alpha, A, W0, total; };
+struct HessLayout { size_t gamma, row_m, row_linv, Oh, U, alpha, A, W0, total; };
 HessLayout hess_layout(int n_kv, int n_q, long long S) {
     const int G = n_q / n_kv, NP = G * (G + 1) / 2;
     HessLayout L;
@@ -589,7 +589,6 @@ HessLayout hess_layout(int n_kv, int n_q, long long S) {
     L.row_linv = off; off = align256(off + static_cast<size_t>(S) * n_q * sizeof(float));
     L.Oh = off;       off = align256(off + static_cast<size_t>(S) * n_q * D * sizeof(float));
     L.U = off;        off = align256(off + static_cast<size_t>(S) * n_kv * NP * D * sizeof(float));
-    L.kappa = off;    off = align256(off + static_cast<size_t>(S) * n_kv * NP * sizeof(float));
     L.alpha = off;    off = align256(off + static_cast<size_t>(S) * n_kv * NP * sizeof(float));
     L.A = off;        off = align256(off + static_cast<size_t>(S) * n_kv * NP * sizeof(float));
     L.W0 = off;       off = align256(off + static_cast<size_t>(S) * n_kv * NP * sizeof(float));
@@ -626,11 +625,11 @@ extern "C" int wushkv_accumulate_attention_hessians_device(int32_t n_kv, int32_t
     P.gamma = reinterpret_cast<float*>(ws + L.gamma);
     P.row_m = reinterpret_cast<float*>(ws + L.row_m); P.row_linv = reinterpret_cast<float*>(ws + L.row_linv);
     P.Oh = reinterpret_cast<float*>(ws + L.Oh); P.U = reinterpret_cast<float*>(ws + L.U);
-    P.kappa = reinterpret_cast<float*>(ws + L.kappa);
-    P.alpha = reinterpret_cast<float*>(ws + L.alpha); P.A = reinterpret_cast<float*>(ws + L.A); P.W0 = reinterpret_cast<float*>(ws + L.W0);
+    P.kappa = P.A = reinterpret_cast<float*>(ws + L.A);
+    P.alpha = reinterpret_cast<float*>(ws + L.alpha); P.W0 = reinterpret_cast<float*>(ws + L.W0);
     P.H_K = H_K; P.H_V = H_V;
     // Slices of 64 positions or more: no more of them than give every SM two waves of CTAs, nor than fit over Oh and U.
-    const long long room = static_cast<long long>(L.kappa - L.Oh) / (static_cast<long long>(n_kv) * KEY_BLOCKS * 256 * 8);
+    const long long room = static_cast<long long>(L.alpha - L.Oh) / (static_cast<long long>(n_kv) * KEY_BLOCKS * 256 * 8);
     const long long want = std::max<long long>(1, std::min<long long>({(n_tokens + KEY_SLICE - 1) / KEY_SLICE, room, 2LL * sm_count() / n_kv}));
     P.slice_len = static_cast<int>((n_tokens + want - 1) / want);
     P.n_slices = static_cast<int>((n_tokens + P.slice_len - 1) / P.slice_len);

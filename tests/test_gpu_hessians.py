@@ -70,3 +70,26 @@ def test_group_sizes_beyond_eight_are_refused():
     from paper_2609_38121_b200 import binding as B
     assert B.lib.wushkv_attention_hessians_workspace_bytes(1, 9, 128, 64) == 0
     assert B.lib.wushkv_attention_hessians_workspace_bytes(1, 8, 128, 64) > 0
+
+
+def test_workspace_of_one_head_per_group():
+    """Gamma, softmax statistics, outputs, one projection, and three numbers per position and head: what such a call asks for, and what
+    is enough for it."""
+    import torch
+    from paper_2609_38121_b200 import binding as B
+    wl, K, Q, V, WO = _inputs(2, 2, 40, 16)
+    up = lambda x: (x + 255) // 256 * 256  # noqa: E731
+    n, row = 2, 40 * 2 * 4
+    nbytes = n * 128 * 128 * 4 + 2 * up(row) + 2 * 40 * 2 * 512 + 3 * up(row)
+    assert B.lib.wushkv_attention_hessians_workspace_bytes(2, 2, 128, 40) <= nbytes
+    bits = lambda x: torch.from_numpy(W.f32_to_bf16_bits(x).view(np.int16)).cuda()  # noqa: E731
+    k, q, v, w = bits(K), bits(Q), bits(V), torch.from_numpy(WO).cuda()
+    H = torch.zeros((2, 2, 128, 128), dtype=torch.float64, device="cuda")
+    ws = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+    tau = float(np.sqrt(128))
+    status = B.lib.wushkv_accumulate_attention_hessians_device(2, 2, 128, 16, 40, k.data_ptr(), q.data_ptr(), v.data_ptr(), w.data_ptr(), tau,
+                                                               H[0].data_ptr(), H[1].data_ptr(), ws.data_ptr(), nbytes, torch.cuda.current_stream().cuda_stream)
+    assert status == B.OK
+    for h in range(2):
+        rk, _ = O.attention_hessians(Q[:, h:h + 1], K[:, h], V[:, h], WO[h:h + 1], tau)
+        assert np.max(np.abs(H[0, h].cpu().numpy() - rk)) <= TOL * np.max(np.abs(rk))
