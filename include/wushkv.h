@@ -184,7 +184,8 @@ int wushkv_build_transforms_device(int32_t n_heads, int32_t d, const double* M, 
  * Chunks (max_new >= 128, or many shorter ones) take the tensor-core transform path (tcgen05, fp32 accumulation in
  * tensor memory), max_new == 1 a single-launch decode-time path, anything else a CUDA-core path.
  * All produce the same codes up to fp32 summation order (wushkv_set_test_option("append_path_cuda", 1)
- * forces the CUDA-core path for chunks).
+ * forces the CUDA-core path for chunks) for a T_K of bf16 values, as the library builds it.  Another T_K is taken as
+ * it is by calls with max_new < 128 and rounded to bf16 by longer chunks.
  */
 int wushkv_append(const wushkv_cache* cache, int32_t batch, const int32_t* slot, int32_t* seq_len,
                   const int32_t* cu_new, int32_t total_new, int32_t max_new,

@@ -16,6 +16,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 #include <cstdlib>
 
 #include "host_common.h"
@@ -600,8 +601,10 @@ __device__ __forceinline__ void quad_quantize(const float (&x)[32], ClipRule rul
 }
 
 // KK_K / KK_V: list length of the quad quantizer for keys / values (8 or 16, >= the rule's rounds), 0 for
-// the warp-per-vector quantizer (any kappa), or -1 for the QuEST rule (Eq. 5, no order statistics).
-template <int BITS, int KK_K, int KK_V>
+// the warp-per-vector quantizer (any kappa), or -1 for the QuEST rule (Eq. 5, no order statistics).  EXACT: T_K as it is given, for
+// calls that would take the CUDA cores if their chunks were fewer; otherwise rounded to bf16 (which changes nothing in the
+// transforms that the library builds).  A kernel of its own, as the other has no register to spare: 1 us of a 300-token chunk.
+template <int BITS, int KK_K, int KK_V, bool EXACT>
 __global__ void __launch_bounds__(TC_THREADS, 2) append_chunk_kernel(AppendParams P, const __grid_constant__ CUtensorMap map_k,
                                                                      const __grid_constant__ CUtensorMap map_v) {
     extern __shared__ __align__(1024) unsigned char tc_smem[];
@@ -630,6 +633,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2) append_chunk_kernel(AppendParam
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(tbar) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    unsigned inexact = 0;
     {
         const float* T = P.c.T_K + static_cast<long long>(head) * D * D;
         const int r8 = lane & 7, cq = lane >> 3;
@@ -644,6 +648,8 @@ __global__ void __launch_bounds__(TC_THREADS, 2) append_chunk_kernel(AppendParam
         for (int k = 0; k < 4; ++k) {
             const int item = warp + k * (TC_THREADS / 32), rg = item >> 2, kc = (item & 3) * 4 + cq;
             const float4 a = ta[k], b = tb[k];
+            if (EXACT) inexact |= (__float_as_uint(a.x) | __float_as_uint(a.y) | __float_as_uint(a.z) | __float_as_uint(a.w) |
+                        __float_as_uint(b.x) | __float_as_uint(b.y) | __float_as_uint(b.z) | __float_as_uint(b.w)) & 0xffffu;
             uint4 v;
             v.x = float_to_bf16_bits(a.x) | (static_cast<unsigned>(float_to_bf16_bits(a.y)) << 16);
             v.y = float_to_bf16_bits(a.z) | (static_cast<unsigned>(float_to_bf16_bits(a.w)) << 16);
@@ -653,14 +659,32 @@ __global__ void __launch_bounds__(TC_THREADS, 2) append_chunk_kernel(AppendParam
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
+    // The transforms that the library builds hold bf16 values, one term.  Another one is exact in three: hi, then what hi left, twice,
+    // multiplied one after the other out of the same operand buffer (8 MMAs and 32 KB from L2 each).
+    volatile int* three_terms = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    if (EXACT) {
+        const int any = __syncthreads_or(static_cast<int>(inexact));
+        if (tid == 0) *three_terms = any;                    // (read behind the barriers of a tile)
+    } else __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const unsigned tmem_base = *tmem_slot;
     unsigned phase = 0;
     bool failed = false;
+    auto store_term = [&](const int term) {
+        const float* T = P.c.T_K + static_cast<long long>(head) * D * D;
+#pragma unroll 1
+        for (int idx = 2 * tid; idx < D * D; idx += 2 * TC_THREADS) {
+            const int i = idx >> 7, j = idx & 127;
+            float x = ld_in(T + idx), y = ld_in(T + idx + 1);
+            for (int k = 0; k < term; ++k) { x -= bf16_bits_to_float(float_to_bf16_bits(x)); y -= bf16_bits_to_float(float_to_bf16_bits(y)); }
+            *reinterpret_cast<unsigned*>(sB + (i >> 3) * TC_SBO + (j >> 3) * TC_LBO + (i & 7) * 16 + (j & 7) * 2) =
+                float_to_bf16_bits(x) | (static_cast<unsigned>(float_to_bf16_bits(y)) << 16);
+        }
+    };
 
     for (int tile = blockIdx.x; tile < n_tiles && !failed; tile += gridDim.x) {
         const int tok0 = tile * TC_TILE;
+        if (EXACT && tile != static_cast<int>(blockIdx.x) && *three_terms) store_term(0);
         // ---- A operand: key rows of this tile (zero rows past the end of the batch), and the value rows of the
         // tile into the part of the fp32 tile that is free until the MMAs are done; both as 16-byte
         // asynchronous copies, so that no register waits for them
@@ -782,12 +806,14 @@ __global__ void __launch_bounds__(TC_THREADS, 2) append_chunk_kernel(AppendParam
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");       // generic-proxy writes -> visible to the tensor core
         __syncthreads();
         // ---- one thread issues the 8 k-steps and commits them to the barrier
+#pragma unroll 1
+        for (int term = 0;; ++term) {
         if (tid == 0) {
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const unsigned long long adesc = umma_smem_desc(smem_addr_u32(sA)), bdesc = umma_smem_desc(smem_addr_u32(sB));
 #pragma unroll
             for (int ks = 0; ks < 8; ++ks) {
-                const unsigned accumulate = ks > 0 ? 1u : 0u;
+                const unsigned accumulate = ks > 0 || (EXACT && term > 0) ? 1u : 0u;
                 // swizzled A: channels 0-63 and 64-127 are two boxes of 16 KB, a k-step is 32 bytes inside the 128-byte row
                 const unsigned long long a_ks = P.use_tma ? umma_smem_desc_sw128(smem_addr_u32(sA) + (ks >> 2) * 16384 + (ks & 3) * 32)
                                                           : adesc + static_cast<unsigned long long>(ks * 2 * TC_LBO >> 4);
@@ -802,7 +828,8 @@ __global__ void __launch_bounds__(TC_THREADS, 2) append_chunk_kernel(AppendParam
                 asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_addr_u32(mbar)) : "memory");
         }
         // ---- while the tensor core runs: values of this tile (no transform)
-        if (KK_V != 0) {
+        if (EXACT && term > 0) {
+        } else if (KK_V != 0) {
             constexpr int KQ = KK_V != 0 ? KK_V : 8;
             const int row = 8 * warp + (lane >> 2), qd = lane & 3;
             const RowInfo ri = rows[row];
@@ -927,6 +954,12 @@ __global__ void __launch_bounds__(TC_THREADS, 2) append_chunk_kernel(AppendParam
             }
             phase ^= 1u;
         }
+        if (!EXACT || term == 2 || *three_terms == 0) break;
+        store_term(term + 1);                                 // the operand buffer has been read; the keys are still there
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncthreads();
+        }
+        if (failed) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         {
             const int q = warp & 3, cg = warp >> 2;          // lane quadrant of this warp, 32-column group
@@ -1216,29 +1249,20 @@ static int append_impl(const wushkv_cache* cache, int32_t batch, const int32_t* 
             if (!opt_in_dynamic_smem(reinterpret_cast<const void*>(kernel), TC_SMEM_TOTAL)) return false;
             return launch_pdl(kernel, grid_tc, dim3(TC_THREADS), TC_SMEM_TOTAL, st, P, map_k, map_v) == cudaSuccess;
         };
-        bool ok;
-        if (P.c.bits == 2) {
-            if (kk_k < 0) ok = launch(append_chunk_kernel<2, -1, -1>);
-            else if (kk_k == 0) ok = launch(append_chunk_kernel<2, 0, 0>);
-            else if (kk_k == 8 && kk_v == 8) ok = launch(append_chunk_kernel<2, 8, 8>);
-            else if (kk_k == 8) ok = launch(append_chunk_kernel<2, 8, 16>);
-            else if (kk_v == 8) ok = launch(append_chunk_kernel<2, 16, 8>);
-            else ok = launch(append_chunk_kernel<2, 16, 16>);
-        } else if (P.c.bits == 3) {
-            if (kk_k < 0) ok = launch(append_chunk_kernel<3, -1, -1>);
-            else if (kk_k == 0) ok = launch(append_chunk_kernel<3, 0, 0>);
-            else if (kk_k == 8 && kk_v == 8) ok = launch(append_chunk_kernel<3, 8, 8>);
-            else if (kk_k == 8) ok = launch(append_chunk_kernel<3, 8, 16>);
-            else if (kk_v == 8) ok = launch(append_chunk_kernel<3, 16, 8>);
-            else ok = launch(append_chunk_kernel<3, 16, 16>);
-        } else {
-            if (kk_k < 0) ok = launch(append_chunk_kernel<4, -1, -1>);
-            else if (kk_k == 0) ok = launch(append_chunk_kernel<4, 0, 0>);
-            else if (kk_k == 8 && kk_v == 8) ok = launch(append_chunk_kernel<4, 8, 8>);
-            else if (kk_k == 8) ok = launch(append_chunk_kernel<4, 8, 16>);
-            else if (kk_v == 8) ok = launch(append_chunk_kernel<4, 16, 8>);
-            else ok = launch(append_chunk_kernel<4, 16, 16>);
-        }
+        auto launch_for = [&](auto bits, auto exact) -> bool {
+            constexpr int B = decltype(bits)::value;
+            constexpr bool E = decltype(exact)::value;
+            if (kk_k < 0) return launch(append_chunk_kernel<B, -1, -1, E>);
+            if (kk_k == 0) return launch(append_chunk_kernel<B, 0, 0, E>);
+            if (kk_k == 8) return kk_v == 8 ? launch(append_chunk_kernel<B, 8, 8, E>) : launch(append_chunk_kernel<B, 8, 16, E>);
+            return kk_v == 8 ? launch(append_chunk_kernel<B, 16, 8, E>) : launch(append_chunk_kernel<B, 16, 16, E>);
+        };
+        auto launch_bits = [&](auto exact) -> bool {
+            return P.c.bits == 2   ? launch_for(std::integral_constant<int, 2>{}, exact)
+                   : P.c.bits == 3 ? launch_for(std::integral_constant<int, 3>{}, exact)
+                                   : launch_for(std::integral_constant<int, 4>{}, exact);
+        };
+        const bool ok = max_new < TC_TILE ? launch_bits(std::true_type{}) : launch_bits(std::false_type{});
         if (!ok) return WUSHKV_ECUDA;
         if (cudaGetLastError() != cudaSuccess) return WUSHKV_ECUDA;
         return launch_pdl(advance_len_kernel, dim3((batch + 7) / 8), dim3(256), 0, st, P.c, batch, slot, seq_len, cu_new) == cudaSuccess ? WUSHKV_OK : WUSHKV_ECUDA;

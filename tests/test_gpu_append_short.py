@@ -1,5 +1,6 @@
 """Many short chunks on the tensor-core append path (its tiles then mix sequences): ragged counts, sequences without new tokens, a
-token count that is no multiple of the tile, projected keys; codes, scales and offsets against the oracle's."""
+token count that is no multiple of the tile, projected keys, transforms that are not bf16-valued; codes, scales and offsets against
+the oracle's."""
 import numpy as np
 import pytest
 
@@ -30,3 +31,38 @@ def test_many_short_chunks(bits, projected):
         assert L.cache.status() == 0
     assert L.check_append_parity() <= CODE_MISMATCH_MAX
     assert np.array_equal(L.seq_len.cpu().numpy(), first + more)
+
+
+@pytest.mark.parametrize("bits,n", [(2, 20), (4, 60)])
+def test_transforms_of_full_precision(bits, n):
+    """A T_K whose entries are no bf16 values (the library's own are): short chunks are transformed by it as it is (several
+    tiles per CTA: test_full_precision_over_several_tiles)."""
+    from oracle import wushkv_oracle as O
+    import torch
+    wl = W.LayerWorkload(dict(seed=151, batch=n, n_q=8, n_kv=8, ctx=0, theta=1e4, bits=bits, s_sink=4, s_keep=64, rmsnorm=False, ragged=None,
+                              prefill_chunk=0))
+    new = np.random.default_rng(4).integers(30, 100, n)
+    L = Layer(wl, new, bits, 4, 64, 1)
+    T = (np.asarray(L.T) * 1.003).astype(np.float32)
+    assert np.any(T != W.bf16_round_f32(T))
+    L.cache.T_K.copy_(torch.from_numpy(T))
+    L.oracle = [O.LayerCache(wl.n_kv, 128, bits, L.kappa_k, L.kappa_v, T.astype(np.float64)) for _ in range(n)]
+    L.append_step(new)
+    assert L.cache.status() == 0
+    assert L.check_append_parity() <= CODE_MISMATCH_MAX
+
+
+def test_full_precision_over_several_tiles():
+    """64 heads leave four CTAs per head: each multiplies several tiles and puts the first term of T_K back between them."""
+    from oracle import wushkv_oracle as O
+    import torch
+    wl = W.LayerWorkload(dict(seed=153, batch=12, n_q=64, n_kv=64, ctx=0, theta=1e4, bits=2, s_sink=4, s_keep=64, rmsnorm=False, ragged=None,
+                              prefill_chunk=0))
+    new = np.full(12, 110)                              # 1320 tokens: 11 tiles
+    L = Layer(wl, new, 2, 4, 64, 1)
+    T = (np.asarray(L.T) * 1.003).astype(np.float32)
+    L.cache.T_K.copy_(torch.from_numpy(T))
+    L.oracle = [O.LayerCache(wl.n_kv, 128, 2, L.kappa_k, L.kappa_v, T.astype(np.float64)) for _ in range(12)]
+    L.append_step(new)
+    assert L.cache.status() == 0
+    assert L.check_append_parity() <= CODE_MISMATCH_MAX
