@@ -6,31 +6,44 @@ import pytest
 
 from paper_2609_38121_b200 import workloads as W
 from tests.harness import CODE_MISMATCH_MAX, Layer
+from tests.test_gpu_projected import _compare_caches, _pair, _wl
 
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("bits,projected", [(2, False), (3, False), (4, True)])
-def test_many_short_chunks(bits, projected):
-    n = 20                                              # about 45 new tokens each, 8 heads: over two (three) tokens per warp
+@pytest.mark.parametrize("bits", [2, 3, 4])
+def test_many_short_chunks(bits):
+    n = 20                                              # about 45 new tokens each, 8 heads: over one token per warp of the rows path
     wl = W.LayerWorkload(dict(seed=141, batch=n, n_q=8, n_kv=8, ctx=0, theta=1e4, bits=bits, s_sink=4, s_keep=64, rmsnorm=False, ragged=None,
                               prefill_chunk=0))
     rng = np.random.default_rng(3)
     first, more = rng.integers(1, 70, n), rng.integers(30, 100, n)
     more[[2, 9]] = 0
     L = Layer(wl, first + more, bits, 4, 64, 1)
-    if projected:                                       # keys as given, rotated by the angle 0 of a table whose base is huge
-        from paper_2609_38121_b200 import binding as B
-        L.prologue = B.Prologue(1e300, 1)
-        L.prologue.table[..., 0], L.prologue.table[..., 1] = 1.0, 0.0
     L.append_step(first)
     L.append_step(more)
-    if projected:
-        assert L.cache.status() & ~L.B.DEV_ROPE_RANGE == 0
-    else:
-        assert L.cache.status() == 0
+    assert L.cache.status() == 0
     assert L.check_append_parity() <= CODE_MISMATCH_MAX
     assert np.array_equal(L.seq_len.cpu().numpy(), first + more)
+
+
+@pytest.mark.parametrize("bits,normalise,weights", [(2, True, True), (4, True, False), (3, False, False)])
+def test_many_short_projected_chunks(bits, normalise, weights):
+    """Every token of a tile is normalised and rotated for its own sequence's position, in tiles that mix sequences of different
+    lengths, with sequences that bring nothing between them: against the same keys prepared by the oracle."""
+    wl = _wl(47, 24, 8, 8, bits, theta=1e4)
+    rng = np.random.default_rng(5)
+    first, more = rng.integers(1, 70, 24), rng.integers(30, 100, 24)
+    more[[0, 7, 8, 23]] = 0
+    assert sum(first) > 592 and sum(more) > 592         # 17 tokens and more per CTA of the rows path: three per warp
+    plain, fused, masks, _ = _pair(wl, first + more, bits, normalise, weights)
+    for L in (plain, fused):
+        L.append_step(first)
+        L.append_step(more)
+        assert L.cache.status() == 0
+    assert plain.check_append_parity() <= CODE_MISMATCH_MAX
+    share, rate = _compare_caches(plain, fused, masks, first + more, wl.n_kv)
+    assert share <= 0.25 and rate <= 0.05
 
 
 @pytest.mark.parametrize("bits,n", [(2, 20), (4, 60)])

@@ -29,6 +29,19 @@ def test_shares_by_amount_of_work(ctx, new, n_q, n_kv, bits):
     assert L.cache.status() == 0
 
 
+def test_more_sequences_than_the_table_takes_at_once():
+    """Above 512 sequences the table of shares is put together in two trips, and with more shares than SMs the pairs are sorted by the
+    size of their shares: 560 short chunks on uneven contexts."""
+    rng = np.random.default_rng(7)
+    ctx, new = rng.integers(0, 200, 560), rng.integers(1, 6, 560)
+    ctx[[3, 300, 530]] = [2000, 900, 1500]
+    new[[10, 511, 512]] = 0
+    L = Layer(_wl(8, 1, 560), ctx + new, 2, 4, 64, 1)
+    L.append_step(ctx)
+    assert L.check_prefill_parity(new) <= 2e-3
+    assert L.cache.status() == 0
+
+
 def test_smaller_workspaces():
     import torch
     from paper_2609_38121_b200 import binding as B
