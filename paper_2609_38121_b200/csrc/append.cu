@@ -1228,8 +1228,8 @@ static int append_impl(const wushkv_cache* cache, int32_t batch, const int32_t* 
     const int want_ctas = std::max(1, 2 * sm_count() / P.c.n_kv);
     const int tpc = std::max(8, ((total_new + want_ctas - 1) / want_ctas + 7) / 8 * 8);
     // The tensor-core path takes about 15 us whatever it gets (23 us with projected keys) while one wave of it suffices, the
-    // warp-per-vector path about 10 us for every token of a warp: the line is at two tokens per warp (three).  16 ragged
-    // chunks of 5 to 90 tokens, 8 heads, 3 bits: 34.7 -> 20.2 us.
+    // warp-per-vector path about 10 us for every token of a warp: it is left as soon as some warp would get a second token (a third
+    // one, projected).  16 ragged chunks of 5 to 90 tokens, 8 heads, 3 bits: 34.7 -> 20.2 us.
     const bool many_short = max_new > 1 && tpc >= (P.pro.rope ? 24 : 16);
     if ((max_new >= TC_TILE || many_short) && !force_cuda) {    // prefill chunk: tensor-core transform
         const int n_tiles = (total_new + TC_TILE - 1) / TC_TILE;

@@ -260,8 +260,9 @@ __device__ bool cholesky_pivoted(double* S, int* perm, int* pivot_s, int* fail) 
 //   L L^T = H (damped);  A = L^T M L (M damped), scaled to trace 1;  C C^T = A with its rows and columns in pivot order.
 //   One-sided Jacobi on the columns of C: rotations from the right until they are orthogonal, W = C V.  Then A = W W^T: the
 //   eigenvectors of A are W's columns over their lengths, the eigenvalues the lengths' squares.
-// What bounds it: 127 steps of 64 disjoint rotations per sweep, each step reading and writing the whole matrix, 128 KB, in shared
-// memory, and a chain of about 1000 cycles from the dot products to the rotated columns.  A two-sided Jacobi on A with the
+// What bounds it: 127 steps of 64 disjoint rotations per sweep.  A step reads and writes the whole matrix, 128 KB, in shared memory:
+// 2048 cycles at 128 bytes per cycle, and behind the reads a chain of about 1000 cycles from the dot products to the rotated
+// columns.  In a capture the shared-memory pipe is busy 65 % of the cycles of the eight SMs that work, the fp64 pipe 27 %.  A two-sided Jacobi on A with the
 // rotations applied to A's columns, A's rows and the eigenvectors in global memory, four barriers per step, took 50.6 ms
 // for 8 heads.
 __global__ void __launch_bounds__(BT_THREADS) build_transforms_kernel(const double* Mall, const double* Hall, double gamma, float* Tall,

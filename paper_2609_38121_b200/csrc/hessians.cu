@@ -12,7 +12,9 @@
 //
 // Every step is a contraction over 128 channels or over positions, done as register-blocked fp32 products out of shared
 // memory (with a warp per row, a CTA per position and the sums over s as vectors of 128 channels per pair, 1024 tokens of 32 / 8
-// heads took 6.0 ms, every value fetched being used for one or two multiplications; now 1.36 ms, pairs_kernel 0.59, rows_kernel 0.35):
+// heads took 6.0 ms, every value fetched being used for one or two multiplications; now 1.34 ms, pairs_kernel 0.59, rows_kernel 0.35.  In
+// a capture of pairs_kernel two warps per scheduler keep the fp32 pipe busy 46 % of the cycles and the shared-memory pipe 52 %, and its
+// last wave leaves SMs idle for a fifth of the time):
 //   gamma_kernel      Gamma_{gg'}, 128 x 128 x d_model, float64 across groups of 16
 //   rows_kernel       causal softmax statistics (max, 1 / sum) and head outputs o_{g,t}: 64 x 64 tiles
 //   project_kernel    U, kappa and alpha: 64 x 128 tiles
@@ -447,6 +449,9 @@ __device__ __forceinline__ void add_key_entry(const HessParams& P, int h, int i,
 // 384 threads; lane (r, c) = (lane >> 2, lane & 3) holds rows 2 r .. and columns 4 c .. of its warp's block.  With one slice the
 // sums go to H_K, else they are left in the workspace (over U and the head outputs, which nothing reads any more) and
 // finish_kernel adds them up in the order of the slices: the same bits on every run.
+// Three CTAs per slice keep short sequences from being one CTA's chain; what bounds it is shared-memory reads and fp32 issue alike
+// (two wavefronts for eight multiply-adds per warp) and the conversions to float64.  With all 64 blocks, 512 threads, loads waited for
+// and float64 atomics the whole call took 1352 us for 1024 tokens of 32 / 8 heads and 310 us for 300 tokens of 16 / 4, now 1344 and 267.
 constexpr int KEY_SLICE = 64, KEY_BLOCKS = 36, KEY_WARPS = 12;
 __device__ __forceinline__ void key_block(int k, int& bi, int& bj) { pair_heads(k, 8, bi, bj); }
 template <int G>
