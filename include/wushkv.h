@@ -66,7 +66,8 @@ extern "C" {
 #define WUSHKV_DEV_BAD_SLOT        4  /* slot[b] outside [0, n_slots): sequence skipped          */
 #define WUSHKV_DEV_COPY_TIMEOUT    8  /* a staged page copy did not arrive within the wait limit */
 #define WUSHKV_DEV_BAD_COUNT      16  /* max_new == 1 was promised but a sequence brought more than one token: sequence skipped;
-                                         chunk attention: a sequence brought more than max_new tokens, those beyond it may have no output */
+                                         chunk attention that splits its tiles: a sequence brought more than max_new tokens, those
+                                         beyond it may have no output */
 #define WUSHKV_DEV_VALUE_RANGE    32  /* a stored value step Delta_v >= 1024: beyond the fp16 range of the decode value contraction */
 #define WUSHKV_DEV_ROPE_RANGE     64  /* a position beyond the rotary table of a *_projected call: rotated by the table's last angle */
 /* After PAGE_TABLE_FULL, BAD_PAGE_ID, BAD_SLOT or BAD_COUNT in wushkv_append the length of the affected

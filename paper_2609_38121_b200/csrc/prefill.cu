@@ -1339,10 +1339,23 @@ __device__ __forceinline__ int key_shares(const PrefillParams& P, int tiles, flo
     if (P.fixed_split > 0) return min(P.fixed_split, P.max_split);
     return max(1, min(static_cast<int>(static_cast<float>(tiles) * per_tile), min(P.max_split, tiles)));
 }
+// A sequence that brings more tokens than the tile pairs of max_new cover: that is reported, and the rows past them are marked as
+// having nothing to merge.  (Here rather than in the attention kernel, where the code cost every call 0.3 to 0.7 us.)
+__device__ __forceinline__ void leave_rest(const PrefillParams& P, int first, int n_new) {
+    const int covered = 2 * (TM / P.c.G) * P.max_pairs;
+    if (n_new <= covered) return;
+    atomicOr(P.c.dev_status, WUSHKV_DEV_BAD_COUNT);
+    for (int t = covered; t < min(n_new, P.total_new - first); ++t)
+        for (int j = 0; j < P.c.n_q; ++j) P.part[(static_cast<long long>(first + t) * P.c.n_q + j) * PART_W + D + 2] = 0.f;
+}
 constexpr int SHARE_THREADS = 512;
 __device__ __noinline__ void make_share_table(const PrefillParams& P, ShareScratch& sc) {       // the first 512 threads of a CTA
     const CacheView& c = P.c;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, R = TM / c.G;
+    if (P.shares == nullptr) {                                   // all pairs are split alike: no table
+        for (int b = tid; b < P.batch; b += SHARE_THREADS) { const int f = ld_in(P.cu_new + b); leave_rest(P, f, ld_in(P.cu_new + b + 1) - f); }
+        return;
+    }
     auto sync = [] { asm volatile("bar.sync 4, 512;" ::: "memory"); };
     auto exclusive = [&](int mine, int& all) {                   // prefix sum over the 512 threads
         int incl = mine;
@@ -1364,7 +1377,9 @@ __device__ __noinline__ void make_share_table(const PrefillParams& P, ShareScrat
         const int b = base + tid;
         int pairs = 0, old_tiles = 0, n_new = 0;
         if (b < P.batch) {
-            n_new = ld_in(P.cu_new + b + 1) - ld_in(P.cu_new + b);
+            const int first_tok = ld_in(P.cu_new + b);
+            n_new = ld_in(P.cu_new + b + 1) - first_tok;
+            leave_rest(P, first_tok, n_new);
             const int S = __ldcg(P.seq_len + b), S0 = max(S - n_new, 0);
             const int q_hi = min(c.s_sink + n_quantized(S - c.lag, c.s_sink, c.s_keep, c.s_flush), S0);
             pairs = n_new > 0 ? min((n_new + 2 * R - 1) / (2 * R), P.max_pairs) : 0;
@@ -1479,12 +1494,6 @@ __global__ void __launch_bounds__(WS_THREADS, 1) prefill_attn_ws_kernel(PrefillP
     const int first = ld_in(P.cu_new + b), n_new = ld_in(P.cu_new + b + 1) - first;
     const int S = ld_in(P.seq_len + b), sl = ld_in(P.slot + b);        // (requested together)
     if (2 * pr * R >= n_new) return;
-    if (n_new > 2 * R * P.max_pairs) {                           // rows past the tile pairs of max_new tokens are left alone: nothing to merge
-        if (tid == 0) atomicOr(c.dev_status, WUSHKV_DEV_BAD_COUNT);
-        if (P.max_split > 1 && sp == 0 && pr == P.max_pairs - 1)
-            for (int k = 2 * R * P.max_pairs * G + tid; k < min(n_new, P.total_new - first) * G; k += WS_THREADS)
-                P.part[(static_cast<long long>(first + k / G) * c.n_q + h * G + k % G) * PART_W + D + 2] = 0.f;
-    }
     const bool bad = sl < 0 || sl >= c.n_slots || S < n_new;
     if (P.max_split > 1 && sp == 0)                              // for the merge: how many shares the pair's rows have (none to merge if it is skipped)
         for (int k = tid; k < min(2 * R, n_new - 2 * pr * R) * G; k += WS_THREADS)
@@ -2107,20 +2116,16 @@ __global__ void __launch_bounds__(WS_THREADS, 1) prefill_attn_ws_kernel(PrefillP
 constexpr int MERGE_WARPS = 8;
 __global__ void __launch_bounds__(32 * MERGE_WARPS) prefill_merge_kernel(PrefillParams P) {
     pdl_wait();
+    if (P.shares != nullptr && __ldcg(&P.shares[P.n_slots].x) == 0) return;      // no pair is shared
     // Rows behind the last sequence's were visited by no CTA: the workspace holds there what it held.  So it does in a sequence whose
     // pairs found no room in the table; a count that no CTA can have written is passed over, and nothing is read outside the workspace.
-    const int lane = threadIdx.x & 31;
-    const long long first_row = static_cast<long long>(blockIdx.x) * MERGE_WARPS + (threadIdx.x >> 5), row_step = static_cast<long long>(gridDim.x) * MERGE_WARPS;
-    auto count_of = [&](long long row) { return __ldcg(P.part + min(row, static_cast<long long>(P.total_new) * P.c.n_q - 1) * PART_W + D + 2); };
-    float next = count_of(first_row);                            // (requested together with the two that say whether it is used)
-    const long long n_rows = static_cast<long long>(min(ld_in(P.cu_new + P.batch), P.total_new)) * P.c.n_q;
-    if (P.shares != nullptr && __ldcg(&P.shares[P.n_slots].x) == 0) return;      // no pair is shared
-    for (long long row = first_row; row < n_rows; row += row_step) {
-    const float count = next;
-    next = count_of(row + row_step);
+    const int lane = threadIdx.x & 31, last = ld_in(P.cu_new + P.batch);
+    for (long long row = static_cast<long long>(blockIdx.x) * MERGE_WARPS + (threadIdx.x >> 5); row < static_cast<long long>(P.total_new) * P.c.n_q;
+         row += static_cast<long long>(gridDim.x) * MERGE_WARPS) {
     const long long stride = static_cast<long long>(P.total_new) * P.c.n_q * PART_W;
     const float* p0 = P.part + row * PART_W;
-    if (!(count >= 2.f && count <= static_cast<float>(P.max_split))) continue;       // a pair that one CTA finished
+    const float count = __ldcg(p0 + D + 2);                      // (requested together with the last sequence's end)
+    if (!(count >= 2.f && count <= static_cast<float>(P.max_split)) || row >= static_cast<long long>(last) * P.c.n_q) continue;      // a pair that one CTA finished
     const int n_share = static_cast<int>(count);
     float m = -INFINITY, l = 0.f;
     float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -2247,7 +2252,7 @@ __global__ void __launch_bounds__(PT_THREADS, 1) prefill_prep_tc_kernel(const __
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     pdl_wait();
     pdl_launch_dependents();
-    if (hs == 2 * P.c.n_kv + P.c.n_q) {                          // one CTA more: the attention kernel's table of shares
+    if (hs == 2 * P.c.n_kv + P.c.n_q) {                          // one CTA more, where pairs may be shared: the attention kernel's table
         if (blockIdx.x == 0 && warp < SHARE_THREADS / 32) make_share_table(P, *reinterpret_cast<ShareScratch*>(sm_pt));
         return;
     }
@@ -2610,7 +2615,7 @@ static int prefill_attn_impl(const wushkv_cache* cache, int32_t batch, const int
         }
         if (tc_prep) {      // head slots: key heads, query heads, then one per KV head for the values
             const int slots_tc = slots + P.c.n_kv, per_slot_tc = std::max(1, std::min(n_tok_tiles, sm_count() / slots_tc));
-            if (launch_pdl(prefill_prep_tc_kernel, dim3(per_slot_tc, slots_tc + (P.shares ? 1 : 0)), dim3(PT_THREADS), PT_SMEM, st, P, in_k, in_q) != cudaSuccess) return WUSHKV_ECUDA;
+            if (launch_pdl(prefill_prep_tc_kernel, dim3(per_slot_tc, slots_tc + (P.max_split > 1 ? 1 : 0)), dim3(PT_THREADS), PT_SMEM, st, P, in_k, in_q) != cudaSuccess) return WUSHKV_ECUDA;
         }
 #if WUSHKV_WS_TIMING
         if (tc_prep) {
@@ -2628,7 +2633,7 @@ static int prefill_attn_impl(const wushkv_cache* cache, int32_t batch, const int
 #endif
         else {
             prefill_prep_kernel<<<dim3(per_slot, slots), 256, smem_prep, st>>>(P);
-            if (P.shares) prefill_shares_kernel<<<1, SHARE_THREADS, 0, st>>>(P);
+            if (P.max_split > 1) prefill_shares_kernel<<<1, SHARE_THREADS, 0, st>>>(P);
         }
     }
     if (cudaGetLastError() != cudaSuccess) return WUSHKV_ECUDA;

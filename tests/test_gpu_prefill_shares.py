@@ -108,7 +108,8 @@ def test_rows_without_a_sequence_are_left_alone(word):
     assert np.max(np.abs(out[:60] - full)) <= 1e-3 * np.max(np.abs(full))
 
 
-def test_more_tokens_than_promised():
+@pytest.mark.parametrize("with_table", [True, False])
+def test_more_tokens_than_promised(with_table):
     """A sequence with more new tokens than max_new: its rows past the tile pairs of max_new tokens have no output, and that is reported."""
     import torch
     from paper_2609_38121_b200 import binding as B
@@ -119,6 +120,9 @@ def test_more_tokens_than_promised():
     full = L.first
     K, V, Q, cu = _chunk(L, ctx, new, 220)
     nbytes = B.prefill_workspace_bytes(L.cache.desc, 2, 220)
+    if not with_table:                                  # 8 pairs over the two KV heads: 16 shares at most, behind the operands
+        up = lambda x: (x + 255) // 256 * 256  # noqa: E731
+        nbytes = up(2 * up(220 * 2 * 256) + up(2 * 220 * 8 * 256) + up(220 * 8 * 4) + 16 * 220 * 8 * 528)
     ws = torch.full((nbytes,), 0x40, dtype=torch.uint8, device="cuda")
     O = torch.full((220, 8, 128), float("nan"), device="cuda")
     B.prefill_attn(L.cache.desc, 2, L.slot, L.seq_len, cu, 220, 64, K, V, Q, O, ws, nbytes)
