@@ -3,9 +3,8 @@
 // Definition 1).  Same results as the host entry points wushkv_accumulate_gram / wushkv_build_transforms up to
 // summation order; meant for calibration sets of millions of tokens, where the host loops take hours.
 //
-//   gram_kernel             X^T X of one head over a slice of tokens on tensor cores (bf16 operands are the inputs
-//                           themselves, products exact, fp32 accumulation within the slice), added to the float64
-//                           statistics with atomics.
+//   gram_kernel             X^T X of the heads on tensor cores (bf16 operands are the inputs themselves, products exact, fp32
+//                           accumulation over 128 tokens, float64 beyond), added to the float64 statistics with atomics.
 //   the transform builder   float64 throughout: damping, Cholesky, L^T M L, one-sided Jacobi on its Cholesky factor with a round-robin
 //                           ordering (64 disjoint rotations per step), canonical order / sign, T = c Had Lam^(-1/4) U^T L^T
 //                           rounded to bf16, Gauss-Jordan inverse of the rounded matrix.
@@ -19,86 +18,158 @@
 namespace wushkv {
 namespace {
 
-constexpr int GR_TOK = 64;                 // tokens per staged tile
-constexpr int GR_PITCH = D + 8;            // bf16 per staged row (272 bytes: conflict-free ldmatrix)
-constexpr int GR_SLICE = 2048;             // tokens per CTA
-constexpr int GR_FLUSH = 128;              // tokens whose products are summed in fp32 (8 tensor-core accumulations) before they move to float64
-
 __device__ __forceinline__ unsigned saddr(const void* p) { return static_cast<unsigned>(__cvta_generic_to_shared(p)); }
-__device__ __forceinline__ void ldsm4t(unsigned addr, unsigned& a, unsigned& b, unsigned& c, unsigned& d) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(a), "=r"(b), "=r"(c), "=r"(d) : "r"(addr));
-}
-__device__ __forceinline__ void mma_bf16_acc(float (&c)[4], unsigned a0, unsigned a1, unsigned a2, unsigned a3, unsigned b0, unsigned b1) {
-    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
 
-// grid (token slices, n_kv + n_q head slots), 256 threads: warp w owns output rows 16w .. 16w+15 (all 128 columns).  One CTA fits
-// on an SM (64 float64 and 64 fp32 sums per thread), so the next tile is requested while this one is multiplied; the bound
-// is the mma.sync rate.  32768 tokens of 32 / 8 heads: 575 us with the loads waited for, now 255 us.
-__global__ void __launch_bounds__(256) gram_kernel(int n_kv, int n_q, long long n_tok, const unsigned short* __restrict__ K,
-                                                   const unsigned short* __restrict__ Q, double* M, double* H) {
-    __shared__ __align__(16) unsigned short xs2[2][GR_TOK][GR_PITCH];
-    const int hs = blockIdx.y;
-    const bool is_key = hs < n_kv;
-    const int head = is_key ? hs : hs - n_kv, n_heads = is_key ? n_kv : n_q, G = n_q / n_kv;
-    const unsigned short* X = is_key ? K : Q;
-    double* out = is_key ? M + static_cast<long long>(head) * D * D : H + static_cast<long long>(head / G) * D * D;
-    const double weight = is_key ? 1.0 : 2.0;                 // H = 2 sum_g sum_t q q^T (Eq. 4)
-    const long long t0 = static_cast<long long>(blockIdx.x) * GR_SLICE, t1 = min(t0 + GR_SLICE, n_tok);
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
-    float acc[16][4];
-    double dacc[16][4];
-#pragma unroll
-    for (int nb = 0; nb < 16; ++nb) {
-        acc[nb][0] = acc[nb][1] = acc[nb][2] = acc[nb][3] = 0.f;
-        dacc[nb][0] = dacc[nb][1] = dacc[nb][2] = dacc[nb][3] = 0.0;
+// ---- X^T X of all heads -------------------------------------------------------------------------------------------------
+// A unit is 128 tokens of one head: a 128 x 128 tile of bf16 rows, fetched by two bulk tensor copies (64 channels each, 128-byte
+// swizzle), which stands for both operands of 8 tcgen05.mma M128 N128 K16 (channels on M and N, tokens on K: both operands MN-major).  The
+// fp32 sums over 128 tokens (8 accumulations) come back from tensor memory and move to float64 in registers.  One CTA per SM takes a
+// consecutive part of the list (head, tokens); where the matrix changes, and at the end, a thread adds its 64 sums to the statistics
+// with atomics (to the mirror image of their places, which makes a warp's addresses consecutive).
+// Warps 0-7: float64 sums of the 32 tensor-memory lanes that their number allows, half the columns each.  Warp 8: copies, six tiles ahead.
+// Warp 9: MMAs, into one of four accumulators.  32768 tokens of 32 / 8 heads: mma.sync with the sums in the same warps 255 us (its rate),
+// this 106.
+constexpr int GR_TOK = 128, GR_STAGES = 6, GR_ACC = 4, GR_THREADS = 320;
+constexpr int GR_TILE_BYTES = GR_TOK * D * 2;
+constexpr size_t GRAM_SMEM = static_cast<size_t>(GR_STAGES) * GR_TILE_BYTES + 1024;      // and alignment
+constexpr unsigned GR_IDESC = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | ((static_cast<unsigned>(D) >> 3) << 17) |
+                              ((static_cast<unsigned>(D) >> 4) << 24);                   // fp32 <- bf16 x bf16, both MN-major
+struct GramParams {
+    int n_kv, n_q;
+    long long groups, units;                         // groups of tokens; groups times heads (those of K, then those of Q)
+    double *M, *H;
+};
+// False when the wait ran out (about a second), here or in another warp.
+__device__ __forceinline__ bool gram_wait(unsigned bar, unsigned parity, volatile int* stop) {
+#pragma unroll 1
+    for (int n = 0; n < (1 << 20); ++n) {
+        unsigned done;
+        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                     : "=r"(done) : "r"(bar), "r"(parity), "r"(1000u) : "memory");
+        if (done) return true;
+        if (stop && *stop) return false;
     }
-    auto request = [&](long long base, int buf) {                        // 16-byte pieces; rows past the end are zero
+    if (stop) *stop = 1;
+    return false;
+}
+__device__ __forceinline__ void gram_commit(unsigned bar) {
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+__global__ void __launch_bounds__(GR_THREADS, 1) gram_kernel(GramParams P, const __grid_constant__ CUtensorMap k_map, const __grid_constant__ CUtensorMap q_map) {
+    extern __shared__ __align__(16) unsigned char gram_smem[];
+    __shared__ unsigned long long full_bar[GR_STAGES], free_bar[GR_STAGES], acc_bar[GR_ACC], read_bar[GR_ACC], drain_bar;
+    __shared__ unsigned tmem_s;
+    __shared__ int stop_s;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const unsigned tiles = (saddr(gram_smem) + 1023u) & ~1023u;
+    const long long u0 = P.units * blockIdx.x / gridDim.x, u1 = P.units * (blockIdx.x + 1) / gridDim.x;
+    const int n_units = static_cast<int>(u1 - u0);
+    if (tid == 0) {
+        auto init = [](unsigned long long* bar, unsigned count) { asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(saddr(bar)), "r"(count) : "memory"); };
+        for (int k = 0; k < GR_STAGES; ++k) { init(&full_bar[k], 1); init(&free_bar[k], 1); }
+        for (int k = 0; k < GR_ACC; ++k) { init(&acc_bar[k], 1); init(&read_bar[k], 8); }
+        init(&drain_bar, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        stop_s = 0;
+    }
+    if (warp == 9) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(saddr(&tmem_s)), "r"(static_cast<unsigned>(GR_ACC * D)) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const unsigned tmem = tmem_s;
+    volatile int* stop = &stop_s;
+    if (warp == 8) {
+        if (lane == 0) {
+            int slot = static_cast<int>(u0 / P.groups), k = 0;
+            long long group = u0 % P.groups;
+            for (; k < n_units; ++k) {
+                const int stage = k % GR_STAGES;
+                if (k >= GR_STAGES && !gram_wait(saddr(&free_bar[stage]), (k / GR_STAGES - 1) & 1, stop)) break;
+                const unsigned bar = saddr(&full_bar[stage]), dst = tiles + stage * GR_TILE_BYTES;
+                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(static_cast<unsigned>(GR_TILE_BYTES)) : "memory");
+                const CUtensorMap* map = slot < P.n_kv ? &k_map : &q_map;
+                const int head = slot < P.n_kv ? slot : slot - P.n_kv, row = static_cast<int>(group * GR_TOK);
 #pragma unroll
-        for (int item = tid; item < GR_TOK * 16; item += 256) {
-            const int r = item >> 4, piece = item & 15;
-            const bool in = base + r < t1;
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(saddr(&xs2[buf][r][8 * piece])),
-                         "l"(X + ((in ? base + r : t0) * n_heads + head) * D + 8 * piece), "r"(in ? 16u : 0u) : "memory");
+                for (int half = 0; half < 2; ++half)
+                    asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
+                                 ::"r"(dst + half * (GR_TILE_BYTES / 2)), "l"(reinterpret_cast<unsigned long long>(map)), "r"(64 * half), "r"(head), "r"(row), "r"(bar) : "memory");
+                if (++group == P.groups) { group = 0; ++slot; }
+            }
+            if (*stop)                               // nothing may arrive after the CTA has gone
+                for (int n = k > GR_STAGES ? k - GR_STAGES : 0; n < k; ++n) gram_wait(saddr(&full_bar[n % GR_STAGES]), (n / GR_STAGES) & 1, nullptr);
         }
-        asm volatile("cp.async.commit_group;" ::: "memory");
-    };
-    request(t0, 0);
-    int buf = 0;
-    for (long long base = t0; base < t1; base += GR_TOK, buf ^= 1) {
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
-        __syncthreads();                                                 // this tile has landed; the other buffer has been read
-        if (base + GR_TOK < t1) request(base + GR_TOK, buf ^ 1);
-        const unsigned short (*xs)[GR_PITCH] = xs2[buf];
+    } else if (warp == 9) {
+        if (lane == 0) {
+            for (int k = 0; k < n_units; ++k) {
+                const int stage = k % GR_STAGES, acc = k % GR_ACC;
+                if (!gram_wait(saddr(&full_bar[stage]), (k / GR_STAGES) & 1, stop)) break;
+                if (k >= GR_ACC && !gram_wait(saddr(&read_bar[acc]), (k / GR_ACC - 1) & 1, stop)) break;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                // rows of 128 bytes (64 channels of a token), groups of 8 tokens 1024 bytes apart, the other 64 channels half a tile behind
+                const unsigned long long desc = (static_cast<unsigned long long>(((tiles + stage * GR_TILE_BYTES) >> 4) & 0x3FFFu)) |
+                                                (static_cast<unsigned long long>((GR_TILE_BYTES / 2) >> 4) << 16) |
+                                                (static_cast<unsigned long long>(1024u >> 4) << 32) | (1ull << 46) | (2ull << 61);
 #pragma unroll
-        for (int ks = 0; ks < GR_TOK / 16; ++ks) {
-            // A = X^T (channel x token): registers (rows i0.., tokens lo), (rows i0+8.., lo), (rows i0.., hi), (rows i0+8.., hi)
-            unsigned a0, a1, a2, a3;
-            ldsm4t(saddr(&xs[16 * ks + 8 * (lane >> 4) + (lane & 7)][16 * warp + 8 * ((lane >> 3) & 1)]), a0, a1, a2, a3);
-#pragma unroll
-            for (int nb2 = 0; nb2 < 8; ++nb2) {
-                unsigned b0, b1, b2, b3;                                 // B = X (token x channel): (tokens lo, cols), (hi, cols), (lo, cols+8), (hi, cols+8)
-                ldsm4t(saddr(&xs[16 * ks + 8 * ((lane >> 3) & 1) + (lane & 7)][16 * nb2 + 8 * (lane >> 4)]), b0, b1, b2, b3);
-                mma_bf16_acc(acc[2 * nb2], a0, a1, a2, a3, b0, b1);
-                mma_bf16_acc(acc[2 * nb2 + 1], a0, a1, a2, a3, b2, b3);
+                for (int ks = 0; ks < GR_TOK / 16; ++ks)
+                    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %3, 0;\n\t"
+                                 "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %1, %2, {%4, %4, %4, %4}, p;\n\t}"
+                                 ::"r"(tmem + acc * D), "l"(desc + static_cast<unsigned long long>(ks * 2048 >> 4)), "r"(GR_IDESC), "r"(ks), "r"(0u) : "memory");
+                gram_commit(saddr(&free_bar[stage]));
+                gram_commit(saddr(&acc_bar[acc]));
+            }
+            if (*stop) {
+                gram_commit(saddr(&drain_bar));
+                gram_wait(saddr(&drain_bar), 0, nullptr);
             }
         }
-        if (((base - t0) / GR_TOK) % (GR_FLUSH / GR_TOK) == GR_FLUSH / GR_TOK - 1 || base + GR_TOK >= t1) {
+    } else {
+        double sum[64];
 #pragma unroll
-            for (int nb = 0; nb < 16; ++nb)
+        for (int e = 0; e < 64; ++e) sum[e] = 0.0;
+        const int i = 32 * (warp & 3) + lane, c0 = 64 * (warp >> 2), G = P.n_q / P.n_kv;
+        int slot = static_cast<int>(u0 / P.groups);
+        long long group = u0 % P.groups;
+        for (int k = 0; k < n_units; ++k) {
+            const int acc = k % GR_ACC;
+            if (!gram_wait(saddr(&acc_bar[acc]), (k / GR_ACC) & 1, stop)) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
-                for (int e = 0; e < 4; ++e) { dacc[nb][e] += static_cast<double>(acc[nb][e]); acc[nb][e] = 0.f; }
+            for (int part = 0; part < 2; ++part) {
+                unsigned v[32];
+                const unsigned addr = tmem + acc * D + c0 + 32 * part + (static_cast<unsigned>(32 * (warp & 3)) << 16);
+                asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+                             "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+                             : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]), "=r"(v[9]),
+                               "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]),
+                               "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]),
+                               "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+                             : "r"(addr));
+                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                if (part == 1) {                     // the accumulator has been read
+                    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                    if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(saddr(&read_bar[acc])) : "memory");
+                }
+#pragma unroll
+                for (int e = 0; e < 32; ++e) sum[32 * part + e] += static_cast<double>(__uint_as_float(v[e]));
+            }
+            const int matrix = slot < P.n_kv ? slot : P.n_kv + (slot - P.n_kv) / G;
+            if (++group == P.groups) { group = 0; ++slot; }
+            if (k == n_units - 1 || matrix != (slot < P.n_kv ? slot : P.n_kv + (slot - P.n_kv) / G)) {
+                double* out = (matrix < P.n_kv ? P.M + static_cast<long long>(matrix) * D * D : P.H + static_cast<long long>(matrix - P.n_kv) * D * D) + c0 * D + i;
+                const double weight = matrix < P.n_kv ? 1.0 : 2.0;       // H = 2 sum_g sum_t q q^T (Eq. 4)
+#pragma unroll
+                for (int e = 0; e < 64; ++e) { atomicAdd(out + e * D, weight * sum[e]); sum[e] = 0.0; }
+            }
         }
     }
-#pragma unroll
-    for (int nb = 0; nb < 16; ++nb) {
-        const int i0 = 16 * warp + g, j0 = 8 * nb + 2 * t;
-        atomicAdd(out + i0 * D + j0, weight * dacc[nb][0]);
-        atomicAdd(out + i0 * D + j0 + 1, weight * dacc[nb][1]);
-        atomicAdd(out + (i0 + 8) * D + j0, weight * dacc[nb][2]);
-        atomicAdd(out + (i0 + 8) * D + j0 + 1, weight * dacc[nb][3]);
-    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (warp == 9) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(static_cast<unsigned>(GR_ACC * D)) : "memory");
+    if (tid == 0 && stop_s) atomicAdd(P.M, static_cast<double>(NAN));    // a wait ran out: the statistics must not look usable
 }
 
 // ---- float64 helpers of the transform builder -----------------------------------------------------
@@ -712,9 +783,17 @@ extern "C" int wushkv_accumulate_gram_device(int32_t n_kv, int32_t n_q, int32_t 
     if (!K || !Q || !M || !H || n_kv <= 0 || n_q <= 0 || d != D || n_tok < 0 || n_q % n_kv != 0) return WUSHKV_EINVAL;
     if (!aligned(K, 16) || !aligned(Q, 16) || !aligned(M, 8) || !aligned(H, 8)) return WUSHKV_EINVAL;
     if (n_tok == 0) return WUSHKV_OK;
-    const long long slices = (n_tok + GR_SLICE - 1) / GR_SLICE;
-    if (slices > 0x7fffffffLL) return WUSHKV_EINVAL;
-    gram_kernel<<<dim3(static_cast<unsigned>(slices), n_kv + n_q), 256, 0, static_cast<cudaStream_t>(stream)>>>(n_kv, n_q, n_tok, K, Q, M, H);
+    GramParams P;
+    P.n_kv = n_kv; P.n_q = n_q; P.M = M; P.H = H;
+    P.groups = (n_tok + GR_TOK - 1) / GR_TOK;
+    P.units = P.groups * (static_cast<long long>(n_kv) + n_q);
+    if (n_tok > 0x7fffffffLL - GR_TOK || P.units > 0x7fffffffLL) return WUSHKV_EINVAL;
+    CUtensorMap k_map, q_map;
+    if (!make_row_tensor_map(k_map, true, K, n_kv, n_tok, GR_TOK) || !make_row_tensor_map(q_map, true, Q, n_q, n_tok, GR_TOK) ||
+        !opt_in_dynamic_smem(reinterpret_cast<const void*>(gram_kernel), static_cast<int>(GRAM_SMEM)))
+        return WUSHKV_ECUDA;
+    const unsigned ctas = static_cast<unsigned>(P.units < sm_count() ? P.units : sm_count());
+    gram_kernel<<<ctas, GR_THREADS, GRAM_SMEM, static_cast<cudaStream_t>(stream)>>>(P, k_map, q_map);
     return cudaGetLastError() == cudaSuccess ? WUSHKV_OK : WUSHKV_ECUDA;
 }
 

@@ -1,4 +1,5 @@
-"""The calibration kernels at the edges of their tiles: one head and more heads than there are clusters at a time."""
+"""The calibration kernels at the edges of their tiles: groups of 128 tokens and matrices that end within a thread block's part of the
+list, one head and more heads than there are clusters at a time."""
 import numpy as np
 import pytest
 
@@ -7,6 +8,23 @@ from paper_2609_38121_b200 import workloads as W
 from tests.test_gpu_builder import _build, _spd
 
 pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n_tok,n_q,n_kv", [(1, 1, 1), (127, 2, 1), (129, 6, 2), (128, 8, 8), (5000, 12, 4), (2561, 21, 3)])
+def test_gram_sums_to_the_last_token(n_tok, n_q, n_kv):
+    """Products of bf16 numbers are exact, 128 of them are summed in fp32 and the rest in float64: 2e-6 of the largest entry is the bound of
+    the other Gram test.  What was in M and H before stays in the sum."""
+    import torch
+    from paper_2609_38121_b200 import binding as B
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    K, Q = (torch.randn((n_tok, n, 128), generator=gen, device="cuda").to(torch.bfloat16) for n in (n_kv, n_q))
+    M, H = (torch.randn((n_kv, 128, 128), generator=gen, device="cuda", dtype=torch.float64) for _ in range(2))
+    k, q, G = K.double(), Q.double(), n_q // n_kv
+    M_ref = M + torch.stack([k[:, h].T @ k[:, h] for h in range(n_kv)])
+    H_ref = H + torch.stack([2 * sum(q[:, j].T @ q[:, j] for j in range(h * G, (h + 1) * G)) for h in range(n_kv)])
+    B.accumulate_gram_device(K.view(torch.int16), Q.view(torch.int16), M, H)
+    for got, ref in ((M, M_ref), (H, H_ref)):
+        assert (got - ref).abs().max().item() <= 2e-6 * ref.abs().max().item()
 
 
 @pytest.mark.parametrize("heads", [1, 7, 41])
