@@ -10,21 +10,22 @@
 //   A_{gg'}(t) = sum_s w_s (alpha_{gg'}(s) - v_s . U_{gg'}(t) + kappa_{gg'}(t)),   alpha = v_s . Gamma_{gg'} v_s,
 //   U = Gamma_{gg'} o_{g',t} + Gamma_{g'g} o_{g,t},   kappa = o_{g,t} . Gamma_{gg'} o_{g',t},   A_{gg'} = A_{g'g}.
 //
-// Every step is a contraction over 128 channels or over positions, done as register-blocked fp32 products out of shared
-// memory (with a warp per row, a CTA per position and the sums over s as vectors of 128 channels per pair, 1024 tokens of 32 / 8
-// heads took 6.0 ms, every value fetched being used for one or two multiplications; now 1.34 ms, pairs_kernel 0.59, rows_kernel 0.35.  In
-// a capture of pairs_kernel two warps per scheduler keep the fp32 pipe busy 46 % of the cycles and the shared-memory pipe 52 %, and its
-// last wave leaves SMs idle for a fifth of the time):
-//   gamma_kernel      Gamma_{gg'}, 128 x 128 x d_model, float64 across groups of 16
+// Every step is a contraction over 128 channels or over positions.  Where one operand is bf16 already and the other fp32 (or
+// both fp32), the fp32 one is split into three bf16 terms, 24 bits, and the products run on the tensor cores (mma.sync: the
+// logits of all heads and v . U of a pair meet entry by entry in one thread's accumulators, which is what the sum over s needs).
+// 1024 tokens of 32 / 8 heads: 1343 us as register-blocked fp32 products out of shared memory, bound by fp32 issue and shared-memory
+// reads alike (pairs_kernel 626, rows_kernel 366, project_kernel 215); now 624 us (243, 96, 136), error against 64 bits 2.8e-7 -> 1.3e-7:
+//   gamma_kernel      Gamma_{gg'}, 128 x 128 x d_model, fp32 products, float64 across groups of 16
 //   rows_kernel       causal softmax statistics (max, 1 / sum) and head outputs o_{g,t}: 64 x 64 tiles
-//   project_kernel    U, kappa and alpha: 64 x 128 tiles
-//   pairs_kernel      logits and v_s . U for (position t; 4 keys s) per thread, all query heads and up to 10 pairs; A, W0
+//   project_kernel    U, kappa and alpha: 128 x 128 tiles
+//   pairs_kernel      logits of all query heads and v_s . U of up to 10 pairs over tiles of 128 keys; A, W0
 //   key_kernel        H_K: sum over (t, g) of q_{g,t} (sum_g' A_{gg'}(t) q_{g',t})^T, float64 across positions
 //   finish_kernel     H_V = 2 sum_{gg'} (sum_t W0) Gamma_{gg'}; the slices of H_K added up in order
 #include <cuda_runtime.h>
 
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "host_common.h"
 #include "layout.cuh"
@@ -36,14 +37,14 @@ constexpr int HS_PITCH = D + 4;            // floats per staged row
 
 struct HessParams {
     int S, n_kv, n_q, G, d_model, n_pairs;
-    float inv_tau;
+    float inv_tau, scale2;       // 1 / tau; log2(e) / tau
     const unsigned short* Q;     // [S][n_q][D] bf16
     const unsigned short* K;     // [S][n_kv][D]
     const unsigned short* V;     // [S][n_kv][D]
     const float* W_O;            // [n_q][D][d_model]
     float* gamma;                // [n_kv][G][G][D][D]
-    float* row_m;                // [S][n_q] maximum of the logits (natural log domain)
-    float* row_linv;             // [S][n_q] 1 / sum exp
+    float* row_m;                // [S][n_q] maximum of the logits times log2(e)
+    float* row_linv;             // [S][n_q] 1 / sum of the exponentials
     float* Oh;                   // [S][n_q][D]
     float* U;                    // [S][n_kv][n_pairs][D]
     float* kappa;                // [S][n_kv][n_pairs], where A goes: pairs_kernel reads a position's before it writes its A
@@ -60,11 +61,57 @@ __device__ __forceinline__ void pair_heads(int k, int G, int& g, int& gp) {
     while (k >= G - g) { k -= G - g; ++g; }
     gp = g + k;
 }
-__device__ __forceinline__ float4 bf16x4(const unsigned short* p) {
-    const uint2 r = *reinterpret_cast<const uint2*>(p);
-    return make_float4(bf16_bits_to_float(r.x & 0xffff), bf16_bits_to_float(r.x >> 16), bf16_bits_to_float(r.y & 0xffff), bf16_bits_to_float(r.y >> 16));
+// Products on the tensor cores at fp32's precision: bf16 operands as they are, fp32 operands as three bf16 terms (24 bits), fp32 sums.
+__device__ __forceinline__ unsigned hs_smem_addr(const void* p) { return static_cast<unsigned>(__cvta_generic_to_shared(p)); }
+__device__ __forceinline__ void hs_ldsm(unsigned addr, unsigned (&r)[4]) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
 }
-__device__ __forceinline__ void fma4(float& acc, const float4& a, const float4& b) { acc = fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.x, b.x, acc)))); }
+__device__ __forceinline__ void hs_ldsm_t(unsigned addr, unsigned (&r)[4]) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void hs_mma(float (&c)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// The tensor core cuts the sum it adds to towards zero, and over a chain of products of one sign pattern that adds up (with every sum kept
+// there the whole call's error was 2.4e-6 where fp32 products have 3e-7): long sums are added up in fp32, the tensor core
+// sums 16 products, or terms that are 2^-8 of the result or less.
+__device__ __forceinline__ void hs_mma_add(float (&c)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
+    float d[4];
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
+                 : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));
+#pragma unroll
+    for (int e = 0; e < 4; ++e) c[e] += d[e];
+}
+__device__ __forceinline__ unsigned hs_pack(float lo, float hi) {
+    unsigned r;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
+    return r;
+}
+// (x, y) as three pairs of bf16 whose sum is the fp32 values up to 2^-24 of each
+__device__ __forceinline__ void hs_split(float x, float y, unsigned& hi, unsigned& mid, unsigned& lo) {
+    hi = hs_pack(x, y);
+    const float x1 = x - __uint_as_float(hi << 16), y1 = y - __uint_as_float(hi & 0xffff0000u);
+    mid = hs_pack(x1, y1);
+    lo = hs_pack(x1 - __uint_as_float(mid << 16), y1 - __uint_as_float(mid & 0xffff0000u));
+}
+__device__ __forceinline__ float hs_ex2(float x) { float y; asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
+// rows of 128 bf16 in shared memory, 16-byte pieces exchanged by the row's low bits: eight rows' pieces lie in different banks
+__device__ __forceinline__ unsigned hs_piece(int row, int piece) { return 256u * row + (static_cast<unsigned>(piece ^ (row & 7)) << 4); }
+// rows [s0, s0 + N) of a [S][heads][D] bf16 tensor's head h to shared memory, zeros beyond S
+template <int N, int THREADS>
+__device__ __forceinline__ void hs_request(unsigned dst, const unsigned short* X, int s0, int S, int heads, int h) {
+#pragma unroll
+    for (int n = 0; n < N * 16 / THREADS; ++n) {
+        const int item = threadIdx.x + n * THREADS, row = item >> 4, piece = item & 15;
+        const bool in = s0 + row < S;
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst + hs_piece(row, piece)),
+                     "l"(X + (static_cast<long long>(in ? s0 + row : 0) * heads + h) * D + 8 * piece), "r"(in ? 16u : 0u) : "memory");
+    }
+}
+__device__ __forceinline__ void hs_requested() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int LEFT>
+__device__ __forceinline__ void hs_landed() { asm volatile("cp.async.wait_group %0;" ::"n"(LEFT) : "memory"); }
 
 // C[i][j] += sum_k a[k][i] b[k][j] for one staged group of 16 k; thread: rows 4 (tid >> 4) .., columns (tid & 15) + 16 e.
 constexpr int OUTER_K = 16;
@@ -140,298 +187,446 @@ __global__ void __launch_bounds__(128) gamma_kernel(HessParams P) {
         }
 }
 
-// Causal softmax statistics and o = sum_s p_s v_s of 64 positions of one query head, over tiles of 64 keys.  256 threads: thread
-// (r, c) = (tid >> 4, tid & 15) holds the logits of positions 4 r .. and keys c + 16 e, then the outputs of the same positions
-// and channels 4 c .., 64 + 4 c ...  grid (position tiles, n_q), the longest first.
+// Causal softmax statistics and o = sum_s p_s v_s of 64 positions of one query head, over tiles of 64 keys: a warp per 16 positions,
+// logits as exact bf16 products, probabilities as three bf16 terms against V; the next key and value tiles arrive during the products.
+// grid (position tiles, n_q), the longest first, 128 threads, two CTAs per SM.  Bound by the tensor pipe (256 MMAs of 16 x 8 x 16 per
+// warp and tile, 35 us of it for 1024 tokens of 32 heads) and the exponentials between them.  (Register-blocked fp32 products out
+// of shared memory took 366 us there, this 96.)
 constexpr int RT = 64;
-struct RowsSmem { float q[RT][HS_PITCH], kv[RT][HS_PITCH], p[RT][RT + 4]; };
-__global__ void __launch_bounds__(256, 2) rows_kernel(HessParams P) {
-    extern __shared__ __align__(16) unsigned char hs_smem[];
-    RowsSmem& sm = *reinterpret_cast<RowsSmem*>(hs_smem);
-    const int t0 = (gridDim.x - 1 - blockIdx.x) * RT, j = blockIdx.y, h = j / P.G, tid = threadIdx.x, r = tid >> 4, c = tid & 15;
-    for (int item = tid; item < RT * 32; item += 256) {
-        const int row = item >> 5, piece = item & 31;
-        *reinterpret_cast<float4*>(&sm.q[row][4 * piece]) =
-            t0 + row < P.S ? bf16x4(P.Q + (static_cast<long long>(t0 + row) * P.n_q + j) * D + 4 * piece) : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    float m[4], l[4], o[4][8];
+constexpr int ROWS_SMEM = 5 * RT * 256;                 // queries, two stages of keys and values
+__global__ void __launch_bounds__(128, 2) rows_kernel(HessParams P) {
+    extern __shared__ __align__(128) unsigned char hs_smem[];
+    const int t0 = (gridDim.x - 1 - blockIdx.x) * RT, j = blockIdx.y, h = j / P.G, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const unsigned sq = hs_smem_addr(hs_smem), skv = sq + RT * 256;
+    const int s_end = min(t0 + RT, P.S);
+    hs_request<RT, 128>(sq, P.Q, t0, P.S, P.n_q, j);
+    hs_request<RT, 128>(skv, P.K, 0, P.S, P.n_kv, h);
+    hs_request<RT, 128>(skv + RT * 256, P.V, 0, P.S, P.n_kv, h);
+    hs_requested();
+    float m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f}, o[16][4];
 #pragma unroll
-    for (int a = 0; a < 4; ++a) {
-        m[a] = -INFINITY; l[a] = 0.f;
-#pragma unroll
-        for (int e = 0; e < 8; ++e) o[a][e] = 0.f;
-    }
-    for (int s0 = 0; s0 < min(t0 + RT, P.S); s0 += RT) {
-        auto stage = [&](const unsigned short* X) {
-            for (int item = tid; item < RT * 32; item += 256) {
-                const int row = item >> 5, piece = item & 31;
-                *reinterpret_cast<float4*>(&sm.kv[row][4 * piece]) =
-                    s0 + row < P.S ? bf16x4(X + (static_cast<long long>(s0 + row) * P.n_kv + h) * D + 4 * piece) : make_float4(0.f, 0.f, 0.f, 0.f);
-            }
-        };
+    for (int n = 0; n < 16; ++n) o[n][0] = o[n][1] = o[n][2] = o[n][3] = 0.f;
+    unsigned q[8][4];
+    const int t_row = t0 + 16 * warp + (lane >> 2);     // this thread's positions: t_row, t_row + 8
+    for (int s0 = 0, st = 0; s0 < s_end; s0 += RT, st ^= 1) {
+        const unsigned sk = skv + 2 * RT * 256 * st, sv = sk + RT * 256;
+        hs_landed<0>();
         __syncthreads();
-        stage(P.K);
-        __syncthreads();
-        float z[4][4] = {};
-#pragma unroll 4
-        for (int k = 0; k < D; k += 4) {
-            float4 qa[4], kb[4];
-#pragma unroll
-            for (int a = 0; a < 4; ++a) { qa[a] = *reinterpret_cast<const float4*>(&sm.q[4 * r + a][k]); kb[a] = *reinterpret_cast<const float4*>(&sm.kv[c + 16 * a][k]); }
-#pragma unroll
-            for (int a = 0; a < 4; ++a)
-#pragma unroll
-                for (int e = 0; e < 4; ++e) fma4(z[a][e], qa[a], kb[e]);
+        if (s0 + RT < s_end) {
+            hs_request<RT, 128>(skv + 2 * RT * 256 * (st ^ 1), P.K, s0 + RT, P.S, P.n_kv, h);
+            hs_request<RT, 128>(skv + 2 * RT * 256 * (st ^ 1) + RT * 256, P.V, s0 + RT, P.S, P.n_kv, h);
+            hs_requested();
         }
-        __syncthreads();
-        stage(P.V);
+        if (s0 == 0) {
 #pragma unroll
-        for (int a = 0; a < 4; ++a) {
-            const int t = t0 + 4 * r + a;
+            for (int ks = 0; ks < 8; ++ks) hs_ldsm(sq + hs_piece(16 * warp + (lane & 15), 2 * ks + (lane >> 4)), q[ks]);
+        }
+        float z[8][4];
+#pragma unroll
+        for (int n = 0; n < 8; ++n) z[n][0] = z[n][1] = z[n][2] = z[n][3] = 0.f;
+#pragma unroll
+        for (int ks = 0; ks < 8; ++ks)
+#pragma unroll
+            for (int n = 0; n < 8; n += 2) {
+                unsigned b[4];
+                hs_ldsm(sk + hs_piece(8 * n + (lane & 7) + ((lane >> 4) << 3), 2 * ks + ((lane >> 3) & 1)), b);
+                hs_mma_add(z[n], q[ks], b[0], b[1]);
+                hs_mma_add(z[n + 1], q[ks], b[2], b[3]);
+            }
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
             float mx = -INFINITY;
 #pragma unroll
-            for (int e = 0; e < 4; ++e) { z[a][e] = s0 + c + 16 * e <= t ? z[a][e] * P.inv_tau : -INFINITY; mx = fmaxf(mx, z[a][e]); }
+            for (int n = 0; n < 8; ++n)
 #pragma unroll
-            for (int off = 8; off >= 1; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-            const float mn = fmaxf(m[a], mx), sc = __expf(m[a] - mn);        // every position sees a key of the first tile: mn is finite
+                for (int e = 2 * r; e < 2 * r + 2; ++e) {
+                    if (s0 + 8 * n + 2 * (lane & 3) + (e & 1) > t_row + 8 * r) z[n][e] = -INFINITY;
+                    mx = fmaxf(mx, z[n][e]);
+                }
+            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+            const float mn = fmaxf(m[r], mx * P.scale2), sc = hs_ex2(m[r] - mn);      // every position sees a key of the first tile: mn is finite
             float sum = 0.f;
 #pragma unroll
-            for (int e = 0; e < 4; ++e) { const float p = __expf(z[a][e] - mn); sm.p[4 * r + a][c + 16 * e] = p; sum += p; }
-            l[a] = l[a] * sc + sum;                                      // of this thread's keys
-            m[a] = mn;
+            for (int n = 0; n < 8; ++n)
 #pragma unroll
-            for (int e = 0; e < 8; ++e) o[a][e] *= sc;
+                for (int e = 2 * r; e < 2 * r + 2; ++e) { z[n][e] = hs_ex2(fmaf(z[n][e], P.scale2, -mn)); sum += z[n][e]; }
+            l[r] = l[r] * sc + sum;                                             // of this thread's keys
+            m[r] = mn;
+#pragma unroll
+            for (int n = 0; n < 16; ++n) { o[n][2 * r] *= sc; o[n][2 * r + 1] *= sc; }
         }
-        __syncthreads();
-#pragma unroll 2
-        for (int k = 0; k < RT; k += 4) {
-            float4 pa[4];
+        unsigned p0[4][4], p1[4][4], p2[4][4];
 #pragma unroll
-            for (int a = 0; a < 4; ++a) pa[a] = *reinterpret_cast<const float4*>(&sm.p[4 * r + a][k]);
+        for (int ks = 0; ks < 4; ++ks)
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk) {
-                const float4 va = *reinterpret_cast<const float4*>(&sm.kv[k + kk][4 * c]), vb = *reinterpret_cast<const float4*>(&sm.kv[k + kk][64 + 4 * c]);
+            for (int i = 0; i < 4; ++i)
+                hs_split(z[2 * ks + (i >> 1)][2 * (i & 1)], z[2 * ks + (i >> 1)][2 * (i & 1) + 1], p0[ks][i], p1[ks][i], p2[ks][i]);
 #pragma unroll
-                for (int a = 0; a < 4; ++a) {
-                    const float p = kk == 0 ? pa[a].x : kk == 1 ? pa[a].y : kk == 2 ? pa[a].z : pa[a].w;
-                    o[a][0] = fmaf(p, va.x, o[a][0]); o[a][1] = fmaf(p, va.y, o[a][1]); o[a][2] = fmaf(p, va.z, o[a][2]); o[a][3] = fmaf(p, va.w, o[a][3]);
-                    o[a][4] = fmaf(p, vb.x, o[a][4]); o[a][5] = fmaf(p, vb.y, o[a][5]); o[a][6] = fmaf(p, vb.z, o[a][6]); o[a][7] = fmaf(p, vb.w, o[a][7]);
-                }
+        for (int n = 0; n < 16; n += 2) {
+            float small[2][4] = {};
+#pragma unroll
+            for (int ks = 0; ks < 4; ++ks) {
+                unsigned b[4];
+                hs_ldsm_t(sv + hs_piece(16 * ks + (lane & 15), n + (lane >> 4)), b);
+                hs_mma(small[0], p2[ks], b[0], b[1]); hs_mma(small[1], p2[ks], b[2], b[3]);
+                hs_mma(small[0], p1[ks], b[0], b[1]); hs_mma(small[1], p1[ks], b[2], b[3]);
+                hs_mma_add(o[n], p0[ks], b[0], b[1]); hs_mma_add(o[n + 1], p0[ks], b[2], b[3]);
             }
+#pragma unroll
+            for (int e = 0; e < 4; ++e) { o[n][e] += small[0][e]; o[n + 1][e] += small[1][e]; }
         }
     }
 #pragma unroll
-    for (int a = 0; a < 4; ++a) {
-#pragma unroll
-        for (int off = 8; off >= 1; off >>= 1) l[a] += __shfl_xor_sync(0xffffffffu, l[a], off);
-        const int t = t0 + 4 * r + a;
+    for (int r = 0; r < 2; ++r) {
+        l[r] += __shfl_xor_sync(0xffffffffu, l[r], 1);
+        l[r] += __shfl_xor_sync(0xffffffffu, l[r], 2);
+        const int t = t_row + 8 * r;
         if (t >= P.S) continue;
-        const float linv = 1.f / l[a];
-        if (c == 0) { P.row_m[static_cast<long long>(t) * P.n_q + j] = m[a]; P.row_linv[static_cast<long long>(t) * P.n_q + j] = linv; }
-        float* dst = P.Oh + (static_cast<long long>(t) * P.n_q + j) * D + 4 * c;
-        *reinterpret_cast<float4*>(dst) = make_float4(o[a][0] * linv, o[a][1] * linv, o[a][2] * linv, o[a][3] * linv);
-        *reinterpret_cast<float4*>(dst + 64) = make_float4(o[a][4] * linv, o[a][5] * linv, o[a][6] * linv, o[a][7] * linv);
+        const float linv = 1.f / l[r];
+        if ((lane & 3) == 0) { P.row_m[static_cast<long long>(t) * P.n_q + j] = m[r]; P.row_linv[static_cast<long long>(t) * P.n_q + j] = linv; }
+        float* dst = P.Oh + (static_cast<long long>(t) * P.n_q + j) * D + 2 * (lane & 3);
+#pragma unroll
+        for (int n = 0; n < 16; ++n) *reinterpret_cast<float2*>(dst + 8 * n) = make_float2(o[n][2 * r] * linv, o[n][2 * r + 1] * linv);
     }
 }
 
-// U, kappa and alpha of 64 positions and one pair: y = Gamma x for 64 rows x, 256 threads; thread (r, c) holds positions 4 r .. and
-// channels 4 c .., 64 + 4 c ...  grid (position tiles, pairs, n_kv).
-struct ProjectSmem { float x[RT][HS_PITCH], gam[D][D]; };
-__global__ void __launch_bounds__(256, 2) project_kernel(HessParams P) {
-    extern __shared__ __align__(16) unsigned char hs_smem[];
-    ProjectSmem& sm = *reinterpret_cast<ProjectSmem*>(hs_smem);
+// U, kappa and alpha of 128 positions and one pair: y = Gamma x, a warp per 16 positions, Gamma as three bf16 terms in shared memory and x
+// as three terms in registers; of the nine products the three below 2^-26 of the result are left out.  alpha uses the first Gamma
+// that is staged (v . Gamma_{gg'} v = v . Gamma_{g'g} v); for g = g' both halves of U are the same product.  grid (position tiles, pairs,
+// n_kv), 256 threads.  Bound by the tensor pipe.  1024 tokens of 32 / 8 heads: 215 us as register-blocked fp32 products, now 136.
+constexpr int PROJECT_T = 128, PROJECT_SMEM = 3 * D * 256;
+__global__ void __launch_bounds__(256, 1) project_kernel(HessParams P) {
+    extern __shared__ __align__(128) unsigned char hs_smem[];
+    const unsigned base = hs_smem_addr(hs_smem);
     int g, gp;
     pair_heads(blockIdx.y, P.G, g, gp);
-    const int t0 = blockIdx.x * RT, h = blockIdx.z, tid = threadIdx.x, r = tid >> 4, c = tid & 15;
-    float y[4][8];
+    const int h = blockIdx.z, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int t_row = blockIdx.x * PROJECT_T + 16 * warp + (lane >> 2);      // this thread's positions: t_row, t_row + 8
+    const bool active = blockIdx.x * PROJECT_T + 16 * warp < P.S;
+    const long long t_in[2] = {min(t_row, P.S - 1), min(t_row + 8, P.S - 1)};
+    float y[16][4];
+    unsigned x[3][8][4];
     auto clear = [&] {
 #pragma unroll
-        for (int a = 0; a < 4; ++a)
+        for (int n = 0; n < 16; ++n) y[n][0] = y[n][1] = y[n][2] = y[n][3] = 0.f;
+    };
+    auto stage_gamma = [&](int ga, int gb) {
+        const float* src = P.gamma + (static_cast<long long>(h * P.G + ga) * P.G + gb) * D * D;
+#pragma unroll 4
+        for (int item = tid; item < D * 16; item += 256) {
+            const float4 u = reinterpret_cast<const float4*>(src)[2 * item], v = reinterpret_cast<const float4*>(src)[2 * item + 1];
+            uint4 w[3];
+            hs_split(u.x, u.y, w[0].x, w[1].x, w[2].x);
+            hs_split(u.z, u.w, w[0].y, w[1].y, w[2].y);
+            hs_split(v.x, v.y, w[0].z, w[1].z, w[2].z);
+            hs_split(v.z, v.w, w[0].w, w[1].w, w[2].w);
 #pragma unroll
-            for (int e = 0; e < 8; ++e) y[a][e] = 0.f;
-    };
-    auto stage_gamma = [&](int ga, int gb) {             // Gamma_{ga gb} x = sum_j x_j Gamma_{gb ga}[j][.]: rows of the transpose
-        const float4* src = reinterpret_cast<const float4*>(P.gamma + (static_cast<long long>(h * P.G + gb) * P.G + ga) * D * D);
-        float4* dst = reinterpret_cast<float4*>(&sm.gam[0][0]);
-#pragma unroll 4
-        for (int k = tid; k < D * D / 4; k += 256) dst[k] = src[k];
-    };
-    auto stage_o = [&](int gx) {
-#pragma unroll 4
-        for (int item = tid; item < RT * 32; item += 256) {
-            const int row = item >> 5, piece = item & 31;
-            *reinterpret_cast<float4*>(&sm.x[row][4 * piece]) =
-                t0 + row < P.S ? *reinterpret_cast<const float4*>(P.Oh + (static_cast<long long>(t0 + row) * P.n_q + h * P.G + gx) * D + 4 * piece) : make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int i = 0; i < 3; ++i) *reinterpret_cast<uint4*>(hs_smem + i * D * 256 + hs_piece(item >> 4, item & 15)) = w[i];
         }
     };
-    auto product = [&] {
-#pragma unroll 2
-        for (int k = 0; k < D; k += 4) {
-            float4 xa[4];
+    auto output_of = [&](int gx, int r, int col) -> float2 {                 // two channels of a head's output at position t_row + 8 r
+        return *reinterpret_cast<const float2*>(P.Oh + (t_in[r] * P.n_q + h * P.G + gx) * D + col + 2 * (lane & 3));
+    };
+    auto load_o = [&](int gx) {
 #pragma unroll
-            for (int a = 0; a < 4; ++a) xa[a] = *reinterpret_cast<const float4*>(&sm.x[4 * r + a][k]);
+        for (int ks = 0; ks < 8; ++ks)
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk) {
-                const float4 ga = *reinterpret_cast<const float4*>(&sm.gam[k + kk][4 * c]), gb = *reinterpret_cast<const float4*>(&sm.gam[k + kk][64 + 4 * c]);
-#pragma unroll
-                for (int a = 0; a < 4; ++a) {
-                    const float x = kk == 0 ? xa[a].x : kk == 1 ? xa[a].y : kk == 2 ? xa[a].z : xa[a].w;
-                    y[a][0] = fmaf(x, ga.x, y[a][0]); y[a][1] = fmaf(x, ga.y, y[a][1]); y[a][2] = fmaf(x, ga.z, y[a][2]); y[a][3] = fmaf(x, ga.w, y[a][3]);
-                    y[a][4] = fmaf(x, gb.x, y[a][4]); y[a][5] = fmaf(x, gb.y, y[a][5]); y[a][6] = fmaf(x, gb.z, y[a][6]); y[a][7] = fmaf(x, gb.w, y[a][7]);
-                }
+            for (int i = 0; i < 4; ++i) {
+                const float2 v = output_of(gx, i & 1, 16 * ks + 8 * (i >> 1));
+                hs_split(v.x, v.y, x[0][ks][i], x[1][ks][i], x[2][ks][i]);
             }
+    };
+    auto product = [&](auto terms_tag) {                                     // y += Gamma x with x in one or three terms
+        constexpr int TERMS = decltype(terms_tag)::value;
+#pragma unroll
+        for (int n = 0; n < 16; n += 4) {
+            float small[4][4] = {};
+#pragma unroll
+            for (int ks = 0; ks < 8; ++ks) {
+                unsigned b[3][2][4];
+#pragma unroll
+                for (int i = 0; i < 3; ++i)
+#pragma unroll
+                    for (int q = 0; q < 2; ++q)
+                        hs_ldsm(base + i * D * 256 + hs_piece(8 * n + 16 * q + (lane & 7) + ((lane >> 4) << 3), 2 * ks + ((lane >> 3) & 1)), b[i][q]);
+#pragma unroll
+                for (int sum = 2; sum >= 0; --sum)                           // the small products first
+#pragma unroll
+                    for (int i = 0; i <= sum; ++i) {
+                        if (sum - i >= TERMS) continue;
+#pragma unroll
+                        for (int q = 0; q < 2; ++q)
+#pragma unroll
+                            for (int w = 0; w < 2; ++w) {
+                                if (sum > 0) hs_mma(small[2 * q + w], x[sum - i][ks], b[i][q][2 * w], b[i][q][2 * w + 1]);
+                                else hs_mma_add(y[n + 2 * q + w], x[0][ks], b[0][q][2 * w], b[0][q][2 * w + 1]);
+                            }
+                    }
+            }
+#pragma unroll
+            for (int w = 0; w < 4; ++w)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) y[n + w][e] += small[w][e];
         }
     };
-    auto dot_rows = [&](float* out) {                    // out[t] = x_t . y_t with the staged rows
+    auto row_sums = [&](const float (&d)[2], float* out) {                   // over the four lanes of a row
 #pragma unroll
-        for (int a = 0; a < 4; ++a) {
-            const float4 xa = *reinterpret_cast<const float4*>(&sm.x[4 * r + a][4 * c]), xb = *reinterpret_cast<const float4*>(&sm.x[4 * r + a][64 + 4 * c]);
-            float d = 0.f;
-            fma4(d, xa, make_float4(y[a][0], y[a][1], y[a][2], y[a][3]));
-            fma4(d, xb, make_float4(y[a][4], y[a][5], y[a][6], y[a][7]));
-#pragma unroll
-            for (int off = 8; off >= 1; off >>= 1) d += __shfl_xor_sync(0xffffffffu, d, off);
-            if (c == 0 && t0 + 4 * r + a < P.S) out[(static_cast<long long>(t0 + 4 * r + a) * P.n_kv + h) * P.n_pairs + blockIdx.y] = d;
+        for (int r = 0; r < 2; ++r) {
+            float v = d[r];
+            v += __shfl_xor_sync(0xffffffffu, v, 1);
+            v += __shfl_xor_sync(0xffffffffu, v, 2);
+            if ((lane & 3) == 0 && t_row + 8 * r < P.S) out[(t_in[r] * P.n_kv + h) * P.n_pairs + blockIdx.y] = v;
         }
     };
-    // Gamma_{gg'} o_{g'}, its product with o_g, then + Gamma_{g'g} o_g
-    clear();
     stage_gamma(g, gp);
-    stage_o(gp);
     __syncthreads();
-    product();
-    __syncthreads();
-    stage_o(g);
-    if (g != gp) stage_gamma(gp, g);
-    __syncthreads();
-    dot_rows(P.kappa);
-    product();                                           // (g = g': the same once more)
+    if (active) {
 #pragma unroll
-    for (int a = 0; a < 4; ++a) {
-        const int t = t0 + 4 * r + a;
-        if (t >= P.S) continue;
-        float* dst = P.U + ((static_cast<long long>(t) * P.n_kv + h) * P.n_pairs + blockIdx.y) * D + 4 * c;
-        *reinterpret_cast<float4*>(dst) = make_float4(y[a][0], y[a][1], y[a][2], y[a][3]);
-        *reinterpret_cast<float4*>(dst + 64) = make_float4(y[a][4], y[a][5], y[a][6], y[a][7]);
+        for (int ks = 0; ks < 8; ++ks)
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                x[0][ks][i] = *reinterpret_cast<const unsigned*>(P.V + (t_in[i & 1] * P.n_kv + h) * D + 16 * ks + 8 * (i >> 1) + 2 * (lane & 3));
+        clear();
+        product(std::integral_constant<int, 1>{});
+        float d[2] = {0.f, 0.f};
+#pragma unroll
+        for (int n = 0; n < 16; ++n)
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                const unsigned v = x[0][n >> 1][2 * (n & 1) + r];
+                d[r] = fmaf(__uint_as_float(v << 16), y[n][2 * r], d[r]);
+                d[r] = fmaf(__uint_as_float(v & 0xffff0000u), y[n][2 * r + 1], d[r]);
+            }
+        row_sums(d, P.alpha);
+        load_o(gp);
+        clear();
+        product(std::integral_constant<int, 3>{});
+        d[0] = d[1] = 0.f;
+#pragma unroll
+        for (int n = 0; n < 16; ++n)
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                const float2 v = output_of(g, r, 8 * n);
+                d[r] = fmaf(v.x, y[n][2 * r], d[r]);
+                d[r] = fmaf(v.y, y[n][2 * r + 1], d[r]);
+            }
+        row_sums(d, P.kappa);
     }
-    __syncthreads();
-    for (int item = tid; item < RT * 32; item += 256) {
-        const int row = item >> 5, piece = item & 31;
-        *reinterpret_cast<float4*>(&sm.x[row][4 * piece]) =
-            t0 + row < P.S ? bf16x4(P.V + (static_cast<long long>(t0 + row) * P.n_kv + h) * D + 4 * piece) : make_float4(0.f, 0.f, 0.f, 0.f);
+    if (g != gp) {
+        __syncthreads();
+        stage_gamma(gp, g);
+        __syncthreads();
+        if (active) {
+            load_o(g);
+            product(std::integral_constant<int, 3>{});
+        }
+    } else {
+#pragma unroll
+        for (int n = 0; n < 16; ++n)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) y[n][e] += y[n][e];
     }
-    __syncthreads();
-    clear();
-    product();                                           // v . Gamma_{g'g} v = v . Gamma_{gg'} v
-    dot_rows(P.alpha);
+    if (!active) return;
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        if (t_row + 8 * r >= P.S) continue;
+        float* dst = P.U + ((t_in[r] * P.n_kv + h) * P.n_pairs + blockIdx.y) * D + 2 * (lane & 3);
+#pragma unroll
+        for (int n = 0; n < 16; ++n) *reinterpret_cast<float2*>(dst + 8 * n) = make_float2(y[n][2 * r], y[n][2 * r + 1]);
+    }
 }
 
-// A and W0 of 16 positions and NC pairs (from pair0 on): thread (t, c) holds the logits of all heads and v . U of the pairs for its
-// position and keys c + 16 e of a tile of 64.  grid (position tiles, pair chunks, n_kv), 256 threads.
-template <int G, int NC>
-struct PairsSmem { float q[G][16][HS_PITCH], u[NC][16][HS_PITCH], k[RT][HS_PITCH], v[RT][HS_PITCH], al[NC][RT]; };
-constexpr int pair_chunks(int G) { return (G * (G + 1) / 2 + 9) / 10; }      // what fits in shared memory beside the heads' queries
+// A and W0 of T positions and up to NC pairs of query heads, over tiles of 128 keys: a warp takes 16 positions x NT tiles of 8 keys and
+// holds the probabilities of all heads, then v . U of one pair after the other, in the same places of its accumulators, so that
+// nothing but the sums over the keys crosses threads.  U is split into three bf16 terms while it is staged; a tile's values are held as operands
+// in registers, so the next tile arrives while the pairs are multiplied.  grid (position tiles, pair chunks, n_kv), 256 threads.
+// Up to 4 heads two position tiles of 16 and chunks of up to 5 pairs, beyond that one and up to 10: what fits in shared memory beside
+// the heads' queries.  1024 tokens of 32 / 8 heads: 626 us as register-blocked fp32 products (fp32 and shared-memory pipes half
+// busy each), now 243.
+constexpr int KT = 128;                                 // keys per tile
+constexpr int pairs_m_tiles(int G) { return G <= 4 ? 2 : 1; }
+constexpr int pair_chunks(int G) { return (G * (G + 1) / 2 + (G <= 4 ? 4 : 9)) / (G <= 4 ? 5 : 10); }
 constexpr int pairs_per_chunk(int G) { return (G * (G + 1) / 2 + pair_chunks(G) - 1) / pair_chunks(G); }
-template <int G, int NC>
+template <int G>
+struct PairsShape {
+    static constexpr int MT = pairs_m_tiles(G), T = 16 * MT, NC = pairs_per_chunk(G), KW = 8 / MT, NT = KT / KW / 8, CHUNKS = pair_chunks(G);
+    static constexpr int OFF_U = G * T * 256, OFF_K = OFF_U + 3 * NC * T * 256, OFF_V = OFF_K + KT * 256, OFF_AL = OFF_V + KT * 256,
+                         OFF_STAT = OFF_AL + NC * KT * 4, OFF_KAPPA = OFF_STAT + G * T * 8, SMEM = OFF_KAPPA + NC * T * 4;
+    static_assert(SMEM <= 232448 && KW * T * NC * 2 * 4 <= KT * 256, "shared memory; the warps' sums over the keys' place");
+};
+template <int G>
 __global__ void __launch_bounds__(256, 1) pairs_kernel(HessParams P) {
-    extern __shared__ __align__(16) unsigned char hs_smem[];
-    PairsSmem<G, NC>& sm = *reinterpret_cast<PairsSmem<G, NC>*>(hs_smem);
-    const int t0 = (gridDim.x - 1 - blockIdx.x) * 16, pair0 = blockIdx.y * NC, h = blockIdx.z, tid = threadIdx.x, tr = tid >> 4, c = tid & 15;
-    const int t = t0 + tr, n_pairs = min(NC, P.n_pairs - pair0);
-    for (int item = tid; item < G * 16 * 32; item += 256) {
-        const int g = item >> 9, row = (item >> 5) & 15, piece = item & 31;
-        *reinterpret_cast<float4*>(&sm.q[g][row][4 * piece]) =
-            t0 + row < P.S ? bf16x4(P.Q + (static_cast<long long>(t0 + row) * P.n_q + h * G + g) * D + 4 * piece) : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    for (int item = tid; item < NC * 16 * 32; item += 256) {
-        const int k = item >> 9, row = (item >> 5) & 15, piece = item & 31;
-        *reinterpret_cast<float4*>(&sm.u[k][row][4 * piece]) =
-            t0 + row < P.S && k < n_pairs ? *reinterpret_cast<const float4*>(P.U + ((static_cast<long long>(t0 + row) * P.n_kv + h) * P.n_pairs + pair0 + k) * D + 4 * piece)
-                                          : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    float rm[G], rl[G], kap[NC], asum[NC], wsum[NC];
+    using Sh = PairsShape<G>;
+    constexpr int MT = Sh::MT, T = Sh::T, NC = Sh::NC, KW = Sh::KW, NT = Sh::NT;
+    extern __shared__ __align__(128) unsigned char hs_smem[];
+    const unsigned base = hs_smem_addr(hs_smem);
+    float* al = reinterpret_cast<float*>(hs_smem + Sh::OFF_AL);
+    const int t0 = (gridDim.x - 1 - blockIdx.x) * T, pair0 = blockIdx.y * NC, h = blockIdx.z, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int wm = MT == 2 ? warp >> 2 : 0, wk = MT == 2 ? warp & 3 : warp, n_pairs = min(NC, P.n_pairs - pair0), s_end = min(t0 + T, P.S);
+    auto request = [&](int s0) {
+        hs_request<KT, 256>(base + Sh::OFF_K, P.K, s0, P.S, P.n_kv, h);
+        hs_request<KT, 256>(base + Sh::OFF_V, P.V, s0, P.S, P.n_kv, h);
+        hs_requested();
+    };
 #pragma unroll
-    for (int g = 0; g < G; ++g) {
-        const long long row = static_cast<long long>(min(t, P.S - 1)) * P.n_q + h * G + g;
-        rm[g] = P.row_m[row]; rl[g] = P.row_linv[row];
-    }
-#pragma unroll
-    for (int k = 0; k < NC; ++k) {
-        kap[k] = k < n_pairs ? P.kappa[(static_cast<long long>(min(t, P.S - 1)) * P.n_kv + h) * P.n_pairs + pair0 + k] : 0.f;
-        asum[k] = wsum[k] = 0.f;
-    }
-    for (int s0 = 0; s0 < min(t0 + 16, P.S); s0 += RT) {
-        __syncthreads();
+    for (int g = 0; g < G; ++g) hs_request<T, 256>(base + g * T * 256, P.Q, t0, P.S, P.n_q, h * G + g);
+    request(0);
 #pragma unroll 2
-        for (int item = tid; item < RT * 32; item += 256) {
-            const int row = item >> 5, piece = item & 31;
-            const bool in = s0 + row < P.S;
-            const long long off = (static_cast<long long>(in ? s0 + row : 0) * P.n_kv + h) * D + 4 * piece;
-            *reinterpret_cast<float4*>(&sm.k[row][4 * piece]) = in ? bf16x4(P.K + off) : make_float4(0.f, 0.f, 0.f, 0.f);
-            *reinterpret_cast<float4*>(&sm.v[row][4 * piece]) = in ? bf16x4(P.V + off) : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int item = tid; item < NC * T * 16; item += 256) {
+        const int k = item / (T * 16), row = (item >> 4) % T, piece = item & 15;
+        uint4 w[3] = {make_uint4(0, 0, 0, 0), make_uint4(0, 0, 0, 0), make_uint4(0, 0, 0, 0)};
+        if (t0 + row < P.S && k < n_pairs) {
+            const float4* src = reinterpret_cast<const float4*>(P.U + ((static_cast<long long>(t0 + row) * P.n_kv + h) * P.n_pairs + pair0 + k) * D + 8 * piece);
+            const float4 x = src[0], y = src[1];
+            hs_split(x.x, x.y, w[0].x, w[1].x, w[2].x);
+            hs_split(x.z, x.w, w[0].y, w[1].y, w[2].y);
+            hs_split(y.x, y.y, w[0].z, w[1].z, w[2].z);
+            hs_split(y.z, y.w, w[0].w, w[1].w, w[2].w);
         }
-        for (int item = tid; item < NC * RT; item += 256) {
-            const int k = item / RT, row = item % RT;
-            sm.al[k][row] = s0 + row < P.S && k < n_pairs ? P.alpha[(static_cast<long long>(s0 + row) * P.n_kv + h) * P.n_pairs + pair0 + k] : 0.f;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) *reinterpret_cast<uint4*>(hs_smem + Sh::OFF_U + (k * 3 + i) * T * 256 + hs_piece(row, piece)) = w[i];
+    }
+    const int t_row = t0 + 16 * wm + (lane >> 2);        // this thread's positions: t_row, t_row + 8
+    const int row0 = 16 * wm + (lane >> 2);
+    // (maximum, 1 / sum) of each head and kappa of each pair for the tile's positions, read again where they are used
+    float2* stat = reinterpret_cast<float2*>(hs_smem + Sh::OFF_STAT);
+    float* kap = reinterpret_cast<float*>(hs_smem + Sh::OFF_KAPPA);
+    for (int item = tid; item < (G + NC) * T; item += 256) {
+        const int k = item / T, row = item % T;
+        const long long t = min(t0 + row, P.S - 1);
+        if (k < G) stat[item] = make_float2(P.row_m[t * P.n_q + h * G + k], P.row_linv[t * P.n_q + h * G + k]);
+        else kap[item - G * T] = k - G < n_pairs ? P.kappa[(t * P.n_kv + h) * P.n_pairs + pair0 + k - G] : 0.f;
+    }
+    float asum[NC][2], wsum[NC][2];
+#pragma unroll
+    for (int k = 0; k < NC; ++k) asum[k][0] = asum[k][1] = wsum[k][0] = wsum[k][1] = 0.f;
+    const unsigned a_row = hs_piece(16 * wm + (lane & 15), 0), a_xor = lane & 7, a_half = lane >> 4;       // piece p of the row: (p ^ a_xor) << 4 beyond its start
+    const unsigned a_base = a_row - (a_xor << 4);
+    for (int s0 = 0; s0 < s_end; s0 += KT) {
+        const int key0 = 8 * NT * wk;                    // this warp's keys of the tile
+        const bool active = s0 + key0 <= t0 + 16 * wm + 15;
+        hs_landed<0>();
+        for (int item = tid; item < NC * KT; item += 256) {
+            const int k = item / KT, row = item % KT;
+            al[item] = s0 + row < P.S && k < n_pairs ? P.alpha[(static_cast<long long>(s0 + row) * P.n_kv + h) * P.n_pairs + pair0 + k] : 0.f;
         }
         __syncthreads();
-        float p[G][4], rr[NC][4];
+        float p[G][NT][4];
+        unsigned v[8][NT][2];
+        if (active) {
 #pragma unroll
-        for (int g = 0; g < G; ++g) p[g][0] = p[g][1] = p[g][2] = p[g][3] = 0.f;
+            for (int g = 0; g < G; ++g)
 #pragma unroll
-        for (int k = 0; k < NC; ++k) rr[k][0] = rr[k][1] = rr[k][2] = rr[k][3] = 0.f;
-#pragma unroll 2
-        for (int k4 = 0; k4 < D; k4 += 4) {
-            float4 b[4];
+                for (int n = 0; n < NT; ++n) p[g][n][0] = p[g][n][1] = p[g][n][2] = p[g][n][3] = 0.f;
 #pragma unroll
-            for (int e = 0; e < 4; ++e) b[e] = *reinterpret_cast<const float4*>(&sm.k[c + 16 * e][k4]);
+            for (int ks = 0; ks < 8; ++ks) {
+                unsigned b[NT][2];
 #pragma unroll
-            for (int g = 0; g < G; ++g) {
-                const float4 a = *reinterpret_cast<const float4*>(&sm.q[g][tr][k4]);
+                for (int n = 0; n < NT; n += 2) {
+                    unsigned w[4];
+                    hs_ldsm(base + Sh::OFF_K + hs_piece(key0 + 8 * n + (lane & 7) + ((lane >> 4) << 3), 2 * ks + ((lane >> 3) & 1)), w);
+                    b[n][0] = w[0]; b[n][1] = w[1]; b[n + 1][0] = w[2]; b[n + 1][1] = w[3];
+                    hs_ldsm(base + Sh::OFF_V + hs_piece(key0 + 8 * n + (lane & 7) + ((lane >> 4) << 3), 2 * ks + ((lane >> 3) & 1)), w);
+                    v[ks][n][0] = w[0]; v[ks][n][1] = w[1]; v[ks][n + 1][0] = w[2]; v[ks][n + 1][1] = w[3];
+                }
 #pragma unroll
-                for (int e = 0; e < 4; ++e) fma4(p[g][e], a, b[e]);
-            }
+                for (int g = 0; g < G; ++g) {
+                    unsigned a[4];
+                    hs_ldsm(base + g * T * 256 + a_base + (((2 * ks + a_half) ^ a_xor) << 4), a);
 #pragma unroll
-            for (int e = 0; e < 4; ++e) b[e] = *reinterpret_cast<const float4*>(&sm.v[c + 16 * e][k4]);
-#pragma unroll
-            for (int k = 0; k < NC; ++k) {
-                const float4 a = *reinterpret_cast<const float4*>(&sm.u[k][tr][k4]);
-#pragma unroll
-                for (int e = 0; e < 4; ++e) fma4(rr[k][e], a, b[e]);
-            }
-        }
-#pragma unroll
-        for (int g = 0; g < G; ++g)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) p[g][e] = s0 + c + 16 * e <= t ? __expf(p[g][e] * P.inv_tau - rm[g]) * rl[g] : 0.f;
-        // pairs in order, from the chunk's first one on (chunk boundaries are the same for every thread)
-        int index = 0;
-#pragma unroll
-        for (int g = 0; g < G; ++g)
-#pragma unroll
-            for (int gp = g; gp < G; ++gp, ++index) {
-#pragma unroll
-                for (int k = 0; k < NC; ++k) {
-                    if (NC < G * (G + 1) / 2 ? index == pair0 + k : index == k) {
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const float w = p[g][e] * p[gp][e];
-                            wsum[k] += w;
-                            asum[k] = fmaf(w, (sm.al[k][c + 16 * e] - rr[k][e]) + kap[k], asum[k]);
-                        }
-                    }
+                    for (int n = 0; n < NT; ++n) hs_mma_add(p[g][n], a, b[n][0], b[n][1]);
                 }
             }
-    }
 #pragma unroll
-    for (int k = 0; k < NC; ++k) {
+            for (int g = 0; g < G; ++g)
 #pragma unroll
-        for (int off = 8; off >= 1; off >>= 1) { asum[k] += __shfl_xor_sync(0xffffffffu, asum[k], off); wsum[k] += __shfl_xor_sync(0xffffffffu, wsum[k], off); }
-        if (c == 0 && t < P.S && k < n_pairs) {
-            const long long o = (static_cast<long long>(t) * P.n_kv + h) * P.n_pairs + pair0 + k;
-            P.A[o] = asum[k];
-            P.W0[o] = wsum[k];
+                for (int r = 0; r < 2; ++r) {
+                    const float2 st = stat[g * T + row0 + 8 * r];
+#pragma unroll
+                    for (int n = 0; n < NT; ++n)
+#pragma unroll
+                        for (int e = 2 * r; e < 2 * r + 2; ++e)
+                            p[g][n][e] = s0 + key0 + 8 * n + 2 * (lane & 3) + (e & 1) <= t_row + 8 * r ? hs_ex2(fmaf(p[g][n][e], P.scale2, -st.x)) * st.y : 0.f;
+                }
         }
+        __syncthreads();
+        if (s0 + KT < s_end) request(s0 + KT);
+        if (active) {
+            auto pair = [&](const int k, const float (&pa)[NT][4], const float (&pb)[NT][4]) {
+                float rr[NT][4], small[NT][4];
+#pragma unroll
+                for (int n = 0; n < NT; ++n)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) rr[n][e] = small[n][e] = 0.f;
+                const unsigned u0 = base + Sh::OFF_U + k * 3 * T * 256 + a_base;
+#pragma unroll
+                for (int ks = 0; ks < 8; ++ks) {
+                    const unsigned off = u0 + (((2 * ks + a_half) ^ a_xor) << 4);
+                    unsigned a[3][4];
+#pragma unroll
+                    for (int i = 0; i < 3; ++i) hs_ldsm(off + i * T * 256, a[i]);
+#pragma unroll
+                    for (int i = 2; i >= 1; --i)
+#pragma unroll
+                        for (int n = 0; n < NT; ++n) hs_mma(small[n], a[i], v[ks][n][0], v[ks][n][1]);
+#pragma unroll
+                    for (int n = 0; n < NT; ++n) hs_mma_add(rr[n], a[0], v[ks][n][0], v[ks][n][1]);
+                }
+                const float kp[2] = {kap[k * T + row0], kap[k * T + row0 + 8]};
+#pragma unroll
+                for (int n = 0; n < NT; ++n) {
+                    const float2 av = *reinterpret_cast<const float2*>(al + k * KT + key0 + 8 * n + 2 * (lane & 3));
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const float w = pa[n][e] * pb[n][e];
+                        wsum[k][e >> 1] += w;
+                        asum[k][e >> 1] = fmaf(w, ((e & 1 ? av.y : av.x) - (rr[n][e] + small[n][e])) + kp[e >> 1], asum[k][e >> 1]);
+                    }
+                }
+            };
+            // the chunk's pairs in order, each expanded with its heads known
+            auto chunk = [&](auto tag) {
+                constexpr int FIRST = decltype(tag)::value * NC;
+                int index = 0;
+#pragma unroll
+                for (int g = 0; g < G; ++g)
+#pragma unroll
+                    for (int gp = g; gp < G; ++gp, ++index)
+                        if (index >= FIRST && index < FIRST + NC) pair(index - FIRST, p[g], p[gp]);
+            };
+            switch (blockIdx.y) {
+                case 0: chunk(std::integral_constant<int, 0>{}); break;
+                case 1: if constexpr (Sh::CHUNKS > 1) chunk(std::integral_constant<int, 1>{}); break;
+                case 2: if constexpr (Sh::CHUNKS > 2) chunk(std::integral_constant<int, 2>{}); break;
+                default: if constexpr (Sh::CHUNKS > 3) chunk(std::integral_constant<int, 3>{}); break;
+            }
+        }
+        __syncthreads();                                 // alpha is read
+    }
+    // sums over the four lanes of a row, then over the warps' keys in order
+    float* red = reinterpret_cast<float*>(hs_smem + Sh::OFF_K);       // [key warp][position][pair][A, W0]
+#pragma unroll
+    for (int k = 0; k < NC; ++k)
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+#pragma unroll
+            for (int off = 1; off <= 2; off <<= 1) {
+                asum[k][r] += __shfl_xor_sync(0xffffffffu, asum[k][r], off);
+                wsum[k][r] += __shfl_xor_sync(0xffffffffu, wsum[k][r], off);
+            }
+            if ((lane & 3) == 0) *reinterpret_cast<float2*>(red + ((wk * T + 16 * wm + (lane >> 2) + 8 * r) * NC + k) * 2) = make_float2(asum[k][r], wsum[k][r]);
+        }
+    __syncthreads();
+    for (int item = tid; item < T * NC; item += 256) {
+        const int row = item / NC, k = item % NC;
+        if (t0 + row >= P.S || k >= n_pairs) continue;
+        float a = 0.f, w = 0.f;
+#pragma unroll
+        for (int i = 0; i < KW; ++i) { const float2 x = *reinterpret_cast<const float2*>(red + (i * T * NC + item) * 2); a += x.x; w += x.y; }
+        const long long o = (static_cast<long long>(t0 + row) * P.n_kv + h) * P.n_pairs + pair0 + k;
+        P.A[o] = a;
+        P.W0[o] = w;
     }
 }
 
@@ -554,6 +749,7 @@ __global__ void __launch_bounds__(256) finish_kernel(HessParams P) {
     }
     for (int k = tid >> 5; k < P.n_pairs; k += 8) {
         double sum = 0.0;
+#pragma unroll 8
         for (int t = lane; t < P.S; t += 32) sum += static_cast<double>(P.W0[(static_cast<long long>(t) * P.n_kv + h) * P.n_pairs + k]);
 #pragma unroll
         for (int o = 16; o >= 1; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
@@ -575,9 +771,9 @@ __global__ void __launch_bounds__(256) finish_kernel(HessParams P) {
 
 template <int G>
 bool launch_pairs(const HessParams& P, cudaStream_t st) {
-    constexpr int NC = pairs_per_chunk(G);
-    if (!opt_in_dynamic_smem(reinterpret_cast<const void*>(pairs_kernel<G, NC>), static_cast<int>(sizeof(PairsSmem<G, NC>)))) return false;
-    pairs_kernel<G, NC><<<dim3((P.S + 15) / 16, pair_chunks(G), P.n_kv), 256, sizeof(PairsSmem<G, NC>), st>>>(P);
+    using Sh = PairsShape<G>;
+    if (!opt_in_dynamic_smem(reinterpret_cast<const void*>(pairs_kernel<G>), Sh::SMEM)) return false;
+    pairs_kernel<G><<<dim3((P.S + Sh::T - 1) / Sh::T, pair_chunks(G), P.n_kv), 256, Sh::SMEM, st>>>(P);
     key_kernel<G><<<dim3(P.n_slices, P.n_kv, KEY_BLOCKS / KEY_WARPS), 32 * KEY_WARPS, 0, st>>>(P);
     return true;
 }
@@ -626,6 +822,7 @@ extern "C" int wushkv_accumulate_attention_hessians_device(int32_t n_kv, int32_t
     HessParams P;
     P.S = static_cast<int>(n_tokens); P.n_kv = n_kv; P.n_q = n_q; P.G = G; P.d_model = d_model; P.n_pairs = G * (G + 1) / 2;
     P.inv_tau = static_cast<float>(1.0 / tau);
+    P.scale2 = static_cast<float>(1.4426950408889634 / tau);
     P.Q = Q; P.K = K; P.V = V; P.W_O = W_O;
     P.gamma = reinterpret_cast<float*>(ws + L.gamma);
     P.row_m = reinterpret_cast<float*>(ws + L.row_m); P.row_linv = reinterpret_cast<float*>(ws + L.row_linv);
@@ -640,13 +837,13 @@ extern "C" int wushkv_accumulate_attention_hessians_device(int32_t n_kv, int32_t
     P.n_slices = static_cast<int>((n_tokens + P.slice_len - 1) / P.slice_len);
     P.key_part = reinterpret_cast<double*>(ws + L.Oh);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (!opt_in_dynamic_smem(reinterpret_cast<const void*>(rows_kernel), static_cast<int>(sizeof(RowsSmem))) ||
-        !opt_in_dynamic_smem(reinterpret_cast<const void*>(project_kernel), static_cast<int>(sizeof(ProjectSmem))))
+    if (!opt_in_dynamic_smem(reinterpret_cast<const void*>(rows_kernel), ROWS_SMEM) ||
+        !opt_in_dynamic_smem(reinterpret_cast<const void*>(project_kernel), PROJECT_SMEM))
         return WUSHKV_ECUDA;
     const unsigned tiles = (P.S + RT - 1) / RT;
     gamma_kernel<<<dim3(P.n_pairs, n_kv, D / 32), 128, 0, st>>>(P);
-    rows_kernel<<<dim3(tiles, n_q), 256, sizeof(RowsSmem), st>>>(P);
-    project_kernel<<<dim3(tiles, P.n_pairs, n_kv), 256, sizeof(ProjectSmem), st>>>(P);
+    rows_kernel<<<dim3(tiles, n_q), 128, ROWS_SMEM, st>>>(P);
+    project_kernel<<<dim3((P.S + PROJECT_T - 1) / PROJECT_T, P.n_pairs, n_kv), 256, PROJECT_SMEM, st>>>(P);
     bool ok;
     switch (G) {
         case 1: ok = launch_pairs<1>(P, st); break;

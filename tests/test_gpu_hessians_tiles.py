@@ -56,3 +56,18 @@ def test_seven_heads_and_a_long_sequence():
         rk, rv = O.attention_hessians(Q, K[:, 0], V[:, 0], WO, tau)
         assert np.max(np.abs(HK[0] - rk)) <= TOL * np.max(np.abs(rk))
         assert np.max(np.abs(HV[0] - rv)) <= TOL * np.max(np.abs(rv))
+
+
+@pytest.mark.parametrize("n_q,n_kv,n_tok,d_model", [(4, 1, 129, 33), (3, 1, 257, 7), (8, 1, 161, 15), (5, 1, 128, 16), (2, 1, 127, 31), (12, 3, 33, 17)])
+def test_tensor_core_products(n_q, n_kv, n_tok, d_model):
+    """Edges of the tiles of 128 keys and of 16, 32 and 128 positions, chunks of 1 to 9 pairs, odd d_model (rows of W_O that do not start
+    on 8 bytes).  Three bf16 terms keep 24 bits of an operand, so what is left is fp32 summation: at most 2 (128 + 24) 2^-24 = 1.8e-5 of a
+    product's largest term for the two chained contractions."""
+    wl, K, Q, V, WO = _inputs(n_q, n_kv, n_tok, d_model, seed=83)
+    tau = float(np.sqrt(128))
+    HK, HV = _gpu(K, Q, V, WO, tau)
+    G = n_q // n_kv
+    for h in range(n_kv):
+        rk, rv = O.attention_hessians(Q[:, h * G:(h + 1) * G], K[:, h], V[:, h], WO[h * G:(h + 1) * G], tau)
+        assert np.max(np.abs(HK[h] - rk)) <= 1.8e-5 * np.max(np.abs(rk)), np.max(np.abs(HK[h] - rk)) / np.max(np.abs(rk))
+        assert np.max(np.abs(HV[h] - rv)) <= 1.8e-5 * np.max(np.abs(rv)), np.max(np.abs(HV[h] - rv)) / np.max(np.abs(rv))
