@@ -595,6 +595,13 @@ __device__ __forceinline__ void tc_mma(unsigned tmem, unsigned long long adesc, 
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
         ::"r"(tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
 }
+// the same with the descriptors' lower and upper words apart
+__device__ __forceinline__ void tc_mma2(unsigned tmem, unsigned alo, unsigned ahi, unsigned blo, unsigned bhi, unsigned idesc, unsigned accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\tsetp.ne.b32 p, %6, 0;\n\tmov.b64 a, {%1, %2};\n\tmov.b64 b, {%3, %4};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, p;\n\t}"
+        ::"r"(tmem), "r"(alo), "r"(ahi), "r"(blo), "r"(bhi), "r"(idesc), "r"(accumulate) : "memory");
+}
 // the same with the A operand in tensor memory (lane = row, a 32-bit column = two consecutive K elements)
 __device__ __forceinline__ void tc_mma_ts(unsigned tmem_d, unsigned tmem_a, unsigned long long bdesc, unsigned idesc, unsigned accumulate) {
     asm volatile(
@@ -1230,7 +1237,8 @@ __global__ void __launch_bounds__(TM, 2) prefill_attn_tc_kernel(PrefillParams P,
 //                     arrive on the tile's "probabilities ready" barrier.
 //   warps 8 / 11      issue the tcgen05.mma of query tile 0 / 1 (one lane each): per key tile g, once the probabilities
 //                     are ready, O_t += P_t(g) V(g) and then S_t(g+2) = Q'_t K(g+2)^T (into the score buffer P_t(g) sat in);
-//                     commits release the key / value stages (two arrivals each) and signal the softmax warps.
+//                     commits signal the softmax warps and release the value stages (and the key stages that the staging
+//                     threads fill next), two arrivals each.
 //   warps 9 / 10      one lane each requests the chunk's own key / value tiles (and warp 9 the query tiles) as bulk tensor
 //                     copies into rings of two / three stages.
 //   warps 12-15       write the other key / value tiles into the same rings: bf16 window rows, and packed pages (the raw
@@ -1251,8 +1259,9 @@ constexpr int WS_OFF_RAW = WS_OFF_V + WS_VS * TC_K_BYTES;        // two raw reco
 enum { WB_KFULL = 0, WB_KEMPTY = WB_KFULL + WS_KS, WB_VFULL = WB_KEMPTY + WS_KS, WB_VEMPTY = WB_VFULL + WS_VS,
        WB_S = WB_VEMPTY + WS_VS, WB_PV = WB_S + 4, WB_PREADY = WB_PV + 4, WB_RAW = WB_PREADY + 4, WB_Q = WB_RAW + 2,
        WB_STAGED, WB_DRAIN, WB_RAWFREE, WB_COUNT = WB_RAWFREE + 2 };
-// The rest of the layout depends on the record size.  Per-key factors of a packed tile, per value stage: (step, offset) of
-// the key side for the 64 keys as fp32 pairs (the softmax threads load them ready to use, two keys per 16-byte load).
+// The rest of the layout depends on the record size.  Per-key factors of a packed tile, per value stage: the steps, then the
+// offsets, of the key side for the 64 keys as fp32 (the softmax threads load them ready for two-lane instructions, four keys per 16 bytes; with
+// pairs of (step, offset) and one lane 2048 tokens on 8 x 32k took 11.74 ms, so 11.39).
 __host__ __device__ constexpr int ws_meta_stage(int) { return TN * 8; }
 __host__ __device__ constexpr int ws_off_meta(int bits) { return WS_OFF_RAW + 2 * record_bytes(bits); }
 __host__ __device__ constexpr int ws_off_live(int bits) { return ws_off_meta(bits) + WS_VS * ws_meta_stage(bits); }      // uint2[WS_VS]: which keys of a packed tile exist
@@ -1260,6 +1269,7 @@ __host__ __device__ constexpr int ws_off_bar(int bits) { return ws_off_live(bits
 __host__ __device__ constexpr int ws_off_misc(int bits) { return ws_off_bar(bits) + WB_COUNT * 8; }                       // [0] tensor-memory slot, [4] abort flag
 __host__ __device__ constexpr int ws_smem(int bits) { return ws_off_misc(bits) + 16; }
 static_assert(ws_smem(2) <= 232448 && ws_smem(3) <= 232448 && ws_smem(4) <= 232448, "the dynamic shared memory of one CTA");
+static_assert(WS_KS == 2, "a key stage and a score buffer per tile parity");
 static_assert(WS_OFF_K % 1024 == 0 && WS_OFF_V % 1024 == 0 && WS_OFF_RAW % 16 == 0, "alignment of the stages");
 static_assert(record_bytes(2) % 16 == 0 && record_bytes(3) % 16 == 0 && record_bytes(4) % 16 == 0, "raw records are copied in 16-byte units");
 
@@ -1300,6 +1310,14 @@ __device__ __forceinline__ bool ws_stagers_and(bool pred) {
                  : "=r"(r) : "r"(pred ? 1u : 0u) : "memory");
     return r != 0;
 }
+
+// two fp32 lanes per instruction
+__device__ __forceinline__ unsigned long long pack_f2(float x, float y) { unsigned long long r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y)); return r; }
+__device__ __forceinline__ void unpack_f2(unsigned long long v, float& x, float& y) { asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v)); }
+__device__ __forceinline__ unsigned long long fma_f2(unsigned long long a, unsigned long long b, unsigned long long c) {
+    unsigned long long r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r; }
+__device__ __forceinline__ unsigned long long mul_f2(unsigned long long a, unsigned long long b) {
+    unsigned long long r; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
 
 #ifndef WUSHKV_WS_TIMING
 #define WUSHKV_WS_TIMING 0      // timing experiments only: per-role cycle counters of CTA (0, 0)
@@ -1555,6 +1573,13 @@ __global__ void __launch_bounds__(WS_THREADS, 1) prefill_attn_ws_kernel(PrefillP
     const int gb_first = max(-nA, 0), gb_end = max(min(gC, NT) - nA, gb_first);      // this CTA's packed pages [gb_first, gb_end)
     const int wait_limit = P.wait_limit > 0 ? P.wait_limit : (1 << 24);      // polls of at least ~60 ns each: a second or more
 
+    // the scores of key tile g are done for the query tiles that have it: its key stage is free
+    auto scores_done = [&](const int g) -> bool {
+        bool done = true;
+        if (g < n_tiles[0]) done = ws_wait(bar(WB_S + (g & 1)), (g >> 1) & 1, wait_limit, abort_flag);
+        if (done && g < n_tiles[1]) done = ws_wait(bar(WB_S + 2 + (g & 1)), (g >> 1) & 1, wait_limit, abort_flag);
+        return done;
+    };
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -1607,8 +1632,8 @@ __global__ void __launch_bounds__(WS_THREADS, 1) prefill_attn_ws_kernel(PrefillP
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const unsigned char* kmeta = meta_all + (g % WS_VS) * META_STAGE;
                 auto factors4 = [&](const unsigned char* side, const int j4, float2 (&f)[4]) {      // (step, offset) of keys 4 j4 .. 4 j4 + 3
-                    const float4 a = reinterpret_cast<const float4*>(side)[2 * j4], b2 = reinterpret_cast<const float4*>(side)[2 * j4 + 1];
-                    f[0] = make_float2(a.x, a.y); f[1] = make_float2(a.z, a.w); f[2] = make_float2(b2.x, b2.y); f[3] = make_float2(b2.z, b2.w);
+                    const float4 a = reinterpret_cast<const float4*>(side)[j4], b2 = reinterpret_cast<const float4*>(side + TN * 4)[j4];
+                    f[0] = make_float2(a.x, b2.x); f[1] = make_float2(a.y, b2.y); f[2] = make_float2(a.z, b2.z); f[3] = make_float2(a.w, b2.w);
                 };
                 if (PACKED) {
                     if (!__all_sync(FULLM, ws_wait(bar(WB_VFULL + g % WS_VS), (g / WS_VS) & 1, wait_limit, abort_flag))) { ok = false; return; }
@@ -1625,10 +1650,10 @@ __global__ void __launch_bounds__(WS_THREADS, 1) prefill_attn_ws_kernel(PrefillP
                 if (PACKED && (live_lo & live_hi) == 0xffffffffu) {
 #pragma unroll
                     for (int j4 = 0; j4 < TN / 4; ++j4) {
-                        float2 mk[4];
-                        factors4(kmeta, j4, mk);
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) s[4 * j4 + q] = fmaf(mk[q].y, my_qsum, mk[q].x * s[4 * j4 + q]);
+                        const float4 step = reinterpret_cast<const float4*>(kmeta)[j4], offs = reinterpret_cast<const float4*>(kmeta + TN * 4)[j4];
+                        const unsigned long long qs = pack_f2(my_qsum, my_qsum);
+                        unpack_f2(fma_f2(pack_f2(offs.x, offs.y), qs, mul_f2(pack_f2(step.x, step.y), pack_f2(s[4 * j4], s[4 * j4 + 1]))), s[4 * j4], s[4 * j4 + 1]);
+                        unpack_f2(fma_f2(pack_f2(offs.z, offs.w), qs, mul_f2(pack_f2(step.z, step.w), pack_f2(s[4 * j4 + 2], s[4 * j4 + 3]))), s[4 * j4 + 2], s[4 * j4 + 3]);
                     }
                 } else if (PACKED || MASKED) {
 #pragma unroll
@@ -1782,37 +1807,44 @@ __global__ void __launch_bounds__(WS_THREADS, 1) prefill_attn_ws_kernel(PrefillP
         WST(0);
         // Descriptors are built once; their low bits hold the start address / 16, so a byte offset is added as offset / 16.
         const bool q_swz = P.use_tma != 0;                      // query tiles written by bulk tensor copies: 128-byte-swizzled rows, two 16 KB boxes
+        // (as two words: the offsets inside shared memory only touch the lower one)
         const unsigned long long q_desc = q_swz ? tc_desc_sw128(smem_addr(sm_ws + WS_OFF_Q + 2 * t * TC_Q_BYTES), 16, 1024)
                                                 : tc_desc(smem_addr(sm_ws + WS_OFF_Q + 2 * t * TC_Q_BYTES), 128, 2048);
         const unsigned long long k_plain0 = tc_desc(smem_addr(sm_ws + WS_OFF_K), 128, 2048), k_swz0 = tc_desc_sw128(smem_addr(sm_ws + WS_OFF_K), 16, 1024);
         const unsigned long long v_plain0 = tc_desc(smem_addr(sm_ws + WS_OFF_V), 128, 1024), v_swz0 = tc_desc_sw128(smem_addr(sm_ws + WS_OFF_V), 8192, 1024);
         const unsigned acc_o = tmem_base + 256u * t;
-        auto scores_of = [&](auto swz_tag, const int g, const int st) {      // lane 0: the MMAs of S_t(g)
-            constexpr bool SWZ = decltype(swz_tag)::value;
-            const unsigned long long kb = (SWZ ? k_swz0 : k_plain0) + static_cast<unsigned>(st * (TC_K_BYTES >> 4));
+        // lane 0: the score MMAs of key tile g; k-steps 0-3 and 4-7 of either operand have a base each, a k-step of 16 channels is
+        // 32 bytes of a swizzled row (channels 64-127 in another box) or two core matrices of the plain layout
+        auto scores_of = [&](const int g) {
+            const bool swz = g >= gC && P.use_tma;
+            const unsigned long long kd = swz ? k_swz0 : k_plain0;
+            const unsigned k0 = static_cast<unsigned>(kd) + static_cast<unsigned>((g & 1) * (TC_K_BYTES >> 4));
+            const unsigned k1 = k0 + (swz ? 8192u >> 4 : 1024u >> 4), kstep = swz ? 32u >> 4 : 256u >> 4;
+            const unsigned q0 = static_cast<unsigned>(q_desc), q1 = q0 + (q_swz ? 16384u >> 4 : 1024u >> 4), qstep = q_swz ? 32u >> 4 : 256u >> 4;
+            const unsigned khi = static_cast<unsigned>(kd >> 32), qhi = static_cast<unsigned>(q_desc >> 32);
             const unsigned acc = acc_o + 128u + 64u * (g & 1);
 #pragma unroll
             for (int ks = 0; ks < 8; ++ks) {
-                // swizzled: channels 0-63 and 64-127 are two boxes of 8 KB; a k-step of 16 channels is 32 bytes inside the 128-byte row
-                const unsigned long long bdesc = kb + static_cast<unsigned>((SWZ ? (ks >> 2) * 8192 + (ks & 3) * 32 : ks * 256) >> 4);
-                const unsigned long long adesc = q_desc + static_cast<unsigned>((q_swz ? (ks >> 2) * 16384 + (ks & 3) * 32 : ks * 256) >> 4);
-                tc_mma(acc, adesc, bdesc, TC_IDESC_S, ks > 0 ? 1u : 0u);
-                tc_mma(acc, adesc + static_cast<unsigned>(TC_Q_BYTES >> 4), bdesc, TC_IDESC_S, 1u);
+                const unsigned b = (ks < 4 ? k0 : k1) + (ks & 3) * kstep, a = (ks < 4 ? q0 : q1) + (ks & 3) * qstep;
+                tc_mma2(acc, a, qhi, b, khi, TC_IDESC_S, ks > 0 ? 1u : 0u);
+                tc_mma2(acc, a + (TC_Q_BYTES >> 4), qhi, b, khi, TC_IDESC_S, 1u);
             }
             if (!(P.drop == 1 && g == 0)) ws_commit(bar(WB_S + 2 * t + (g & 1)));
-            ws_commit(bar(WB_KEMPTY + st));
+        };
+        // The scores of tile g, whose key stage has landed.  The stage is free again when both query tiles' scores are done: the warp that
+        // requests bulk copies waits for those, the staging threads for one barrier of their own (a wait costs each of them some
+        // hundred cycles, a commit the tensor pipe about 60: 5.51 -> 5.26 ms for 8 prompts of 8192 tokens without it).
+        auto scores = [&](const int g) {
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const bool staged_next = g + WS_KS < n_staged;
+            if (g < mine) {
+                scores_of(g);
+                if (staged_next) ws_commit(bar(WB_KEMPTY + (g & 1)));
+            } else if (staged_next) ws_arrive(bar(WB_KEMPTY + (g & 1)));      // a tile only the other query tile reads: just release the stage
         };
         // Only lane 0 runs the loop.  Order per tile g: wait for the probabilities, O_t += P_t(g) V(g), S_t(g+2) (its score
         // buffer is the one P_t(g) sits in, so it must follow that product in the pipe), then, off the critical path, the
         // wait for the value stage the next round needs.
-        auto scores = [&](const int g) -> bool {                // key stage of tile g has landed (awaited by the caller)
-            const int st = g % WS_KS;
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            if (g >= mine) ws_arrive(bar(WB_KEMPTY + st));      // a tile only the other query tile reads: just release the stage
-            else if (g >= gC && P.use_tma) scores_of(std::true_type{}, g, st);
-            else scores_of(std::false_type{}, g, st);
-            return true;
-        };
         // Two streams of work, each in tile order: the scores S_t(sc) (once the key tile has landed and O += P V of tile
         // sc - 2, which reads the probabilities out of the same score buffer, has been issued) and the products O_t += P_t(pv)
         // V(pv) (once the value tile has landed and the probabilities are ready).  Neither may wait for the other: a key tile
@@ -1917,7 +1949,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) prefill_attn_ws_kernel(PrefillP
             for (int g = max(gC, 0); g < NT && ok; ++g) {
                 const int st = g % depth, row = first + (g - gC) * TN;
                 WST(0);
-                if (g >= depth && !__all_sync(FULLM, ws_wait(bar(empty0 + st), ((g / depth) - 1) & 1, wait_limit, abort_flag))) { ok = false; break; }
+                if (g >= depth && !__all_sync(FULLM, keys ? scores_done(g - WS_KS) : ws_wait(bar(empty0 + st), ((g / depth) - 1) & 1, wait_limit, abort_flag))) { ok = false; break; }
                 WST(1);
                 if (lane == 0) {
                     ws_expect_tx(bar(full0 + st), TC_K_BYTES);
@@ -2052,7 +2084,9 @@ __global__ void __launch_bounds__(WS_THREADS, 1) prefill_attn_ws_kernel(PrefillP
                     const bool live = page_ok && pos >= q_lo && pos < q_hi;
                     const unsigned mk = live ? *reinterpret_cast<const unsigned*>(raw + meta_location(BITS, ptid)) : 0u;
                     unsigned char* kside = meta_all + vs * META_STAGE;
-                    reinterpret_cast<float2*>(kside)[ptid] = h2f2u(mk);
+                    const float2 fk = h2f2u(mk);
+                    reinterpret_cast<float*>(kside)[ptid] = fk.x;
+                    reinterpret_cast<float*>(kside)[TN + ptid] = fk.y;
                     const unsigned word = __ballot_sync(FULLM, live);
                     if (lane == 0) reinterpret_cast<unsigned*>(live_all + vs)[ptid >> 5] = word;
                 }
