@@ -736,8 +736,11 @@ __device__ __forceinline__ void unpack_chunk8(const unsigned char* raw, int r, i
     vout = make_uint4(vo[0], vo[1], vo[2], vo[3]);
 }
 
-// A whole page (all 64 tokens live) as fp16 key codes and fp16 values, by 128 threads: instead of gathering eight channels of a token
-// from 16-bit loads (unpack_chunk8), a thread reads the record the way it is laid out and scatters 16-byte chunks.
+// A page as fp16 key codes and fp16 values, by 128 threads: instead of gathering eight channels of a token
+// from 16-bit loads (unpack_chunk8), a thread reads the record the way it is laid out and scatters 16-byte chunks.  Tokens outside
+// [live_lo, live_hi) get values of zero; their key codes are whatever integers the record holds, for the softmax to mask.  (Pages with such
+// tokens took the gathering way, 1200 instructions per thread against 400: with them, window rows requested four pieces at a time and the
+// byte tables below, 16 short turns at 3 bits 233 -> 206 us, 2048 tokens on 8 x 32k 11.44 -> 11.07 ms.)
 //   keys:   thread (block bi, k-step s, fragment row g) loads the four 16-byte pieces of row g (fragment lanes t = 0..3: words
 //           j = rs + 2 hh, bytes b = 2 b1 + b0; the field of k-step s in a byte = channel 32 s + 16 hh + 8 b1 + 2 t + b0 of
 //           token g + 8 rs) and writes, for (rs, hh, b1), the chunk of channels 8 (4 s + 2 hh + b1) .. + 7 of that token:
@@ -750,7 +753,7 @@ __device__ __forceinline__ void unpack_chunk8(const unsigned char* raw, int r, i
 // dequantized, step * code + offset in one fp16 rounding: the probabilities that multiply them are fp16 already, and the
 // softmax then treats a packed page's values like any other's.
 template <int BITS>
-__device__ __forceinline__ void unpack_page(const unsigned char* raw, unsigned char* sK, unsigned char* sV, const int p) {
+__device__ __forceinline__ void unpack_page(const unsigned char* raw, unsigned char* sK, unsigned char* sV, const int p, const int live_lo, const int live_hi) {
     constexpr bool TWO = BITS != 4;                         // 2-bit fields (also the low plane of 3-bit records)
     constexpr unsigned MASK = TWO ? 3u : 15u, MASK2 = MASK * 0x00010001u;
     constexpr int CB = code_block_bytes(BITS);
@@ -758,7 +761,7 @@ __device__ __forceinline__ void unpack_page(const unsigned char* raw, unsigned c
     // fused multiply-add (exact: c 2^f < 1024); mul = 2^-f and add = -2^(10 - f) in both halves.  3 bits: `high` holds the
     // codes' third bits, already at bit f + 2 of each half.
     auto field_h2 = [](const unsigned bytes, const unsigned mask, const unsigned high, const unsigned mul, const unsigned add) {
-        const unsigned w = (bytes & mask) | 0x64006400u | high;
+        const unsigned w = (bytes & mask) | high;
         const __half2 hv = __hfma2(*reinterpret_cast<const __half2*>(&w), *reinterpret_cast<const __half2*>(&mul),
                                    *reinterpret_cast<const __half2*>(&add));
         return *reinterpret_cast<const unsigned*>(&hv);
@@ -781,6 +784,25 @@ __device__ __forceinline__ void unpack_page(const unsigned char* raw, unsigned c
                 wh[t][0] = y.x; wh[t][1] = y.y;
             }
         }
+        if constexpr (BITS == 3) {
+            // The upper byte of the fp16 integers 0 .. 7 (the lower one is 0), picked four at a time: both planes' bits of the k-step are rotated to bits
+            // 4-6 of their bytes, where they are the odd digits of a byte selector; its even digits are 0 and pick the zero byte.
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {                   // j = rs + 2 hh
+                unsigned pair[2][4];                        // [b1][t]
+#pragma unroll
+                for (int t = 0; t < 4; ++t) {
+                    const unsigned low = __funnelshift_r(w[t][j], w[t][j], 2 * s + 28) & 0x30303030u;
+                    const unsigned z = (__funnelshift_r(wh[t][j & 1], wh[t][j & 1], 2 * s + (j >> 1) + 26) & 0x40404040u) | low;
+                    pair[0][t] = __byte_perm(0x42403C00u, 0x47464544u, z);
+                    pair[1][t] = __byte_perm(0x42403C00u, 0x47464544u, z >> 16);
+                }
+#pragma unroll
+                for (int b1 = 0; b1 < 2; ++b1)
+                    *reinterpret_cast<uint4*>(sK + (2 * bi + (j & 1)) * 2048 + (4 * s + 2 * (j >> 1) + b1) * 128 + g * 16) =
+                        make_uint4(pair[b1][0], pair[b1][1], pair[b1][2], pair[b1][3]);
+            }
+        } else
 #pragma unroll
         for (int j = 0; j < 4; ++j) {                       // j = rs + 2 hh
 #pragma unroll
@@ -789,9 +811,9 @@ __device__ __forceinline__ void unpack_page(const unsigned char* raw, unsigned c
 #pragma unroll
                 for (int t = 0; t < 4; ++t) {
                     // bytes 2 b1 and 2 b1 + 1 of the word to bytes 0 and 2, then the thread's field of each
-                    unsigned high = 0u;
+                    unsigned high = 0x64006400u;
                     if constexpr (BITS == 3)            // the same bytes of the 1-bit plane: bit 2 s + hh of each goes to bit 2 s + 2
-                        high = (__byte_perm(wh[t][j & 1], 0u, b1 ? 0x4342u : 0x4140u) << (2 - (j >> 1))) & khigh;
+                        high = (__byte_perm(wh[t][j & 1], 0u, b1 ? 0x4342u : 0x4140u) << (2 - (j >> 1))) & khigh | 0x64006400u;
                     out[t] = field_h2(__byte_perm(w[t][j], 0u, b1 ? 0x4342u : 0x4140u), kmask, high, kmul, kadd);
                 }
                 *reinterpret_cast<uint4*>(sK + (2 * bi + (j & 1)) * 2048 + (4 * s + 2 * (j >> 1) + b1) * 128 + g * 16) =
@@ -804,7 +826,8 @@ __device__ __forceinline__ void unpack_page(const unsigned char* raw, unsigned c
         const int tt = p & 3, hi = (p >> 2) & 1, m = (p >> 3) & 3, bi = p >> 5, ps = m >> 1, rsel = m & 1;
         const unsigned char* src = raw + v_codes_offset(BITS) + bi * CB + (TWO ? 4 * m : 512 * ps + 8 * rsel) + 16 * tt;
         // the values are staged dequantized: step and offset of this thread's token, in both halves of a pair
-        const unsigned mv = *reinterpret_cast<const unsigned*>(raw + meta_location(BITS, 16 * bi + 8 * ps + 2 * tt + hi) + 4);
+        const int token = 16 * bi + 8 * ps + 2 * tt + hi;
+        const unsigned mv = token >= live_lo && token < live_hi ? *reinterpret_cast<const unsigned*>(raw + meta_location(BITS, token) + 4) : 0u;
         const unsigned step2 = __byte_perm(mv, mv, 0x1010u), offs2 = __byte_perm(mv, mv, 0x3232u);
         auto dequant = [&](const unsigned codes) {
             const __half2 hv = __hfma2(*reinterpret_cast<const __half2*>(&codes), *reinterpret_cast<const __half2*>(&step2),
@@ -837,8 +860,8 @@ __device__ __forceinline__ void unpack_page(const unsigned char* raw, unsigned c
                 unsigned out[4];
 #pragma unroll
                 for (int e2 = 0; e2 < 4; ++e2) {
-                    unsigned high = 0u;
-                    if constexpr (BITS == 3) high = __funnelshift_r(hw[e2], hw[e2], (hb - (f + 2)) & 31) & (0x00010001u << (f + 2));
+                    unsigned high = 0x64006400u;
+                    if constexpr (BITS == 3) high = __funnelshift_r(hw[e2], hw[e2], (hb - (f + 2)) & 31) & (0x00010001u << (f + 2)) | 0x64006400u;
                     const unsigned both = __byte_perm(w[2 * e2], w[2 * e2 + 1], 0x0400u + 0x0101u * static_cast<unsigned>(byte));
                     out[e2] = dequant(field_h2(both, MASK2 << f, high, pow2_neg(f), bias_neg(f)));
                 }
@@ -2016,32 +2039,36 @@ __global__ void __launch_bounds__(WS_THREADS, 1) prefill_attn_ws_kernel(PrefillP
             WST(1);
             if (g < nA) {
                 // ---- full-precision old positions: sink [0, a_hi) and recent window [c_lo, S0), bf16 rows
-                for (int item = ptid; item < TN * 16 && mine; item += 128) {
-                    const int r = item & (TN - 1), piece = item >> 6, idx = (g + g0) * TN + r;
-                    uint4 kh = make_uint4(0, 0, 0, 0), vh = kh;
-                    if (idx < n_old_fp) {
-                        const long long plane = (static_cast<long long>(sl) * c.n_kv + h) * 2;
-                        const unsigned short *ksrc, *vsrc;
-                        if (idx < a_hi) {
-                            ksrc = c.sink_kv + (plane * c.s_sink + idx) * D;
-                            vsrc = c.sink_kv + ((plane + 1) * c.s_sink + idx) * D;
-                        } else {
-                            const int p = c_lo + (idx - a_hi);
-                            ksrc = c.ring_kv + (plane * c.ring_cap + p % c.ring_cap) * D;
-                            vsrc = c.ring_kv + ((plane + 1) * c.ring_cap + p % c.ring_cap) * D;
-                        }
-                        const uint4 kb16 = *reinterpret_cast<const uint4*>(ksrc + 8 * piece), vb16 = *reinterpret_cast<const uint4*>(vsrc + 8 * piece);
-                        const unsigned kw[4] = {kb16.x, kb16.y, kb16.z, kb16.w}, vw[4] = {vb16.x, vb16.y, vb16.z, vb16.w};
-                        unsigned ko[4], vo[4];
+                // (row r of both by this thread and the one 64 before or behind it, every other 16-byte piece; four pieces of each requested together)
+                const int r = ptid & (TN - 1), idx = (g + g0) * TN + r;
+                const long long plane = (static_cast<long long>(sl) * c.n_kv + h) * 2;
+                const bool in = idx < n_old_fp, sink = idx < a_hi;
+                const long long cap = sink ? c.s_sink : c.ring_cap;
+                const long long row = sink ? idx : (c_lo + (idx - a_hi)) % c.ring_cap;
+                const unsigned short* base = sink ? c.sink_kv : c.ring_kv;
+                const uint4* ksrc = reinterpret_cast<const uint4*>(base + (plane * cap + (in ? row : 0)) * D) + (ptid >> 6);
+                const uint4* vsrc = reinterpret_cast<const uint4*>(base + ((plane + 1) * cap + (in ? row : 0)) * D) + (ptid >> 6);
 #pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            ko[e] = pack_half2(bf16_bits_to_float(kw[e] & 0xffff), bf16_bits_to_float(kw[e] >> 16));
-                            vo[e] = pack_half2(bf16_bits_to_float(vw[e] & 0xffff), bf16_bits_to_float(vw[e] >> 16));
-                        }
-                        kh = make_uint4(ko[0], ko[1], ko[2], ko[3]); vh = make_uint4(vo[0], vo[1], vo[2], vo[3]);
+                for (int half = 0; half < 2 && mine; ++half) {
+                    uint4 x[2][4];
+#pragma unroll
+                    for (int n = 0; n < 4; ++n) {
+                        x[0][n] = in ? ksrc[8 * half + 2 * n] : make_uint4(0, 0, 0, 0);
+                        x[1][n] = in ? vsrc[8 * half + 2 * n] : make_uint4(0, 0, 0, 0);
                     }
-                    *reinterpret_cast<uint4*>(sK + (r >> 3) * 2048 + piece * 128 + (r & 7) * 16) = kh;
-                    *reinterpret_cast<uint4*>(sV + piece * 1024 + (r >> 3) * 128 + (r & 7) * 16) = vh;
+#pragma unroll
+                    for (int n = 0; n < 4; ++n) {
+                        const int piece = 8 * half + 2 * n + (ptid >> 6);
+#pragma unroll
+                        for (int side = 0; side < 2; ++side) {
+                            const unsigned w[4] = {x[side][n].x, x[side][n].y, x[side][n].z, x[side][n].w};
+                            unsigned o[4];
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) o[e] = pack_half2(bf16_bits_to_float(w[e] & 0xffff), bf16_bits_to_float(w[e] >> 16));
+                            unsigned char* dst = side == 0 ? sK + (r >> 3) * 2048 + piece * 128 + (r & 7) * 16 : sV + piece * 1024 + (r >> 3) * 128 + (r & 7) * 16;
+                            *reinterpret_cast<uint4*>(dst) = make_uint4(o[0], o[1], o[2], o[3]);
+                        }
+                    }
                 }
             } else if (g < gC) {
                 // ---- a packed page: the record was requested one tile ahead; unpack it into integer codes (exact in fp16)
@@ -2052,33 +2079,11 @@ __global__ void __launch_bounds__(WS_THREADS, 1) prefill_attn_ws_kernel(PrefillP
                 if (page_ok) ++raw_uses[rb];
                 WST(5);
                 const unsigned char* raw = sm_ws + WS_OFF_RAW + rb * REC;
-                const uint4 zero4 = make_uint4(0, 0, 0, 0);
                 const int page_pos = (page_first + gb) * PAGE_TOKENS;
-                const bool whole = page_ok && page_pos >= q_lo && page_pos + PAGE_TOKENS <= q_hi;
-                if (whole && mine) unpack_page<BITS>(raw, sK, sV, ptid);
+                // (at an end of the quantized range, or where the page cannot be read, the missing tokens' values become zeros and
+                // their key codes some integers, which the softmax warps mask)
+                if (mine) unpack_page<BITS>(raw, sK, sV, ptid, page_ok ? q_lo - page_pos : PAGE_TOKENS, q_hi - page_pos);
                 WST(6);
-#pragma unroll 4
-                for (int item = ptid; item < (mine && !whole ? TN * 16 : 0); item += 128) {      // first / last page of the range
-                    const int r = item & (TN - 1), kc = item >> 6;
-                    const int pos = (page_first + gb) * PAGE_TOKENS + r;
-                    const bool live = page_ok && pos >= q_lo && pos < q_hi;
-                    uint4 kq = zero4, vq = zero4;
-                    if (live) {
-                        unpack_chunk8<BITS>(raw, r, kc, kq, vq);
-                        // values are staged dequantized (see unpack_page)
-                        const unsigned mv = *reinterpret_cast<const unsigned*>(raw + meta_location(BITS, r) + 4);
-                        const unsigned step2 = __byte_perm(mv, mv, 0x1010u), offs2 = __byte_perm(mv, mv, 0x3232u);
-                        unsigned* vw = reinterpret_cast<unsigned*>(&vq);
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const __half2 hv = __hfma2(*reinterpret_cast<const __half2*>(vw + e), *reinterpret_cast<const __half2*>(&step2),
-                                                       *reinterpret_cast<const __half2*>(&offs2));
-                            vw[e] = *reinterpret_cast<const unsigned*>(&hv);
-                        }
-                    }
-                    *reinterpret_cast<uint4*>(sK + (r >> 3) * 2048 + kc * 128 + (r & 7) * 16) = kq;
-                    *reinterpret_cast<uint4*>(sV + kc * 1024 + (r >> 3) * 128 + (r & 7) * 16) = vq;
-                }
                 if (mine && ptid < TN) {                        // warps 12 and 13: key factors and existence of key ptid
                     const int pos = (page_first + gb) * PAGE_TOKENS + ptid;
                     const bool live = page_ok && pos >= q_lo && pos < q_hi;
