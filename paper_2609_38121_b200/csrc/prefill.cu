@@ -2230,8 +2230,9 @@ static_assert(PT_OFF_X % 1024 == 0, "swizzled tiles need 1024-byte alignment");
 
 // Projected inputs (Algorithm 2 lines 1-2), ahead of the transforms: one warp per chunk token and group of heads; a lane keeps the
 // (cos, sin) of its channels for all of them.  The rows go where the transforms leave their results (keys in KP, queries in the
-// second half of QP): a tile of rows is read there by the one CTA that then writes it.  Bound by instruction issue (about 120
-// per row and warp).  With
+// second half of QP): a tile of rows is read there by the one CTA that then writes it.  Bound by instruction issue: about 80
+// per row and warp, 120 when every row's sum was exchanged and its root taken on its own (five ragged prompts, 7400 tokens of 32 / 8 heads:
+// 518 -> 508 us).  With
 // the rows normalised and rotated inside the transform kernel, tile by tile in shared memory, the table was read for every
 // head and its wait held up that kernel's threads: 220 us for 8000 tokens of 32 / 8 heads against 65 us here and 75 us there.
 constexpr int ROT_WARPS = 8;
@@ -2261,16 +2262,32 @@ __global__ void __launch_bounds__(32 * ROT_WARPS) prefill_rotate_kernel(PrefillP
             pro.weight = j < 0 ? P.pro.weight : P.q_weight;
             w[e] = prologue_weights(pro, lane, j < 0 ? h : j);
         }
+        float x[AHEAD][4], ss[AHEAD];
+#pragma unroll
+        for (int e = 0; e < AHEAD; ++e) {
+            x[e][0] = bf16_bits_to_float(raw[e].x & 0xffff); x[e][1] = bf16_bits_to_float(raw[e].x >> 16);
+            x[e][2] = bf16_bits_to_float(raw[e].y & 0xffff); x[e][3] = bf16_bits_to_float(raw[e].y >> 16);
+            ss[e] = square_sum(x[e]);
+        }
+        // the four rows' sums over the lanes in the order of norm_rope_warp's, six exchanges for all of them: lane L ends up with row
+        // 2 (bit 3) + (bit 4) of L, and one root and reciprocal serve four rows
+        const bool up = lane & 16, up2 = lane & 8;
+        float s0 = (up ? ss[1] : ss[0]) + __shfl_xor_sync(0xffffffffu, up ? ss[0] : ss[1], 16);
+        float s1 = (up ? ss[3] : ss[2]) + __shfl_xor_sync(0xffffffffu, up ? ss[2] : ss[3], 16);
+        float sum = (up2 ? s1 : s0) + __shfl_xor_sync(0xffffffffu, up2 ? s0 : s1, 8);
+#pragma unroll
+        for (int o = 4; o >= 1; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        const float root = norm_factor(sum, P.pro);
 #pragma unroll
         for (int e = 0; e < AHEAD; ++e) {
             const int h = h0 + e, j = h - c.n_kv;
+            const float r = __shfl_sync(0xffffffffu, root, 16 * (e & 1) + 8 * (e >> 1));
             if (h >= h1) break;
-            float x[4] = {bf16_bits_to_float(raw[e].x & 0xffff), bf16_bits_to_float(raw[e].x >> 16), bf16_bits_to_float(raw[e].y & 0xffff), bf16_bits_to_float(raw[e].y >> 16)};
             pro.weight = j < 0 ? P.pro.weight : P.q_weight;
-            norm_rope_warp_loaded(x, lane, pro, w[e], cs0, cs1);
+            norm_rope_scaled(x[e], r, lane, pro, w[e], cs0, cs1);
             unsigned short* dst = j < 0 ? reinterpret_cast<unsigned short*>(P.KP) + (static_cast<long long>(tok) * c.n_kv + h) * D : q_out + (static_cast<long long>(tok) * c.n_q + j) * D;
-            reinterpret_cast<uint2*>(dst)[lane] = make_uint2(__byte_perm(__float_as_uint(x[0]), __float_as_uint(x[1]), 0x7632),       // bf16-valued: the upper halves
-                                                             __byte_perm(__float_as_uint(x[2]), __float_as_uint(x[3]), 0x7632));
+            reinterpret_cast<uint2*>(dst)[lane] = make_uint2(__byte_perm(__float_as_uint(x[e][0]), __float_as_uint(x[e][1]), 0x7632),       // bf16-valued: the upper halves
+                                                             __byte_perm(__float_as_uint(x[e][2]), __float_as_uint(x[e][3]), 0x7632));
         }
     }
 }

@@ -34,16 +34,15 @@ __device__ __forceinline__ int prologue_position(const Prologue& pro, int pos, i
     return pos;
 }
 
-// Warp-wide form: lane L holds channels 4L..4L+3 of one head vector in x[0..3].  This form takes what it needs from
+// Warp-wide form: lane L holds channels 4L..4L+3 of one head vector in x[0..3].  Its steps take what they need from
 // memory as arguments (w: the lane's four weights, read only if pro.weight is set; cs0, cs1: (cos, sin) of the lane's
 // four channel pairs), so that a caller with several vectors can have their loads in flight together.
-__device__ __forceinline__ void norm_rope_warp_loaded(float (&x)[4], int lane, const Prologue& pro, const float4& w,
-                                                      const float4& cs0, const float4& cs1) {
+__device__ __forceinline__ float square_sum(const float (&x)[4]) { return fmaf(x[0], x[0], fmaf(x[1], x[1], fmaf(x[2], x[2], x[3] * x[3]))); }
+__device__ __forceinline__ float norm_factor(float ss, const Prologue& pro) { return ss > 0.f ? 1.f / sqrtf(ss * (1.f / D) + pro.eps) : 0.f; }
+// r: norm_factor of the vector's sum of squares
+__device__ __forceinline__ void norm_rope_scaled(float (&x)[4], float r, int lane, const Prologue& pro, const float4& w,
+                                                 const float4& cs0, const float4& cs1) {
     if (pro.normalise) {
-        float ss = fmaf(x[0], x[0], fmaf(x[1], x[1], fmaf(x[2], x[2], x[3] * x[3])));
-#pragma unroll
-        for (int o = 16; o >= 1; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-        const float r = ss > 0.f ? 1.f / sqrtf(ss * (1.f / D) + pro.eps) : 0.f;
         if (pro.weight) {
             x[0] *= r * w.x; x[1] *= r * w.y; x[2] *= r * w.z; x[3] *= r * w.w;
         } else {
@@ -58,6 +57,17 @@ __device__ __forceinline__ void norm_rope_warp_loaded(float (&x)[4], int lane, c
         const float y = lane < 16 ? fmaf(x[e], c[e], -other * s[e]) : fmaf(other, s[e], x[e] * c[e]);
         x[e] = prologue_bf16_round(y);
     }
+}
+__device__ __forceinline__ void norm_rope_warp_loaded(float (&x)[4], int lane, const Prologue& pro, const float4& w,
+                                                      const float4& cs0, const float4& cs1) {
+    float r = 1.f;
+    if (pro.normalise) {
+        float ss = square_sum(x);
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+        r = norm_factor(ss, pro);
+    }
+    norm_rope_scaled(x, r, lane, pro, w, cs0, cs1);
 }
 // the lane's weights of `head` and its (cos, sin) table entries at `pos`
 __device__ __forceinline__ float4 prologue_weights(const Prologue& pro, int lane, int head) {
