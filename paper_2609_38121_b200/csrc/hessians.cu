@@ -14,7 +14,7 @@
 // both fp32), the fp32 one is split into three bf16 terms, 24 bits, and the products run on the tensor cores (mma.sync: the
 // logits of all heads and v . U of a pair meet entry by entry in one thread's accumulators, which is what the sum over s needs).
 // 1024 tokens of 32 / 8 heads: 1343 us as register-blocked fp32 products out of shared memory, bound by fp32 issue and shared-memory
-// reads alike (pairs_kernel 626, rows_kernel 366, project_kernel 215); now 624 us (243, 96, 136), error against 64 bits 2.8e-7 -> 1.3e-7:
+// reads alike (pairs_kernel 626, rows_kernel 366, project_kernel 215); now 610 us (243, 96, 136), error against 64 bits 2.8e-7 -> 1e-7:
 //   gamma_kernel      Gamma_{gg'}, 128 x 128 x d_model, fp32 products, float64 across groups of 16
 //   rows_kernel       causal softmax statistics (max, 1 / sum) and head outputs o_{g,t}: 64 x 64 tiles
 //   project_kernel    U, kappa and alpha: 128 x 128 tiles
@@ -113,10 +113,11 @@ __device__ __forceinline__ void hs_requested() { asm volatile("cp.async.commit_g
 template <int LEFT>
 __device__ __forceinline__ void hs_landed() { asm volatile("cp.async.wait_group %0;" ::"n"(LEFT) : "memory"); }
 
-// C[i][j] += sum_k a[k][i] b[k][j] for one staged group of 16 k; thread: rows 4 (tid >> 4) .., columns (tid & 15) + 16 e.
+// C[i][j] += sum_k a[k][i] b[k][j] for one staged group of 16 k; thread: rows 4 (tid >> 4) .., columns outer_column(tid, e).
 constexpr int OUTER_K = 16;
+__device__ __forceinline__ int outer_column(int tid, int e) { return 4 * (tid & 15) + (e < 4 ? e : 60 + e); }
 __device__ __forceinline__ void outer_group(const float (*a)[HS_PITCH], const float (*b)[HS_PITCH], double (&acc)[4][8]) {
-    const int i0 = 4 * (threadIdx.x >> 4), j0 = threadIdx.x & 15;
+    const int i0 = 4 * (threadIdx.x >> 4), j0 = 4 * (threadIdx.x & 15);
     float part[4][8];
 #pragma unroll
     for (int r = 0; r < 4; ++r)
@@ -125,9 +126,8 @@ __device__ __forceinline__ void outer_group(const float (*a)[HS_PITCH], const fl
 #pragma unroll 4
     for (int k = 0; k < OUTER_K; ++k) {
         const float4 av = *reinterpret_cast<const float4*>(&a[k][i0]);
-        float bv[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) bv[e] = b[k][j0 + 16 * e];
+        const float4 b0 = *reinterpret_cast<const float4*>(&b[k][j0]), b1 = *reinterpret_cast<const float4*>(&b[k][64 + j0]);
+        const float bv[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
             part[0][e] = fmaf(av.x, bv[e], part[0][e]); part[1][e] = fmaf(av.y, bv[e], part[1][e]);
@@ -143,7 +143,7 @@ __device__ __forceinline__ void outer_group(const float (*a)[HS_PITCH], const fl
 // Gamma_{gg'}[i][j] = sum_m W_g[i][m] W_g'[j][m] and its transpose Gamma_{g'g}; grid (pairs, n_kv, 4 blocks of 32 rows i), 128
 // threads: with few pairs the time is that of one CTA's groups of 16 m, whose loads are in flight while the group before
 // is multiplied (a CTA per pair with its loads waited for: 58 us for one pair and d_model 320).
-__global__ void __launch_bounds__(128) gamma_kernel(HessParams P) {
+__global__ void __launch_bounds__(128, 3) gamma_kernel(HessParams P) {
     __shared__ __align__(16) float a_s[OUTER_K][HS_PITCH], b_s[OUTER_K][HS_PITCH];
     int g, gp;
     pair_heads(blockIdx.x, P.G, g, gp);
@@ -176,14 +176,15 @@ __global__ void __launch_bounds__(128) gamma_kernel(HessParams P) {
     }
     float* out = P.gamma + (static_cast<long long>(h * P.G + g) * P.G + gp) * D * D;
     float* outT = P.gamma + (static_cast<long long>(h * P.G + gp) * P.G + g) * D * D;
-    const int i0 = r0 + 4 * (tid >> 4), j0 = tid & 15;
+    const int i0 = r0 + 4 * (tid >> 4);
 #pragma unroll
     for (int r = 0; r < 4; ++r)
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
+            const int j = outer_column(tid, e);
             const float v = static_cast<float>(acc[r][e]);
-            out[(i0 + r) * D + j0 + 16 * e] = v;
-            if (g != gp) outT[(j0 + 16 * e) * D + i0 + r] = v;
+            out[(i0 + r) * D + j] = v;
+            if (g != gp) outT[j * D + i0 + r] = v;
         }
 }
 
@@ -756,17 +757,21 @@ __global__ void __launch_bounds__(256) finish_kernel(HessParams P) {
         if (lane == 0) c_s[k] = sum;
     }
     __syncthreads();
-    for (int idx = tid; idx < D * D / 16; idx += 256) {
-        const int ij = blockIdx.x * (D * D / 16) + idx;
-        double hv = 0.0;
-        int k = 0;
-        for (int g = 0; g < P.G; ++g)
-            for (int gp = g; gp < P.G; ++gp, ++k) {
-                const double a = P.gamma[(static_cast<long long>(h * P.G + g) * P.G + gp) * D * D + ij];
-                hv += c_s[k] * (g == gp ? a : a + static_cast<double>(P.gamma[(static_cast<long long>(h * P.G + gp) * P.G + g) * D * D + ij]));
+    double hv[D * D / 16 / 256] = {};                    // the thread's entries side by side: their loads are in flight together
+    const int ij = blockIdx.x * (D * D / 16) + tid;
+    int k = 0;
+    for (int g = 0; g < P.G; ++g)
+        for (int gp = g; gp < P.G; ++gp, ++k) {
+            const float* up = P.gamma + (static_cast<long long>(h * P.G + g) * P.G + gp) * D * D + ij;
+            const float* down = P.gamma + (static_cast<long long>(h * P.G + gp) * P.G + g) * D * D + ij;
+#pragma unroll
+            for (int e = 0; e < D * D / 16 / 256; ++e) {
+                const double a = up[256 * e];
+                hv[e] += c_s[k] * (g == gp ? a : a + static_cast<double>(down[256 * e]));
             }
-        P.H_V[static_cast<long long>(h) * D * D + ij] += 2.0 * hv;
-    }
+        }
+#pragma unroll
+    for (int e = 0; e < D * D / 16 / 256; ++e) P.H_V[static_cast<long long>(h) * D * D + ij + 256 * e] += 2.0 * hv[e];
 }
 
 template <int G>
