@@ -1854,9 +1854,9 @@ __global__ void __launch_bounds__(WS_THREADS, 1) prefill_attn_ws_kernel(PrefillP
             }
             if (!(P.drop == 1 && g == 0)) ws_commit(bar(WB_S + 2 * t + (g & 1)));
         };
-        // The scores of tile g, whose key stage has landed.  The stage is free again when both query tiles' scores are done: the warp that
-        // requests bulk copies waits for those, the staging threads for one barrier of their own (a wait costs each of them some
-        // hundred cycles, a commit the tensor pipe about 60: 5.51 -> 5.26 ms for 8 prompts of 8192 tokens without it).
+        // The scores of tile g, whose key stage has landed.  The stage is free again when the scores of the query tiles that have it are done: the
+        // warp that requests bulk copies waits for those, the staging threads for one barrier of their own (a wait costs each of them some
+        // hundred cycles, a commit the tensor pipe about 60: 5.46 -> 5.29 ms for 8 prompts of 8192 tokens without it).
         auto scores = [&](const int g) {
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const bool staged_next = g + WS_KS < n_staged;
@@ -1880,6 +1880,9 @@ __global__ void __launch_bounds__(WS_THREADS, 1) prefill_attn_ws_kernel(PrefillP
             return ready != 0;
         };
         if (lane == 0 && ok) {
+            // From here on the key tiles are not looked for: this warp does not read them and no staging thread waits for its arrival.  The
+            // copies do not wait for it either, and a stage that they have refilled meanwhile would not read as landed any more.
+            const int unread = max(mine, n_staged - WS_KS);
             int sc = 0, pv = 0, idle = 0;
             while (pv < NT) {
                 bool progressed = false;
@@ -1910,7 +1913,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) prefill_attn_ws_kernel(PrefillP
                         }
                     }
                 }
-                if (sc < NT && sc < pv + 2 && landed(WB_KFULL, WS_KS, sc)) {
+                if (sc < NT && sc < pv + 2 && (sc >= unread || landed(WB_KFULL, WS_KS, sc))) {
                     WST(6);
                     scores(sc);
                     ++sc; progressed = true;

@@ -37,3 +37,17 @@ def test_prompt_lengths_around_tiles(n, test_option):
     L = Layer(wl, [n], 2, 4, 64, 1)
     assert L.check_prefill_parity([n]) <= 2e-3
     assert L.cache.status() == 0
+
+
+@pytest.mark.parametrize("n,ctx,split", [(522, 0, 1), (522, 300, 1), (538, 300, 2), (1030, 0, 3)])
+def test_last_pair_without_a_second_tile(n, ctx, split, test_option):
+    """Four heads per key/value head: a query tile is 32 positions, a pair 64.  The last pair has positions for its first tile only, and more
+    copied key tiles than stages, which the second tile's issuing warp passes over."""
+    test_option("prefill_split", split)
+    wl = W.LayerWorkload(dict(seed=103, batch=1, n_q=8, n_kv=2, ctx=0, theta=1e4, bits=2, s_sink=4, s_keep=64, rmsnorm=False, ragged=None,
+                              prefill_chunk=0))
+    L = Layer(wl, [ctx + n], 2, 4, 64, 1)
+    if ctx:
+        L.append_step([ctx])
+    assert L.check_prefill_parity([n]) <= 2e-3
+    assert L.cache.status() == 0
