@@ -154,6 +154,7 @@ int wushkv_build_transforms(int32_t n_heads, int32_t d, const double* M, const d
  *   wushkv_accumulate_gram_device: K, Q (device) bf16 as above, 16-byte aligned; M, H (device, in/out) float64
  *     [n_kv][d][d], zeroed by the caller before the first sequence.  d must be 128.  Products of the bf16
  *     inputs are exact, sums are fp32 within groups of 128 tokens and float64 beyond (relative error below 1e-6).
+ *     Should a wait inside the kernel run out (about a second; not expected), the diagonals of every M and H become NaN.
  *   wushkv_build_transforms_device: M, H (device) float64 [n_heads][d][d]; T, T_invT (device, out) fp32
  *     [n_heads][d][d] with the same canonical form and bf16 rounding as the host call; status (device, out):
  *     one int32 the caller zeroes, set to WUSHKV_ENOTPD if a damped matrix is not positive definite;
@@ -426,6 +427,8 @@ int wushkv_set_profile_events(void* start, void* stop);
  *   "drop_prefill"      1: the tcgen05 chunk attention never commits the score MMAs of a CTA's first tile; 2: it announces
  *                       but never issues one bulk copy of a CTA's first chunk tile; 3: the tcgen05 transform kernel does the
  *                       same with a copy of its first token tile (the bounded wait runs out in each case).
+ *   "drop_gram"         wushkv_accumulate_gram_device: 1: a CTA's first products are never signalled; 2: one of its first bulk
+ *                       copies is announced but never issued (the bounded wait runs out in both cases).
  * Returns WUSHKV_EINVAL for an unknown name.
  */
 int wushkv_set_test_option(const char* name, long long value);

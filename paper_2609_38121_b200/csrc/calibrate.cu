@@ -10,6 +10,7 @@
 //                           rounded to bf16, Gauss-Jordan inverse of the rounded matrix.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 
 #include "host_common.h"
@@ -38,11 +39,13 @@ struct GramParams {
     int n_kv, n_q;
     long long groups, units;                         // groups of tokens; groups times heads (those of K, then those of Q)
     double *M, *H;
+    int wait_limit;                                  // polls of about a microsecond each
+    int drop;                                        // testing aid: 1 the first unit's products are never signalled, 2 one bulk copy is never issued
 };
-// False when the wait ran out (about a second), here or in another warp.
-__device__ __forceinline__ bool gram_wait(unsigned bar, unsigned parity, volatile int* stop) {
+// False when the wait ran out, here or in another warp.
+__device__ __forceinline__ bool gram_wait(unsigned bar, unsigned parity, int limit, volatile int* stop) {
 #pragma unroll 1
-    for (int n = 0; n < (1 << 20); ++n) {
+    for (int n = 0; n < limit; ++n) {
         unsigned done;
         asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\tselp.u32 %0, 1, 0, p;\n\t}"
                      : "=r"(done) : "r"(bar), "r"(parity), "r"(1000u) : "memory");
@@ -81,32 +84,34 @@ __global__ void __launch_bounds__(GR_THREADS, 1) gram_kernel(GramParams P, const
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const unsigned tmem = tmem_s;
     volatile int* stop = &stop_s;
+    int copied = 0;                                  // by this thread
     if (warp == 8) {
         if (lane == 0) {
             int slot = static_cast<int>(u0 / P.groups), k = 0;
             long long group = u0 % P.groups;
             for (; k < n_units; ++k) {
                 const int stage = k % GR_STAGES;
-                if (k >= GR_STAGES && !gram_wait(saddr(&free_bar[stage]), (k / GR_STAGES - 1) & 1, stop)) break;
+                if (k >= GR_STAGES && !gram_wait(saddr(&free_bar[stage]), (k / GR_STAGES - 1) & 1, P.wait_limit, stop)) break;
                 const unsigned bar = saddr(&full_bar[stage]), dst = tiles + stage * GR_TILE_BYTES;
                 asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(static_cast<unsigned>(GR_TILE_BYTES)) : "memory");
                 const CUtensorMap* map = slot < P.n_kv ? &k_map : &q_map;
                 const int head = slot < P.n_kv ? slot : slot - P.n_kv, row = static_cast<int>(group * GR_TOK);
 #pragma unroll
-                for (int half = 0; half < 2; ++half)
+                for (int half = 0; half < 2; ++half) {
+                    if (P.drop == 2 && k == 0 && half == 0) continue;
                     asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
                                  ::"r"(dst + half * (GR_TILE_BYTES / 2)), "l"(reinterpret_cast<unsigned long long>(map)), "r"(64 * half), "r"(head), "r"(row), "r"(bar) : "memory");
+                }
                 if (++group == P.groups) { group = 0; ++slot; }
             }
-            if (*stop)                               // nothing may arrive after the CTA has gone
-                for (int n = k > GR_STAGES ? k - GR_STAGES : 0; n < k; ++n) gram_wait(saddr(&full_bar[n % GR_STAGES]), (n / GR_STAGES) & 1, nullptr);
+            copied = k;
         }
     } else if (warp == 9) {
         if (lane == 0) {
             for (int k = 0; k < n_units; ++k) {
                 const int stage = k % GR_STAGES, acc = k % GR_ACC;
-                if (!gram_wait(saddr(&full_bar[stage]), (k / GR_STAGES) & 1, stop)) break;
-                if (k >= GR_ACC && !gram_wait(saddr(&read_bar[acc]), (k / GR_ACC - 1) & 1, stop)) break;
+                if (!gram_wait(saddr(&full_bar[stage]), (k / GR_STAGES) & 1, P.wait_limit, stop)) break;
+                if (k >= GR_ACC && !gram_wait(saddr(&read_bar[acc]), (k / GR_ACC - 1) & 1, P.wait_limit, stop)) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 // rows of 128 bytes (64 channels of a token), groups of 8 tokens 1024 bytes apart, the other 64 channels half a tile behind
                 const unsigned long long desc = (static_cast<unsigned long long>(((tiles + stage * GR_TILE_BYTES) >> 4) & 0x3FFFu)) |
@@ -118,11 +123,7 @@ __global__ void __launch_bounds__(GR_THREADS, 1) gram_kernel(GramParams P, const
                                  "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %1, %2, {%4, %4, %4, %4}, p;\n\t}"
                                  ::"r"(tmem + acc * D), "l"(desc + static_cast<unsigned long long>(ks * 2048 >> 4)), "r"(GR_IDESC), "r"(ks), "r"(0u) : "memory");
                 gram_commit(saddr(&free_bar[stage]));
-                gram_commit(saddr(&acc_bar[acc]));
-            }
-            if (*stop) {
-                gram_commit(saddr(&drain_bar));
-                gram_wait(saddr(&drain_bar), 0, nullptr);
+                if (!(P.drop == 1 && k == 0)) gram_commit(saddr(&acc_bar[acc]));
             }
         }
     } else {
@@ -134,7 +135,7 @@ __global__ void __launch_bounds__(GR_THREADS, 1) gram_kernel(GramParams P, const
         long long group = u0 % P.groups;
         for (int k = 0; k < n_units; ++k) {
             const int acc = k % GR_ACC;
-            if (!gram_wait(saddr(&acc_bar[acc]), (k / GR_ACC) & 1, stop)) break;
+            if (!__all_sync(0xffffffffu, gram_wait(saddr(&acc_bar[acc]), (k / GR_ACC) & 1, P.wait_limit, stop))) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
             for (int part = 0; part < 2; ++part) {
@@ -168,8 +169,22 @@ __global__ void __launch_bounds__(GR_THREADS, 1) gram_kernel(GramParams P, const
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (stop_s) {                                    // a wait ran out
+        // no copy or product may be under way when the CTA has gone
+        for (int n = copied > GR_STAGES ? copied - GR_STAGES : 0; n < copied; ++n) gram_wait(saddr(&full_bar[n % GR_STAGES]), (n / GR_STAGES) & 1, P.wait_limit, nullptr);
+        if (warp == 9 && lane == 0) {
+            gram_commit(saddr(&drain_bar));
+            gram_wait(saddr(&drain_bar), 0, P.wait_limit, nullptr);
+        }
+        __syncwarp();
+        // the statistics must not look usable: not a number on the diagonal of every matrix
+        for (long long n = tid; n < static_cast<long long>(P.n_kv) * D; n += GR_THREADS) {
+            const long long at = n / D * (D * D) + n % D * (D + 1);
+            atomicAdd(P.M + at, static_cast<double>(NAN));
+            atomicAdd(P.H + at, static_cast<double>(NAN));
+        }
+    }
     if (warp == 9) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(static_cast<unsigned>(GR_ACC * D)) : "memory");
-    if (tid == 0 && stop_s) atomicAdd(P.M, static_cast<double>(NAN));    // a wait ran out: the statistics must not look usable
 }
 
 // ---- float64 helpers of the transform builder -----------------------------------------------------
@@ -785,6 +800,8 @@ extern "C" int wushkv_accumulate_gram_device(int32_t n_kv, int32_t n_q, int32_t 
     if (n_tok == 0) return WUSHKV_OK;
     GramParams P;
     P.n_kv = n_kv; P.n_q = n_q; P.M = M; P.H = H;
+    P.wait_limit = knobs().wait_limit > 0 ? static_cast<int>(std::min(knobs().wait_limit, 1LL << 20)) : 1 << 20;      // about a second
+    P.drop = knobs().drop_gram;
     P.groups = (n_tok + GR_TOK - 1) / GR_TOK;
     P.units = P.groups * (static_cast<long long>(n_kv) + n_q);
     if (n_tok > 0x7fffffffLL - GR_TOK || P.units > 0x7fffffffLL) return WUSHKV_EINVAL;

@@ -92,6 +92,29 @@ def test_chunk_attention_wait_that_runs_out_is_flagged(what, one_tile, test_opti
     assert ok.cache.status() == 0
 
 
+@pytest.mark.parametrize("what", [1, 2])
+def test_gram_wait_that_runs_out_leaves_no_usable_statistics(what, test_option):
+    """Products that are never signalled (1), a bulk copy that is announced but never issued (2): the kernel returns, no matrix of
+    any head looks usable, and the next call is healthy."""
+    import torch
+    from paper_2609_38121_b200 import binding as B
+    gen = torch.Generator(device="cuda").manual_seed(68)
+    K, Q = (torch.randn((9000, n, 128), generator=gen, device="cuda").to(torch.bfloat16) for n in (3, 6))
+    sums = lambda: [torch.zeros((3, 128, 128), dtype=torch.float64, device="cuda") for _ in range(2)]  # noqa: E731
+    test_option("drop_gram", what)
+    test_option("wait_limit", 2000)
+    M, H = sums()
+    B.accumulate_gram_device(K.view(torch.int16), Q.view(torch.int16), M, H)
+    for X in (M, H):
+        assert torch.all(torch.isnan(torch.diagonal(X, dim1=1, dim2=2)))
+    test_option("drop_gram", 0)
+    test_option("wait_limit", 0)
+    M, H = sums()
+    B.accumulate_gram_device(K.view(torch.int16), Q.view(torch.int16), M, H)
+    ref = torch.stack([K[:, h].double().T @ K[:, h].double() for h in range(3)])
+    assert (M - ref).abs().max().item() <= 2e-6 * ref.abs().max().item() and torch.all(torch.isfinite(H))
+
+
 def test_more_tokens_than_the_decode_hint_promised():
     """max_new == 1 selects the single-token kernel; a sequence that brings two tokens is flagged and left alone."""
     import torch
