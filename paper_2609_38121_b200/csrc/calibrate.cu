@@ -28,8 +28,9 @@ __device__ __forceinline__ unsigned saddr(const void* p) { return static_cast<un
 // consecutive part of the list (head, tokens); where the matrix changes, and at the end, a thread adds its 64 sums to the statistics
 // with atomics (to the mirror image of their places, which makes a warp's addresses consecutive).
 // Warps 0-7: float64 sums of the 32 tensor-memory lanes that their number allows, half the columns each.  Warp 8: copies, six tiles ahead.
-// Warp 9: MMAs, into one of four accumulators.  32768 tokens of 32 / 8 heads: mma.sync with the sums in the same warps 255 us (its rate),
-// this 106.
+// Warp 9: MMAs, into one of four accumulators.  What bounds it: the conversions to float64 and their sums, in eight warps that hold 64 of them
+// per thread.  32768 tokens of 32 / 8 heads: mma.sync with the sums in the same warps 255 us (its rate), this 92; with 32 columns
+// loaded at a time, which spills, 106.
 constexpr int GR_TOK = 128, GR_STAGES = 6, GR_ACC = 4, GR_THREADS = 320;
 constexpr int GR_TILE_BYTES = GR_TOK * D * 2;
 constexpr size_t GRAM_SMEM = static_cast<size_t>(GR_STAGES) * GR_TILE_BYTES + 1024;      // and alignment
@@ -62,7 +63,7 @@ __global__ void __launch_bounds__(GR_THREADS, 1) gram_kernel(GramParams P, const
     extern __shared__ __align__(16) unsigned char gram_smem[];
     __shared__ unsigned long long full_bar[GR_STAGES], free_bar[GR_STAGES], acc_bar[GR_ACC], read_bar[GR_ACC], drain_bar;
     __shared__ unsigned tmem_s;
-    __shared__ int stop_s;
+    __shared__ int stop_s, copied_s;                // a wait ran out; tiles requested by bulk copies
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const unsigned tiles = (saddr(gram_smem) + 1023u) & ~1023u;
     const long long u0 = P.units * blockIdx.x / gridDim.x, u1 = P.units * (blockIdx.x + 1) / gridDim.x;
@@ -73,7 +74,7 @@ __global__ void __launch_bounds__(GR_THREADS, 1) gram_kernel(GramParams P, const
         for (int k = 0; k < GR_ACC; ++k) { init(&acc_bar[k], 1); init(&read_bar[k], 8); }
         init(&drain_bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        stop_s = 0;
+        stop_s = copied_s = 0;
     }
     if (warp == 9) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(saddr(&tmem_s)), "r"(static_cast<unsigned>(GR_ACC * D)) : "memory");
@@ -84,7 +85,6 @@ __global__ void __launch_bounds__(GR_THREADS, 1) gram_kernel(GramParams P, const
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const unsigned tmem = tmem_s;
     volatile int* stop = &stop_s;
-    int copied = 0;                                  // by this thread
     if (warp == 8) {
         if (lane == 0) {
             int slot = static_cast<int>(u0 / P.groups), k = 0;
@@ -104,7 +104,7 @@ __global__ void __launch_bounds__(GR_THREADS, 1) gram_kernel(GramParams P, const
                 }
                 if (++group == P.groups) { group = 0; ++slot; }
             }
-            copied = k;
+            copied_s = k;
         }
     } else if (warp == 9) {
         if (lane == 0) {
@@ -135,27 +135,27 @@ __global__ void __launch_bounds__(GR_THREADS, 1) gram_kernel(GramParams P, const
         long long group = u0 % P.groups;
         for (int k = 0; k < n_units; ++k) {
             const int acc = k % GR_ACC;
-            if (!__all_sync(0xffffffffu, gram_wait(saddr(&acc_bar[acc]), (k / GR_ACC) & 1, P.wait_limit, stop))) break;
+            // (the lanes decide together whether to go on, but only after the loads: in front of them the vote takes 104 us instead of 92)
+            const bool landed = gram_wait(saddr(&acc_bar[acc]), (k / GR_ACC) & 1, P.wait_limit, stop);
+            __syncwarp();
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
-            for (int part = 0; part < 2; ++part) {
-                unsigned v[32];
-                const unsigned addr = tmem + acc * D + c0 + 32 * part + (static_cast<unsigned>(32 * (warp & 3)) << 16);
-                asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-                             "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+            for (int part = 0; part < 4; ++part) {
+                unsigned v[16];
+                const unsigned addr = tmem + acc * D + c0 + 16 * part + (static_cast<unsigned>(32 * (warp & 3)) << 16);
+                asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
                              : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]), "=r"(v[9]),
-                               "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]),
-                               "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]),
-                               "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+                               "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
                              : "r"(addr));
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                if (part == 1) {                     // the accumulator has been read
+                if (part == 3) {                     // the accumulator has been read
                     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                     if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(saddr(&read_bar[acc])) : "memory");
                 }
 #pragma unroll
-                for (int e = 0; e < 32; ++e) sum[32 * part + e] += static_cast<double>(__uint_as_float(v[e]));
+                for (int e = 0; e < 16; ++e) sum[16 * part + e] += static_cast<double>(__uint_as_float(v[e]));
             }
+            if (!__all_sync(0xffffffffu, landed)) break;
             const int matrix = slot < P.n_kv ? slot : P.n_kv + (slot - P.n_kv) / G;
             if (++group == P.groups) { group = 0; ++slot; }
             if (k == n_units - 1 || matrix != (slot < P.n_kv ? slot : P.n_kv + (slot - P.n_kv) / G)) {
@@ -171,8 +171,8 @@ __global__ void __launch_bounds__(GR_THREADS, 1) gram_kernel(GramParams P, const
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     if (stop_s) {                                    // a wait ran out
         // no copy or product may be under way when the CTA has gone
-        for (int n = copied > GR_STAGES ? copied - GR_STAGES : 0; n < copied; ++n) gram_wait(saddr(&full_bar[n % GR_STAGES]), (n / GR_STAGES) & 1, P.wait_limit, nullptr);
         if (warp == 9 && lane == 0) {
+            for (int n = max(copied_s - GR_STAGES, 0); n < copied_s; ++n) gram_wait(saddr(&full_bar[n % GR_STAGES]), (n / GR_STAGES) & 1, P.wait_limit, nullptr);
             gram_commit(saddr(&drain_bar));
             gram_wait(saddr(&drain_bar), 0, P.wait_limit, nullptr);
         }
