@@ -34,6 +34,7 @@ extern "C" int wushkv_set_test_option(const char* name, long long value) {
     else if (!std::strcmp(name, "prefill_split")) k.prefill_split = static_cast<int>(value);
     else if (!std::strcmp(name, "append_no_tma")) k.append_no_tma = value != 0;
     else if (!std::strcmp(name, "drop_prefill")) k.drop_prefill = static_cast<int>(value);
+    else if (!std::strcmp(name, "gram_no_tma")) k.gram_no_tma = value != 0;
     else if (!std::strcmp(name, "drop_gram")) k.drop_gram = static_cast<int>(value);
     else return WUSHKV_EINVAL;
     return WUSHKV_OK;

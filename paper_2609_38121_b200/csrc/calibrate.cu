@@ -40,6 +40,9 @@ struct GramParams {
     int n_kv, n_q;
     long long groups, units;                         // groups of tokens; groups times heads (those of K, then those of Q)
     double *M, *H;
+    const unsigned short *K, *Q;                     // read where there is no tensor map
+    long long n_tok;
+    int use_tma;
     int wait_limit;                                  // polls of about a microsecond each
     int drop;                                        // testing aid: 1 the first unit's products are never signalled, 2 one bulk copy is never issued
 };
@@ -85,7 +88,29 @@ __global__ void __launch_bounds__(GR_THREADS, 1) gram_kernel(GramParams P, const
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const unsigned tmem = tmem_s;
     volatile int* stop = &stop_s;
-    if (warp == 8) {
+    if (warp == 8 && !P.use_tma) {                   // the same tiles by 16-byte loads and stores of the warp's lanes
+        int slot = static_cast<int>(u0 / P.groups);
+        long long group = u0 % P.groups;
+        for (int k = 0; k < n_units; ++k) {
+            const int stage = k % GR_STAGES;
+            if (!__all_sync(0xffffffffu, k < GR_STAGES || gram_wait(saddr(&free_bar[stage]), (k / GR_STAGES - 1) & 1, P.wait_limit, stop))) break;
+            const bool key = slot < P.n_kv;
+            const int head = key ? slot : slot - P.n_kv, heads = key ? P.n_kv : P.n_q;
+            const unsigned short* X = (key ? P.K : P.Q) + static_cast<long long>(head) * D;
+#pragma unroll 4
+            for (int item = lane; item < GR_TOK * 16; item += 32) {
+                const int r = item >> 4, piece = item & 15;
+                const long long token = group * GR_TOK + r;
+                const uint4 v = token < P.n_tok ? *reinterpret_cast<const uint4*>(X + token * heads * D + 8 * piece) : make_uint4(0, 0, 0, 0);
+                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};"
+                             ::"r"(tiles + stage * GR_TILE_BYTES + (piece >> 3) * (GR_TILE_BYTES / 2) + r * 128 + (((piece ^ r) & 7) << 4)), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(saddr(&full_bar[stage])) : "memory");
+            if (++group == P.groups) { group = 0; ++slot; }
+        }
+    } else if (warp == 8) {
         if (lane == 0) {
             int slot = static_cast<int>(u0 / P.groups), k = 0;
             long long group = u0 % P.groups;
@@ -798,19 +823,24 @@ extern "C" int wushkv_accumulate_gram_device(int32_t n_kv, int32_t n_q, int32_t 
     if (!K || !Q || !M || !H || n_kv <= 0 || n_q <= 0 || d != D || n_tok < 0 || n_q % n_kv != 0) return WUSHKV_EINVAL;
     if (!aligned(K, 16) || !aligned(Q, 16) || !aligned(M, 8) || !aligned(H, 8)) return WUSHKV_EINVAL;
     if (n_tok == 0) return WUSHKV_OK;
+    if (n_tok > 0x7fffffffLL * 2048) return WUSHKV_EINVAL;
     GramParams P;
     P.n_kv = n_kv; P.n_q = n_q; P.M = M; P.H = H;
     P.wait_limit = knobs().wait_limit > 0 ? static_cast<int>(std::min(knobs().wait_limit, 1LL << 20)) : 1 << 20;      // about a second
     P.drop = knobs().drop_gram;
-    P.groups = (n_tok + GR_TOK - 1) / GR_TOK;
-    P.units = P.groups * (static_cast<long long>(n_kv) + n_q);
-    if (n_tok > 0x7fffffffLL - GR_TOK || P.units > 0x7fffffffLL) return WUSHKV_EINVAL;
-    CUtensorMap k_map, q_map;
-    if (!make_row_tensor_map(k_map, true, K, n_kv, n_tok, GR_TOK) || !make_row_tensor_map(q_map, true, Q, n_q, n_tok, GR_TOK) ||
-        !opt_in_dynamic_smem(reinterpret_cast<const void*>(gram_kernel), static_cast<int>(GRAM_SMEM)))
-        return WUSHKV_ECUDA;
-    const unsigned ctas = static_cast<unsigned>(P.units < sm_count() ? P.units : sm_count());
-    gram_kernel<<<ctas, GR_THREADS, GRAM_SMEM, static_cast<cudaStream_t>(stream)>>>(P, k_map, q_map);
+    if (!opt_in_dynamic_smem(reinterpret_cast<const void*>(gram_kernel), static_cast<int>(GRAM_SMEM))) return WUSHKV_ECUDA;
+    constexpr long long LAUNCH_TOK = 1LL << 29;      // keeps rows and a CTA's units within 32 bits
+    for (long long t0 = 0; t0 < n_tok; t0 += LAUNCH_TOK) {
+        P.K = K + t0 * n_kv * D; P.Q = Q + t0 * n_q * D;
+        P.n_tok = std::min(LAUNCH_TOK, n_tok - t0);
+        P.groups = (P.n_tok + GR_TOK - 1) / GR_TOK;
+        P.units = P.groups * (static_cast<long long>(n_kv) + n_q);
+        CUtensorMap k_map, q_map;
+        const bool mk = make_row_tensor_map(k_map, true, P.K, n_kv, P.n_tok, GR_TOK), mq = make_row_tensor_map(q_map, true, P.Q, n_q, P.n_tok, GR_TOK);
+        P.use_tma = mk && mq && !knobs().gram_no_tma;
+        const unsigned ctas = static_cast<unsigned>(P.units < sm_count() ? P.units : sm_count());
+        gram_kernel<<<ctas, GR_THREADS, GRAM_SMEM, static_cast<cudaStream_t>(stream)>>>(P, k_map, q_map);
+    }
     return cudaGetLastError() == cudaSuccess ? WUSHKV_OK : WUSHKV_ECUDA;
 }
 

@@ -59,6 +59,7 @@ struct Knobs {
     int prefill_split = 0;          // > 0: CTAs per tile pair of the warp-specialised chunk attention (capped by what the workspace holds); 0: chosen by the grid size
     int prefill_no_tma = 0;         // 1: the tcgen05 kernel stages the chunk's tiles with 16-byte copies instead of bulk tensor copies
     int drop_prefill = 0;           // chunk attention: 1 the first tile's score MMAs are never committed, 2 one bulk copy is never issued, 3 one bulk copy of the transform kernel is never issued
+    int gram_no_tma = 0;            // 1: the Gram accumulation stages its tiles with 16-byte copies instead of bulk tensor copies
     int drop_gram = 0;              // Gram accumulation: 1 a CTA's first products are never signalled, 2 one of its bulk copies is never issued
     int append_no_tma = 0;          // 1: the chunk append stages its tiles with 16-byte copies instead of bulk tensor copies
 };

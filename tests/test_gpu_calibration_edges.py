@@ -38,3 +38,20 @@ def test_builder_for_one_and_for_many_heads(heads):
     assert np.all(np.abs(T - ref) <= unit) and np.mean(T != ref) < 1e-3
     for h in range(heads):
         np.testing.assert_allclose(Ti[h].T @ T[h], np.eye(128), atol=1e-4)
+
+
+@pytest.mark.parametrize("n_tok,n_q,n_kv", [(1, 1, 1), (127, 2, 1), (32768 + 77, 7, 1)])
+def test_gram_without_tensor_maps_sums_the_same(n_tok, n_q, n_kv, test_option):
+    """Tiles staged by 16-byte copies: the same products.  The float64 sums are grouped alike; the CTAs' parts of a matrix meet in any order."""
+    import torch
+    from paper_2609_38121_b200 import binding as B
+    gen = torch.Generator(device="cuda").manual_seed(6)
+    K, Q = (torch.randn((n_tok, n, 128), generator=gen, device="cuda").to(torch.bfloat16).view(torch.int16) for n in (n_kv, n_q))
+    sums = []
+    for copies in (0, 1):
+        test_option("gram_no_tma", copies)
+        M, H = (torch.zeros((n_kv, 128, 128), dtype=torch.float64, device="cuda") for _ in range(2))
+        B.accumulate_gram_device(K, Q, M, H)
+        sums.append((M, H))
+    for a, b in zip(*sums):
+        assert (a - b).abs().max().item() <= 148 * 2.0 ** -52 * a.abs().max().item()
