@@ -25,6 +25,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <limits>
 #include <type_traits>
 
 #include "host_common.h"
@@ -827,7 +828,8 @@ extern "C" int wushkv_accumulate_attention_hessians_device(int32_t n_kv, int32_t
     HessParams P;
     P.S = static_cast<int>(n_tokens); P.n_kv = n_kv; P.n_q = n_q; P.G = G; P.d_model = d_model; P.n_pairs = G * (G + 1) / 2;
     P.inv_tau = static_cast<float>(1.0 / tau);
-    P.scale2 = static_cast<float>(1.4426950408889634 / tau);
+    // (never 0: masked logits are -infinity when they meet it; at the smallest fp32 number any finite logit's exponential is 1)
+    P.scale2 = std::max(static_cast<float>(1.4426950408889634 / tau), std::numeric_limits<float>::denorm_min());
     P.Q = Q; P.K = K; P.V = V; P.W_O = W_O;
     P.gamma = reinterpret_cast<float*>(ws + L.gamma);
     P.row_m = reinterpret_cast<float*>(ws + L.row_m); P.row_linv = reinterpret_cast<float*>(ws + L.row_linv);

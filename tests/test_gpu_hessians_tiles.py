@@ -71,3 +71,12 @@ def test_tensor_core_products(n_q, n_kv, n_tok, d_model):
         rk, rv = O.attention_hessians(Q[:, h * G:(h + 1) * G], K[:, h], V[:, h], WO[h * G:(h + 1) * G], tau)
         assert np.max(np.abs(HK[h] - rk)) <= 1.8e-5 * np.max(np.abs(rk)), np.max(np.abs(HK[h] - rk)) / np.max(np.abs(rk))
         assert np.max(np.abs(HV[h] - rv)) <= 1.8e-5 * np.max(np.abs(rv)), np.max(np.abs(HV[h] - rv)) / np.max(np.abs(rv))
+
+
+@pytest.mark.parametrize("tau", [1e42, 1e46, 1e300, float("inf")])
+def test_temperatures_beyond_the_fp32_range(tau):
+    """The probabilities are uniform, as at 1e30; 2 / tau^2 leaves next to nothing of H_K (1 / tau is a number of fp32 and becomes 0)."""
+    wl, K, Q, V, WO = _inputs(4, 1, 150, 16, seed=89)
+    ref, got = _gpu(K, Q, V, WO, 1e30), _gpu(K, Q, V, WO, tau)
+    assert np.max(np.abs(got[1] - ref[1])) <= TOL * np.max(np.abs(ref[1]))
+    assert np.max(np.abs(got[0])) <= 1e-60
