@@ -266,7 +266,9 @@ int wushkv_prefill_attn(const wushkv_cache* cache, int32_t batch, const int32_t*
  *   H_K, H_V (device, in/out): float64 [n_kv][d][d], accumulated.
  *   workspace (device): >= wushkv_attention_hessians_workspace_bytes() bytes, 256-byte aligned, scratch.
  * d must be 128 and the group size n_q / n_kv at most 8 (WUSHKV_EINVAL otherwise).  Cost O(n_tokens^2) per head.
- * Arithmetic: fp32 with float64 accumulation of the sums over tokens.
+ * Arithmetic: fp32 with float64 accumulation of the sums over tokens.  fp32 operands of the long products are taken as three
+ * bf16 terms, 24 bits of them from 2^-109 up; head outputs and products with Gamma = W_O W_O^T that are smaller lose bits.
+ * Where a product overflows or an input is not finite, the entries of H_K are not numbers.
  */
 size_t wushkv_attention_hessians_workspace_bytes(int32_t n_kv, int32_t n_q, int32_t d, int64_t n_tokens);
 int wushkv_accumulate_attention_hessians_device(int32_t n_kv, int32_t n_q, int32_t d, int32_t d_model, int64_t n_tokens,

@@ -89,9 +89,10 @@ __device__ __forceinline__ unsigned hs_pack(float lo, float hi) {
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
     return r;
 }
-// (x, y) as three pairs of bf16 whose sum is the fp32 values up to 2^-24 of each
+// (x, y) as three pairs of bf16 whose sum is the fp32 values up to 2^-24 of each.  The first term stops at bf16's largest number, which
+// fp32's range exceeds (the second makes up for it).
 __device__ __forceinline__ void hs_split(float x, float y, unsigned& hi, unsigned& mid, unsigned& lo) {
-    hi = hs_pack(x, y);
+    asm("cvt.rn.satfinite.bf16x2.f32 %0, %1, %2;" : "=r"(hi) : "f"(y), "f"(x));
     const float x1 = x - __uint_as_float(hi << 16), y1 = y - __uint_as_float(hi & 0xffff0000u);
     mid = hs_pack(x1, y1);
     lo = hs_pack(x1 - __uint_as_float(mid << 16), y1 - __uint_as_float(mid & 0xffff0000u));

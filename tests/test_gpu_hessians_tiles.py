@@ -4,6 +4,7 @@ import numpy as np
 import pytest
 
 from oracle import wushkv_oracle as O
+from paper_2609_38121_b200 import workloads as W
 from tests.test_gpu_hessians import TOL, _gpu, _inputs
 
 pytestmark = pytest.mark.gpu
@@ -80,3 +81,17 @@ def test_temperatures_beyond_the_fp32_range(tau):
     ref, got = _gpu(K, Q, V, WO, 1e30), _gpu(K, Q, V, WO, tau)
     assert np.max(np.abs(got[1] - ref[1])) <= TOL * np.max(np.abs(ref[1]))
     assert np.max(np.abs(got[0])) <= 1e-60
+
+
+def test_gamma_between_the_largest_numbers_of_bf16_and_fp32():
+    """Gamma[3][3] = 3.3989e38 rounds to infinity in bf16; with small values everything else is far inside the range."""
+    wl, K, Q, V, WO = _inputs(1, 1, 150, 16, seed=91)
+    WO = np.zeros_like(WO)
+    WO[0, 3, 5] = np.float32(1.8436e19)
+    assert 3.3962e38 < float(WO[0, 3, 5]) ** 2 < 3.4028e38
+    V = W.bf16_round_f32(V * np.float32(1e-4))
+    tau = float(np.sqrt(128))
+    HK, HV = _gpu(K, Q, V, WO, tau)
+    rk, rv = O.attention_hessians(Q, K[:, 0], V[:, 0], WO, tau)
+    assert np.max(np.abs(HK[0] - rk)) <= TOL * np.max(np.abs(rk))
+    assert np.max(np.abs(HV[0] - rv)) <= TOL * np.max(np.abs(rv))
