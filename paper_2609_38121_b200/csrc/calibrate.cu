@@ -269,7 +269,7 @@ __global__ void __launch_bounds__(BT_THREADS) factor_kernel(const double* Mall, 
     __shared__ __align__(16) unsigned key_s[2][4];
     const int h = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     double* ws = wsall + h * WS_HEAD;
-    double scale;
+    double scale, lift = 1.0;
     if (PIVOT) {
         if (ws[META_FAIL] != 0.0) return;
         const double tr = trace(ws + WS_A);
@@ -278,7 +278,8 @@ __global__ void __launch_bounds__(BT_THREADS) factor_kernel(const double* Mall, 
             return;
         }
         if (tid == 0) ws[META_TR_A] = tr;
-        scale = 0.5 / tr;
+        if (!(tr > 0x1p-900 && tr < 0x1p900)) lift = tr < 1.0 ? 0x1p200 : 0x1p-200;      // where 1 / tr is beyond the range, or has lost bits
+        scale = 0.5 / (lift * tr);
     } else {
         const double tr_m = trace(Mall + static_cast<long long>(h) * D * D);
         if (tid == 0) { ws[META_TR_M] = tr_m; ws[META_FAIL] = 0.0; }
@@ -288,7 +289,7 @@ __global__ void __launch_bounds__(BT_THREADS) factor_kernel(const double* Mall, 
     for (int idx = tid; idx < D * D; idx += BT_THREADS) {
         const int i = idx >> 7, j = idx & 127;
         if (i < j) continue;
-        S[j * BT_PITCH + i] = PIVOT ? scale * (ws[WS_A + idx] + ws[WS_A + j * D + i])
+        S[j * BT_PITCH + i] = PIVOT ? scale * (lift * (ws[WS_A + idx] + ws[WS_A + j * D + i]))
                                     : Hall[static_cast<long long>(h) * D * D + idx] + (i == j ? scale : 0.0);
     }
     __syncthreads();

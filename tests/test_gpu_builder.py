@@ -83,3 +83,20 @@ def test_columns_of_very_different_length(gamma):
     Td = T.cpu().numpy().astype(np.float64)
     unit = np.maximum(np.abs(ref), 1e-9 * np.abs(ref).max()) * 2.0 ** -7
     assert np.all(np.abs(Td - ref) <= unit) and np.mean(Td != ref) < 1e-3
+
+
+@pytest.mark.parametrize("m_scale,h_scale,power,floor", [(1e-155, 1e-156, 512, 1e-4), (1e153, 1e153, -512, 1e-9)])
+def test_statistics_at_the_ends_of_the_float64_range(m_scale, h_scale, power, floor):
+    """The trace of L^T M L is 1e-310 or 1e307: its reciprocal overflows or has fewer bits.  T does not change when M and H are multiplied by
+    a power of 16, so it is compared with that of the same matrices inside the range, with the tolerance of the other tests.  At the lower end
+    L^T M L is summed in multiples of 2^-1074: 128 terms per entry, each rounded by up to half of that, move the matrix by about
+    sqrt(128) sqrt(128) 2^-1075 = 3e-322 (2-norm).  Its eigenvalues lie between 1.7e-313 and 6e-312, the closest 2e-315 apart (numpy, the same matrices
+    times 1e311), so eigenvectors turn by up to 1.5e-7; entries of T near zero differ by that much of the largest, and the floor
+    allows 1e-4 2^-7 = 8e-7."""
+    rng = np.random.default_rng(11)
+    M, H = _spd(rng, 1.0, m_scale)[None], _spd(rng, 1.0, h_scale)[None]
+    T, Ti = _build(M, H, W.GAMMA)
+    ref, _ = _build(M * 2.0 ** power, H * 2.0 ** power, W.GAMMA)
+    unit = np.maximum(np.abs(ref), floor * np.abs(ref).max()) * 2.0 ** -7
+    assert np.all(np.abs(T - ref) <= unit) and np.mean(T != ref) < 1e-3
+    np.testing.assert_allclose(Ti[0].T @ T[0], np.eye(128), atol=1e-4)
