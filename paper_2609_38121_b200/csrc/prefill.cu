@@ -758,8 +758,8 @@ __device__ __forceinline__ void unpack_page(const unsigned char* raw, unsigned c
     constexpr unsigned MASK = TWO ? 3u : 15u, MASK2 = MASK * 0x00010001u;
     constexpr int CB = code_block_bytes(BITS);
     // Two codes that sit at bit f of bytes 0 and 2 of `bytes` -> fp16 pair: (1024 + c 2^f) 2^-f - 1024 2^-f = c, one
-    // fused multiply-add (exact: c 2^f < 1024); mul = 2^-f and add = -2^(10 - f) in both halves.  3 bits: `high` holds the
-    // codes' third bits, already at bit f + 2 of each half.
+    // fused multiply-add (exact: c 2^f < 1024); mul = 2^-f and add = -2^(10 - f) in both halves.  `high` holds fp16's
+    // 1024 in both halves and, at 3 bits, the codes' third bits at bit f + 2 of each.
     auto field_h2 = [](const unsigned bytes, const unsigned mask, const unsigned high, const unsigned mul, const unsigned add) {
         const unsigned w = (bytes & mask) | high;
         const __half2 hv = __hfma2(*reinterpret_cast<const __half2*>(&w), *reinterpret_cast<const __half2*>(&mul),
@@ -772,7 +772,7 @@ __device__ __forceinline__ void unpack_page(const unsigned char* raw, unsigned c
         const int g = p & 7, s = (p >> 3) & 3, bi = p >> 5;
         const unsigned char* src = raw + bi * CB + (TWO ? 0 : 512 * (s >> 1)) + 64 * g;
         const int sh0 = TWO ? 2 * s : 4 * (s & 1);
-        const unsigned kmask = MASK2 << sh0, kmul = pow2_neg(sh0), kadd = bias_neg(sh0), khigh = 0x00010001u << (sh0 + 2);
+        const unsigned kmask = MASK2 << sh0, kmul = pow2_neg(sh0), kadd = bias_neg(sh0);
         unsigned w[4][4];                                   // [t][j]
         unsigned wh[4][2];                                  // 3 bits: [t][rs], bit 2 s + hh of byte b
 #pragma unroll
@@ -811,10 +811,7 @@ __device__ __forceinline__ void unpack_page(const unsigned char* raw, unsigned c
 #pragma unroll
                 for (int t = 0; t < 4; ++t) {
                     // bytes 2 b1 and 2 b1 + 1 of the word to bytes 0 and 2, then the thread's field of each
-                    unsigned high = 0x64006400u;
-                    if constexpr (BITS == 3)            // the same bytes of the 1-bit plane: bit 2 s + hh of each goes to bit 2 s + 2
-                        high = (__byte_perm(wh[t][j & 1], 0u, b1 ? 0x4342u : 0x4140u) << (2 - (j >> 1))) & khigh | 0x64006400u;
-                    out[t] = field_h2(__byte_perm(w[t][j], 0u, b1 ? 0x4342u : 0x4140u), kmask, high, kmul, kadd);
+                    out[t] = field_h2(__byte_perm(w[t][j], 0u, b1 ? 0x4342u : 0x4140u), kmask, 0x64006400u, kmul, kadd);
                 }
                 *reinterpret_cast<uint4*>(sK + (2 * bi + (j & 1)) * 2048 + (4 * s + 2 * (j >> 1) + b1) * 128 + g * 16) =
                     make_uint4(out[0], out[1], out[2], out[3]);
@@ -1284,7 +1281,7 @@ enum { WB_KFULL = 0, WB_KEMPTY = WB_KFULL + WS_KS, WB_VFULL = WB_KEMPTY + WS_KS,
        WB_STAGED, WB_DRAIN, WB_RAWFREE, WB_COUNT = WB_RAWFREE + 2 };
 // The rest of the layout depends on the record size.  Per-key factors of a packed tile, per value stage: the steps, then the
 // offsets, of the key side for the 64 keys as fp32 (the softmax threads load them ready for two-lane instructions, four keys per 16 bytes; with
-// pairs of (step, offset) and one lane 2048 tokens on 8 x 32k took 11.74 ms, so 11.39).
+// pairs of (step, offset) and one lane 2048 tokens on 8 x 32k took 11.78 ms, so 11.44).
 __host__ __device__ constexpr int ws_meta_stage(int) { return TN * 8; }
 __host__ __device__ constexpr int ws_off_meta(int bits) { return WS_OFF_RAW + 2 * record_bytes(bits); }
 __host__ __device__ constexpr int ws_off_live(int bits) { return ws_off_meta(bits) + WS_VS * ws_meta_stage(bits); }      // uint2[WS_VS]: which keys of a packed tile exist
@@ -1547,7 +1544,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) prefill_attn_ws_kernel(PrefillP
     auto bar = [&](int i) -> unsigned { return bar0 + 8u * static_cast<unsigned>(i); };
     unsigned* tmem_slot = reinterpret_cast<unsigned*>(sm_ws + ws_off_misc(BITS));
     volatile int* abort_flag = reinterpret_cast<volatile int*>(sm_ws + ws_off_misc(BITS) + 4);
-    unsigned char* meta_all = sm_ws + ws_off_meta(BITS);         // [stage][key side, value side][key]: (step, offset)
+    unsigned char* meta_all = sm_ws + ws_off_meta(BITS);         // [stage][step, offset][key], fp32
     uint2* live_all = reinterpret_cast<uint2*>(sm_ws + ws_off_live(BITS));
 
     if (warp == 0) {

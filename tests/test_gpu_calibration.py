@@ -22,7 +22,7 @@ def test_gram_accumulation_matches_the_oracle_over_several_sequences():
     M = torch.zeros((n_kv, 128, 128), dtype=torch.float64, device="cuda")
     H = torch.zeros_like(M)
     Mo, Ho = np.zeros((n_kv, 128, 128)), np.zeros((n_kv, 128, 128))
-    for n_tok in (3000, 1, 2048, 77):                      # more than one slice, a single token, exactly one slice, a ragged tile
+    for n_tok in (3000, 1, 2048, 77):                      # several groups of 128 tokens with a ragged end, a single token, whole groups, less than a group
         pos = np.arange(n_tok)
         K = wl._keys(rng, pos)
         Q = wl._queries(rng, pos)

@@ -1,5 +1,5 @@
 """The calibration kernels at the edges of their tiles: groups of 128 tokens and matrices that end within a thread block's part of the
-list, one head and more heads than there are clusters at a time."""
+list, parts of the list that go round the rings of tiles and accumulators, one head and more heads than there are clusters at a time."""
 import numpy as np
 import pytest
 
@@ -55,3 +55,32 @@ def test_gram_without_tensor_maps_sums_the_same(n_tok, n_q, n_kv, test_option):
         sums.append((M, H))
     for a, b in zip(*sums):
         assert (a - b).abs().max().item() <= 148 * 2.0 ** -52 * a.abs().max().item()
+
+
+@pytest.mark.parametrize("n_tok,n_q,n_kv", [(32768 + 77, 32, 8), (65537, 7, 1), (9000, 24, 24)])
+def test_gram_goes_round_its_rings(n_tok, n_q, n_kv):
+    """69, 27 and 23 tiles per thread block on 148 SMs, with six places for tiles and four accumulators: every place is filled again and
+    again, matrices change within a block's part, the last tile is ragged.  Bound as above."""
+    import torch
+    from paper_2609_38121_b200 import binding as B
+    gen = torch.Generator(device="cuda").manual_seed(8)
+    K, Q = (torch.randn((n_tok, n, 128), generator=gen, device="cuda").to(torch.bfloat16) for n in (n_kv, n_q))
+    M, H = (torch.zeros((n_kv, 128, 128), dtype=torch.float64, device="cuda") for _ in range(2))
+    B.accumulate_gram_device(K.view(torch.int16), Q.view(torch.int16), M, H)
+    G = n_q // n_kv
+    for h in range(n_kv):
+        k = K[:, h].double()
+        ref = k.T @ k
+        assert (M[h] - ref).abs().max().item() <= 2e-6 * ref.abs().max().item()
+        ref = sum(2 * Q[:, j].double().T @ Q[:, j].double() for j in range(h * G, (h + 1) * G))
+        assert (H[h] - ref).abs().max().item() <= 2e-6 * ref.abs().max().item()
+
+
+def test_builder_beyond_one_wave_of_clusters():
+    """About 90 clusters of eight thread blocks run at a time; 200 heads made of five: equal statistics give equal transforms, whichever
+    cluster takes them, and they are those of five heads alone."""
+    rng = np.random.default_rng(13)
+    M, H = (np.stack([_spd(rng, 2.0, 1.0) for _ in range(5)]) for _ in range(2))
+    T, Ti = _build(M, H, W.GAMMA)
+    T200, Ti200 = _build(np.tile(M, (40, 1, 1)), np.tile(H, (40, 1, 1)), W.GAMMA)
+    assert np.array_equal(T200, np.tile(T, (40, 1, 1))) and np.array_equal(Ti200, np.tile(Ti, (40, 1, 1)))
