@@ -28,9 +28,10 @@ __device__ __forceinline__ unsigned saddr(const void* p) { return static_cast<un
 // consecutive part of the list (head, tokens); where the matrix changes, and at the end, a thread adds its 64 sums to the statistics
 // with atomics (to the mirror image of their places, which makes a warp's addresses consecutive).
 // Warps 0-7: float64 sums of the 32 tensor-memory lanes that their number allows, half the columns each.  Warp 8: copies, six tiles ahead.
-// Warp 9: MMAs, into one of four accumulators.  What bounds it: the conversions to float64 and their sums, in eight warps that hold 64 of them
-// per thread.  32768 tokens of 32 / 8 heads: mma.sync with the sums in the same warps 255 us (its rate), this 92; with 32 columns
-// loaded at a time, which spills, 106.
+// Warp 9: MMAs, into one of four accumulators.  32768 tokens of 32 / 8 heads: mma.sync with the sums in the same warps 255 us (its rate),
+// this 92; with 32 columns loaded at a time, which spills, 106.  1.07 us per unit, and about 18 us for the launch and the atomics at the end.
+// No unit of the SM binds alone (timing-only variants: tiles out of the L2 92 us, half the copies 91, one MMA instead of eight or no float64
+// sums 88, both 82, all of it 80).
 constexpr int GR_TOK = 128, GR_STAGES = 6, GR_ACC = 4, GR_THREADS = 320;
 constexpr int GR_TILE_BYTES = GR_TOK * D * 2;
 constexpr size_t GRAM_SMEM = static_cast<size_t>(GR_STAGES) * GR_TILE_BYTES + 1024;      // and alignment
@@ -507,7 +508,8 @@ __device__ __forceinline__ void jacobi_rotate(double2 (&p)[4], double2 (&q)[4], 
             q[k] = make_double2(fma(tq, x.x, w.x), fma(tq, x.y, w.y));
         }
     }
-    // c = (1 + t^2)^(-1/2): an fp32 value and one step of third order, which leaves the cube of its error
+    // c = a^(-1/2), a = 1 + t^2: an fp32 value y and one step of third order, which leaves the cube of its error.  With e = 1 - a y^2,
+    // c = y (1 - e)^(-1/2), and the binomial series of that root begins 1 + e / 2 + 3 e^2 / 8.
     const double a = fma(t, t, 1.0), y = static_cast<double>(fast_rsqrt(fmaf(tf, tf, 1.f))), e = fma(-a * y, y, 1.0);
     const double c = fma(y * e, fma(0.375, e, 0.5), y), ic = a * c;
     const ColumnState np = {sp.up * c, sp.down * ic, fma(-t, g, sp.norm2), 0.0}, nq = {sq.up * c, sq.down * ic, fma(t, g, sq.norm2), 0.0};

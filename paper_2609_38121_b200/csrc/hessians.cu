@@ -12,9 +12,10 @@
 //
 // Every step is a contraction over 128 channels or over positions.  Where one operand is bf16 already and the other fp32 (or
 // both fp32), the fp32 one is split into three bf16 terms, 24 bits, and the products run on the tensor cores (mma.sync: the
-// logits of all heads and v . U of a pair meet entry by entry in one thread's accumulators, which is what the sum over s needs).
+// long sums have to be added up outside the tensor core, which cuts them towards zero, so every 16 products come back to registers).
 // 1024 tokens of 32 / 8 heads: 1343 us as register-blocked fp32 products out of shared memory, bound by fp32 issue and shared-memory
-// reads alike (pairs_kernel 626, rows_kernel 366, project_kernel 215); now 610 us (243, 96, 136), error against 64 bits 2.8e-7 -> 1e-7:
+// reads alike (pairs_kernel 626, rows_kernel 366, project_kernel 215); now 610 us (243, 96, 136).  Error of H_K against 64 bits, 2-norm, mean of five seeds:
+// 3.6e-7 -> 1.6e-7; of H_V 4.9e-8 -> 3.3e-8:
 //   gamma_kernel      Gamma_{gg'}, 128 x 128 x d_model, fp32 products, float64 across groups of 16
 //   rows_kernel       causal softmax statistics (max, 1 / sum) and head outputs o_{g,t}: 64 x 64 tiles
 //   project_kernel    U, kappa and alpha: 128 x 128 tiles
@@ -75,7 +76,7 @@ __device__ __forceinline__ void hs_mma(float (&c)[4], const unsigned (&a)[4], un
                  : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 // The tensor core cuts the sum it adds to towards zero, and over a chain of products of one sign pattern that adds up (with every sum kept
-// there the whole call's error was 2.4e-6 where fp32 products have 3e-7): long sums are added up in fp32, the tensor core
+// there H_K's error is 5.7e-7 and H_V's 2.7e-7, 2-norm, where fp32 products have 3.6e-7 and 4.9e-8; 558 us): long sums are added up in fp32, the tensor core
 // sums 16 products, or terms that are 2^-8 of the result or less.
 __device__ __forceinline__ void hs_mma_add(float (&c)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
     float d[4];
@@ -648,8 +649,8 @@ __device__ __forceinline__ void add_key_entry(const HessParams& P, int h, int i,
 // sums go to H_K, else they are left in the workspace (over U and the head outputs, which nothing reads any more) and
 // finish_kernel adds them up in the order of the slices: the same bits on every run.
 // Three CTAs per slice keep short sequences from being one CTA's chain; what bounds it is shared-memory reads and fp32 issue alike
-// (two wavefronts for eight multiply-adds per warp) and the conversions to float64.  With all 64 blocks, 512 threads, loads waited for
-// and float64 atomics the whole call took 1352 us for 1024 tokens of 32 / 8 heads and 310 us for 300 tokens of 16 / 4, now 1344 and 267.
+// (two wavefronts for eight multiply-adds per warp) and the conversions to float64: 57 us for 1024 tokens of 32 / 8 heads.  (With all 64 blocks, 512
+// threads, loads waited for and float64 atomics the whole call, then 1344 us, took 8 us more, and 310 instead of 267 us for 300 tokens of 16 / 4.)
 constexpr int KEY_SLICE = 64, KEY_BLOCKS = 36, KEY_WARPS = 12;
 __device__ __forceinline__ void key_block(int k, int& bi, int& bj) { pair_heads(k, 8, bi, bj); }
 template <int G>
